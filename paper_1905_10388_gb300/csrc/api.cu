@@ -191,6 +191,7 @@ struct Problem {
   // partitioned substitution (few pencils): blocks per pencil and the
   // inflow/outflow vectors of the blocks
   bool spike = false;
+  bool by_group = false;                     // the lane substitution serves the problem (whole or partitioned)
   int spike_blocks = 0;                      // requested (0: automatic)
   int nblk = 0, nblk_f = 0;
   double *d_sp_s0 = nullptr, *d_sp_s = nullptr, *d_sp_o0 = nullptr, *d_sp_u = nullptr;
@@ -325,10 +326,15 @@ cudaError_t reset_spike_guess(Problem* pr, cudaStream_t s) {
 // (two to four chains per GPU sub-partition with its two parts; measured at
 // 256 pencils of 1792 rows: 4 blocks 0.224 ms per solve, 7 blocks 0.254, 14
 // blocks 0.253, 28 blocks 0.274, whole pencils 0.289), each a whole number of
-// 32-row chunks and at least 64 rows.
+// 32-row chunks and at least 64 rows.  From LANE_SPLIT_PENCILS pencils on the
+// lane substitution takes them: about 1024 groups of 16 pencils x blocks, a
+// warp or two for each of the GPU's 608 sub-partitions (Fisher-KPP 2048 x
+// 1024, four steps: 512 warps 5.20 ms, 1024 4.91 ms, 2048 5.77 ms).
 int default_spike_blocks(int npad, int P) {
   const int nch = npad / SOLVE_CHUNK;
-  const int target = std::max(2, (1024 + std::max(P, 1) - 1) / std::max(P, 1));
+  const int groups = (P + LANE_GROUP - 1) / LANE_GROUP;
+  const int target = P >= LANE_SPLIT_PENCILS ? std::max(2, 1024 / groups)
+                                             : std::max(2, (1024 + std::max(P, 1) - 1) / std::max(P, 1));
   int best = 1;
   for (int nb = 2; nb <= nch / 2; ++nb)
     if (nch % nb == 0 && std::abs(nb - target) < std::abs(best - target)) best = nb;
@@ -439,15 +445,9 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
   pr->upad = kuu <= 31 ? 32 : 64;
   // SBDFq keeps q factors (its start-up orders); the Runge-Kutta schemes one
   const int nfactors = is_cnab(pr->scheme) ? 1 : std::max(1, sbdf_order(pr->scheme));
-  // thousands of pencils fill the GPU with one lane per right-hand side
+  // thousands of pencils: one lane per right-hand side, whole pencils
   pr->lanes = pr->solve_kind == SP_SOLVE_LANES ||
-              (pr->solve_kind == SP_SOLVE_AUTO && pr->P >= LANE_MIN_PENCILS && lanes_supported(pr->kl, kuu));
-  const size_t ngroups = (pr->P + LANE_GROUP - 1) / LANE_GROUP;
-  if (pr->lanes) {
-    CK(dalloc(&pr->d_bg, (size_t)pr->P * pr->n));
-    CK(dalloc(&pr->d_xg, (size_t)pr->P * pr->n));
-    CK(dalloc(&pr->d_yg, ngroups * LANE_GROUP * pr->n));
-  }
+              (pr->solve_kind == SP_SOLVE_AUTO && pr->P >= LANE_MIN_PENCILS);
   // mixed precision: the Chebyshev backward transform on the tensor cores
   // (SP_ZT_MMA, or SP_ZT_AUTO on three-dimensional problems), when its sizes fit
   pr->zmma = pr->prec == SP_PREC_MIXED && cheb_mma_supported(pr->Nz, pr->Ngz) &&
@@ -462,15 +462,14 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
   }
   // a few hundred pencils are too few chains for the GPU: cut each pencil's
   // rows into blocks substituted in parallel (spike.cu)
+  pr->by_group = pr->lanes;
   pr->nblk = pr->spike_blocks > 0 ? pr->spike_blocks : default_spike_blocks(pr->npad, pr->P);
   pr->spike = !pr->lanes && spike_supported(pr->kl, kuu, pr->npad, pr->nblk) &&
               (pr->solve_kind == SP_SOLVE_SPIKE ||
                (pr->solve_kind == SP_SOLVE_AUTO && pr->P < SPIKE_MAX_PENCILS && pr->npad >= SPIKE_MIN_ROWS));
   if (pr->spike) {
-    CK(dalloc(&pr->d_bg, (size_t)pr->P * pr->n));
-    CK(dalloc(&pr->d_xg, (size_t)pr->P * pr->n));
-    CK(dalloc(&pr->d_yg, (size_t)pr->P * pr->n));
-    pr->nblk_f = spike_forward_blocks(pr->npad);
+    pr->by_group = pr->P >= LANE_SPLIT_PENCILS;
+    pr->nblk_f = pr->by_group ? pr->nblk : spike_forward_blocks(pr->npad);
     const size_t nv = (size_t)pr->P * pr->nblk * 2, nvf = (size_t)pr->P * pr->nblk_f * 2;
     CK(dalloc(&pr->d_sp_s0, nvf * 8));
     CK(dalloc(&pr->d_sp_s, nvf * 8));
@@ -478,13 +477,17 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
     CK(dalloc(&pr->d_sp_u, nv * 32));
     CK(reset_spike_guess(pr, ctx->stream));
   }
+  if (pr->lanes || pr->spike) {
+    // by group: the rows beyond n and the last group's missing pencils stay zero
+    const size_t nv = !pr->by_group ? (size_t)pr->P * pr->n
+                                    : (size_t)((pr->P + LANE_GROUP - 1) / LANE_GROUP) * LANE_GROUP * pr->npad;
+    for (double2** v : {&pr->d_bg, &pr->d_xg, &pr->d_yg}) {
+      CK(dalloc(v, nv));
+      CK(cudaMemsetAsync(*v, 0, nv * sizeof(double2), s));
+    }
+  }
   for (int fi = 0; fi < nfactors; ++fi) {
     BandFactor& f = pr->fac[fi];
-    if (pr->lanes) {
-      CK(dalloc(&f.Lg, ngroups * pr->n * pr->kl * LANE_GROUP));
-      CK(dalloc(&f.pg, ngroups * pr->n * LANE_GROUP));
-      CK(dalloc(&f.umask, (size_t)pr->n));
-    }
     CK(dalloc(&f.L, (size_t)pr->P * pr->npad * pr->lpad));
     CK(dalloc(&f.piv, (size_t)pr->P * pr->npad));
     CK(dalloc(&f.U, (size_t)pr->P * pr->npad * pr->upad));
@@ -512,7 +515,7 @@ void free_problem(Problem* pr) {
   for (auto b : pr->d_LX) F(b);
   for (auto b : pr->d_Fc) F(b);
   F(pr->d_gz); F(pr->d_gy); F(pr->d_h);
-  for (auto& f : pr->fac) { F(f.L); F(f.piv); F(f.U); F(f.rd); F(f.Lg); F(f.Ug); F(f.pg); F(f.umask); F(f.spD); F(f.spE); }
+  for (auto& f : pr->fac) { F(f.L); F(f.piv); F(f.U); F(f.rd); F(f.spD); F(f.spE); lane_list_free(f.ll); }
   F(pr->d_bg); F(pr->d_xg); F(pr->d_yg);
   F(pr->d_sp_s0); F(pr->d_sp_s); F(pr->d_sp_o0); F(pr->d_sp_u);
   cheb_mma_free(pr->cm);
@@ -617,9 +620,8 @@ SolveArgs base_args(Problem* pr, sp_ctx* ctx, int fac) {
   a.status = ctx->d_status;
   a.xc32_out = pr->d_Xc32;   // null unless mixed precision
   a.xs32_out = pr->zmma ? pr->cm.xs32 : nullptr;
-  a.Lg = pr->fac[fac].Lg; a.Ug = pr->fac[fac].Ug; a.pg = pr->fac[fac].pg;   // null unless lane mode
-  a.cmax = pr->fac[fac].cmax;
-  a.umask = pr->fac[fac].umask;
+  a.ll = pr->by_group ? &pr->fac[fac].ll : nullptr;
+  a.by_group = pr->by_group;
   a.spD = pr->spike ? pr->fac[fac].spD : nullptr;   // null unless partitioned substitution
   a.spE = pr->spike ? pr->fac[fac].spE : nullptr;
   return a;
@@ -637,10 +639,24 @@ void set_ep_L(Problem* pr, SolveArgs& a) {
   a.ep_rows = nullptr; a.ep_nrows = 0;
 }
 
+// Arguments of the lane substitution of `pr` with the listed factor `f`.
+LaneArgs lane_args(sp_ctx* ctx, Problem* pr, const LaneList& f, int kl, int kuu) {
+  LaneArgs la{};
+  la.P = pr->P; la.n = pr->n; la.npad = pr->npad; la.kl = kl; la.kuu = kuu;
+  la.nblk = pr->spike ? pr->nblk : 1; la.m = pr->npad / la.nblk;
+  la.nblk_f = pr->spike ? pr->nblk_f : 1; la.m_f = pr->npad / la.nblk_f;
+  la.lcap = f.lcap; la.ucap = f.ucap; la.lrecs = f.lrecs; la.urecs = f.urecs;
+  la.Lv = f.Lv; la.Uv = f.Uv; la.lco = f.lco; la.uco = f.uco; la.pg = f.pg;
+  la.bg = pr->d_bg; la.yg = reinterpret_cast<double*>(pr->d_yg); la.xg = pr->d_xg;
+  la.status = ctx->d_status;
+  la.s0 = pr->d_sp_s0; la.sst = pr->d_sp_s; la.o0 = pr->d_sp_o0; la.uin = pr->d_sp_u;
+  return la;
+}
+
 sp_status solve(sp_ctx* ctx, Problem* pr, cudaStream_t s, const SolveArgs& a) {
   const bool t = pr->timing && pr->ev_used + 2 <= pr->ev.size();
   if (t) CK(cudaEventRecord(pr->ev[pr->ev_used], s));
-  if (pr->spike && a.Lf && a.Lf == pr->facT.L && pr->facT.spE && pr->d_spT_u) {
+  if (pr->spike && !a.by_group && a.Lf && a.Lf == pr->facT.L && pr->facT.spE && pr->d_spT_u) {
     // transposed solve: assembly and whole-row forward substitution (mode 3),
     // partitioned back substitution from the last transposed solve's inflows,
     // epilogue
@@ -665,14 +681,24 @@ sp_status solve(sp_ctx* ctx, Problem* pr, cudaStream_t s, const SolveArgs& a) {
     }
     return SP_OK;
   }
-  if ((a.Lg && pr->lanes) || (a.spD && pr->spike)) {
-    // assembly -> lane-per-pencil or partitioned substitution -> epilogue
+  if (a.ll || (a.spD && pr->spike)) {
+    // assembly -> lane substitution (whole or partitioned) or partitioned
+    // window substitution -> epilogue
     SolveArgs a1 = a;
     a1.mode = 1; a1.bg = pr->d_bg;
     CK(launch_pencil_solve(s, a1));
     if (pr->lanes) {
-      CK(launch_pencil_lanes(s, pr->P, pr->n, a.kl, a.kuu, a.Lg, a.Ug, a.cmax, a.pg, a.umask, pr->d_bg,
-                             pr->d_yg, pr->d_xg));
+      const LaneArgs la = lane_args(ctx, pr, *a.ll, a.kl, a.kuu);
+      CK(launch_lane_forward(s, la, 0));
+      CK(launch_lane_backward(s, la, 0));
+    } else if (pr->by_group) {
+      const LaneArgs la = lane_args(ctx, pr, *a.ll, a.kl, a.kuu);
+      CK(launch_lane_forward(s, la, 1));
+      CK(launch_spike_forward_rec(s, la, a.spD));
+      CK(launch_lane_forward(s, la, 2));
+      CK(launch_lane_backward(s, la, 1));
+      CK(launch_spike_backward_rec(s, la, a.spE));
+      CK(launch_lane_backward(s, la, 2));
     } else {
       SpikeArgs sa{};
       sa.P = pr->P; sa.n = pr->n; sa.npad = pr->npad; sa.kl = a.kl; sa.kuu = a.kuu; sa.lpad = a.lpad;
@@ -871,7 +897,7 @@ SolveArgs transposed_args(Problem* pr, sp_ctx* ctx) {
   a.n_nl = 0; a.nbc = 0; a.bc_coef = 0.0;
   a.xc32_out = nullptr;
   a.xs32_out = nullptr;
-  a.Lg = nullptr; a.Ug = nullptr; a.pg = nullptr; a.umask = nullptr;
+  a.ll = nullptr; a.by_group = 0;
   a.spD = nullptr; a.spE = nullptr;      // no coupling matrices for the transposed factor
   a.ep_rows = nullptr; a.ep_nrows = 0;   // the transposed patterns carry no row list
   return a;
@@ -1302,39 +1328,13 @@ static sp_status factor_matrices(sp_ctx* ctx, Problem* pr, int nf, const double 
     if (e != cudaSuccess) { cudaFree(work); CK(e); }
     if (pr->spike) {
       e = launch_spike_coupling(ctx->stream, pr->P, pr->npad, pr->nblk_f, pr->nblk, pr->kl, pr->kl + pr->ku,
-                                pr->lpad, pr->upad, pr->fac[f]);
+                                pr->lpad, pr->upad, pr->fac[f], pr->by_group);
       if (e != cudaSuccess) { cudaFree(work); CK(e); }
     }
-    if (pr->lanes) {
-      // lane layout: the union pattern of U over pencils, then the copy with
-      // only the listed entries
+    if (pr->by_group) {
       BandFactor& bf = pr->fac[f];
-      e = cudaMemsetAsync(bf.umask, 0, (size_t)pr->n * sizeof(unsigned long long), ctx->stream);
-      if (e == cudaSuccess)
-        e = launch_u_mask(ctx->stream, pr->P, pr->n, pr->npad, pr->kl + pr->ku, pr->upad, bf.U, bf.umask);
-      std::vector<unsigned long long> hm(pr->n);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(hm.data(), bf.umask, hm.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                            ctx->stream);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-      if (e != cudaSuccess) { cudaFree(work); CK(e); }
-      int cmax = 1;
-      double listed = 0;
-      for (unsigned long long m : hm) {
-        cmax = std::max(cmax, __builtin_popcountll(m));
-        listed += __builtin_popcountll(m) - 1;
-      }
-      bf.u_listed = listed / pr->n;
-      if (cmax != bf.cmax || !bf.Ug) {
-        if (bf.Ug) cudaFree(bf.Ug);
-        bf.Ug = nullptr;
-        const size_t ngroups = (pr->P + LANE_GROUP - 1) / LANE_GROUP;
-        e = cudaMalloc((void**)&bf.Ug, ngroups * pr->n * cmax * LANE_GROUP * sizeof(double));
-        if (e != cudaSuccess) { cudaFree(work); CK(e); }
-        bf.cmax = cmax;
-      }
-      e = launch_factor_relayout(ctx->stream, pr->P, pr->n, pr->npad, pr->kl, pr->kl + pr->ku, pr->lpad, pr->upad,
-                                 bf);
+      e = lane_list_build(ctx->stream, pr->P, pr->n, pr->npad, pr->kl, pr->kl + pr->ku, pr->lpad, pr->upad, bf.L,
+                          bf.piv, bf.U, bf.ll);
       if (e != cudaSuccess) { cudaFree(work); CK(e); }
     }
   }
@@ -1881,7 +1881,7 @@ sp_status sp_adjoint_init(sp_ctx* ctx, int problem) {
   // solves' (kl' + ku' = kl + ku); their forward substitution stays whole-row,
   // since kl' = ku is wider than the partitioned forward windows
   const int kuuT = pr->klT + pr->kuT;
-  if (pr->spike && pr->upad == 32 && spike_bwd_supported(kuuT, pr->npad, pr->nblk)) {
+  if (pr->spike && !pr->by_group && pr->upad == 32 && spike_bwd_supported(kuuT, pr->npad, pr->nblk)) {
     if (!pr->facT.spE) CK(dalloc(&pr->facT.spE, (size_t)pr->P * pr->nblk * kuuT * 32));
     if (!pr->d_spT_u) CK(dalloc(&pr->d_spT_u, (size_t)pr->P * pr->nblk * 2 * 32));
     CK(cudaMemsetAsync(pr->d_spT_u, 0, (size_t)pr->P * pr->nblk * 2 * 32 * sizeof(double), s));
@@ -2225,7 +2225,7 @@ sp_status sp_eig_target(sp_ctx* ctx, int problem, double sigma_t, int iters, con
   a.mv_x = x; a.mv_coef = 1.0; a.mv_store = nullptr;
   set_mv_M(pr, a);
   a.xt_out = y; a.xc_out = nullptr; a.xc32_out = nullptr; a.ep_mv_vals = nullptr;
-  a.Lg = nullptr; a.Ug = nullptr; a.pg = nullptr; a.umask = nullptr;
+  a.ll = nullptr; a.by_group = 0;
   for (int k = 0; e == cudaSuccess && k < iters; ++k) {
     e = launch_pencil_solve(s, a);
     if (e == cudaSuccess) e = launch_eig_update(s, pr->P, pr->n, x, y, mu);
@@ -2361,9 +2361,9 @@ sp_status sp_get_solve_work(sp_ctx* ctx, int problem, double* fma_per_row, doubl
   const BandFactor& f = pr->fac[pr->nfac - 1];
   const double n = pr->n, kl = pr->kl, kuu = pr->kl + pr->ku;
   double fma, bytes;
-  if (pr->lanes) {
-    fma = kl + f.u_listed;
-    bytes = n * (kl + f.cmax) * 8.0 + n;
+  if (pr->by_group) {
+    fma = f.ll.l_listed + f.ll.u_listed;
+    bytes = n * (fma + 1) * 8.0 + n;
   } else {
     fma = kl + kuu;
     bytes = n * (kl + kuu + 1) * 8.0 + n;

@@ -324,11 +324,21 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
   //      left-preconditioned F~ (T-to-U conversion, tau rows dropped) and
   //      boundary values
   const size_t prow = (size_t)pp * n;
+  // element r of this pencil in the substitution kernels' vectors
+  const size_t v0 = a.by_group ? lane_index(pp, 0, a.npad) : prow;
+  const int vstep = a.by_group ? LANE_GROUP : 1;
+  auto vec = [&](int r) { return v0 + (size_t)r * vstep; };
   const int Nz = a.Nz;
   const float invNz = 1.0f / (float)Nz;
   if (mode == 2) {
-    // epilogue only: X~ (already divided by U_jj) from the substitution kernel
-    for (int r = tid; active && r < n; r += nt) sm.B[r] = a.xg[prow + r];
+    // epilogue only: X~ from the substitution kernel, as b = U_jj X~ by group
+    // from the lane substitution
+    const double* rdp = a.rd + (size_t)pp * a.npad;
+    for (int r = tid; active && r < n; r += nt) {
+      const double2 b = a.xg[vec(r)];
+      const double rd = a.by_group ? rdp[r] : 1.0;
+      sm.B[r] = a.by_group ? make_double2(b.x * rd, b.y * rd) : b;
+    }
     __syncthreads();
   } else {
   // modes 0 and 1: two passes over the rows, each with every lane on the
@@ -391,7 +401,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
   }
   __syncthreads();
   if (mode == 1) {
-    for (int r = tid; active && r < n; r += nt) a.bg[prow + r] = sm.B[r];   // B~ for the substitution kernel
+    for (int r = tid; active && r < n; r += nt) a.bg[vec(r)] = sm.B[r];   // B~ for the substitution
     return;
   }
   }
@@ -586,7 +596,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
   const bool work = active && !*sm.abort_flag;
   if (mode == 3) {
     // y = L^-1 P B~ for the partitioned back substitution
-    for (int r = tid; work && r < n; r += nt) a.yg[prow + r] = sm.B[r];
+    for (int r = tid; work && r < n; r += nt) a.yg[vec(r)] = sm.B[r];
     return;
   }
 
@@ -625,7 +635,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
       for (int r = tid; work && r < n; r += nt) {
         double2 s = make_double2(0.0, 0.0);
         if (mode == 2 && a.ep_from_b != 0.0) {
-          const double2 bb = a.bg[prow + r];
+          const double2 bb = a.bg[vec(r)];
           s.x = bb.x * a.ep_from_b;
           s.y = bb.y * a.ep_from_b;
         }
@@ -650,7 +660,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
       }
       if (mode == 2 && a.ep_from_b != 0.0) {
         // L~ X~ = (B~ - alpha M~ X~) / beta for the stage matrix alpha M~ + beta L~
-        const double2 bb = a.bg[prow + r];
+        const double2 bb = a.bg[vec(r)];
         s.x = (bb.x - a.ep_alpha * s.x) * a.ep_from_b;
         s.y = (bb.y - a.ep_alpha * s.y) * a.ep_from_b;
       }
@@ -776,294 +786,8 @@ cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
   return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------------------
-// Lane-per-pencil substitution for problems with many pencils (3D): the
-// window kernel above keeps one pencil's band across a warp's lanes, which
-// leaves most lanes idle in the forward pass (kl of 32) and, with two window
-// registers, in the back substitution (kl + ku of 64); it is the right shape
-// when a few hundred dependent chains cannot fill the GPU anyway.  With tens
-// of thousands of pencils the FP64 pipe is the limit instead, so here each
-// lane carries one real right-hand side (lane 2i: real part, 2i + 1:
-// imaginary part of pencil i of a group of LANE_GROUP) through the whole
-// substitution with its window of pending rows in registers; every warp
-// FMA does useful work on all 32 lanes.  The factor is stored interleaved
-// by pencil within a group, so a warp's load of one factor entry reads 16
-// consecutive doubles.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait2() { asm volatile("cp.async.wait_group 2;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Rows staged ahead in the lane substitution: LANE_BUFS buffers, the copy
-// of row j + LANE_BUFS - 1 in flight while row j is used
-constexpr int LANE_BUFS = 3;
-
-// doubles of shared memory per warp: LANE_BUFS forward buffers (multipliers
-// and pivots) or LANE_BUFS backward buffers (listed U entries), whichever is
-// larger
-__host__ __device__ inline int lane_stride(int kl, int cmax) {
-  const int fw = LANE_BUFS * (kl * LANE_GROUP + 2), bw = LANE_BUFS * cmax * LANE_GROUP;
-  return fw > bw ? fw : bw;
-}
-
-template <int KL, int KUU>
-__global__ void __launch_bounds__(128) k_pencil_lanes(int P, int n, int cmax, const double* __restrict__ Lg,
-                                                      const double* __restrict__ Uc,
-                                                      const uint8_t* __restrict__ pg,
-                                                      const unsigned long long* __restrict__ umask,
-                                                      const double2* __restrict__ b, double2* __restrict__ y,
-                                                      double2* __restrict__ x) {
-  extern __shared__ __align__(16) double lane_stage[];   // [warp][2][cmax][LANE_GROUP]
-  const int gl = blockIdx.x * blockDim.x + threadIdx.x;
-  const int comp = gl & 1;
-  const int pen = gl >> 1;                       // pencil; a warp holds the 16 pencils of one group
-  const bool act = pen < P;                      // idle lanes of the last group keep the warp's rhythm
-  const int g = pen / LANE_GROUP, i = pen - g * LANE_GROUP;
-  if (g * LANE_GROUP >= P) return;               // a whole warp past the last group (no storage there)
-  const int lane = threadIdx.x & 31;
-  const double* bp = reinterpret_cast<const double*>(b + (size_t)(act ? pen : 0) * n) + comp;
-  double* yp = reinterpret_cast<double*>(y + (size_t)g * n * LANE_GROUP + i) + comp;   // row j at yp[2 j LANE_GROUP]
-  const size_t gn = (size_t)g * n;
-  // per-warp staging area (lane_stride doubles): forward rows, then backward rows
-  double* st = lane_stage + (size_t)(threadIdx.x >> 5) * lane_stride(KL, cmax);
-  // forward: row interchanges and unit-lower multipliers; win[t] = row j + t.
-  // Each row's multipliers and pivot offsets for the warp's 16 pencils are
-  // copied into shared memory two rows ahead (cp.async, three buffers).
-  constexpr int FW = KL * LANE_GROUP + 2;        // doubles per forward buffer (+16 bytes of pivots)
-  auto fstage = [&](int jr) {
-    const double* src = Lg + (gn + jr) * KL * LANE_GROUP;
-    double* dst = st + (jr % LANE_BUFS) * FW;
-    for (int c = lane; c < KL * (LANE_GROUP / 2); c += 32) cp_async16(dst + 2 * c, src + 2 * c);
-    if (lane == 31) cp_async16(dst + KL * LANE_GROUP, pg + (gn + jr) * LANE_GROUP);
-    cp_async_commit();
-  };
-  {
-    double win[KL + 1];
-#pragma unroll
-    for (int t = 0; t <= KL; ++t) win[t] = (act && t < n) ? bp[2 * t] : 0.0;
-    fstage(0);
-    if (n > 1) fstage(1);
-    else cp_async_commit();
-    for (int j = 0; j < n; ++j) {
-      if (j + 2 < n) fstage(j + 2);
-      else cp_async_commit();                    // one group per row keeps wait_group 2 exact
-      cp_async_wait2();
-      __syncwarp();
-      const double* Ls = st + (j % LANE_BUFS) * FW;
-      const int off = reinterpret_cast<const uint8_t*>(Ls + KL * LANE_GROUP)[i];
-      const double* Lrow = Ls + i;
-      double piv_val = win[0];
-#pragma unroll
-      for (int t = 1; t <= KL; ++t) piv_val = (off == t) ? win[t] : piv_val;
-#pragma unroll
-      for (int t = 1; t <= KL; ++t) win[t] = (off == t) ? win[0] : win[t];
-      const double yj = piv_val;
-      yp[(size_t)2 * j * LANE_GROUP] = yj;
-#pragma unroll
-      for (int t = 1; t <= KL; ++t) win[t] = fma(-Lrow[(t - 1) * LANE_GROUP], yj, win[t]);
-#pragma unroll
-      for (int t = 0; t < KL; ++t) win[t] = win[t + 1];
-      win[KL] = (act && j + KL + 1 < n) ? bp[2 * (j + KL + 1)] : 0.0;
-      __syncwarp();                              // buffer j % 3 is refilled for row j + 3 next
-    }
-    cp_async_wait0();
-    __syncwarp();
-  }
-  // back substitution with the scaled columns U_{j-t,j} / U_jj.  Only entries
-  // nonzero in some pencil are stored: the k-th set bit t of umask[j] holds
-  // U_{j-t,j} / U_jj at Uc[g][j][k] (k = 0: 1/U_jj).  Each row's entries
-  // are copied into shared memory two rows ahead (cp.async, three buffers per
-  // warp), and only the listed entries issue an FMA: the mask is the same for
-  // the whole warp, so the loop branches (a predicated-off FP64 instruction
-  // would still hold the FP64 pipe) and jumps to the FMA of its window
-  // register.  The rows of y this lane wrote are read back by this lane only.
-  auto stage = [&](int jr) {
-    const int cnt = __popcll(umask[jr]);
-    const double* src = Uc + (gn + jr) * (size_t)cmax * LANE_GROUP;
-    double* dst = st + (jr % LANE_BUFS) * cmax * LANE_GROUP;
-    for (int c = lane; c < cnt * (LANE_GROUP / 2); c += 32) cp_async16(dst + 2 * c, src + 2 * c);
-    cp_async_commit();
-  };
-  double w[KUU + 1];                             // w[t] = pending row j - t
-#pragma unroll
-  for (int t = 0; t <= KUU; ++t) w[t] = (act && n - 1 - t >= 0) ? yp[(size_t)2 * (n - 1 - t) * LANE_GROUP] : 0.0;
-  double* xp = reinterpret_cast<double*>(x + (size_t)(act ? pen : 0) * n) + comp;
-  stage(n - 1);
-  if (n > 1) stage(n - 2);
-  else cp_async_commit();
-  for (int j = n - 1; j >= 0; --j) {
-    if (j >= 2) stage(j - 2);
-    else cp_async_commit();                      // one group per row keeps wait_group 2 exact
-    cp_async_wait2();
-    __syncwarp();
-    const double* vals = st + (j % LANE_BUFS) * cmax * LANE_GROUP + i;
-    const unsigned long long m = umask[j];
-    const double bj = w[0];
-    if (act) xp[2 * j] = bj * vals[0];
-    unsigned long long mm = m & ~1ull;
-    int k = 1;
-    while (mm) {
-      const int t = __ffsll((long long)mm) - 1;
-      mm &= mm - 1;
-      const double ut = vals[(k++) * LANE_GROUP];
-      switch (t) {
-#define SP_LANE_CASE(T)                          \
-  case T:                                        \
-    if (T <= KUU) w[T] = fma(-ut, bj, w[T]);    \
-    break;
-        SP_LANE_CASE(1)
-        SP_LANE_CASE(2)
-        SP_LANE_CASE(3)
-        SP_LANE_CASE(4)
-        SP_LANE_CASE(5)
-        SP_LANE_CASE(6)
-        SP_LANE_CASE(7)
-        SP_LANE_CASE(8)
-        SP_LANE_CASE(9)
-        SP_LANE_CASE(10)
-        SP_LANE_CASE(11)
-        SP_LANE_CASE(12)
-        SP_LANE_CASE(13)
-        SP_LANE_CASE(14)
-        SP_LANE_CASE(15)
-        SP_LANE_CASE(16)
-        SP_LANE_CASE(17)
-        SP_LANE_CASE(18)
-        SP_LANE_CASE(19)
-        SP_LANE_CASE(20)
-        SP_LANE_CASE(21)
-        SP_LANE_CASE(22)
-        SP_LANE_CASE(23)
-        SP_LANE_CASE(24)
-        SP_LANE_CASE(25)
-        SP_LANE_CASE(26)
-        SP_LANE_CASE(27)
-        SP_LANE_CASE(28)
-        SP_LANE_CASE(29)
-        SP_LANE_CASE(30)
-        SP_LANE_CASE(31)
-        SP_LANE_CASE(32)
-        SP_LANE_CASE(33)
-        SP_LANE_CASE(34)
-        SP_LANE_CASE(35)
-        SP_LANE_CASE(36)
-        SP_LANE_CASE(37)
-        SP_LANE_CASE(38)
-        SP_LANE_CASE(39)
-        SP_LANE_CASE(40)
-        SP_LANE_CASE(41)
-        SP_LANE_CASE(42)
-        SP_LANE_CASE(43)
-        SP_LANE_CASE(44)
-        SP_LANE_CASE(45)
-        SP_LANE_CASE(46)
-        SP_LANE_CASE(47)
-        SP_LANE_CASE(48)
-        SP_LANE_CASE(49)
-        SP_LANE_CASE(50)
-        SP_LANE_CASE(51)
-        SP_LANE_CASE(52)
-        SP_LANE_CASE(53)
-        SP_LANE_CASE(54)
-        SP_LANE_CASE(55)
-        SP_LANE_CASE(56)
-        SP_LANE_CASE(57)
-        SP_LANE_CASE(58)
-        SP_LANE_CASE(59)
-        SP_LANE_CASE(60)
-        SP_LANE_CASE(61)
-        SP_LANE_CASE(62)
-        SP_LANE_CASE(63)
-#undef SP_LANE_CASE
-        default:
-          break;
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < KUU; ++t) w[t] = w[t + 1];
-    const int row = j - KUU - 1;
-    w[KUU] = (act && row >= 0) ? yp[(size_t)2 * row * LANE_GROUP] : 0.0;
-    __syncwarp();                                // buffer j % 3 is refilled for row j - 3 next
-  }
-  cp_async_wait0();
-}
-
+// bands for which the lane substitution can be asked for by name
 bool lanes_supported(int kl, int kuu) { return (kl == 9 && kuu == 38) || (kl == 7 && kuu == 29); }
-
-cudaError_t launch_pencil_lanes(cudaStream_t s, int P, int n, int kl, int kuu, const double* Lg, const double* Uc,
-                                int cmax, const uint8_t* pg, const unsigned long long* umask, const double2* b,
-                                double2* y, double2* x) {
-  const int threads = 2 * P;
-  const int grid = (threads + 127) / 128;
-  const size_t smem = (size_t)4 * lane_stride(kl, cmax) * sizeof(double);
-  cudaError_t e = cudaSuccess;
-  if (kl == 9 && kuu == 38) {
-    if ((e = cudaFuncSetAttribute(k_pencil_lanes<9, 38>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) ==
-        cudaSuccess)
-      k_pencil_lanes<9, 38><<<grid, 128, smem, s>>>(P, n, cmax, Lg, Uc, pg, umask, b, y, x);
-  } else if (kl == 7 && kuu == 29) {
-    if ((e = cudaFuncSetAttribute(k_pencil_lanes<7, 29>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) ==
-        cudaSuccess)
-      k_pencil_lanes<7, 29><<<grid, 128, smem, s>>>(P, n, cmax, Lg, Uc, pg, umask, b, y, x);
-  } else {
-    return cudaErrorInvalidValue;
-  }
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
-}
-
-__global__ void k_u_mask(int P, int n, int npad, int kuu, int upad, const double* __restrict__ U,
-                         unsigned long long* __restrict__ umask) {
-  const size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (idx >= (size_t)P * n) return;
-  const int p = (int)(idx / n), j = (int)(idx - (size_t)p * n);
-  const double* col = U + ((size_t)p * npad + j) * upad;
-  unsigned long long m = 1ull;
-  for (int t = 1; t <= kuu; ++t)
-    if (col[t] != 0.0) m |= 1ull << t;
-  if ((m & ~umask[j]) != 0ull) atomicOr(umask + j, m);
-}
-
-cudaError_t launch_u_mask(cudaStream_t s, int P, int n, int npad, int kuu, int upad, const double* U,
-                          unsigned long long* umask) {
-  if (kuu > 63) return cudaErrorInvalidValue;
-  const size_t total = (size_t)P * n;
-  k_u_mask<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(P, n, npad, kuu, upad, U, umask);
-  return cudaGetLastError();
-}
-
-// Copy a factor into the lane layout (one thread per pencil row): dense
-// multipliers and pivots, and the U entries listed in umask[j] in order of t.
-__global__ void k_factor_relayout(int P, int n, int npad, int kl, int kuu, int lpad, int upad, int cmax,
-                                  const double* __restrict__ L, const uint8_t* __restrict__ piv,
-                                  const double* __restrict__ U, const unsigned long long* __restrict__ umask,
-                                  double* __restrict__ Lg, double* __restrict__ Uc, uint8_t* __restrict__ pg) {
-  const size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (idx >= (size_t)P * n) return;
-  const int p = (int)(idx / n), j = (int)(idx - (size_t)p * n);
-  const int g = p / LANE_GROUP, i = p - g * LANE_GROUP;
-  const size_t row = (size_t)g * n + j;
-  for (int t = 0; t < kl; ++t) Lg[(row * kl + t) * LANE_GROUP + i] = L[((size_t)p * npad + j) * lpad + t];
-  const double* col = U + ((size_t)p * npad + j) * upad;
-  const unsigned long long m = umask[j];
-  int k = 0;
-  for (int t = 0; t <= kuu && k < cmax; ++t)
-    if ((m >> t) & 1ull) Uc[(row * cmax + k++) * LANE_GROUP + i] = col[t];
-  pg[row * LANE_GROUP + i] = piv[(size_t)p * npad + j];
-}
-
-cudaError_t launch_factor_relayout(cudaStream_t s, int P, int n, int npad, int kl, int kuu, int lpad, int upad,
-                                   const BandFactor& f) {
-  const size_t total = (size_t)P * n;
-  k_factor_relayout<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(P, n, npad, kl, kuu, lpad, upad, f.cmax, f.L,
-                                                                   f.piv, f.U, f.umask, f.Lg, f.Ug, f.pg);
-  return cudaGetLastError();
-}
 
 // ---------------------------------------------------------------------------
 // state conversion and Chebyshev derivative (set-up kernels)

@@ -16,6 +16,32 @@ namespace spectau {
 constexpr int SOLVE_CHUNK = 32;
 constexpr int SOLVE_RING = 2;
 
+// Pencils per warp in the lane-per-right-hand-side substitution (two lanes
+// each: real and imaginary part).
+constexpr int LANE_GROUP = 16;
+// Its right-hand sides are stored by group, [G][npad][16] complex: element (p, r).
+__host__ __device__ inline size_t lane_index(int p, int r, int npad) {
+  return ((size_t)(p / LANE_GROUP) * npad + r) * LANE_GROUP + p % LANE_GROUP;
+}
+
+// A factor's entries listed for the lane substitution (lanes.cu), by groups of
+// LANE_GROUP pencils (G of them), 16 values per entry.
+struct LaneList {
+  // records of two entries: [16 pencils][2] values, the byte offsets of their
+  // rows in the shared-memory ring (bit 0 of the second: the row's last record)
+  double* Lv = nullptr;         // [G][lcap]  multipliers, rows rising, band offset rising
+  double* Uv = nullptr;         // [G][ucap]  scaled U entries, rows falling, offset falling
+  uint32_t* lmask = nullptr;    // [G][npad] bit t: L_{j+t,j} listed
+  unsigned long long* umask = nullptr;   // [G][npad] bit t: U_{j,j+t} listed
+  int32_t* lco = nullptr;       // [G][npad/4 + 1] first record of each four-row chunk
+  int32_t* uco = nullptr;
+  uint16_t* pg = nullptr;       // [G][npad][16] the pivot row's byte offset in the ring
+  int32_t* tot = nullptr;       // [G][4] record counts (lane_list_build's scratch)
+  int lcap = 0, ucap = 0;       // records allocated per group
+  int lrecs = 0, urecs = 0;     // most records of a four-row chunk
+  double l_listed = 0, u_listed = 0;     // mean entries per row, pads included
+};
+
 // Banded LU factors of one matrix a*M~ + b*L~ for all pencils.
 struct BandFactor {
   double alpha = 0, beta = 0;   // A = alpha M~ + beta L~
@@ -23,17 +49,35 @@ struct BandFactor {
   uint8_t* piv = nullptr;       // [P][npad]        pivot row offset (piv - j) in [0, kl]
   double* U = nullptr;          // [P][npad][upad]  t=0: 1/U_jj, t>=1: U_{j-t,j}/U_jj
   double* rd = nullptr;         // [P][npad]        1/U_jj (0 on padding columns)
-  // lane-interleaved copies for k_pencil_lanes (groups of LANE_GROUP pencils):
-  double* Lg = nullptr;         // [G][n][kl][16]
-  double* Ug = nullptr;         // [G][n][cmax][16]  the listed U entries of column j (k = 0: 1/U_jj)
-  int cmax = 0;                 // most entries listed for one column
-  double u_listed = 0;          // mean listed entries per column, the diagonal excluded
-  uint8_t* pg = nullptr;        // [G][n][16]
-  unsigned long long* umask = nullptr;   // [n] bit t: U_{j-t,j} != 0 in some pencil (bit 0 set)
   // partitioned substitution (spike.cu): coupling matrices of the row blocks
   double* spD = nullptr;        // [P][nblk_f][7][8]   forward window after a block from the window before
   double* spE = nullptr;        // [P][nblk][kuu][32]  back-substitution outflow from the inflow
+  LaneList ll;                  // lists of the lane substitution (whole or partitioned)
 };
+
+// Lane substitution of one problem's pencils, whole (nblk = nblk_f = 1) or in
+// row blocks.
+struct LaneArgs {
+  int P, n, npad, kl, kuu;
+  int nblk, m, nblk_f, m_f;     // blocks per pencil and their rows, back and forward
+  int lcap, ucap, lrecs, urecs;
+  const double* Lv; const double* Uv;
+  const int32_t* lco; const int32_t* uco;
+  const uint16_t* pg;
+  // right-hand sides by group, [G][npad][16 pencils] complex, zero beyond n
+  const double2* bg;            // B~
+  double* yg;                   // y = L^-1 P B~
+  double2* xg;                  // b = U_jj x~
+  double* s0; double* sst;      // forward outflows / inflows [p][nblk_f][2][8]
+  double* o0; double* uin;      // backward outflows / inflows [p][nblk][2][32]
+  DevStatus* status;
+};
+// pass 0: whole pencils; 1: blocks from zero / guessed inflows; 2: from the true ones
+cudaError_t launch_lane_forward(cudaStream_t s, const LaneArgs& a, int pass);
+cudaError_t launch_lane_backward(cudaStream_t s, const LaneArgs& a, int pass);
+cudaError_t lane_list_build(cudaStream_t s, int P, int n, int npad, int kl, int kuu, int lpad, int upad,
+                            const double* L, const uint8_t* piv, const double* U, LaneList& f);
+void lane_list_free(LaneList& f);
 
 // Partitioned substitution of problems with few pencils (spike.cu).
 struct SpikeArgs {
@@ -50,16 +94,22 @@ struct SpikeArgs {
   DevStatus* status;
 };
 // Problems with fewer pencils than this (and kl <= 7, kl + ku <= 31, at
-// least SPIKE_MIN_ROWS rows) use the partitioned substitution by default.
-constexpr int SPIKE_MAX_PENCILS = 608;
+// least SPIKE_MIN_ROWS rows) use the partitioned substitution by default,
+// from LANE_SPLIT_PENCILS pencils on in its lane form (Fisher-KPP 2048 x 1024,
+// 1024 pencils: 0.41 ms per solve against 0.78 ms with the window kernel; with
+// 256 pencils of 2D Rayleigh-Benard the window form's passes over fewer,
+// longer blocks are the faster ones, 0.17 against 0.21 ms).
+constexpr int SPIKE_MAX_PENCILS = 4096;
+constexpr int LANE_SPLIT_PENCILS = 608;
 constexpr int SPIKE_MIN_ROWS = 512;
 bool spike_supported(int kl, int kuu, int npad, int nblk);
 bool spike_bwd_supported(int kuu, int npad, int nblk);
 cudaError_t launch_spike_coupling_bwd(cudaStream_t s, int P, int npad, int nblk, int kuu, int upad, const double* U,
                                       double* E);
-cudaError_t launch_spike_backward(cudaStream_t st, const SpikeArgs& s);
 cudaError_t launch_spike_coupling(cudaStream_t s, int P, int npad, int nblk_f, int nblk, int kl, int kuu, int lpad,
-                                  int upad, const BandFactor& f);
+                                  int upad, const BandFactor& f, bool by_row);
+cudaError_t launch_spike_backward(cudaStream_t st, const SpikeArgs& s);
+cudaError_t launch_spike_solve(cudaStream_t s, const SpikeArgs& a);
 // forward blocks of the partitioned substitution: 128 rows, or 64 or 32 when
 // those divide the padded rows
 inline int spike_forward_blocks(int npad) {
@@ -67,14 +117,15 @@ inline int spike_forward_blocks(int npad) {
     if (npad % m == 0) return npad / m;
   return 1;
 }
-cudaError_t launch_spike_solve(cudaStream_t s, const SpikeArgs& a);
+cudaError_t launch_spike_forward_rec(cudaStream_t s, const LaneArgs& a, const double* D);
+cudaError_t launch_spike_backward_rec(cudaStream_t s, const LaneArgs& a, const double* E);
 
-// Pencils per warp in the lane-per-pencil substitution (two lanes each:
-// real and imaginary part).
-constexpr int LANE_GROUP = 16;
-// Problems with at least this many pencils use the lane-per-pencil
-// substitution (2 P lanes = P / 16 warps: several per SM).
-constexpr int LANE_MIN_PENCILS = 4096;
+// Problems with at least this many pencils use the lane substitution on whole
+// pencils.  Its time is the chain's (about 0.93 us per row and solve) up to
+// 608 groups, the window kernel's grows with the pencils: 288 rows of 3D
+// Rayleigh-Benard take 0.27 ms against 0.17 ms for 1024 pencils and 0.34 ms
+// for 2048.
+constexpr int LANE_MIN_PENCILS = 2048;
 
 // Chebyshev backward transform on the tensor cores (chebmma.cu): the split
 // FP32 copy of the coefficients it reads, the transform matrix halves, and
@@ -159,7 +210,7 @@ struct SolveArgs {
   const int32_t* bc_rows; const double2* bc_values;
   DevStatus* status;
   // mode 0: assembly, substitution and epilogue in one kernel; 1: assembly
-  // only, B~ to bg [p][n]; 2: epilogue only, from xg [p][n] (x~ = y / U_jj)
+  // only, B~ to bg; 2: epilogue only, from xg; [p][n] or by group
   // (the substitution then runs in k_pencil_lanes or the partitioned
   // kernels); 3: assembly and forward substitution, y = L^-1 P B~ to yg
   // [p][n] (the partitioned back substitution follows)
@@ -170,8 +221,10 @@ struct SolveArgs {
   // FP64 pipe, sets it; a lone problem's whole-row chains are bound by their
   // latency and keep a 32-lane window per part)
   int fwd16;
-  // factor in the lane-interleaved layout (null: not available)
-  const double* Lg; const double* Ug; const uint8_t* pg; const unsigned long long* umask; int cmax;
+  // the factor's lists (host pointer; null: no lane substitution); by_group:
+  // bg, xg and yg are stored by group, xg holds b = U_jj x~
+  const LaneList* ll;
+  int by_group;
   // coupling matrices of the partitioned substitution (null: not available)
   const double* spD; const double* spE;
 };
@@ -243,20 +296,7 @@ size_t pencil_solve_smem(int npad, int lpad, int upad);
 // batched pencil solves: one CTA per (problem, pencil) work item
 cudaError_t launch_pencil_solve_batched(cudaStream_t s, const SolveArgs* args, const int4* work, int nwork,
                                         int max_kuu, size_t smem);
-// Lane-per-pencil substitution (many-pencil problems): forward and back
-// substitution of P pencils, B~ [p][n] in, x~ = y / U_jj [p][n] out, y scratch
-// [G][n][16] complex.  Returns cudaErrorInvalidValue when (kl, kl + ku) has
-// no compiled instance (lanes_supported).
 bool lanes_supported(int kl, int kuu);
-cudaError_t launch_pencil_lanes(cudaStream_t s, int P, int n, int kl, int kuu, const double* Lg, const double* Uc,
-                                int cmax, const uint8_t* pg, const unsigned long long* umask, const double2* b,
-                                double2* y, double2* x);
-// umask[j] |= bit t for every t <= kuu with U_{j-t,j} != 0 in some pencil
-// (umask zeroed by the caller)
-cudaError_t launch_u_mask(cudaStream_t s, int P, int n, int npad, int kuu, int upad, const double* U,
-                          unsigned long long* umask);
-cudaError_t launch_factor_relayout(cudaStream_t s, int P, int n, int npad, int kl, int kuu, int lpad, int upad,
-                                   const BandFactor& f);
 cudaError_t launch_coef_to_solve(cudaStream_t s, int P, int S, int Nz, const double2* xc,
                                  double2* xt, const int32_t* col_map, const int32_t* var_recombine,
                                  const int32_t* var_phase);

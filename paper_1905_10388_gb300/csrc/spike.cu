@@ -51,12 +51,14 @@ constexpr int SPK_CHUNK = 32;         // U columns per bulk copy
 // factorization time: the coupling matrices, one thread per (pencil, block,
 // unit inflow).  D_k[r][i]: forward window row r after block k for window
 // row i = 1 before it (no fresh right-hand side); E_k[r][t]: backward
-// outflow r (row j0 - kuu + r) for unit inflow t (row j1 - kuu + t).  The
-// arithmetic is the substitution's own, written per row.
+// outflow r (row j0 - kuu + r) for unit inflow t (row j1 - kuu + t), or, for
+// the lane substitution (by_row), b of row j0 + r for unit b of row j1 + t.
+// The arithmetic is the substitution's own, written per row.
 // ---------------------------------------------------------------------------
 __global__ void k_spike_coupling(int P, int npad, int nblk_f, int nblk, int kl, int kuu, int lpad, int upad,
                                  const double* __restrict__ L, const uint8_t* __restrict__ piv,
-                                 const double* __restrict__ U, double* __restrict__ D, double* __restrict__ E) {
+                                 const double* __restrict__ U, double* __restrict__ D, double* __restrict__ E,
+                                 bool by_row) {
   const long long nf = (long long)P * nblk_f * SPK_FS;
   const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (idx >= nf + (long long)P * nblk * kuu) return;
@@ -86,28 +88,31 @@ __global__ void k_spike_coupling(int P, int npad, int nblk_f, int nblk, int kl, 
     const int p = (int)(jdx / ((long long)kuu * nblk));
     const int m = npad / nblk, j0 = k * m, j1 = j0 + m;
     double w[SPK_BW];                   // w[t]: pending row j - t
-    for (int t = 0; t < SPK_BW; ++t) w[t] = 0.0;
-    w[kuu - 1 - t0] = 1.0;
     const double* Up = U + (size_t)p * npad * upad;
+    double* Ek = E + ((size_t)p * nblk + k) * kuu * SPK_BW;
+    // inflow t0: partial sum of row j1 - kuu + t0, or (by_row) b of row j1 + t0
+    for (int t = 0; t < SPK_BW; ++t)
+      w[t] = by_row ? ((t0 + 1 + t <= kuu && j1 + t0 < npad) ? -Up[(size_t)(j1 + t0) * upad + t0 + 1 + t] : 0.0)
+                    : (t == kuu - 1 - t0 ? 1.0 : 0.0);
     for (int j = j1 - 1; j >= j0; --j) {
       const double bj = w[0];
+      if (by_row && j - j0 < kuu) Ek[(j - j0) * SPK_BW + t0] = bj;
       for (int t = 1; t <= kuu; ++t) w[t] = fma(-Up[(size_t)j * upad + t], bj, w[t]);
       for (int t = 0; t < SPK_BW - 1; ++t) w[t] = w[t + 1];
       w[SPK_BW - 1] = 0.0;
     }
-    double* Ek = E + ((size_t)p * nblk + k) * kuu * SPK_BW;
-    for (int r = 0; r < kuu; ++r) Ek[r * SPK_BW + t0] = w[kuu - 1 - r];
+    for (int r = 0; r < kuu && !by_row; ++r) Ek[r * SPK_BW + t0] = w[kuu - 1 - r];
   }
 }
 
 cudaError_t launch_spike_coupling(cudaStream_t s, int P, int npad, int nblk_f, int nblk, int kl, int kuu, int lpad,
-                                  int upad, const BandFactor& f) {
+                                  int upad, const BandFactor& f, bool by_row) {
   if (kl > SPK_FS || kuu >= SPK_BW || nblk < 1 || nblk_f < 1 || npad % (nblk * SPK_CHUNK) ||
       npad % (nblk_f * SPK_FW))
     return cudaErrorInvalidValue;
   const long long total = (long long)P * (nblk_f * SPK_FS + nblk * kuu);
   k_spike_coupling<<<(unsigned)((total + 127) / 128), 128, 0, s>>>(P, npad, nblk_f, nblk, kl, kuu, lpad, upad, f.L,
-                                                                  f.piv, f.U, f.spD, f.spE);
+                                                                  f.piv, f.U, f.spD, f.spE, by_row);
   return cudaGetLastError();
 }
 
@@ -180,25 +185,32 @@ __global__ void __launch_bounds__(128) k_spike_fwd(SpikeArgs s) {
   if (PASS == 1 && act && q < SPK_FS) s.s0[(((size_t)p * s.nblk_f + k + 1) * 2 + c) * SPK_FW + q] = v;
 }
 
+// row r of pencil p's B~
+__device__ __forceinline__ const double2* spike_row(const SpikeArgs& s, int p, int r) { return s.bg + (size_t)p * s.n + r; }
+__device__ __forceinline__ const double2* spike_row(const LaneArgs& s, int p, int r) {
+  return s.bg + lane_index(p, r, s.npad);
+}
+
 // forward inflows: s_0 = rows 0..6 of B~, s_1 from block 0 (exact), then
 // s_{k+1} = s0_{k+1} + D_k s_k; one warp per (pencil, part), lanes 0..6.
 // The next step's matrix row and outflow are loaded before this step's FMAs.
-__global__ void __launch_bounds__(128) k_spike_fwd_rec(SpikeArgs s) {
+template <typename A>
+__global__ void __launch_bounds__(128) k_spike_fwd_rec(A s, const double* __restrict__ D) {
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= s.P * 2) return;
   const int p = w >> 1, c = w & 1;
   const int i = lane < SPK_FS ? lane : 0;
-  const double* Bp = reinterpret_cast<const double*>(s.bg + (size_t)p * s.n) + c;
+  const double* Bp = reinterpret_cast<const double*>(spike_row(s, p, i < s.n ? i : 0)) + c;
   auto at = [&](int k) { return (((size_t)p * s.nblk_f + k) * 2 + c) * SPK_FW; };
-  double st = i < s.n ? Bp[2 * i] : 0.0;
+  double st = i < s.n ? Bp[0] : 0.0;
   if (lane < SPK_FS) s.sst[at(0) + i] = st;
   if (s.nblk_f < 2) return;
   st = s.s0[at(1) + i];
   if (lane < SPK_FS) s.sst[at(1) + i] = st;
   double dn[SPK_FS], sn = 0.0;
   auto load = [&](int k) {
-    const double* Dk = s.D + ((size_t)p * s.nblk_f + k) * SPK_FS * SPK_FW + i * SPK_FW;
+    const double* Dk = D + ((size_t)p * s.nblk_f + k) * SPK_FS * SPK_FW + i * SPK_FW;
 #pragma unroll
     for (int t = 0; t < SPK_FS; ++t) dn[t] = Dk[t];
     sn = s.s0[at(k + 1) + i];
@@ -329,7 +341,8 @@ __global__ void __launch_bounds__(64, 10) k_spike_bwd(SpikeArgs s) {
 // sums.  The next step's matrix entries are loaded before this step's FMAs.
 constexpr int SPK_REC_WARPS = 4;
 constexpr int SPK_REC_COLS = SPK_BW / SPK_REC_WARPS;
-__global__ void __launch_bounds__(SPK_REC_WARPS * 32) k_spike_bwd_rec(SpikeArgs s) {
+template <typename A>
+__global__ void __launch_bounds__(SPK_REC_WARPS * 32) k_spike_bwd_rec(A s, const double* __restrict__ E) {
   __shared__ double part[SPK_REC_WARPS][SPK_BW];
   __shared__ double ucur[SPK_BW];
   const int p = blockIdx.x >> 1, c = blockIdx.x & 1;
@@ -345,7 +358,7 @@ __global__ void __launch_bounds__(SPK_REC_WARPS * 32) k_spike_bwd_rec(SpikeArgs 
   }
   double en[SPK_REC_COLS];
   auto load = [&](int k) {
-    const double* Ek = s.E + ((size_t)p * s.nblk + k) * kuu * SPK_BW + (size_t)(r < kuu ? r : 0) * SPK_BW;
+    const double* Ek = E + ((size_t)p * s.nblk + k) * kuu * SPK_BW + (size_t)(r < kuu ? r : 0) * SPK_BW;
 #pragma unroll
     for (int tt = 0; tt < SPK_REC_COLS; ++tt) {
       const int t = wq * SPK_REC_COLS + tt;
@@ -393,7 +406,7 @@ cudaError_t launch_spike_coupling_bwd(cudaStream_t s, int P, int npad, int nblk,
   if (!spike_bwd_supported(kuu, npad, nblk) || upad != SPK_BW) return cudaErrorInvalidValue;
   const long long total = (long long)P * nblk * kuu;
   k_spike_coupling<<<(unsigned)((total + 127) / 128), 128, 0, s>>>(P, npad, 0, nblk, 0, kuu, 0, upad, nullptr,
-                                                                  nullptr, U, nullptr, E);
+                                                                  nullptr, U, nullptr, E, false);
   return cudaGetLastError();
 }
 
@@ -404,7 +417,7 @@ cudaError_t launch_spike_backward(cudaStream_t st, const SpikeArgs& s) {
     return cudaErrorInvalidValue;
   k_spike_bwd<1><<<s.P * (s.nblk > 1 ? s.nblk - 1 : 1), 64, 0, st>>>(s);
   if (s.nblk > 1) {
-    k_spike_bwd_rec<<<s.P * 2, SPK_REC_WARPS * 32, 0, st>>>(s);
+    k_spike_bwd_rec<<<s.P * 2, SPK_REC_WARPS * 32, 0, st>>>(s, s.E);
     k_spike_bwd<2><<<s.P * (s.nblk - 1), 64, 0, st>>>(s);
   }
   return cudaGetLastError();
@@ -420,14 +433,27 @@ cudaError_t launch_spike_solve(cudaStream_t st, const SpikeArgs& s) {
     const long long lanes1 = (long long)s.P * (s.nblk_f - 1) * 2 * SPK_FW;
     k_spike_fwd<1><<<(unsigned)((lanes1 + T - 1) / T), T, 0, st>>>(s);
   }
-  k_spike_fwd_rec<<<(unsigned)((s.P * 2 * 32 + T - 1) / T), T, 0, st>>>(s);
+  k_spike_fwd_rec<<<(unsigned)((s.P * 2 * 32 + T - 1) / T), T, 0, st>>>(s, s.D);
   const long long lanes2 = (long long)s.P * s.nblk_f * 2 * SPK_FW;
   k_spike_fwd<2><<<(unsigned)((lanes2 + T - 1) / T), T, 0, st>>>(s);
   k_spike_bwd<1><<<s.P * (s.nblk > 1 ? s.nblk - 1 : 1), 64, 0, st>>>(s);
   if (s.nblk > 1) {
-    k_spike_bwd_rec<<<s.P * 2, SPK_REC_WARPS * 32, 0, st>>>(s);
+    k_spike_bwd_rec<<<s.P * 2, SPK_REC_WARPS * 32, 0, st>>>(s, s.E);
     k_spike_bwd<2><<<s.P * (s.nblk - 1), 64, 0, st>>>(s);
   }
+  return cudaGetLastError();
+}
+
+// the recurrences alone, between the passes of the lane substitution
+cudaError_t launch_spike_forward_rec(cudaStream_t st, const LaneArgs& s, const double* D) {
+  const int T = 128;
+  k_spike_fwd_rec<<<(unsigned)((s.P * 2 * 32 + T - 1) / T), T, 0, st>>>(s, D);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_spike_backward_rec(cudaStream_t st, const LaneArgs& s, const double* E) {
+  if (s.nblk < 2) return cudaSuccess;
+  k_spike_bwd_rec<<<s.P * 2, SPK_REC_WARPS * 32, 0, st>>>(s, E);
   return cudaGetLastError();
 }
 
