@@ -322,23 +322,34 @@ cudaError_t reset_spike_guess(Problem* pr, cudaStream_t s) {
   return e;
 }
 
-// Blocks per pencil of the partitioned back substitution: about 1024 / P
-// (two to four chains per GPU sub-partition with its two parts; measured at
-// 256 pencils of 1792 rows: 4 blocks 0.224 ms per solve, 7 blocks 0.254, 14
-// blocks 0.253, 28 blocks 0.274, whole pencils 0.289), each a whole number of
-// 32-row chunks and at least 64 rows.  From LANE_SPLIT_PENCILS pencils on the
-// lane substitution takes them: about 1024 groups of 16 pencils x blocks, a
-// warp or two for each of the GPU's 608 sub-partitions (Fisher-KPP 2048 x
-// 1024, four steps: 512 warps 5.20 ms, 1024 4.91 ms, 2048 5.77 ms).
+// the divisor of `whole` nearest to `target`
+int near_divisor(int whole, int target) {
+  int best = 1;
+  for (int d = 2; d <= whole; ++d)
+    if (whole % d == 0 && std::abs(d - target) < std::abs(best - target)) best = d;
+  return best;
+}
+
+// Blocks per pencil of the partitioned back substitution, each a whole number
+// of 32-row chunks.  In the one-CTA-per-pencil form (split.cu) a block and
+// part is a warp's: eight blocks for a CTA of 16 warps, four for one of 8
+// (512 x 256 SBDF2 mixed, 16 steps: 2 blocks 4.79 ms, 4 blocks 3.76, 8 blocks
+// 4.15; 500-step adjoint sizes, 20 steps: 4 blocks 17.8 ms, 7 16.6, 14 18.7).
+// From LANE_SPLIT_PENCILS pencils on the lane substitution takes them: about
+// 1024 groups of 16 pencils x blocks, a warp or two for each of the GPU's 608
+// sub-partitions (Fisher-KPP 2048 x 1024, four steps: 512 warps 5.20 ms, 1024
+// 4.91 ms, 2048 5.77 ms).
 int default_spike_blocks(int npad, int P) {
   const int nch = npad / SOLVE_CHUNK;
   const int groups = (P + LANE_GROUP - 1) / LANE_GROUP;
-  const int target = P >= LANE_SPLIT_PENCILS ? std::max(2, 1024 / groups)
-                                             : std::max(2, (1024 + std::max(P, 1) - 1) / std::max(P, 1));
-  int best = 1;
-  for (int nb = 2; nb <= nch / 2; ++nb)
-    if (nch % nb == 0 && std::abs(nb - target) < std::abs(best - target)) best = nb;
-  return best;
+  if (P >= LANE_SPLIT_PENCILS) return near_divisor(nch, std::max(2, 1024 / groups));
+  return near_divisor(nch, P <= 152 ? 8 : 4);
+}
+// Forward blocks: of about 32 rows, 64 for long pencils (a block costs a step
+// of the recurrence over blocks, about as long as three rows of its two passes).
+int default_forward_blocks(int npad) {
+  const int nch = npad / SOLVE_CHUNK;
+  return npad <= 1024 ? nch : near_divisor(nch, nch / 2);
 }
 
 sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
@@ -464,23 +475,29 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
   // rows into blocks substituted in parallel (spike.cu)
   pr->by_group = pr->lanes;
   pr->nblk = pr->spike_blocks > 0 ? pr->spike_blocks : default_spike_blocks(pr->npad, pr->P);
-  pr->spike = !pr->lanes && spike_supported(pr->kl, kuu, pr->npad, pr->nblk) &&
+  pr->nblk_f = pr->P >= LANE_SPLIT_PENCILS ? pr->nblk : default_forward_blocks(pr->npad);
+  const bool split_fits = pr->P >= LANE_SPLIT_PENCILS ||
+                          pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false) <= 227 * 1024;
+  pr->spike = !pr->lanes && split_fits && spike_supported(pr->kl, kuu, pr->npad, pr->nblk) &&
               (pr->solve_kind == SP_SOLVE_SPIKE ||
-               (pr->solve_kind == SP_SOLVE_AUTO && pr->P < SPIKE_MAX_PENCILS && pr->npad >= SPIKE_MIN_ROWS));
+               (pr->solve_kind == SP_SOLVE_AUTO && pr->P < SPIKE_MAX_PENCILS &&
+                (pr->npad >= SPIKE_MIN_ROWS || (pr->P <= SPLIT_MAX_PENCILS && pr->npad >= SPLIT_MIN_ROWS))));
   if (pr->spike) {
     pr->by_group = pr->P >= LANE_SPLIT_PENCILS;
-    pr->nblk_f = pr->by_group ? pr->nblk : spike_forward_blocks(pr->npad);
     const size_t nv = (size_t)pr->P * pr->nblk * 2, nvf = (size_t)pr->P * pr->nblk_f * 2;
-    CK(dalloc(&pr->d_sp_s0, nvf * 8));
-    CK(dalloc(&pr->d_sp_s, nvf * 8));
-    CK(dalloc(&pr->d_sp_o0, nv * 32));
     CK(dalloc(&pr->d_sp_u, nv * 32));
     CK(reset_spike_guess(pr, ctx->stream));
+    if (pr->by_group) {
+      CK(dalloc(&pr->d_sp_s0, nvf * 8));
+      CK(dalloc(&pr->d_sp_s, nvf * 8));
+      CK(dalloc(&pr->d_sp_o0, nv * 32));
+    } else {
+      CK(dalloc(&pr->d_bg, (size_t)pr->P * pr->n));
+    }
   }
-  if (pr->lanes || pr->spike) {
+  if (pr->by_group) {
     // by group: the rows beyond n and the last group's missing pencils stay zero
-    const size_t nv = !pr->by_group ? (size_t)pr->P * pr->n
-                                    : (size_t)((pr->P + LANE_GROUP - 1) / LANE_GROUP) * LANE_GROUP * pr->npad;
+    const size_t nv = (size_t)((pr->P + LANE_GROUP - 1) / LANE_GROUP) * LANE_GROUP * pr->npad;
     for (double2** v : {&pr->d_bg, &pr->d_xg, &pr->d_yg}) {
       CK(dalloc(v, nv));
       CK(cudaMemsetAsync(*v, 0, nv * sizeof(double2), s));
@@ -520,7 +537,7 @@ void free_problem(Problem* pr) {
   F(pr->d_sp_s0); F(pr->d_sp_s); F(pr->d_sp_o0); F(pr->d_sp_u);
   cheb_mma_free(pr->cm);
   F(pr->d_lb_F); F(pr->d_lb_eq); F(pr->d_eigx); F(pr->d_eigsig);
-  F(pr->facT.L); F(pr->facT.piv); F(pr->facT.U); F(pr->facT.rd); F(pr->facT.spE); F(pr->d_spT_u);
+  F(pr->facT.L); F(pr->facT.piv); F(pr->facT.U); F(pr->facT.rd); F(pr->facT.spD); F(pr->facT.spE); F(pr->d_spT_u);
   F(pr->d_indptrT); F(pr->d_indicesT); F(pr->d_MvT); F(pr->d_LvT);
   F(pr->d_mu[0]); F(pr->d_mu[1]); F(pr->d_LTmu); F(pr->d_MTmu); F(pr->d_JF); F(pr->d_lamx);
   F(pr->d_Xbar); F(pr->d_Fbar); F(pr->d_Fbar32); F(pr->d_gzadj);
@@ -621,9 +638,10 @@ SolveArgs base_args(Problem* pr, sp_ctx* ctx, int fac) {
   a.xc32_out = pr->d_Xc32;   // null unless mixed precision
   a.xs32_out = pr->zmma ? pr->cm.xs32 : nullptr;
   a.ll = pr->by_group ? &pr->fac[fac].ll : nullptr;
-  a.by_group = pr->by_group;
   a.spD = pr->spike ? pr->fac[fac].spD : nullptr;   // null unless partitioned substitution
   a.spE = pr->spike ? pr->fac[fac].spE : nullptr;
+  a.sp_nblk = pr->nblk; a.sp_nblk_f = pr->nblk_f; a.sp_u = pr->d_sp_u;
+  a.bg = pr->d_bg; a.xg = pr->d_xg;
   return a;
 }
 
@@ -653,85 +671,52 @@ LaneArgs lane_args(sp_ctx* ctx, Problem* pr, const LaneList& f, int kl, int kuu)
   return la;
 }
 
-sp_status solve(sp_ctx* ctx, Problem* pr, cudaStream_t s, const SolveArgs& a) {
+// L~ X~ of a stage.  FP64 form: the product with L~ itself.  Mixed form: from
+// the stage's own right-hand side, (B~ - alpha M~ X~) / beta with the factored
+// alpha M~ + beta L~, M~'s compact pattern instead of L~'s (3D: 1508 against
+// 6073 entries per pencil, ~0.5 ms of FP64 pipe per stage at 256 x 256 x 128).
+// B~ is alpha M~ X~ up to O(beta), so the difference cancels; the error it
+// leaves in a later stage's right-hand side, dt a_ij L~X~ = (a_ij / a_jj)(B~ -
+// alpha M~ X~), is a few FP64 roundings of M~X~, far below the FP32
+// transforms' 1e-7 but above the FP64 form's own rounding (the 500-step RK222
+// adjoint gradient drifts 15x past the oracle floor), hence FP64 keeps L~.
+void stage_lx(Problem* pr, SolveArgs& a) {
+  if (a.ep_mv_vals != pr->d_Lv || !pr->prec) return;
+  int fi = 0;
+  for (int q = 1; q < 4; ++q)
+    if (a.Lf == pr->fac[q].L && pr->fac[q].L) fi = q;
+  const BandFactor& f = pr->fac[fi];
+  set_ep_M(pr, a);
+  a.ep_alpha = f.alpha;
+  a.ep_from_b = 1.0 / f.beta;
+}
+
+sp_status solve(sp_ctx* ctx, Problem* pr, cudaStream_t s, const SolveArgs& args) {
   const bool t = pr->timing && pr->ev_used + 2 <= pr->ev.size();
   if (t) CK(cudaEventRecord(pr->ev[pr->ev_used], s));
-  if (pr->spike && !a.by_group && a.Lf && a.Lf == pr->facT.L && pr->facT.spE && pr->d_spT_u) {
-    // transposed solve: assembly and whole-row forward substitution (mode 3),
-    // partitioned back substitution from the last transposed solve's inflows,
-    // epilogue
-    SolveArgs a3 = a;
-    a3.mode = 3; a3.yg = pr->d_yg;
-    CK(launch_pencil_solve(s, a3));
-    SpikeArgs sa{};
-    sa.P = pr->P; sa.n = pr->n; sa.npad = pr->npad; sa.kl = a.kl; sa.kuu = a.kuu; sa.lpad = a.lpad;
-    sa.upad = a.upad; sa.nblk = pr->nblk; sa.m = pr->npad / pr->nblk;
-    sa.nblk_f = pr->nblk_f; sa.m_f = pr->npad / pr->nblk_f;
-    sa.U = a.Uf; sa.rd = a.rd; sa.E = pr->facT.spE;
-    sa.yg = pr->d_yg; sa.xg = pr->d_xg;
-    sa.o0 = pr->d_sp_o0; sa.uin = pr->d_spT_u;
-    sa.status = ctx->d_status;
-    CK(launch_spike_backward(s, sa));
-    SolveArgs a2 = a;
-    a2.mode = 2; a2.xg = pr->d_xg; a2.bg = pr->d_bg;
-    CK(launch_pencil_solve(s, a2));
-    if (t) {
-      CK(cudaEventRecord(pr->ev[pr->ev_used + 1], s));
-      pr->ev_used += 2;
-    }
-    return SP_OK;
-  }
-  if (a.ll || (a.spD && pr->spike)) {
-    // assembly -> lane substitution (whole or partitioned) or partitioned
-    // window substitution -> epilogue
-    SolveArgs a1 = a;
-    a1.mode = 1; a1.bg = pr->d_bg;
-    CK(launch_pencil_solve(s, a1));
+  SolveArgs a = args;
+  if (a.ll) {
+    // assembly -> lane substitution, whole or partitioned -> epilogue
+    a.mode = 1;
+    CK(launch_pencil_solve(s, a));
+    const LaneArgs la = lane_args(ctx, pr, *a.ll, a.kl, a.kuu);
     if (pr->lanes) {
-      const LaneArgs la = lane_args(ctx, pr, *a.ll, a.kl, a.kuu);
       CK(launch_lane_forward(s, la, 0));
       CK(launch_lane_backward(s, la, 0));
-    } else if (pr->by_group) {
-      const LaneArgs la = lane_args(ctx, pr, *a.ll, a.kl, a.kuu);
+    } else {
       CK(launch_lane_forward(s, la, 1));
       CK(launch_spike_forward_rec(s, la, a.spD));
       CK(launch_lane_forward(s, la, 2));
       CK(launch_lane_backward(s, la, 1));
       CK(launch_spike_backward_rec(s, la, a.spE));
       CK(launch_lane_backward(s, la, 2));
-    } else {
-      SpikeArgs sa{};
-      sa.P = pr->P; sa.n = pr->n; sa.npad = pr->npad; sa.kl = a.kl; sa.kuu = a.kuu; sa.lpad = a.lpad;
-      sa.upad = a.upad; sa.nblk = pr->nblk; sa.m = pr->npad / pr->nblk;
-      sa.nblk_f = pr->nblk_f; sa.m_f = pr->npad / pr->nblk_f;
-      sa.L = a.Lf; sa.piv = a.piv; sa.U = a.Uf; sa.rd = a.rd; sa.D = a.spD; sa.E = a.spE;
-      sa.bg = pr->d_bg; sa.yg = pr->d_yg; sa.xg = pr->d_xg;
-      sa.s0 = pr->d_sp_s0; sa.sst = pr->d_sp_s; sa.o0 = pr->d_sp_o0; sa.uin = pr->d_sp_u;
-      sa.status = ctx->d_status;
-      CK(launch_spike_solve(s, sa));
     }
-    SolveArgs a2 = a;
-    a2.mode = 2; a2.xg = pr->d_xg; a2.bg = pr->d_bg;
-    if (a2.ep_mv_vals == pr->d_Lv && pr->prec) {
-      // L~ X~ of a stage.  FP64 form: the product with L~ itself.  Mixed
-      // form: from the stage's own right-hand side, (B~ - alpha M~ X~) / beta
-      // with the factored alpha M~ + beta L~, M~'s compact pattern instead of
-      // L~'s (3D: 1508 against 6073 entries per pencil, ~0.5 ms of FP64 pipe
-      // per stage at 256 x 256 x 128).  B~ is alpha M~ X~ up to O(beta), so
-      // the difference cancels; the error it leaves in a later stage's
-      // right-hand side, dt a_ij L~X~ = (a_ij / a_jj)(B~ - alpha M~ X~), is a
-      // few FP64 roundings of M~X~, far below the FP32 transforms' 1e-7 but
-      // above the FP64 form's own rounding (the 500-step RK222 adjoint
-      // gradient drifts 15x past the oracle floor), hence FP64 keeps L~.
-      int fi = 0;
-      for (int q = 1; q < 4; ++q)
-        if (a.Lf == pr->fac[q].L && pr->fac[q].L) fi = q;
-      const BandFactor& f = pr->fac[fi];
-      set_ep_M(pr, a2);
-      a2.ep_alpha = f.alpha;
-      a2.ep_from_b = 1.0 / f.beta;
-    }
-    CK(launch_pencil_solve(s, a2));
+    a.mode = 2;
+    stage_lx(pr, a);
+    CK(launch_pencil_solve(s, a));
+  } else if (a.spE) {
+    stage_lx(pr, a);
+    CK(launch_pencil_split(s, a));
   } else {
     CK(launch_pencil_solve(s, a));
   }
@@ -897,8 +882,9 @@ SolveArgs transposed_args(Problem* pr, sp_ctx* ctx) {
   a.n_nl = 0; a.nbc = 0; a.bc_coef = 0.0;
   a.xc32_out = nullptr;
   a.xs32_out = nullptr;
-  a.ll = nullptr; a.by_group = 0;
-  a.spD = nullptr; a.spE = nullptr;      // no coupling matrices for the transposed factor
+  a.ll = nullptr;
+  a.spD = pr->facT.spD; a.spE = pr->facT.spE;    // null unless partitioned
+  a.sp_nblk_f = pr->nblk; a.sp_u = pr->d_spT_u;
   a.ep_rows = nullptr; a.ep_nrows = 0;   // the transposed patterns carry no row list
   return a;
 }
@@ -944,6 +930,7 @@ struct Batch {
   int tile = 8;
   int max_ngz = 0, max_kuu = 0;
   size_t x_smem = 0, s_smem = 0;
+  bool split = false;                        // every problem's solves in the partitioned kernel
   int4 *d_wzb = nullptr, *d_wx = nullptr, *d_wzf = nullptr, *d_ws = nullptr;
   int nzb = 0, nx = 0, nzf = 0, ns = 0;
   std::vector<BatchStage> stages;
@@ -979,6 +966,15 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
   b->tile = tile;
   b->parity = parity;
   std::vector<std::pair<long long, int4>> zb, xr, zf, sv;
+  // few pencils in all: the solves' latency counts, so each problem's
+  // partitioned form; more: the FP64 pipe does, so whole pencils
+  int pencils = 0;
+  b->split = true;
+  for (Problem* pr : ps) {
+    pencils += pr->P;
+    b->split = b->split && pr->spike && !pr->by_group;
+  }
+  b->split = b->split && pencils <= SPLIT_MAX_PENCILS;
   for (size_t q = 0; q < ps.size(); ++q) {
     Problem* pr = ps[q];
     const int nt = (pr->P + tile - 1) / tile;
@@ -993,7 +989,8 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
     b->max_kuu = std::max(b->max_kuu, pr->kl + pr->ku);
     b->x_smem = std::max(b->x_smem, x_smem_bytes(pr->prec, pr->Ngx, 7, (int)pr->gfields.size(),
                                                  (int)pr->nl_eqs.size()));
-    b->s_smem = std::max(b->s_smem, pencil_solve_smem(pr->npad, pr->lpad, pr->upad));
+    b->s_smem = std::max(b->s_smem, b->split ? pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false)
+                                             : pencil_solve_smem(pr->npad, pr->lpad, pr->upad));
   }
   auto finish = [](std::vector<std::pair<long long, int4>>& v) {
     std::stable_sort(v.begin(), v.end(), [](const auto& a, const auto& c) { return a.first > c.first; });
@@ -1028,6 +1025,7 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
       zfv.push_back(zdesc_forward(ps[q], plans[q][i].fc_out));
       av.push_back(plans[q][i].args);
       av.back().fwd16 = 1;            // throughput-bound: both parts' forward in one warp
+      if (b->split) stage_lx(ps[q], av.back());
       fill_f_halves(av.back());
     }
     BatchStage st;
@@ -1066,7 +1064,8 @@ sp_status batch_step(sp_ctx* ctx, Batch* b, cudaStream_t s) {
     CK(launch_cheb_backward_batched(s, b->prec, b->tile, st.d_zb, b->d_wzb, b->nzb, b->max_ngz, q));
     CK(launch_fourier_rows_batched(s, b->prec, st.d_x, b->d_wx, b->nx, b->x_smem, q ? q + 1 : nullptr));
     CK(launch_cheb_forward_batched(s, b->prec, b->tile, st.d_zf, b->d_wzf, b->nzf, b->max_ngz, q ? q + 2 : nullptr));
-    CK(launch_pencil_solve_batched(s, st.d_args, b->d_ws, b->ns, b->max_kuu, b->s_smem));
+    if (b->split) CK(launch_pencil_split_batched(s, st.d_args, b->d_ws, b->ns, b->s_smem));
+    else CK(launch_pencil_solve_batched(s, st.d_args, b->d_ws, b->ns, b->max_kuu, b->s_smem));
   }
   return SP_OK;
 }
@@ -1692,6 +1691,7 @@ sp_status sp_step_batched(sp_ctx* ctx, int nproblems, const int* problem_ids, co
       for (double2* b : pr->d_MX) if (b) bufs.push_back({b, nvec});
       for (double2* b : pr->d_LX) if (b) bufs.push_back({b, nvec});
       for (double2* b : pr->d_Fc) if (b) bufs.push_back({b, nfc});
+      if (pr->d_sp_u) bufs.push_back({pr->d_sp_u, (size_t)pr->P * pr->nblk * 2 * 32 * sizeof(double)});
       if (pr->zmma) bufs.push_back({pr->cm.xs32, (size_t)pr->S * 2 * pr->P * pr->Nz * sizeof(float)});
     }
     size_t total = 0;
@@ -1877,15 +1877,18 @@ sp_status sp_adjoint_init(sp_ctx* ctx, int problem) {
   CK(e);
   pr->facT.alpha = pr->fac[0].alpha;
   pr->facT.beta = pr->fac[0].beta;
-  // the transposed solves' back substitution is partitioned like the forward
-  // solves' (kl' + ku' = kl + ku); their forward substitution stays whole-row,
-  // since kl' = ku is wider than the partitioned forward windows
+  // the transposed solves are partitioned like the forward ones, their wider
+  // lower band (kl' = ku) in forward blocks as long as the back ones
   const int kuuT = pr->klT + pr->kuT;
-  if (pr->spike && !pr->by_group && pr->upad == 32 && spike_bwd_supported(kuuT, pr->npad, pr->nblk)) {
+  if (pr->spike && !pr->by_group && pr->upad == 32 && pr->klT <= 30 &&
+      spike_bwd_supported(kuuT, pr->npad, pr->nblk) &&
+      pencil_split_smem(pr->npad, pr->nblk, pr->nblk, kuuT, pr->klT > 7) <= 227 * 1024) {
+    if (!pr->facT.spD) CK(dalloc(&pr->facT.spD, (size_t)pr->P * pr->nblk * (pr->klT > 7 ? 31 * 32 : 7 * 8)));
     if (!pr->facT.spE) CK(dalloc(&pr->facT.spE, (size_t)pr->P * pr->nblk * kuuT * 32));
     if (!pr->d_spT_u) CK(dalloc(&pr->d_spT_u, (size_t)pr->P * pr->nblk * 2 * 32));
     CK(cudaMemsetAsync(pr->d_spT_u, 0, (size_t)pr->P * pr->nblk * 2 * 32 * sizeof(double), s));
-    CK(launch_spike_coupling_bwd(s, pr->P, pr->npad, pr->nblk, kuuT, pr->upad, pr->facT.U, pr->facT.spE));
+    CK(launch_spike_coupling(s, pr->P, pr->npad, pr->nblk, pr->nblk, pr->klT, kuuT, pr->lpadT, pr->upad, pr->facT,
+                             false));
     CK(cudaStreamSynchronize(s));
   }
   return SP_OK;
@@ -2200,6 +2203,13 @@ sp_status sp_eig_target(sp_ctx* ctx, int problem, double sigma_t, int iters, con
   cudaError_t e = launch_band_factor(s, pr->P, pr->n, (int)pr->nnz, pr->kl, pr->ku, pr->d_indptr, pr->d_indices,
                                      pr->d_Mv, pr->d_Lv, sigma_t, 1.0, work, pr->fac[0], pr->npad, pr->lpad,
                                      pr->upad, ctx->d_status);
+  const bool split = pr->spike && !pr->by_group;
+  if (e == cudaSuccess && split) {
+    e = reset_spike_guess(pr, s);
+    if (e == cudaSuccess)
+      e = launch_spike_coupling(s, pr->P, pr->npad, pr->nblk_f, pr->nblk, pr->kl, pr->kl + pr->ku, pr->lpad, pr->upad,
+                                pr->fac[0], false);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFree(work);
   CK(e);
@@ -2225,9 +2235,9 @@ sp_status sp_eig_target(sp_ctx* ctx, int problem, double sigma_t, int iters, con
   a.mv_x = x; a.mv_coef = 1.0; a.mv_store = nullptr;
   set_mv_M(pr, a);
   a.xt_out = y; a.xc_out = nullptr; a.xc32_out = nullptr; a.ep_mv_vals = nullptr;
-  a.ll = nullptr; a.by_group = 0;
+  a.ll = nullptr;
   for (int k = 0; e == cudaSuccess && k < iters; ++k) {
-    e = launch_pencil_solve(s, a);
+    e = split ? launch_pencil_split(s, a) : launch_pencil_solve(s, a);
     if (e == cudaSuccess) e = launch_eig_update(s, pr->P, pr->n, x, y, mu);
   }
   std::vector<double2> hm(pr->P);

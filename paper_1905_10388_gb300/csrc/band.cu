@@ -23,6 +23,7 @@
 #include <cstdio>
 
 #include "internal.h"
+#include "pencil.cuh"
 #include "tma.cuh"
 
 namespace spectau {
@@ -190,42 +191,6 @@ __device__ __forceinline__ double2 shfl2(double2 v, int src) {
 // ---------------------------------------------------------------------------
 // pencil solve: prologue (B~ assembly) -> L pass -> U pass -> epilogue
 // ---------------------------------------------------------------------------
-// acc + the left-preconditioned F~ entry of row (slot sl, mode m): the
-// combination sum_k c_k F_k of the stored right-hand sides, through the
-// T-to-U conversion P^L for differential equations (Appendix: row m holds
-// (1 + delta_m0)/2 F_m - F_{m+2}/2) and the phase i^-q of the equation's
-// real-ification.  One FMA per term and component: on GB300 every FP64
-// instruction holds the sub-partition's FP64 pipe for 64 cycles, so the
-// halves c/2 and -c/2 come precomputed with the arguments and the phase is
-// applied to the loaded values (a sign and swap, no arithmetic).
-__device__ __forceinline__ double2 add_f_row(const SolveArgs& a, int sl, int m, int p, double2 acc) {
-  const int Nz = a.Nz;
-  const int e = a.nl_eq[sl];
-  const bool dif = a.eq_differential[e] != 0;
-  const int ph = -a.eq_phase[e];
-#pragma unroll
-  for (int k = 0; k < SP_MAX_TERMS; ++k) {
-    if (k >= a.nfc) break;
-    const double2* F = a.fc[k] + ((size_t)sl * a.P + p) * Nz;
-    const double2 v0 = cipow_d(F[m], ph);
-    const double c = (dif && m > 0) ? a.fc_half[k] : a.fc_coef[k];
-    acc.x = fma(c, v0.x, acc.x);
-    acc.y = fma(c, v0.y, acc.y);
-    if (dif && m + 2 < Nz) {
-      const double2 v2 = cipow_d(F[m + 2], ph);
-      acc.x = fma(a.fc_mhalf[k], v2.x, acc.x);
-      acc.y = fma(a.fc_mhalf[k], v2.y, acc.y);
-    }
-  }
-  return acc;
-}
-
-// c v, exactly v when c = 1 (tested on the bit pattern: no FP64 compare)
-__device__ __forceinline__ double2 scale_first(double c, double2 v) {
-  if (__double_as_longlong(c) == 0x3FF0000000000000LL) return v;
-  return make_double2(c * v.x, c * v.y);
-}
-
 struct SolveSmem {
   double2* B;
   double* Lring;
@@ -250,25 +215,20 @@ __host__ __device__ inline size_t solve_smem_bytes(int npad, int lpad, int upad)
   return off;
 }
 
-// PPC pencils per CTA of NT threads (1 or 2); with PPC = 2 threads
-// [0, NT/2) serve pencil 2b and [NT/2, NT) pencil 2b + 1, each half with its
-// own shared-memory region.  Warps 0 and 1 of a pencil substitute; all NT/PPC
-// threads share the assembly and the epilogue.
-template <int RU, int PPC, int MODE = -1, int NT = 128>
+// One pencil per CTA of NT threads.  Warps 0 and 1 substitute; all threads
+// share the assembly and the epilogue.
+template <int RU, int MODE = -1, int NT = 128>
 __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block, unsigned char* smem_raw) {
   // MODE >= 0 fixes the stage at compile time (assembly-only and
   // epilogue-only kernels carry neither the factor ring nor the substitution)
   const int mode = MODE >= 0 ? MODE : a.mode;
-  const int lp = (mode == 0 || mode == 3) ? a.lpad : 0, up = mode == 0 ? a.upad : 0;
-  const int half = (PPC == 2) ? (int)(threadIdx.x / (NT / 2)) : 0;
-  const int p = block * PPC + half;
-  const bool active = p < a.P;
-  const int tid = (PPC == 2) ? (int)(threadIdx.x % (NT / 2)) : (int)threadIdx.x;
-  const int nt = NT / PPC;
+  const int lp = mode == 0 ? a.lpad : 0, up = mode == 0 ? a.upad : 0;
+  const int pp = block, tid = threadIdx.x;
+  constexpr int nt = NT;
   const int n = a.n;
   SolveSmem sm;
   {
-    size_t off = (size_t)half * solve_smem_bytes(a.npad, lp, up);
+    size_t off = 0;
     sm.B = reinterpret_cast<double2*>(smem_raw + off);
     off += align_up((size_t)(a.npad + 64) * 16, 128);
     sm.Lring = reinterpret_cast<double*>(smem_raw + off);
@@ -283,7 +243,6 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
     sm.abort_flag = reinterpret_cast<int*>(smem_raw + off);
   }
   const int nchunks = a.npad / SOLVE_CHUNK;
-  const int pp = active ? p : 0;             // keeps addresses valid on an idle half
   const double* Lsrc = a.Lf + (size_t)pp * a.npad * a.lpad;
   const double* Usrc = a.Uf + (size_t)pp * a.npad * a.upad;
   const uint8_t* Psrc = a.piv + (size_t)pp * a.npad;
@@ -304,104 +263,40 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
              &sm.barU[s]);
   };
 
-  if (tid == 0 && active) {
+  if (tid == 0) {
     *sm.abort_flag = 0;
-    if (mode == 0 || mode == 3) {
+    if (mode == 0) {
       for (int s = 0; s < SOLVE_RING; ++s) {
         mbar_init(&sm.barL[s], 1);
         mbar_init(&sm.barU[s], 1);
       }
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       // the factor does not depend on the prologue: start streaming now
-      // (mode 3, forward substitution only: L alone)
       for (int c = 0; c < min(SOLVE_RING, nchunks); ++c) issue_L(c);
-      if (mode == 0)
-        for (int k = 0; k < min(SOLVE_RING, nchunks); ++k) issue_U(k);
+      for (int k = 0; k < min(SOLVE_RING, nchunks); ++k) issue_U(k);
     }
   }
 
   // ---- prologue: B~ = linear combination of stored vectors, one matvec,
   //      left-preconditioned F~ (T-to-U conversion, tau rows dropped) and
   //      boundary values
-  const size_t prow = (size_t)pp * n;
-  // element r of this pencil in the substitution kernels' vectors
-  const size_t v0 = a.by_group ? lane_index(pp, 0, a.npad) : prow;
-  const int vstep = a.by_group ? LANE_GROUP : 1;
-  auto vec = [&](int r) { return v0 + (size_t)r * vstep; };
-  const int Nz = a.Nz;
-  const float invNz = 1.0f / (float)Nz;
+  // element r of this pencil in the lane substitution's vectors
+  const size_t v0 = lane_index(pp, 0, a.npad);
+  auto vec = [&](int r) { return v0 + (size_t)r * LANE_GROUP; };
   if (mode == 2) {
-    // epilogue only: X~ from the substitution kernel, as b = U_jj X~ by group
-    // from the lane substitution
+    // epilogue only: X~ = b / U_jj, b from the lane substitution
     const double* rdp = a.rd + (size_t)pp * a.npad;
-    for (int r = tid; active && r < n; r += nt) {
+    for (int r = tid; r < n; r += nt) {
       const double2 b = a.xg[vec(r)];
-      const double rd = a.by_group ? rdp[r] : 1.0;
-      sm.B[r] = a.by_group ? make_double2(b.x * rd, b.y * rd) : b;
+      const double rd = rdp[r];
+      sm.B[r] = make_double2(b.x * rd, b.y * rd);
     }
     __syncthreads();
   } else {
-  // modes 0 and 1: two passes over the rows, each with every lane on the
-  // same kind of row, since on GB300 an FP64 warp instruction holds the FP64
-  // pipe for 64 cycles whatever its active mask: stored vectors and matvec
-  // for every row, then the F~ entries by (slot, mode), then the boundary
-  // rows.  Mode 1 (assembly only) then stores B~ for the substitution
-  // kernel.
-  for (int r = tid; active && r < n; r += nt) {
-    double2 acc = make_double2(0.0, 0.0);
-    if (a.nvec > 0) acc = scale_first(a.vec_coef[0], a.vec[0][prow + r]);
-    for (int k = 1; k < a.nvec; ++k) {
-      const double2 v = a.vec[k][prow + r];
-      acc.x = fma(a.vec_coef[k], v.x, acc.x);
-      acc.y = fma(a.vec_coef[k], v.y, acc.y);
-    }
-    if (a.mv_x != nullptr) {
-      double2 s = make_double2(0.0, 0.0);
-      const double* vals = a.mv_vals + (size_t)p * a.mv_nnz;
-      for (int e = a.mv_indptr[r]; e < a.mv_indptr[r + 1]; ++e) {
-        const double m = vals[e];
-        const double2 x = a.mv_x[prow + a.mv_indices[e]];
-        s.x = fma(m, x.x, s.x);
-        s.y = fma(m, x.y, s.y);
-      }
-      if (a.mv_store != nullptr) a.mv_store[prow + r] = s;
-      acc.x = fma(a.mv_coef, s.x, acc.x);
-      acc.y = fma(a.mv_coef, s.y, acc.y);
-    }
-    if (a.mv2_vals != nullptr) {                 // a second matrix on the same vector (CNAB: L~ X~^n)
-      double2 s = make_double2(0.0, 0.0);
-      const double* vals = a.mv2_vals + (size_t)p * a.mv2_nnz;
-      for (int e = a.mv2_indptr[r]; e < a.mv2_indptr[r + 1]; ++e) {
-        const double m = vals[e];
-        const double2 x = a.mv_x[prow + a.mv2_indices[e]];
-        s.x = fma(m, x.x, s.x);
-        s.y = fma(m, x.y, s.y);
-      }
-      acc.x = fma(a.mv2_coef, s.x, acc.x);
-      acc.y = fma(a.mv2_coef, s.y, acc.y);
-    }
-    sm.B[r] = acc;
-  }
-  for (int r = n + tid; active && r < a.npad + 64; r += nt) sm.B[r] = make_double2(0.0, 0.0);
-  __syncthreads();
-  for (int idx = tid; active && idx < a.n_nl * Nz; idx += nt) {
-    const int sl = div_idx(idx, invNz), m = idx - sl * Nz;
-    const int e = a.nl_eq[sl];
-    const int row = a.row_map[e * Nz + m];
-    if (row < 0) continue;
-    sm.B[row] = add_f_row(a, sl, m, p, sm.B[row]);
-  }
-  for (int q = tid; active && q < a.nbc; q += nt) {
-    const int row = a.bc_rows[q];
-    const double2 g = a.bc_values[(size_t)p * a.nbc + q];
-    double2 b = sm.B[row];
-    b.x = fma(a.bc_coef, g.x, b.x);
-    b.y = fma(a.bc_coef, g.y, b.y);
-    sm.B[row] = b;
-  }
-  __syncthreads();
+  // (mode 1, assembly only, then stores B~ for the substitution kernel)
+  pencil_assemble(a, pp, tid, nt, a.npad + 64, sm.B);
   if (mode == 1) {
-    for (int r = tid; active && r < n; r += nt) a.bg[vec(r)] = sm.B[r];   // B~ for the substitution
+    for (int r = tid; r < n; r += nt) a.bg[vec(r)] = sm.B[r];   // B~ for the substitution
     return;
   }
   }
@@ -422,7 +317,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
   //      Both warps read each ring slot; named barrier 1 (64 threads) at the
   //      top of every chunk both agrees on a timed-out wait and frees the
   //      previous slot for refilling.
-  if ((mode == 0 || mode == 3) && active && tid < 64) {
+  if (mode == 0 && tid < 64) {
     const int lane = tid & 31;
     const int comp = tid >> 5;                 // 0: real part, 1: imaginary part
     double* Bd = reinterpret_cast<double*>(sm.B) + comp;   // element j at Bd[2 j]
@@ -431,10 +326,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
     auto chunk_sync = [&](uint64_t* bar, int k, int& done) -> bool {
       const bool got = bounded_wait(bar, (k / SOLVE_RING) & 1);
       if (!got) atomicOr(sm.abort_flag, 1);
-      if (half == 0)
-        asm volatile("bar.sync 1, 64;" ::: "memory");
-      else
-        asm volatile("bar.sync 2, 64;" ::: "memory");
+      asm volatile("bar.sync 1, 64;" ::: "memory");
       if (*sm.abort_flag) return false;
       done = k + 1;
       return true;
@@ -519,14 +411,9 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
       }
     }
     // both parts' y in B before either warp's back substitution
-    if (half == 0)
-      asm volatile("bar.sync 1, 64;" ::: "memory");
-    else
-      asm volatile("bar.sync 2, 64;" ::: "memory");
+    asm volatile("bar.sync 1, 64;" ::: "memory");
     // backward: scaled U columns (U_{j-t,j}/U_jj), window of 32*RU entries;
     // x_j = b_j / U_jj is applied once per chunk, lane l to row j0 + l
-    // (mode 3 stops after the forward pass: y is in B)
-    if (mode == 0) {
     constexpr int W = 32 * RU;
     const double* rdp = a.rd + (size_t)pp * a.npad;
     const int npad = a.npad;
@@ -581,126 +468,44 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
       }
       Bd[2 * (j0 + lane)] = xo * rdl;
     }
-    }
     if (!ok && tid == 0) {
       // report, then let every copy in flight land before the CTA exits
-      raise_status(a.status, SP_ERR_TIMEOUT, p);
+      raise_status(a.status, SP_ERR_TIMEOUT, pp);
       // chunks issued: RING up front, then chunk q - 1 + RING at the top of chunk q
       const int issL = min(nchunks, doneL == 0 ? SOLVE_RING : doneL - 1 + SOLVE_RING);
-      const int issU = mode == 0 ? min(nchunks, doneU == 0 ? SOLVE_RING : doneU - 1 + SOLVE_RING) : 0;
+      const int issU = min(nchunks, doneU == 0 ? SOLVE_RING : doneU - 1 + SOLVE_RING);
       for (int q = doneL; q < issL; ++q) bounded_wait(&sm.barL[q % SOLVE_RING], (q / SOLVE_RING) & 1);
       for (int q = doneU; q < issU; ++q) bounded_wait(&sm.barU[q % SOLVE_RING], (q / SOLVE_RING) & 1);
     }
   }
   __syncthreads();
-  const bool work = active && !*sm.abort_flag;
-  if (mode == 3) {
-    // y = L^-1 P B~ for the partitioned back substitution
-    for (int r = tid; work && r < n; r += nt) a.yg[vec(r)] = sm.B[r];
-    return;
-  }
-
-  // ---- epilogue: store X~, recombine to T coefficients, optional M~ X~
-  bool finite = true;
-  for (int r = tid; work && r < n; r += nt) {
-    const double2 x = sm.B[r];
-    finite = finite && dfinite(x.x) && dfinite(x.y);
-    if (a.xt_out) a.xt_out[prow + r] = x;
-  }
-  if (a.xc_out) {
-    for (int idx = tid; work && idx < a.S * Nz; idx += nt) {
-      const int v = div_idx(idx, invNz), m = idx - v * Nz;
-      double2 x = sm.B[a.col_map[idx]];
-      if (a.var_recombine[v] && m + 2 < Nz) {
-        const double2 x2 = sm.B[a.col_map[idx + 2]];
-        x.x -= x2.x;
-        x.y -= x2.y;
-      }
-      const double2 xv = cipow_d(x, a.var_phase[v]);
-      a.xc_out[((size_t)v * a.P + p) * Nz + m] = xv;
-      if (a.xc32_out) a.xc32_out[((size_t)v * a.P + p) * Nz + m] = make_float2((float)xv.x, (float)xv.y);
-      if (a.xs32_out) {
-        a.xs32_out[(((size_t)v * a.P + p) * 2) * Nz + m] = (float)xv.x;
-        a.xs32_out[(((size_t)v * a.P + p) * 2 + 1) * Nz + m] = (float)xv.y;
-      }
-    }
-  }
-  if (a.ep_mv_vals) {
-    const double* vals = a.ep_mv_vals + (size_t)p * a.ep_nnz;
-    const bool listed = a.ep_rows != nullptr;
-    if (listed) {
-      // rows without entries first (zero, or B~/beta for L~X~ from the
-      // stage right-hand side), then the listed rows with every lane on a
-      // row that has entries; the barrier orders the two stores of a row
-      for (int r = tid; work && r < n; r += nt) {
-        double2 s = make_double2(0.0, 0.0);
-        if (mode == 2 && a.ep_from_b != 0.0) {
-          const double2 bb = a.bg[vec(r)];
-          s.x = bb.x * a.ep_from_b;
-          s.y = bb.y * a.ep_from_b;
-        }
-        a.ep_mv_store[prow + r] = s;
-      }
-      __syncthreads();
-    }
-    const int nrows = listed ? a.ep_nrows : n;
-    for (int i = tid; work && i < nrows; i += nt) {
-      const int r = listed ? a.ep_rows[i] : i;
-      double2 s = make_double2(0.0, 0.0);
-      for (int e = a.ep_indptr[r]; e < a.ep_indptr[r + 1]; ++e) {
-        const double m = vals[e];
-        double2 x = sm.B[a.ep_indices[e]];
-        if (a.ep_mv_addvec) {
-          const double2 y = a.ep_mv_addvec[prow + a.ep_indices[e]];
-          x.x += y.x;
-          x.y += y.y;
-        }
-        s.x = fma(m, x.x, s.x);
-        s.y = fma(m, x.y, s.y);
-      }
-      if (mode == 2 && a.ep_from_b != 0.0) {
-        // L~ X~ = (B~ - alpha M~ X~) / beta for the stage matrix alpha M~ + beta L~
-        const double2 bb = a.bg[vec(r)];
-        s.x = (bb.x - a.ep_alpha * s.x) * a.ep_from_b;
-        s.y = (bb.y - a.ep_alpha * s.y) * a.ep_from_b;
-      }
-      a.ep_mv_store[prow + r] = s;
-    }
-  }
-  if (!finite) raise_status(a.status, SP_ERR_NONFINITE, p);
+  const bool work = !*sm.abort_flag;
+  if (work) pencil_epilogue(a, pp, tid, nt, mode == 2, vec, sm.B);
 }
 
 // 256 threads: two pencils' CTAs fit on one SM (registers capped at 128 per
 // thread), and the assembly and epilogue, bound by dependent global loads,
 // run twice as wide as with the two substituting warps' 128
 constexpr int SOLVE_THREADS = 256;
-template <int RU, int PPC>
+template <int RU>
 __global__ void __launch_bounds__(SOLVE_THREADS, 2) k_pencil_solve(SolveArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  pencil_solve_body<RU, PPC, -1, SOLVE_THREADS>(a, blockIdx.x, smem_raw);
+  pencil_solve_body<RU, -1, SOLVE_THREADS>(a, blockIdx.x, smem_raw);
 }
 // 128 threads, three CTAs per SM: for more pencils than two CTAs per SM
 // hold, more concurrent chains outweigh the narrower assembly and epilogue
 template <int RU>
 __global__ void __launch_bounds__(128, 3) k_pencil_solve_narrow(SolveArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  pencil_solve_body<RU, 1, -1, 128>(a, blockIdx.x, smem_raw);
+  pencil_solve_body<RU, -1, 128>(a, blockIdx.x, smem_raw);
 }
 
 // right-hand-side assembly only (MODE 1) or epilogue only (MODE 2), around
-// k_pencil_lanes: shared memory for B~ alone, several CTAs per SM
+// the lane substitution: shared memory for B~ alone, several CTAs per SM
 template <int MODE>
 __global__ void __launch_bounds__(128, 6) k_pencil_stage(SolveArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  pencil_solve_body<1, 1, MODE>(a, blockIdx.x, smem_raw);
-}
-
-// the same with 512-thread CTAs, for problems with few pencils (one CTA
-// per pencil would leave most of the GPU idle at 128 threads)
-template <int MODE>
-__global__ void __launch_bounds__(512, 2) k_pencil_stage_wide(SolveArgs a) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  pencil_solve_body<1, 1, MODE, 512>(a, blockIdx.x, smem_raw);
+  pencil_solve_body<1, MODE>(a, blockIdx.x, smem_raw);
 }
 
 // a batch of problems: work item (problem, pencil) per CTA
@@ -711,7 +516,7 @@ __global__ void __launch_bounds__(128, 4) k_pencil_solve_batched(const SolveArgs
                                                                  const int4* __restrict__ work) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int4 w = work[blockIdx.x];
-  pencil_solve_body<RU, 1>(args[w.x], w.y, smem_raw);
+  pencil_solve_body<RU>(args[w.x], w.y, smem_raw);
 }
 
 size_t pencil_solve_smem(int npad, int lpad, int upad) { return solve_smem_bytes(npad, lpad, upad); }
@@ -735,16 +540,6 @@ cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
   if (a.mode == 1 || a.mode == 2) {
     const size_t smem = solve_smem_bytes(a.npad, 0, 0);
     if (smem > 227 * 1024) return cudaErrorInvalidValue;
-    if (a.P < 2 * 152) {
-      if (a.mode == 1) {
-        cudaFuncSetAttribute(k_pencil_stage_wide<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_pencil_stage_wide<1><<<a.P, 512, smem, s>>>(a);
-      } else {
-        cudaFuncSetAttribute(k_pencil_stage_wide<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_pencil_stage_wide<2><<<a.P, 512, smem, s>>>(a);
-      }
-      return cudaGetLastError();
-    }
     if (a.mode == 1) {
       cudaFuncSetAttribute(k_pencil_stage<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       k_pencil_stage<1><<<a.P, 128, smem, s>>>(a);
@@ -754,10 +549,9 @@ cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
     }
     return cudaGetLastError();
   }
-  constexpr int PPC = 1;
-  const size_t smem = PPC * solve_smem_bytes(a.npad, a.lpad, a.upad);
+  const size_t smem = solve_smem_bytes(a.npad, a.lpad, a.upad);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  const int grid = (a.P + PPC - 1) / PPC;
+  const int grid = a.P;
   static int sms = 0;
   if (sms == 0) {
     int dev = 0;
@@ -777,11 +571,11 @@ cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
     return cudaGetLastError();
   }
   if (a.kuu <= 31) {
-    cudaFuncSetAttribute(k_pencil_solve<1, PPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_pencil_solve<1, PPC><<<grid, SOLVE_THREADS, smem, s>>>(a);
+    cudaFuncSetAttribute(k_pencil_solve<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_pencil_solve<1><<<grid, SOLVE_THREADS, smem, s>>>(a);
   } else {
-    cudaFuncSetAttribute(k_pencil_solve<2, PPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_pencil_solve<2, PPC><<<grid, SOLVE_THREADS, smem, s>>>(a);
+    cudaFuncSetAttribute(k_pencil_solve<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_pencil_solve<2><<<grid, SOLVE_THREADS, smem, s>>>(a);
   }
   return cudaGetLastError();
 }

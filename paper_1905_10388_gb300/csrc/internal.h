@@ -79,44 +79,24 @@ cudaError_t lane_list_build(cudaStream_t s, int P, int n, int npad, int kl, int 
                             const double* L, const uint8_t* piv, const double* U, LaneList& f);
 void lane_list_free(LaneList& f);
 
-// Partitioned substitution of problems with few pencils (spike.cu).
-struct SpikeArgs {
-  int P, n, npad, kl, kuu, lpad, upad;
-  int nblk, m;                  // back-substitution blocks per pencil and their rows
-  int nblk_f, m_f;              // forward-substitution blocks and rows (multiples of 8)
-  const double* L; const uint8_t* piv; const double* U; const double* rd;
-  const double* D; const double* E;
-  const double2* bg;            // B~ [p][n]
-  double2* yg;                  // y = L^-1 P B~ [p][n]
-  double2* xg;                  // x~ = y / U_jj [p][n] (the epilogue's input)
-  double* s0; double* sst;      // forward outflows / inflows [p][nblk_f][2][8]
-  double* o0; double* uin;      // backward outflows / inflows [p][nblk][2][32]
-  DevStatus* status;
-};
 // Problems with fewer pencils than this (and kl <= 7, kl + ku <= 31, at
 // least SPIKE_MIN_ROWS rows) use the partitioned substitution by default,
 // from LANE_SPLIT_PENCILS pencils on in its lane form (Fisher-KPP 2048 x 1024,
-// 1024 pencils: 0.41 ms per solve against 0.78 ms with the window kernel; with
-// 256 pencils of 2D Rayleigh-Benard the window form's passes over fewer,
-// longer blocks are the faster ones, 0.17 against 0.21 ms).
+// 1024 pencils: 0.41 ms per solve against 0.78 ms with the window kernel),
+// below that one CTA per pencil (2D Rayleigh-Benard 256 x 128, 128 pencils: 65
+// us per solve; eight launches of separate pass kernels took 110 us; 512 x 256,
+// 256 pencils: 188 us, the lane form 207 us).
 constexpr int SPIKE_MAX_PENCILS = 4096;
 constexpr int LANE_SPLIT_PENCILS = 608;
 constexpr int SPIKE_MIN_ROWS = 512;
+// Problems that have at most two CTAs per SM take it from fewer rows on (64 x
+// 32, 224 rows: 16 RK222 steps 2.27 ms with the window kernel, 2.10 ms).
+constexpr int SPLIT_MAX_PENCILS = 304;
+constexpr int SPLIT_MIN_ROWS = 96;
 bool spike_supported(int kl, int kuu, int npad, int nblk);
 bool spike_bwd_supported(int kuu, int npad, int nblk);
-cudaError_t launch_spike_coupling_bwd(cudaStream_t s, int P, int npad, int nblk, int kuu, int upad, const double* U,
-                                      double* E);
 cudaError_t launch_spike_coupling(cudaStream_t s, int P, int npad, int nblk_f, int nblk, int kl, int kuu, int lpad,
                                   int upad, const BandFactor& f, bool by_row);
-cudaError_t launch_spike_backward(cudaStream_t st, const SpikeArgs& s);
-cudaError_t launch_spike_solve(cudaStream_t s, const SpikeArgs& a);
-// forward blocks of the partitioned substitution: 128 rows, or 64 or 32 when
-// those divide the padded rows
-inline int spike_forward_blocks(int npad) {
-  for (int m = 128; m >= 32; m /= 2)
-    if (npad % m == 0) return npad / m;
-  return 1;
-}
 cudaError_t launch_spike_forward_rec(cudaStream_t s, const LaneArgs& a, const double* D);
 cudaError_t launch_spike_backward_rec(cudaStream_t s, const LaneArgs& a, const double* E);
 
@@ -210,23 +190,22 @@ struct SolveArgs {
   const int32_t* bc_rows; const double2* bc_values;
   DevStatus* status;
   // mode 0: assembly, substitution and epilogue in one kernel; 1: assembly
-  // only, B~ to bg; 2: epilogue only, from xg; [p][n] or by group
-  // (the substitution then runs in k_pencil_lanes or the partitioned
-  // kernels); 3: assembly and forward substitution, y = L^-1 P B~ to yg
-  // [p][n] (the partitioned back substitution follows)
+  // only, B~ to bg; 2: epilogue only, from xg (the lane substitution runs in
+  // between: bg, xg by group, xg holds b = U_jj x~).  The partitioned kernel
+  // keeps B~ [p][n] in bg for the epilogue's L~X~
   int mode;
-  double2* bg; const double2* xg; double2* yg;
+  double2* bg; const double2* xg;
   // 1: with kl <= 15, one warp runs both parts' forward substitution in two
   // 16-lane windows (half the FP64 issue; the batched solve, bound by the
   // FP64 pipe, sets it; a lone problem's whole-row chains are bound by their
   // latency and keep a 32-lane window per part)
   int fwd16;
-  // the factor's lists (host pointer; null: no lane substitution); by_group:
-  // bg, xg and yg are stored by group, xg holds b = U_jj x~
+  // the factor's lists (host pointer; null: no lane substitution)
   const LaneList* ll;
-  int by_group;
   // coupling matrices of the partitioned substitution (null: not available)
   const double* spD; const double* spE;
+  int sp_nblk, sp_nblk_f;       // back- and forward-substitution blocks per pencil
+  double* sp_u;                 // back-substitution inflows, the next solve's guesses [p][nblk][2][32]
 };
 
 // fc_half / fc_mhalf from fc_coef (exact scalings), before a launch
@@ -293,6 +272,11 @@ cudaError_t launch_eig_residual(cudaStream_t s, int P, int n, int nnz, const int
                                 const double* Mv, const double* Lv, const double2* x, const double2* sig,
                                 double* res);
 size_t pencil_solve_smem(int npad, int lpad, int upad);
+// partitioned pencil solve, one CTA per pencil (split.cu)
+cudaError_t launch_pencil_split(cudaStream_t s, const SolveArgs& a);
+cudaError_t launch_pencil_split_batched(cudaStream_t s, const SolveArgs* args, const int4* work, int nwork,
+                                        size_t smem);
+size_t pencil_split_smem(int npad, int nblk, int nblk_f, int kuu, bool wide);
 // batched pencil solves: one CTA per (problem, pencil) work item
 cudaError_t launch_pencil_solve_batched(cudaStream_t s, const SolveArgs* args, const int4* work, int nwork,
                                         int max_kuu, size_t smem);
