@@ -145,6 +145,13 @@ struct Problem {
   int32_t *d_eq_diff = nullptr, *d_eq_ph = nullptr, *d_bc_rows = nullptr, *d_nl_eq = nullptr;
   double2* d_bc_values = nullptr;
   double* d_kx = nullptr;
+  // the right-hand side on compile-time lengths (rows.cuh): variables that go
+  // through z, (variable, y derivative) pairs that go through y, and the grid
+  // fields' sources among them
+  bool rows_fast = false;
+  std::vector<int> zvars;
+  int nyf = 0;
+  int32_t *d_zvar = nullptr, *d_ysrc = nullptr, *d_ydy = nullptr, *d_xsrc = nullptr, *d_xdx = nullptr;
   int32_t *d_gvar = nullptr, *d_gop = nullptr, *d_tslot = nullptr, *d_tfa = nullptr, *d_tfb = nullptr;
   double* d_tcoef = nullptr;
   int32_t *d_ident = nullptr, *d_zero = nullptr;
@@ -412,6 +419,34 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
   for (auto& g : pr->gfields) { gv.push_back(g.var); go.push_back(g.op); }
   CK(upload(&pr->d_gvar, gv, s));
   CK(upload(&pr->d_gop, go, s));
+  {
+    pr->rows_fast = !gv.empty() && fft_planned(pr->Ngx) && fft_planned(pr->Ngz) &&
+                    (pr->ndim == 2 || fft_planned(pr->Ngy)) &&
+                    x_rows_bytes(pr->prec, pr->Ngx, (int)gv.size(), (int)pr->nl_eqs.size()) <= ROWS_SMEM_MAX &&
+                    z_cols_bytes(pr->prec, pr->Ngz) <= ROWS_SMEM_MAX &&
+                    (pr->ndim == 2 || z_cols_bytes(pr->prec, pr->Ngy) <= ROWS_SMEM_MAX);
+    auto place = [](std::vector<int>& v, int x) {
+      const size_t i = std::find(v.begin(), v.end(), x) - v.begin();
+      if (i == v.size()) v.push_back(x);
+      return (int32_t)i;
+    };
+    std::vector<int> yf;                         // 2 (index among zvars) + (1: y derivative)
+    std::vector<int32_t> xs, xd;
+    pr->zvars.clear();
+    for (size_t f = 0; f < gv.size(); ++f) {
+      const int zi = place(pr->zvars, gv[f]);
+      xs.push_back(pr->ndim == 3 ? place(yf, 2 * zi + (go[f] == SP_OP_DY ? 1 : 0)) : zi);
+      xd.push_back(go[f] == SP_OP_DX ? 1 : 0);
+    }
+    pr->nyf = (int)yf.size();
+    std::vector<int32_t> zv(pr->zvars.begin(), pr->zvars.end()), ys, yd;
+    for (int y : yf) { ys.push_back(y / 2); yd.push_back(y % 2); }
+    CK(upload(&pr->d_zvar, zv, s));
+    CK(upload(&pr->d_ysrc, ys, s));
+    CK(upload(&pr->d_ydy, yd, s));
+    CK(upload(&pr->d_xsrc, xs, s));
+    CK(upload(&pr->d_xdx, xd, s));
+  }
   CK(upload(&pr->d_tslot, pr->t_slot, s));
   CK(upload(&pr->d_tfa, pr->t_fa, s));
   CK(upload(&pr->d_tfb, pr->t_fb, s));
@@ -475,10 +510,15 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
   // rows into blocks substituted in parallel (spike.cu)
   pr->by_group = pr->lanes;
   pr->nblk = pr->spike_blocks > 0 ? pr->spike_blocks : default_spike_blocks(pr->npad, pr->P);
-  pr->nblk_f = pr->P >= LANE_SPLIT_PENCILS ? pr->nblk : default_forward_blocks(pr->npad);
+  // (a lower band wider than the 8-lane forward windows: forward blocks as
+  // long as the back ones, in the one-CTA form only)
+  const bool wide = pr->kl > 7;
+  pr->nblk_f = pr->P >= LANE_SPLIT_PENCILS || wide ? pr->nblk : default_forward_blocks(pr->npad);
   const bool split_fits = pr->P >= LANE_SPLIT_PENCILS ||
-                          pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false) <= 227 * 1024;
-  pr->spike = !pr->lanes && split_fits && spike_supported(pr->kl, kuu, pr->npad, pr->nblk) &&
+                          pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, kuu, wide) <= 227 * 1024;
+  const bool bands = wide ? pr->kl <= 30 && pr->P < LANE_SPLIT_PENCILS && spike_bwd_supported(kuu, pr->npad, pr->nblk)
+                          : spike_supported(pr->kl, kuu, pr->npad, pr->nblk);
+  pr->spike = !pr->lanes && split_fits && bands &&
               (pr->solve_kind == SP_SOLVE_SPIKE ||
                (pr->solve_kind == SP_SOLVE_AUTO && pr->P < SPIKE_MAX_PENCILS &&
                 (pr->npad >= SPIKE_MIN_ROWS || (pr->P <= SPLIT_MAX_PENCILS && pr->npad >= SPLIT_MIN_ROWS))));
@@ -510,7 +550,7 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
     CK(dalloc(&f.U, (size_t)pr->P * pr->npad * pr->upad));
     CK(dalloc(&f.rd, (size_t)pr->P * pr->npad));
     if (pr->spike) {
-      CK(dalloc(&f.spD, (size_t)pr->P * pr->nblk_f * 7 * 8));
+      CK(dalloc(&f.spD, (size_t)pr->P * pr->nblk_f * (wide ? 31 * 32 : 7 * 8)));
       CK(dalloc(&f.spE, (size_t)pr->P * pr->nblk * kuu * 32));
     }
   }
@@ -525,7 +565,7 @@ void free_problem(Problem* pr) {
   F(pr->d_var_rec); F(pr->d_var_ph); F(pr->d_eq_diff); F(pr->d_eq_ph); F(pr->d_bc_rows); F(pr->d_nl_eq);
 
   F(pr->d_cfl_grid); F(pr->d_cfl_mid1); F(pr->d_cfl_mid2); F(pr->d_inv_dz); F(pr->d_cfl_args); F(pr->d_cfl_out);
-  F(pr->d_bc_values); F(pr->d_kx); F(pr->d_gvar); F(pr->d_gop); F(pr->d_tslot); F(pr->d_tfa); F(pr->d_tfb);
+  F(pr->d_bc_values); F(pr->d_kx); F(pr->d_gvar); F(pr->d_gop); F(pr->d_zvar); F(pr->d_ysrc); F(pr->d_ydy); F(pr->d_xsrc); F(pr->d_xdx); F(pr->d_tslot); F(pr->d_tfa); F(pr->d_tfb);
   F(pr->d_tcoef); F(pr->d_ident); F(pr->d_zero); F(pr->d_Xt); F(pr->d_Xc); F(pr->d_Xc32); F(pr->d_kx32);
   F(pr->d_tcoef32);
   for (auto b : pr->d_MX) F(b);
@@ -579,6 +619,37 @@ cudaError_t coef_to_grid(Problem* pr, cudaStream_t s, int prec, int nf, Transfor
                              nullptr, nullptr, 0, nullptr);
 }
 
+// Descriptors of a problem's right-hand-side transforms (rows.cuh; the batched
+// run-time-length kernels where rows_fast is not set)
+ZDesc zdesc_backward(Problem* pr) {
+  TransformPlan& pz = pr->plans.at({pr->Nz, pr->Ngz});
+  ZDesc d{};
+  d.Nc = pz.Nc; d.Ng = pz.Ng; d.radix3 = pz.radix3; d.P = pr->P;
+  d.tw = pr->prec ? pz.tw32 : pz.tw64; d.wq = pr->prec ? pz.dct32 : pz.dct64;
+  d.f_var = pr->rows_fast ? pr->d_zvar : pr->d_gvar; d.f_op = pr->d_gop; d.kx = pr->d_kx; d.xc = pr->d_Xc;
+  d.xc_stride = pr->P * pr->Nz;
+  d.gz = pr->d_gz;
+  d.kx32 = pr->d_kx32; d.xc32 = pr->d_Xc32;
+  return d;
+}
+ZDesc zdesc_forward(Problem* pr, double2* fc) {
+  ZDesc d = zdesc_backward(pr);
+  d.h = pr->ndim == 3 ? pr->d_gz : pr->d_h; d.fc = fc;
+  return d;
+}
+XDesc xdesc_rows(Problem* pr) {
+  TransformPlan& px = pr->plans.at({pr->Nx, pr->Ngx});
+  XDesc d{};
+  d.N = px.Ng; d.radix3 = px.radix3; d.rows = pr->Ngz * pr->Ngy; d.K = pr->K; d.mode = 7; d.nf = (int)pr->gfields.size();
+  d.tw = pr->prec ? px.tw32 : px.tw64;
+  d.gz = pr->ndim == 3 ? pr->d_gy : pr->d_gz;
+  d.nterms = (int)pr->t_slot.size(); d.t_eq = pr->d_tslot; d.t_coef = pr->d_tcoef; d.t_fa = pr->d_tfa;
+  d.t_fb = pr->d_tfb; d.ne = (int)pr->nl_eqs.size(); d.h = pr->d_h;
+  d.t_coef32 = pr->d_tcoef32;
+  d.f_src = pr->d_xsrc; d.f_dx = pr->d_xdx; d.kx = pr->d_kx; d.kx32 = pr->d_kx32;
+  return d;
+}
+
 // F(X) for the current coefficient state: z backward -> (y backward) -> x
 // rows (products) -> (y forward) -> z forward
 sp_status eval_rhs(sp_ctx* ctx, Problem* pr, cudaStream_t s, double2* fc_out) {
@@ -599,12 +670,37 @@ sp_status eval_rhs(sp_ctx* ctx, Problem* pr, cudaStream_t s, double2* fc_out) {
       CK(launch_to_f32_split(s, pr->d_Xc, pr->cm.xs32, (size_t)pr->S * pr->P, pr->Nz));
       pr->xs32_valid = true;
     }
-    std::vector<int> fv(nf), fo(nf);
-    for (int f = 0; f < nf; ++f) { fv[f] = pr->gfields[f].var; fo[f] = pr->gfields[f].op; }
-    CK(launch_cheb_backward_mma(s, pr->cm, nf, fv.data(), fo.data(), pr->d_kx32, pr->d_gz, ctx->d_status));
+    std::vector<int> fv(pr->zvars), fo(pr->zvars.size(), SP_OP_ID);
+    if (!pr->rows_fast) {
+      fv.resize(nf);
+      fo.resize(nf);
+      for (int f = 0; f < nf; ++f) { fv[f] = pr->gfields[f].var; fo[f] = pr->gfields[f].op; }
+    }
+    CK(launch_cheb_backward_mma(s, pr->cm, (int)fv.size(), fv.data(), fo.data(), pr->d_kx32, pr->d_gz, ctx->d_status));
+  } else if (pr->rows_fast) {
+    CK(pr->prec ? launch_z_cols<float>(s, zdesc_backward(pr), (int)pr->zvars.size(), false)
+                : launch_z_cols<double>(s, zdesc_backward(pr), (int)pr->zvars.size(), false));
   } else {
     CK(launch_cheb_backward(s, pr->prec, pz, pr->P, nf, pr->d_gvar, pr->d_gop, pr->d_kx, pr->d_Xc,
                             pr->P * pr->Nz, pr->d_gz, pr->d_kx32, pr->d_Xc32));
+  }
+  if (pr->rows_fast) {
+    XDesc x = xdesc_rows(pr);
+    ZDesc z = zdesc_forward(pr, fc_out);
+    YDesc y{};
+    if (pr->ndim == 3) {
+      TransformPlan& py = pr->plans.at({pr->Ny, pr->Ngy});
+      y.Ny = py.Nc; y.Ng = py.Ng; y.K = pr->K; y.nz = pr->Ngz;
+      y.tw = pr->prec ? py.tw32 : py.tw64;
+      y.f_src = pr->d_ysrc; y.f_dy = pr->d_ydy; y.ky = pr->d_kx + pr->P; y.ky32 = pr->prec ? pr->d_kx32 + pr->P : nullptr;
+      y.dir = -1; y.src = pr->d_gz; y.dst = pr->d_gy;
+      CK(pr->prec ? launch_y_cols<float>(s, y, pr->nyf) : launch_y_cols<double>(s, y, pr->nyf));
+      y.dir = 1; y.src = pr->d_h; y.dst = pr->d_gz;
+    }
+    CK(pr->prec ? launch_x_rows<float>(s, x) : launch_x_rows<double>(s, x));
+    if (pr->ndim == 3) CK(pr->prec ? launch_y_cols<float>(s, y, ne) : launch_y_cols<double>(s, y, ne));
+    CK(pr->prec ? launch_z_cols<float>(s, z, ne, true) : launch_z_cols<double>(s, z, ne, true));
+    return SP_OK;
   }
   if (pr->ndim == 3) {
     TransformPlan& py = pr->plans.at({pr->Ny, pr->Ngy});
@@ -845,33 +941,6 @@ sp_status one_step(sp_ctx* ctx, Problem* pr, cudaStream_t s, double dt) {
 // ---------------------------------------------------------------------------
 // batches: every kernel type launched once per stage over all problems
 // ---------------------------------------------------------------------------
-ZDesc zdesc_backward(Problem* pr) {
-  TransformPlan& pz = pr->plans.at({pr->Nz, pr->Ngz});
-  ZDesc d{};
-  d.Nc = pz.Nc; d.Ng = pz.Ng; d.radix3 = pz.radix3; d.P = pr->P;
-  d.tw = pr->prec ? pz.tw32 : pz.tw64; d.wq = pr->prec ? pz.dct32 : pz.dct64;
-  d.f_var = pr->d_gvar; d.f_op = pr->d_gop; d.kx = pr->d_kx; d.xc = pr->d_Xc; d.xc_stride = pr->P * pr->Nz;
-  d.gz = pr->d_gz;
-  d.kx32 = pr->d_kx32; d.xc32 = pr->d_Xc32;
-  return d;
-}
-ZDesc zdesc_forward(Problem* pr, double2* fc) {
-  ZDesc d = zdesc_backward(pr);
-  d.h = pr->d_h; d.fc = fc;
-  return d;
-}
-XDesc xdesc_rows(Problem* pr) {
-  TransformPlan& px = pr->plans.at({pr->Nx, pr->Ngx});
-  XDesc d{};
-  d.N = px.Ng; d.radix3 = px.radix3; d.rows = pr->Ngz; d.K = pr->P; d.mode = 7; d.nf = (int)pr->gfields.size();
-  d.tw = pr->prec ? px.tw32 : px.tw64;
-  d.gz = pr->d_gz;
-  d.nterms = (int)pr->t_slot.size(); d.t_eq = pr->d_tslot; d.t_coef = pr->d_tcoef; d.t_fa = pr->d_tfa;
-  d.t_fb = pr->d_tfb; d.ne = (int)pr->nl_eqs.size(); d.h = pr->d_h;
-  d.t_coef32 = pr->d_tcoef32;
-  return d;
-}
-
 // --- adjoint ---------------------------------------------------------------
 // Solve arguments for A~^T y = rhs with the transposed factor (no right-hand
 // side assembly beyond stored vectors, no boundary values).
@@ -931,6 +1000,8 @@ struct Batch {
   int max_ngz = 0, max_kuu = 0;
   size_t x_smem = 0, s_smem = 0;
   bool split = false;                        // every problem's solves in the partitioned kernel
+  bool fast = false;                         // every problem's transforms on compile-time lengths
+  size_t z_smem = 0;
   int4 *d_wzb = nullptr, *d_wx = nullptr, *d_wzf = nullptr, *d_ws = nullptr;
   int nzb = 0, nx = 0, nzf = 0, ns = 0;
   std::vector<BatchStage> stages;
@@ -969,17 +1040,19 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
   // few pencils in all: the solves' latency counts, so each problem's
   // partitioned form; more: the FP64 pipe does, so whole pencils
   int pencils = 0;
-  b->split = true;
+  b->split = b->fast = true;
   for (Problem* pr : ps) {
     pencils += pr->P;
-    b->split = b->split && pr->spike && !pr->by_group;
+    b->fast = b->fast && pr->rows_fast;
+    b->split = b->split && pr->spike && !pr->by_group && pr->kl <= 7;
   }
   b->split = b->split && pencils <= SPLIT_MAX_PENCILS;
   for (size_t q = 0; q < ps.size(); ++q) {
     Problem* pr = ps[q];
-    const int nt = (pr->P + tile - 1) / tile;
+    const int tl = b->fast ? z_cols_tile(pr->prec) : tile;
+    const int nt = (pr->P + tl - 1) / tl;
     const long long zc = (long long)pr->Ngz * 100 + pr->Nz;
-    for (int f = 0; f < (int)pr->gfields.size(); ++f)
+    for (int f = 0; f < (int)(b->fast ? pr->zvars.size() : pr->gfields.size()); ++f)
       for (int t = 0; t < nt; ++t) zb.push_back({zc, make_int4((int)q, t, f, 0)});
     for (int e = 0; e < (int)pr->nl_eqs.size(); ++e)
       for (int t = 0; t < nt; ++t) zf.push_back({zc, make_int4((int)q, t, e, 0)});
@@ -987,8 +1060,10 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
     for (int p = 0; p < pr->P; ++p) sv.push_back({(long long)pr->n, make_int4((int)q, p, 0, 0)});
     b->max_ngz = std::max(b->max_ngz, pr->Ngz);
     b->max_kuu = std::max(b->max_kuu, pr->kl + pr->ku);
-    b->x_smem = std::max(b->x_smem, x_smem_bytes(pr->prec, pr->Ngx, 7, (int)pr->gfields.size(),
-                                                 (int)pr->nl_eqs.size()));
+    const int nf = (int)pr->gfields.size(), ne = (int)pr->nl_eqs.size();
+    b->x_smem = std::max(b->x_smem, b->fast ? x_rows_bytes(pr->prec, pr->Ngx, nf, ne)
+                                            : x_smem_bytes(pr->prec, pr->Ngx, 7, nf, ne));
+    b->z_smem = std::max(b->z_smem, z_cols_bytes(pr->prec, pr->Ngz));
     b->s_smem = std::max(b->s_smem, b->split ? pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false)
                                              : pencil_solve_smem(pr->npad, pr->lpad, pr->upad));
   }
@@ -1021,6 +1096,7 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
     std::vector<SolveArgs> av;
     for (size_t q = 0; q < ps.size(); ++q) {
       zbv.push_back(zdesc_backward(ps[q]));
+      if (!b->fast) zbv.back().f_var = ps[q]->d_gvar;
       xv.push_back(xdesc_rows(ps[q]));
       zfv.push_back(zdesc_forward(ps[q], plans[q][i].fc_out));
       av.push_back(plans[q][i].args);
@@ -1061,9 +1137,20 @@ sp_status batch_step(sp_ctx* ctx, Batch* b, cudaStream_t s) {
   for (int i = 0; i < b->nstage; ++i) {
     const BatchStage& st = b->stages[i];
     int* q = b->persist ? b->d_queue + 4 * i : nullptr;
-    CK(launch_cheb_backward_batched(s, b->prec, b->tile, st.d_zb, b->d_wzb, b->nzb, b->max_ngz, q));
-    CK(launch_fourier_rows_batched(s, b->prec, st.d_x, b->d_wx, b->nx, b->x_smem, q ? q + 1 : nullptr));
-    CK(launch_cheb_forward_batched(s, b->prec, b->tile, st.d_zf, b->d_wzf, b->nzf, b->max_ngz, q ? q + 2 : nullptr));
+    int *q1 = q ? q + 1 : nullptr, *q2 = q ? q + 2 : nullptr;
+    if (b->fast && b->prec) {
+      CK(launch_z_cols_batched<float>(s, false, st.d_zb, b->d_wzb, b->nzb, b->z_smem, q));
+      CK(launch_x_rows_batched<float>(s, st.d_x, b->d_wx, b->nx, b->x_smem, q1));
+      CK(launch_z_cols_batched<float>(s, true, st.d_zf, b->d_wzf, b->nzf, b->z_smem, q2));
+    } else if (b->fast) {
+      CK(launch_z_cols_batched<double>(s, false, st.d_zb, b->d_wzb, b->nzb, b->z_smem, q));
+      CK(launch_x_rows_batched<double>(s, st.d_x, b->d_wx, b->nx, b->x_smem, q1));
+      CK(launch_z_cols_batched<double>(s, true, st.d_zf, b->d_wzf, b->nzf, b->z_smem, q2));
+    } else {
+      CK(launch_cheb_backward_batched(s, b->prec, b->tile, st.d_zb, b->d_wzb, b->nzb, b->max_ngz, q));
+      CK(launch_fourier_rows_batched(s, b->prec, st.d_x, b->d_wx, b->nx, b->x_smem, q1));
+      CK(launch_cheb_forward_batched(s, b->prec, b->tile, st.d_zf, b->d_wzf, b->nzf, b->max_ngz, q2));
+    }
     if (b->split) CK(launch_pencil_split_batched(s, st.d_args, b->d_ws, b->ns, b->s_smem));
     else CK(launch_pencil_solve_batched(s, st.d_args, b->d_ws, b->ns, b->max_kuu, b->s_smem));
   }
@@ -1658,7 +1745,10 @@ sp_status sp_step_batched(sp_ctx* ctx, int nproblems, const int* problem_ids, co
     CK(cudaEventCreate(&e1));
     int best = 8;
     float best_ms = 1e30f;
+    const bool fast = std::all_of(ps.begin(), ps.end(), [](Problem* pr) { return pr->rows_fast; });
+    if (fast) best = z_cols_tile(ps[0]->prec);   // compile-time lengths: one tile, nothing to choose
     for (int tile : {4, 8, 16}) {
+      if (fast) break;
       Batch* b = get_batch(multistep ? ps[0]->iteration % D : 0, tile, false);
       if (!b) return fail(ctx, SP_ERR_CUDA, "building batch: %s", ctx->err.c_str());
       // the transform kernels write only scratch buffers that the next step overwrites

@@ -1,0 +1,243 @@
+// Shared-memory Stockham FFT passes of compile-time length N = 2^k or 3 * 2^k,
+// two or three per transform, each butterfly in one thread's registers.
+//
+// A pass of radix R over sub-transforms of length Ns: butterfly j < N / R reads
+// the R elements j + t N / R, twiddles element t by W_N^{t k N / (R Ns)}, k = j
+// mod Ns, and writes the R outputs (j / Ns) R Ns + k + q Ns; the first pass has
+// Ns = 1 and no twiddles and takes the factor 3, and the result is in natural
+// order.  With N a template constant every index is a shift, a mask or an
+// immediate: at run-time lengths the index arithmetic alone was most of the
+// FP32 kernels' instructions.
+//
+// Twiddled butterflies split even and odd inputs with one common factor:
+// E_q = sum_s a_{2s} w^{2s} r^{2qs}, O_q the same sum of a_{2s+1}, X_{q, q+R/2} =
+// E_q +- w r^q O_q (r = exp(sign 2 pi i / R)), down to single elements.  Each
+// two-point step is four FMAs for E + w O and two for E - w O = 2 E - (E + w O):
+// 72 FP instructions and 4 twiddle loads for radix 8, against 84 and 7 with
+// the inputs multiplied first.
+//
+// Buffers are padded by one element every 128 bytes, so the first pass's
+// stride-R writes spread over the banks.
+#pragma once
+#include "common.cuh"
+
+namespace spectau {
+
+template <int N>
+struct FftPlan;   // R0, R1, R2 (1: two passes)
+#define SP_FFT_PLAN(n, a, b, c)                       \
+  template <>                                         \
+  struct FftPlan<n> {                                 \
+    static constexpr int R0 = a, R1 = b, R2 = c;      \
+    static_assert(a * b * c == n, "radices");         \
+  };
+SP_FFT_PLAN(16, 4, 4, 1)
+SP_FFT_PLAN(24, 6, 4, 1)
+SP_FFT_PLAN(32, 8, 4, 1)
+SP_FFT_PLAN(48, 3, 4, 4)
+SP_FFT_PLAN(64, 4, 4, 4)
+SP_FFT_PLAN(96, 6, 4, 4)
+SP_FFT_PLAN(128, 8, 4, 4)
+SP_FFT_PLAN(192, 6, 8, 4)
+SP_FFT_PLAN(256, 8, 8, 4)
+SP_FFT_PLAN(384, 6, 8, 8)
+SP_FFT_PLAN(512, 8, 8, 8)
+SP_FFT_PLAN(768, 12, 8, 8)
+SP_FFT_PLAN(1024, 16, 8, 8)
+SP_FFT_PLAN(1536, 12, 16, 8)
+SP_FFT_PLAN(2048, 16, 16, 8)
+SP_FFT_PLAN(3072, 12, 16, 16)
+SP_FFT_PLAN(4096, 16, 16, 16)
+#undef SP_FFT_PLAN
+
+template <typename T>
+__device__ __forceinline__ constexpr int fft_pad(int i) { return i + (sizeof(T) == 4 ? (i >> 4) : (i >> 3)); }
+// elements of a padded buffer of N
+template <typename T>
+__host__ __device__ constexpr int fft_padded(int N) { return N + (sizeof(T) == 4 ? N / 16 : N / 8); }
+
+// z times exp(SIGN i pi / 2)
+template <typename T, int SIGN>
+__device__ __forceinline__ C<T> rot90(C<T> z) { return SIGN < 0 ? mk<T>(z.y, -z.x) : mk<T>(-z.y, z.x); }
+
+// E + w O, E - w O
+template <typename T>
+__device__ __forceinline__ void bfly(C<T> e, C<T> o, C<T> w, C<T>& p, C<T>& m) {
+  p.x = fma(-w.y, o.y, fma(w.x, o.x, e.x));
+  p.y = fma(w.y, o.x, fma(w.x, o.y, e.y));
+  m.x = fma((T)2, e.x, -p.x);
+  m.y = fma((T)2, e.y, -p.y);
+}
+
+// DFT of length R (a power of two) of a[0], a[S], a[2S], ... with the common
+// twiddle w: out[q] = sum_t a[t S] w^t r^{qt}; tw[base] = conj-adjusted powers.
+// `at(m, q, R)` returns w^m exp(SIGN 2 pi i q / R) for q < R / 4.
+template <typename T, int SIGN, int R, int S, int M, typename W>
+struct DitTw {
+  static __device__ __forceinline__ void run(const C<T>* a, C<T>* out, const W& at) {
+    C<T> e[R / 2], o[R / 2];
+    DitTw<T, SIGN, R / 2, 2 * S, 2 * M, W>::run(a, e, at);
+    DitTw<T, SIGN, R / 2, 2 * S, 2 * M, W>::run(a + S, o, at);
+    if (R == 2) {
+      bfly<T>(e[0], o[0], at(M, 0, 2), out[0], out[1]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < R / 4; ++q) {
+        const C<T> w = at(M, q, R);
+        bfly<T>(e[q], o[q], w, out[q], out[q + R / 2]);
+        bfly<T>(e[q + R / 4], o[q + R / 4], rot90<T, SIGN>(w), out[q + R / 4], out[q + 3 * R / 4]);
+      }
+    }
+  }
+};
+template <typename T, int SIGN, int S, int M, typename W>
+struct DitTw<T, SIGN, 1, S, M, W> {
+  static __device__ __forceinline__ void run(const C<T>* a, C<T>* out, const W&) { out[0] = a[0]; }
+};
+
+// The same without twiddles (first pass): constant roots, the trivial ones as
+// sums and differences.
+template <typename T, int SIGN, int R, int S>
+struct Dit {
+  static __device__ __forceinline__ void run(const C<T>* a, C<T>* out) {
+    C<T> e[R / 2], o[R / 2];
+    Dit<T, SIGN, R / 2, 2 * S>::run(a, e);
+    Dit<T, SIGN, R / 2, 2 * S>::run(a + S, o);
+#pragma unroll
+    for (int q = 0; q < R / 2; ++q) {
+      if (q == 0) {
+        out[0] = cadd<T>(e[0], o[0]);
+        out[R / 2] = csub<T>(e[0], o[0]);
+      } else if (4 * q == R) {
+        const C<T> v = rot90<T, SIGN>(o[q]);
+        out[q] = cadd<T>(e[q], v);
+        out[q + R / 2] = csub<T>(e[q], v);
+      } else {
+        constexpr double c1 = 0.92387953251128675613, s1 = 0.38268343236508977173, h = 0.70710678118654752440;
+        const int u = q * 16 / R;                // root exp(SIGN 2 pi i u / 16), u = 1, 2, 3, 5, 6, 7
+        const double cr = u == 1 ? c1 : u == 2 ? h : u == 3 ? s1 : u == 5 ? -s1 : u == 6 ? -h : -c1;
+        const double ci = u == 1 ? s1 : u == 2 ? h : u == 3 ? c1 : u == 5 ? c1 : u == 6 ? h : s1;
+        bfly<T>(e[q], o[q], mk<T>((T)cr, (T)(SIGN < 0 ? -ci : ci)), out[q], out[q + R / 2]);
+      }
+    }
+  }
+};
+template <typename T, int SIGN, int S>
+struct Dit<T, SIGN, 1, S> {
+  static __device__ __forceinline__ void run(const C<T>* a, C<T>* out) { out[0] = a[0]; }
+};
+
+// 3-point DFT: sums, differences and FMAs with -1/2 and sqrt(3)/2
+template <typename T, int SIGN>
+__device__ __forceinline__ void dft3(C<T> a0, C<T> a1, C<T> a2, C<T>& x0, C<T>& x1, C<T>& x2) {
+  const T c = (SIGN < 0 ? (T)-1 : (T)1) * (T)0.86602540378443864676;
+  const C<T> s = cadd<T>(a1, a2), d = csub<T>(a1, a2);
+  const C<T> m = mk<T>(fma((T)-0.5, s.x, a0.x), fma((T)-0.5, s.y, a0.y));
+  x0 = cadd<T>(a0, s);
+  x1 = mk<T>(fma(-c, d.y, m.x), fma(c, d.x, m.y));
+  x2 = mk<T>(fma(c, d.y, m.x), fma(-c, d.x, m.y));
+}
+
+// First-pass DFT of R0 = 2^a or 3 2^a elements.  The factor 3 by the prime
+// factor map (coprime factors need no twiddles): with R = 3 H, input (H n1 + 3
+// n2) mod R and output k = k1 mod 3, k2 mod H.
+template <typename T, int SIGN, int R>
+__device__ __forceinline__ void dft_first(const C<T>* a, C<T>* out) {
+  if constexpr (R % 3 == 0) {
+    constexpr int H = R / 3;
+    C<T> b[3][H];
+#pragma unroll
+    for (int n2 = 0; n2 < H; ++n2)
+      dft3<T, SIGN>(a[(3 * n2) % R], a[(H + 3 * n2) % R], a[(2 * H + 3 * n2) % R], b[0][n2], b[1][n2], b[2][n2]);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+      C<T> o[H];
+      Dit<T, SIGN, H, 1>::run(b[k1], o);
+#pragma unroll
+      for (int k2 = 0; k2 < H; ++k2) {
+        // the k in [0, R) with H k = k1 H (mod 3 H) after the maps: k = k1 (H
+        // H^-1 mod 3) + k2 (3 3^-1 mod H)
+        constexpr int hi = H % 3 == 1 ? 1 : 2;                        // H^-1 mod 3
+        constexpr int ti = H == 1 ? 0 : H == 2 ? 1 : H == 4 ? 3 : 3;  // 3^-1 mod H (H = 1, 2, 4, 8)
+        out[(H * hi * k1 + 3 * ti * k2) % R] = o[k2];
+      }
+    }
+  } else {
+    Dit<T, SIGN, R, 1>::run(a, out);
+  }
+}
+
+// First pass over nb sequences: `in(b, i)` gives element i of sequence b.
+template <typename T, int N, int SIGN, int NT, typename IN, typename OUT>
+__device__ __forceinline__ void fft_pass_first(int nb, IN&& in, OUT&& out) {
+  constexpr int R = FftPlan<N>::R0, Q = N / R;
+  for (int id = threadIdx.x; id < nb * Q; id += NT) {
+    const int b = id / Q, j = id - b * Q;
+    C<T> a[R], y[R];
+#pragma unroll
+    for (int t = 0; t < R; ++t) a[t] = in(b, j + t * Q);
+    dft_first<T, SIGN, R>(a, y);
+#pragma unroll
+    for (int q = 0; q < R; ++q) out(b, j * R + q, y[q]);
+  }
+}
+
+// A twiddled pass of radix R over sub-transforms of length Ns from padded
+// buffers x (sequence stride NP): `out(b, i, v)` takes element i of sequence b.
+template <typename T, int N, int SIGN, int NT, int R, int Ns, typename OUT>
+__device__ __forceinline__ void fft_pass_tw(const C<T>* __restrict__ x, const C<T>* __restrict__ tw, int nb,
+                                            OUT&& out) {
+  constexpr int Q = N / R, NP = fft_padded<T>(N), STEP = N / (R * Ns);
+  for (int id = threadIdx.x; id < nb * Q; id += NT) {
+    const int b = id / Q, j = id - b * Q;
+    const int k = j % Ns, g = j / Ns;
+    const C<T>* xb = x + b * NP;
+    C<T> a[R], y[R];
+#pragma unroll
+    for (int t = 0; t < R; ++t) a[t] = xb[fft_pad<T>(j + t * Q)];
+    const int w0 = k * STEP;
+    auto at = [&](int m, int q, int r) {
+      C<T> w = tw[m * w0 + q * (N / r)];
+      return SIGN > 0 ? mk<T>(w.x, -w.y) : w;
+    };
+    DitTw<T, SIGN, R, 1, 1, decltype(at)>::run(a, y, at);
+    const int o = g * R * Ns + k;
+#pragma unroll
+    for (int q = 0; q < R; ++q) out(b, o + q * Ns, y[q]);
+  }
+}
+
+// Transforms nb sequences: `in` as above, results to `fin(b, i, v)` in natural
+// order.  A three-pass transform goes through buffer u, then v; a two-pass one
+// through v only (fin may write where u is).  Ends after a barrier.
+template <typename T, int N, int SIGN, int NT, typename IN, typename FIN>
+__device__ __forceinline__ void fft_run(int nb, C<T>* u, C<T>* v, const C<T>* tw, IN&& in, FIN&& fin) {
+  using P = FftPlan<N>;
+  constexpr int NP = fft_padded<T>(N);
+  C<T>* first = P::R2 > 1 ? u : v;
+  fft_pass_first<T, N, SIGN, NT>(nb, in, [&](int b, int i, C<T> z) { first[b * NP + fft_pad<T>(i)] = z; });
+  __syncthreads();
+  if constexpr (P::R2 > 1) {
+    fft_pass_tw<T, N, SIGN, NT, P::R1, P::R0>(u, tw, nb, [&](int b, int i, C<T> z) { v[b * NP + fft_pad<T>(i)] = z; });
+    __syncthreads();
+    fft_pass_tw<T, N, SIGN, NT, P::R2, P::R0 * P::R1>(v, tw, nb, fin);
+  } else {
+    fft_pass_tw<T, N, SIGN, NT, P::R1, P::R0>(v, tw, nb, fin);
+  }
+  __syncthreads();
+}
+
+// calls f(std::integral_constant<int, N>) for a length of the plans above
+template <typename F>
+cudaError_t fft_dispatch(int N, F&& f) {
+  switch (N) {
+#define SP_FFT_CASE(n) case n: return f(std::integral_constant<int, n>());
+    SP_FFT_CASE(16) SP_FFT_CASE(24) SP_FFT_CASE(32) SP_FFT_CASE(48) SP_FFT_CASE(64) SP_FFT_CASE(96)
+    SP_FFT_CASE(128) SP_FFT_CASE(192) SP_FFT_CASE(256) SP_FFT_CASE(384) SP_FFT_CASE(512) SP_FFT_CASE(768)
+    SP_FFT_CASE(1024) SP_FFT_CASE(1536) SP_FFT_CASE(2048) SP_FFT_CASE(3072) SP_FFT_CASE(4096)
+#undef SP_FFT_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace spectau

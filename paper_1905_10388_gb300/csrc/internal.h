@@ -251,6 +251,8 @@ struct XDesc {
   const void* hin; void* gzadj;             // adjoint rows: inputs / outputs
   int xscale;                                // bit 1: transpose of forward x on input; bit 2: of backward x on output
   int pairs;                                 // field pairs per backward FFT round (0: two)
+  // rows.cuh: grid field f is input f_src[f], times i k_x where f_dx[f] is set
+  const int32_t* f_src; const int32_t* f_dx; const double* kx; const float* kx32;
 };
 
 // Complex Fourier y transform of nf x nz planes of N_y slots x K columns.
@@ -258,6 +260,9 @@ struct YDesc {
   int Ny, Ng, K, nz, radix3, dir;
   const void* tw;
   const void* src; void* dst;
+  // rows.cuh, dir < 0: output f is input f_src[f], times i k_y where f_dy[f] is
+  // set (ky, ky32: one value per slot, K apart)
+  const int32_t* f_src; const int32_t* f_dy; const double* ky; const float* ky32;
 };
 
 // --- launchers (band.cu) ---------------------------------------------------
@@ -314,6 +319,29 @@ cudaError_t launch_fourier_y(cudaStream_t s, int prec, const TransformPlan& py, 
                              const void* src, void* dst);
 size_t z_smem_bytes(int prec, int Ng, int tile);
 size_t x_smem_bytes(int prec, int N, int mode, int nf, int ne, int pairs = 0);
+// the right-hand side's transforms on compile-time lengths (rows.cuh), float or
+// double; cudaErrorInvalidValue for a length or size they do not take
+constexpr size_t ROWS_SMEM_MAX = 226 * 1024;   // dynamic shared memory of a CTA, its static tables beside it
+inline bool fft_planned(int N) { return N >= 16 && N <= 4096 && (((N & (N - 1)) == 0) || (N % 3 == 0 && (((N / 3) & (N / 3 - 1)) == 0))); }
+inline size_t rows_padded(int prec, int N) { return (size_t)(N + (prec ? N / 16 : N / 8)) * (prec ? 8 : 16); }
+inline size_t x_rows_bytes(int prec, int N, int nf, int ne) {
+  const int nbi = (nf + 1) / 2, nbo = (ne + 1) / 2;
+  return (nbi + (nbi > 2 * nbo ? nbi : 2 * nbo)) * rows_padded(prec, N);
+}
+inline int z_cols_tile(int prec) { return prec ? 8 : 4; }
+inline size_t z_cols_bytes(int prec, int N) {   // two buffers of tile columns, each one element over a multiple of 16
+  const size_t el = N + (prec ? N / 16 : N / 8);
+  return 2 * z_cols_tile(prec) * ((el + 15) / 16 * 16 + 1) * (prec ? 8 : 16);
+}
+template <typename T> cudaError_t launch_x_rows(cudaStream_t s, const XDesc& d);
+template <typename T> cudaError_t launch_y_cols(cudaStream_t s, const YDesc& d, int nf);
+template <typename T> cudaError_t launch_z_cols(cudaStream_t s, const ZDesc& d, int nf, bool forward);
+template <typename T>
+cudaError_t launch_x_rows_batched(cudaStream_t s, const XDesc* ds, const int4* work, int nwork, size_t smem,
+                                  int* queue);
+template <typename T>
+cudaError_t launch_z_cols_batched(cudaStream_t s, bool forward, const ZDesc* ds, const int4* work, int nwork,
+                                  size_t smem, int* queue);
 // batched transforms: queue null: one CTA per work item; else a persistent
 // grid pulling items from the device counter *queue (zero before the launch)
 cudaError_t launch_cheb_backward_batched(cudaStream_t s, int prec, int tile, const ZDesc* ds, const int4* work,

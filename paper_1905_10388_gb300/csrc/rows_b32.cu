@@ -1,0 +1,7 @@
+// batched x rows and z transforms, float (rows.cuh)
+#include "rows.cuh"
+
+namespace spectau {
+template cudaError_t launch_x_rows_batched<float>(cudaStream_t, const XDesc*, const int4*, int, size_t, int*);
+template cudaError_t launch_z_cols_batched<float>(cudaStream_t, bool, const ZDesc*, const int4*, int, size_t, int*);
+}  // namespace spectau

@@ -448,7 +448,7 @@ cudaError_t launch_pencil_split(cudaStream_t s, const SolveArgs& args) {
   SolveArgs a = args;
   fill_f_halves(a);
   const bool wide = a.kl > 7;
-  if (a.kl > 31 || a.kuu >= SPL_W || a.upad != SPL_W || a.npad % (a.sp_nblk * SOLVE_CHUNK) ||
+  if (a.kl > 30 || a.kuu >= SPL_W || a.upad != SPL_W || a.npad % (a.sp_nblk * SOLVE_CHUNK) ||
       a.npad % (a.sp_nblk_f * SOLVE_CHUNK))
     return cudaErrorInvalidValue;
   const size_t smem = pencil_split_smem(a.npad, a.sp_nblk, a.sp_nblk_f, a.kuu, wide);
