@@ -151,6 +151,7 @@ struct Problem {
   bool rows_fast = false;
   std::vector<int> zvars;
   int nyf = 0;
+  void *d_zb = nullptr, *d_zf = nullptr;     // z tables, in the precision
   int32_t *d_zvar = nullptr, *d_ysrc = nullptr, *d_ydy = nullptr, *d_xsrc = nullptr, *d_xdx = nullptr;
   int32_t *d_gvar = nullptr, *d_gop = nullptr, *d_tslot = nullptr, *d_tfa = nullptr, *d_tfb = nullptr;
   double* d_tcoef = nullptr;
@@ -423,6 +424,7 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
     pr->rows_fast = !gv.empty() && fft_planned(pr->Ngx) && fft_planned(pr->Ngz) &&
                     (pr->ndim == 2 || fft_planned(pr->Ngy)) &&
                     x_rows_bytes(pr->prec, pr->Ngx, (int)gv.size(), (int)pr->nl_eqs.size()) <= ROWS_SMEM_MAX &&
+                    x_smem_bytes(pr->prec, pr->Ngx, 7, (int)gv.size(), (int)pr->nl_eqs.size()) <= 227 * 1024 &&
                     z_cols_bytes(pr->prec, pr->Ngz) <= ROWS_SMEM_MAX &&
                     (pr->ndim == 2 || z_cols_bytes(pr->prec, pr->Ngy) <= ROWS_SMEM_MAX);
     auto place = [](std::vector<int>& v, int x) {
@@ -441,6 +443,28 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
     pr->nyf = (int)yf.size();
     std::vector<int32_t> zv(pr->zvars.begin(), pr->zvars.end()), ys, yd;
     for (int y : yf) { ys.push_back(y / 2); yd.push_back(y % 2); }
+    // w_k = exp(-i pi k / (2 N)) with what the transforms fold into it (rows.cuh)
+    std::vector<double2> zb(pr->Ngz), zf(pr->Ngz);
+    const double pi = 3.14159265358979323846;
+    const double hs = 1.0 / (2.0 * pr->Ngx) / (pr->ndim == 3 ? pr->Ngy : 1);
+    for (int k = 0; k < pr->Ngz; ++k) {
+      const double c = std::cos(pi * k / (2.0 * pr->Ngz)), n = -std::sin(pi * k / (2.0 * pr->Ngz));
+      const double b = k == 0 ? 1.0 : (k % 2 ? -0.5 : 0.5), f = (k % 2 ? -1.0 : 1.0) * (k == 0 ? 0.5 : 1.0) * hs / pr->Ngz;
+      zb[k] = make_double2(b * c, b * n);
+      zf[k] = make_double2(f * c, f * n);
+    }
+    if (pr->prec) {
+      std::vector<float2> b32, f32;
+      for (int k = 0; k < pr->Ngz; ++k) {
+        b32.push_back(make_float2((float)zb[k].x, (float)zb[k].y));
+        f32.push_back(make_float2((float)zf[k].x, (float)zf[k].y));
+      }
+      CK(upload((float2**)&pr->d_zb, b32, s));
+      CK(upload((float2**)&pr->d_zf, f32, s));
+    } else {
+      CK(upload((double2**)&pr->d_zb, zb, s));
+      CK(upload((double2**)&pr->d_zf, zf, s));
+    }
     CK(upload(&pr->d_zvar, zv, s));
     CK(upload(&pr->d_ysrc, ys, s));
     CK(upload(&pr->d_ydy, yd, s));
@@ -565,7 +589,7 @@ void free_problem(Problem* pr) {
   F(pr->d_var_rec); F(pr->d_var_ph); F(pr->d_eq_diff); F(pr->d_eq_ph); F(pr->d_bc_rows); F(pr->d_nl_eq);
 
   F(pr->d_cfl_grid); F(pr->d_cfl_mid1); F(pr->d_cfl_mid2); F(pr->d_inv_dz); F(pr->d_cfl_args); F(pr->d_cfl_out);
-  F(pr->d_bc_values); F(pr->d_kx); F(pr->d_gvar); F(pr->d_gop); F(pr->d_zvar); F(pr->d_ysrc); F(pr->d_ydy); F(pr->d_xsrc); F(pr->d_xdx); F(pr->d_tslot); F(pr->d_tfa); F(pr->d_tfb);
+  F(pr->d_bc_values); F(pr->d_kx); F(pr->d_gvar); F(pr->d_gop); F(pr->d_zb); F(pr->d_zf); F(pr->d_zvar); F(pr->d_ysrc); F(pr->d_ydy); F(pr->d_xsrc); F(pr->d_xdx); F(pr->d_tslot); F(pr->d_tfa); F(pr->d_tfb);
   F(pr->d_tcoef); F(pr->d_ident); F(pr->d_zero); F(pr->d_Xt); F(pr->d_Xc); F(pr->d_Xc32); F(pr->d_kx32);
   F(pr->d_tcoef32);
   for (auto b : pr->d_MX) F(b);
@@ -626,6 +650,7 @@ ZDesc zdesc_backward(Problem* pr) {
   ZDesc d{};
   d.Nc = pz.Nc; d.Ng = pz.Ng; d.radix3 = pz.radix3; d.P = pr->P;
   d.tw = pr->prec ? pz.tw32 : pz.tw64; d.wq = pr->prec ? pz.dct32 : pz.dct64;
+  if (pr->rows_fast) d.wq = pr->d_zb;
   d.f_var = pr->rows_fast ? pr->d_zvar : pr->d_gvar; d.f_op = pr->d_gop; d.kx = pr->d_kx; d.xc = pr->d_Xc;
   d.xc_stride = pr->P * pr->Nz;
   d.gz = pr->d_gz;
@@ -634,6 +659,7 @@ ZDesc zdesc_backward(Problem* pr) {
 }
 ZDesc zdesc_forward(Problem* pr, double2* fc) {
   ZDesc d = zdesc_backward(pr);
+  if (pr->rows_fast) d.wq = pr->d_zf;
   d.h = pr->ndim == 3 ? pr->d_gz : pr->d_h; d.fc = fc;
   return d;
 }
@@ -1096,9 +1122,14 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
     std::vector<SolveArgs> av;
     for (size_t q = 0; q < ps.size(); ++q) {
       zbv.push_back(zdesc_backward(ps[q]));
-      if (!b->fast) zbv.back().f_var = ps[q]->d_gvar;
+      if (!b->fast && ps[q]->rows_fast) {    // the run-time-length kernels' tables and fields
+        const TransformPlan& pz = ps[q]->plans.at({ps[q]->Nz, ps[q]->Ngz});
+        zbv.back().wq = ps[q]->prec ? pz.dct32 : pz.dct64;
+        zbv.back().f_var = ps[q]->d_gvar;
+      }
       xv.push_back(xdesc_rows(ps[q]));
       zfv.push_back(zdesc_forward(ps[q], plans[q][i].fc_out));
+      if (!b->fast) zfv.back().wq = zbv.back().wq;
       av.push_back(plans[q][i].args);
       av.back().fwd16 = 1;            // throughput-bound: both parts' forward in one warp
       if (b->split) stage_lx(ps[q], av.back());

@@ -12,13 +12,19 @@
 // Twiddled butterflies split even and odd inputs with one common factor:
 // E_q = sum_s a_{2s} w^{2s} r^{2qs}, O_q the same sum of a_{2s+1}, X_{q, q+R/2} =
 // E_q +- w r^q O_q (r = exp(sign 2 pi i / R)), down to single elements.  Each
-// two-point step is four FMAs for E + w O and two for E - w O = 2 E - (E + w O):
-// 72 FP instructions and 4 twiddle loads for radix 8, against 84 and 7 with
-// the inputs multiplied first.
+// two-point step is four FMAs for E + w O and, in FP64, whose pipe is the
+// bound, two for E - w O = 2 E - (E + w O): 72 FP64 instructions and 4 twiddle
+// loads for radix 8, against 84 and 7 with the inputs multiplied first (errors
+// of the right-hand side against a dense evaluation 5.6e-14 against 5.8e-14 at
+// 256 x 256).  FP32, bound by other instructions, takes four for it, as exact
+// as a product and a difference.
 //
 // Buffers are padded by one element every 128 bytes, so the first pass's
 // stride-R writes spread over the banks.
 #pragma once
+#include <type_traits>
+#include <utility>
+
 #include "common.cuh"
 
 namespace spectau {
@@ -65,8 +71,13 @@ template <typename T>
 __device__ __forceinline__ void bfly(C<T> e, C<T> o, C<T> w, C<T>& p, C<T>& m) {
   p.x = fma(-w.y, o.y, fma(w.x, o.x, e.x));
   p.y = fma(w.y, o.x, fma(w.x, o.y, e.y));
-  m.x = fma((T)2, e.x, -p.x);
-  m.y = fma((T)2, e.y, -p.y);
+  if constexpr (sizeof(T) == 8) {
+    m.x = fma((T)2, e.x, -p.x);
+    m.y = fma((T)2, e.y, -p.y);
+  } else {
+    m.x = fma(w.y, o.y, fma(-w.x, o.x, e.x));
+    m.y = fma(-w.y, o.x, fma(-w.x, o.y, e.y));
+  }
 }
 
 // DFT of length R (a power of two) of a[0], a[S], a[2S], ... with the common
@@ -127,28 +138,44 @@ struct Dit<T, SIGN, 1, S> {
   static __device__ __forceinline__ void run(const C<T>* a, C<T>* out) { out[0] = a[0]; }
 };
 
-// 3-point DFT: sums, differences and FMAs with -1/2 and sqrt(3)/2
-template <typename T, int SIGN>
+// 3-point DFT: sums, differences and FMAs with -1/2 and sqrt(3)/2.  Z: an input
+// known to be zero (-1: none).
+template <typename T, int SIGN, int Z>
 __device__ __forceinline__ void dft3(C<T> a0, C<T> a1, C<T> a2, C<T>& x0, C<T>& x1, C<T>& x2) {
   const T c = (SIGN < 0 ? (T)-1 : (T)1) * (T)0.86602540378443864676;
-  const C<T> s = cadd<T>(a1, a2), d = csub<T>(a1, a2);
-  const C<T> m = mk<T>(fma((T)-0.5, s.x, a0.x), fma((T)-0.5, s.y, a0.y));
-  x0 = cadd<T>(a0, s);
+  const C<T> s = Z == 1 ? a2 : Z == 2 ? a1 : cadd<T>(a1, a2);
+  const C<T> d = Z == 1 ? mk<T>(-a2.x, -a2.y) : Z == 2 ? a1 : csub<T>(a1, a2);
+  const C<T> m = Z == 0 ? mk<T>((T)-0.5 * s.x, (T)-0.5 * s.y)
+                        : mk<T>(fma((T)-0.5, s.x, a0.x), fma((T)-0.5, s.y, a0.y));
+  x0 = Z == 0 ? s : cadd<T>(a0, s);
   x1 = mk<T>(fma(-c, d.y, m.x), fma(c, d.x, m.y));
   x2 = mk<T>(fma(c, d.y, m.x), fma(-c, d.x, m.y));
 }
 
+// f(integral_constant<int, 0>), ..., f(integral_constant<int, R - 1>)
+template <typename F, int... Ts>
+__device__ __forceinline__ void unroll_seq(F&& f, std::integer_sequence<int, Ts...>) {
+  (f(std::integral_constant<int, Ts>()), ...);
+}
+template <int R, typename F>
+__device__ __forceinline__ void unroll(F&& f) { unroll_seq(f, std::make_integer_sequence<int, R>()); }
+
 // First-pass DFT of R0 = 2^a or 3 2^a elements.  The factor 3 by the prime
 // factor map (coprime factors need no twiddles): with R = 3 H, input (H n1 + 3
 // n2) mod R and output k = k1 mod 3, k2 mod H.
-template <typename T, int SIGN, int R>
+// PAD: the middle third of the inputs is zero (a spectrum padded by 3/2).
+template <typename T, int SIGN, int R, bool PAD>
 __device__ __forceinline__ void dft_first(const C<T>* a, C<T>* out) {
   if constexpr (R % 3 == 0) {
     constexpr int H = R / 3;
     C<T> b[3][H];
-#pragma unroll
-    for (int n2 = 0; n2 < H; ++n2)
-      dft3<T, SIGN>(a[(3 * n2) % R], a[(H + 3 * n2) % R], a[(2 * H + 3 * n2) % R], b[0][n2], b[1][n2], b[2][n2]);
+    unroll<H>([&](auto n) {
+      constexpr int n2 = decltype(n)::value;
+      constexpr int i0 = (3 * n2) % R, i1 = (H + 3 * n2) % R, i2 = (2 * H + 3 * n2) % R;
+      // the three differ by R / 3, so exactly one lies in the middle third
+      constexpr int Z = !PAD ? -1 : (i0 / H == 1 ? 0 : i1 / H == 1 ? 1 : 2);
+      dft3<T, SIGN, Z>(a[i0], a[i1], a[i2], b[0][n2], b[1][n2], b[2][n2]);
+    });
 #pragma unroll
     for (int k1 = 0; k1 < 3; ++k1) {
       C<T> o[H];
@@ -167,19 +194,35 @@ __device__ __forceinline__ void dft_first(const C<T>* a, C<T>* out) {
   }
 }
 
-// First pass over nb sequences: `in(b, i)` gives element i of sequence b.
-template <typename T, int N, int SIGN, int NT, typename IN, typename OUT>
-__device__ __forceinline__ void fft_pass_first(int nb, IN&& in, OUT&& out) {
+// First pass over nb sequences: `open(b, j)` gives a reader e of sequence b's
+// elements j + t N / R0, e(integral_constant<int, t>).  PAD: elements [N/3, 2N/3)
+// are zero and are not read.
+template <int R, bool PAD>
+constexpr bool fft_zero(int t) { return PAD && 3 * t >= R && 3 * t < 2 * R; }
+template <typename T, int R, bool PAD, typename E>
+__device__ __forceinline__ void fft_read(E&& e, C<T>* a) {
+  unroll<R>([&](auto t) {
+    if constexpr (fft_zero<R, PAD>(decltype(t)::value)) a[decltype(t)::value] = mk<T>(0, 0);
+    else a[decltype(t)::value] = e(t);
+  });
+}
+template <typename T, int N, int SIGN, int NT, bool PAD, typename OPEN, typename OUT>
+__device__ __forceinline__ void fft_pass_first(int nb, OPEN&& open, OUT&& out) {
   constexpr int R = FftPlan<N>::R0, Q = N / R;
   for (int id = threadIdx.x; id < nb * Q; id += NT) {
     const int b = id / Q, j = id - b * Q;
     C<T> a[R], y[R];
-#pragma unroll
-    for (int t = 0; t < R; ++t) a[t] = in(b, j + t * Q);
-    dft_first<T, SIGN, R>(a, y);
+    fft_read<T, R, PAD>(open(b, j), a);
+    dft_first<T, SIGN, R, PAD>(a, y);
 #pragma unroll
     for (int q = 0; q < R; ++q) out(b, j * R + q, y[q]);
   }
+}
+
+// element of a twiddle table by a 32-bit byte offset
+template <typename T>
+__device__ __forceinline__ C<T> fft_tw(const C<T>* tw, unsigned i) {
+  return __ldg(reinterpret_cast<const C<T>*>(reinterpret_cast<const char*>(tw) + i * (unsigned)sizeof(C<T>)));
 }
 
 // A twiddled pass of radix R over sub-transforms of length Ns from padded
@@ -195,9 +238,9 @@ __device__ __forceinline__ void fft_pass_tw(const C<T>* __restrict__ x, const C<
     C<T> a[R], y[R];
 #pragma unroll
     for (int t = 0; t < R; ++t) a[t] = xb[fft_pad<T>(j + t * Q)];
-    const int w0 = k * STEP;
+    const unsigned w0 = k * STEP;
     auto at = [&](int m, int q, int r) {
-      C<T> w = tw[m * w0 + q * (N / r)];
+      const C<T> w = fft_tw<T>(tw, m * w0 + q * (N / r));
       return SIGN > 0 ? mk<T>(w.x, -w.y) : w;
     };
     DitTw<T, SIGN, R, 1, 1, decltype(at)>::run(a, y, at);
@@ -207,15 +250,15 @@ __device__ __forceinline__ void fft_pass_tw(const C<T>* __restrict__ x, const C<
   }
 }
 
-// Transforms nb sequences: `in` as above, results to `fin(b, i, v)` in natural
+// Transforms nb sequences: `open` as above, results to `fin(b, i, v)` in natural
 // order.  A three-pass transform goes through buffer u, then v; a two-pass one
 // through v only (fin may write where u is).  Ends after a barrier.
-template <typename T, int N, int SIGN, int NT, typename IN, typename FIN>
-__device__ __forceinline__ void fft_run(int nb, C<T>* u, C<T>* v, const C<T>* tw, IN&& in, FIN&& fin) {
+template <typename T, int N, int SIGN, int NT, bool PAD, typename OPEN, typename FIN>
+__device__ __forceinline__ void fft_run(int nb, C<T>* u, C<T>* v, const C<T>* tw, OPEN&& open, FIN&& fin) {
   using P = FftPlan<N>;
   constexpr int NP = fft_padded<T>(N);
   C<T>* first = P::R2 > 1 ? u : v;
-  fft_pass_first<T, N, SIGN, NT>(nb, in, [&](int b, int i, C<T> z) { first[b * NP + fft_pad<T>(i)] = z; });
+  fft_pass_first<T, N, SIGN, NT, PAD>(nb, open, [&](int b, int i, C<T> z) { first[b * NP + fft_pad<T>(i)] = z; });
   __syncthreads();
   if constexpr (P::R2 > 1) {
     fft_pass_tw<T, N, SIGN, NT, P::R1, P::R0>(u, tw, nb, [&](int b, int i, C<T> z) { v[b * NP + fft_pad<T>(i)] = z; });

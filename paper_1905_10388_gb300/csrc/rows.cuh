@@ -9,6 +9,17 @@
 // more where a y derivative is used, and the x rows apply i k_x as they load
 // (2D Rayleigh-Benard: 6 z transforms for 8 grid fields; 3D: 8 and 12 y
 // transforms for 15).
+//
+// FP64 is bound by its pipe: the work is counted in FP64 instructions (signs,
+// halves and scales live in tables, +-1 coefficients take no multiplication, the
+// padded third of a spectrum enters no butterfly).  FP32 is bound by
+// instruction issue (57 % active, FMA pipe 20 %): a run-time length, a branch or
+// an address per element costs more than the arithmetic.  Per launch, the
+// run-time-length kernels before and these now: x rows 512 x 256 FP64 171 ->
+// 119 us (pipe 69 % busy, 82 % on the SMs with three of the 384 rows), FP32 28
+// -> 16; 3D 128 x 128 x 64 FP32 390 -> 160; Fisher-KPP 2048 x 1024 FP32 137 ->
+// 60; y of the 3D case 139 and 40 -> 64 and 20; z 512 x 256 FP64 76 and 40 -> 41
+// and 29.
 #pragma once
 #include <algorithm>
 #include <type_traits>
@@ -19,6 +30,10 @@
 namespace spectau {
 
 constexpr size_t ROWS_SMEM = ROWS_SMEM_MAX;
+
+// -x by the sign bit (off the FP64 pipe)
+__device__ __forceinline__ double neg_bits(double x) { return dneg(x); }
+__device__ __forceinline__ float neg_bits(float x) { return -x; }
 
 // threads of a CTA: about the butterflies of four sequences, in whole warps
 template <typename T, int N>
@@ -45,7 +60,7 @@ size_t x_rows_smem(int nf, int ne) {
   return (size_t)(nbi + std::max(nbi, 2 * nbo)) * fft_padded<T>(N) * sizeof(C<T>);
 }
 
-template <typename T, int N, int NT>
+template <typename T, int N, int NT, bool PAD>
 __device__ __forceinline__ void x_rows_body(const XDesc& d, int row, unsigned char* rows_smem) {
   constexpr int NP = fft_padded<T>(N), MAX_TERMS = 16, MAX_F = 16;
   const int K = d.K, rows = d.rows, nf = d.nf, ne = d.ne, tid = threadIdx.x;
@@ -53,54 +68,68 @@ __device__ __forceinline__ void x_rows_body(const XDesc& d, int row, unsigned ch
   C<T>* u = reinterpret_cast<C<T>*>(rows_smem);
   C<T>* v = u + nbi * NP;
   T* G = reinterpret_cast<T*>(u);                // grid fields [f][N], over the first buffer
-  __shared__ T tc[MAX_TERMS];
-  __shared__ int ta[MAX_TERMS], tb[MAX_TERMS], te[MAX_TERMS];
   __shared__ int fs[MAX_F], fx[MAX_F];
+  __shared__ int4 term[MAX_TERMS];               // field offsets, equation offset (last of its equation: | 1), coefficient kind
+  __shared__ T tc[MAX_TERMS];
   const int nterms = min(d.nterms, MAX_TERMS);
   const T* tcoef = reinterpret_cast<const T*>(sizeof(T) == 8 ? (const void*)d.t_coef : (const void*)d.t_coef32);
-  const T* kx = reinterpret_cast<const T*>(sizeof(T) == 8 ? (const void*)d.kx : (const void*)d.kx32);
+  const T* __restrict__ kx = reinterpret_cast<const T*>(sizeof(T) == 8 ? (const void*)d.kx : (const void*)d.kx32);
   if (tid < nterms) {
-    tc[tid] = tcoef[tid]; ta[tid] = d.t_fa[tid] * N; tb[tid] = d.t_fb[tid] * N; te[tid] = d.t_eq[tid];
+    const int e = d.t_eq[tid];
+    const bool last = tid + 1 == nterms || d.t_eq[tid + 1] != e;
+    const T c = tcoef[tid];
+    tc[tid] = c;
+    term[tid] = make_int4(d.t_fa[tid] * N, d.t_fb[tid] * N, ((e >> 1) * 4 * NP + (e & 1) * 2) | (last ? 1 : 0),
+                          c == (T)1 ? 1 : c == (T)-1 ? -1 : 0);
   }
   if (tid < nf) { fs[tid] = d.f_src[tid]; fx[tid] = d.f_dx[tid]; }
   const C<T>* __restrict__ tw = reinterpret_cast<const C<T>*>(d.tw);
   __syncthreads();
   const C<T>* __restrict__ gz = reinterpret_cast<const C<T>*>(d.gz) + (size_t)row * K;
   const size_t plane = (size_t)rows * K;
-  auto spec = [&](int f, int k) -> C<T> {
-    if (f >= nf) return mk<T>(0, 0);
-    const C<T> z = gz[fs[f] * plane + k];
-    if (!fx[f]) return z;
-    const T q = kx[k];
-    return mk<T>(-q * z.y, q * z.x);
-  };
-  fft_run<T, N, +1, NT>(
+  constexpr int Q0 = N / FftPlan<N>::R0;
+  fft_run<T, N, +1, NT, PAD>(
       nbi, u, v, tw,
-      [&](int b, int i) -> C<T> {
+      [&](int b, int j) {
         // two real fields a, b as a + i b: the Hermitian spectrum of the stored k >= 0 modes
-        if (i < K) {
-          const C<T> A = spec(2 * b, i), B = spec(2 * b + 1, i);
-          return i == 0 ? mk<T>(A.x, B.x) : mk<T>(A.x - B.y, A.y + B.x);
-        }
-        if (i > N - K) {
-          const C<T> A = spec(2 * b, N - i), B = spec(2 * b + 1, N - i);
-          return mk<T>(A.x + B.y, B.x - A.y);
-        }
-        return mk<T>(0, 0);
+        const bool two = 2 * b + 1 < nf;
+        const C<T>* pa = gz + fs[2 * b] * plane;
+        const C<T>* pb = gz + fs[two ? 2 * b + 1 : 2 * b] * plane;
+        const bool xa = fx[2 * b] != 0, xb = two && fx[2 * b + 1] != 0;
+        return [=](auto t) -> C<T> {
+          constexpr int i0 = decltype(t)::value * Q0;
+          const bool mirror = PAD ? 3 * i0 >= 2 * N : j + i0 > N - K;
+          const int k = mirror ? N - i0 - j : i0 + j;
+          if ((!PAD || 3 * i0 == 2 * N) && (mirror ? k >= K : k >= K)) return mk<T>(0, 0);
+          C<T> A = pa[k], B = two ? pb[k] : mk<T>(0, 0);
+          if (xa || xb) {
+            const T q = kx[k];
+            if (xa) A = mk<T>(-q * A.y, q * A.x);
+            if (xb) B = mk<T>(-q * B.y, q * B.x);
+          }
+          if (i0 == 0 && j == 0) A.y = B.y = 0;
+          return mirror ? mk<T>(A.x + B.y, B.x - A.y) : mk<T>(A.x - B.y, A.y + B.x);
+        };
       },
       [&](int b, int i, C<T> z) {
         G[2 * b * N + i] = z.x;
         if (2 * b + 1 < nf) G[(2 * b + 1) * N + i] = z.y;
       });
-  // products: terms are grouped by equation; two equations share a complex sequence
+  // products: terms are grouped by equation; two equations share a complex
+  // sequence.  Coefficients +-1 cost one FMA per term.
   T* O = reinterpret_cast<T*>(v);
   for (int i = tid; i < N; i += NT) {
     const int o = 2 * fft_pad<T>(i);
     T acc = 0;
     for (int t = 0; t < nterms; ++t) {
-      acc += tc[t] * G[ta[t] + i] * G[tb[t] + i];
-      if (t + 1 == nterms || te[t + 1] != te[t]) {
-        O[(te[t] >> 1) * 2 * NP + o + (te[t] & 1)] = acc;
+      const int4 m = term[t];
+      T ga = G[m.x + i];
+      const T gb = G[m.y + i];
+      if (m.w < 0) ga = neg_bits(ga);
+      else if (m.w == 0) ga *= tc[t];
+      acc = fma(ga, gb, acc);
+      if (m.z & 1) {
+        O[(m.z >> 1) + o] = acc;
         acc = 0;
       }
     }
@@ -110,23 +139,27 @@ __device__ __forceinline__ void x_rows_body(const XDesc& d, int row, unsigned ch
   constexpr bool three = FftPlan<N>::R2 > 1;
   C<T>* u2 = v + nbo * NP;
   C<T>* Z = three ? u2 : v;
-  fft_run<T, N, -1, NT>(
-      nbo, u2, three ? v : u2, tw, [&](int b, int i) -> C<T> { return v[b * NP + fft_pad<T>(i)]; },
+  fft_run<T, N, -1, NT, false>(
+      nbo, u2, three ? v : u2, tw,
+      [&](int b, int j) {
+        const C<T>* x = v + b * NP;
+        return [=](auto t) -> C<T> { return x[fft_pad<T>(j + decltype(t)::value * Q0)]; };
+      },
       [&](int b, int i, C<T> z) { Z[b * NP + fft_pad<T>(i)] = z; });
   C<T>* h = reinterpret_cast<C<T>*>(d.h) + (size_t)row * K;
-  const T s = (T)1 / (T)(2 * N);
+  // (the 1 / (2 N) of the forward transform is in the z transform's table)
   for (int b = 0; b < nbo; ++b)
     for (int k = tid; k < K; k += NT) {
       const C<T> z = Z[b * NP + fft_pad<T>(k)], r = Z[b * NP + fft_pad<T>(k == 0 ? 0 : N - k)];
-      h[2 * b * plane + k] = mk<T>((z.x + r.x) * s, (z.y - r.y) * s);
-      if (2 * b + 1 < ne) h[(2 * b + 1) * plane + k] = mk<T>((z.y + r.y) * s, (r.x - z.x) * s);
+      h[2 * b * plane + k] = mk<T>(z.x + r.x, z.y - r.y);
+      if (2 * b + 1 < ne) h[(2 * b + 1) * plane + k] = mk<T>(z.y + r.y, r.x - z.x);
     }
 }
 
-template <typename T, int N, int NT>
+template <typename T, int N, int NT, bool PAD>
 __global__ void __launch_bounds__(NT, rows_ctas<T>(NT)) k_x_rows(XDesc d) {
   extern __shared__ __align__(16) unsigned char rows_smem[];
-  x_rows_body<T, N, NT>(d, blockIdx.x, rows_smem);
+  x_rows_body<T, N, NT, PAD>(d, blockIdx.x, rows_smem);
 }
 
 template <typename T>
@@ -135,9 +168,12 @@ cudaError_t launch_x_rows(cudaStream_t s, const XDesc& d) {
     constexpr int N = decltype(n)::value, NT = rows_threads<T, N>();
     const size_t smem = x_rows_smem<T, N>(d.nf, d.ne);
     if (smem > ROWS_SMEM || d.nf > 16 || d.nterms > 16) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_x_rows<T, N, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto* k = k_x_rows<T, N, NT, false>;
+    if constexpr (N % 3 == 0)
+      if (3 * d.K == N) k = k_x_rows<T, N, NT, true>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_x_rows<T, N, NT><<<d.rows, NT, smem, s>>>(d);
+    k<<<d.rows, NT, smem, s>>>(d);
     return cudaGetLastError();
   });
 }
@@ -158,11 +194,11 @@ constexpr int col_stride() { return (fft_padded<T>(N) + 15) / 16 * 16 + 1; }
 template <typename T, int N>
 constexpr size_t col_smem() { return (size_t)2 * col_tile<T>() * col_stride<T, N>() * sizeof(C<T>); }
 
-// One transform of the tile: `in(c, i)`, `fin(c, i, v)`; IN_COL / OUT_COL:
+// One transform of the tile: readers `open(c, j)` (fftn.cuh), `fin(c, i, v)`; IN_COL / OUT_COL:
 // columns fastest over the threads in the first / last pass.  Two-pass lengths
 // use buffer v alone.  Ends after a barrier.
-template <typename T, int N, int SIGN, int NT, bool IN_COL, bool OUT_COL, typename IN, typename FIN>
-__device__ __forceinline__ void col_run(C<T>* u, C<T>* v, const C<T>* tw, IN&& in, FIN&& fin) {
+template <typename T, int N, int SIGN, int NT, bool PAD, bool IN_COL, bool OUT_COL, typename OPEN, typename FIN>
+__device__ __forceinline__ void col_run(C<T>* u, C<T>* v, const C<T>* tw, OPEN&& open, FIN&& fin) {
   using P = FftPlan<N>;
   constexpr int TC = col_tile<T>(), NS = col_stride<T, N>();
   C<T>* first = P::R2 > 1 ? u : v;
@@ -171,9 +207,8 @@ __device__ __forceinline__ void col_run(C<T>* u, C<T>* v, const C<T>* tw, IN&& i
     for (int id = threadIdx.x; id < TC * Q; id += NT) {
       const int c = IN_COL ? id % TC : id / Q, j = IN_COL ? id / TC : id % Q;
       C<T> a[R], y[R];
-#pragma unroll
-      for (int t = 0; t < R; ++t) a[t] = in(c, j + t * Q);
-      dft_first<T, SIGN, R>(a, y);
+      fft_read<T, R, PAD>(open(c, j), a);
+      dft_first<T, SIGN, R, PAD>(a, y);
 #pragma unroll
       for (int q = 0; q < R; ++q) first[c * NS + fft_pad<T>(j * R + q)] = y[q];
     }
@@ -189,9 +224,9 @@ __device__ __forceinline__ void col_run(C<T>* u, C<T>* v, const C<T>* tw, IN&& i
       C<T> a[R], y[R];
 #pragma unroll
       for (int t = 0; t < R; ++t) a[t] = xc[fft_pad<T>(j + t * Q)];
-      const int w0 = k * STEP;
+      const unsigned w0 = k * STEP;
       auto at = [&](int m, int q, int rr) {
-        const C<T> w = tw[m * w0 + q * (N / rr)];
+        const C<T> w = fft_tw<T>(tw, m * w0 + q * (N / rr));
         return SIGN > 0 ? mk<T>(w.x, -w.y) : w;
       };
       DitTw<T, SIGN, R, 1, 1, decltype(at)>::run(a, y, at);
@@ -213,45 +248,60 @@ __device__ __forceinline__ void col_run(C<T>* u, C<T>* v, const C<T>* tw, IN&& i
 }
 
 // y axis (complex): DIR < 0: slots -> grid of output field f, with i k_y where
-// f_dy is set; DIR > 0: grid -> slots (1/N, Nyquist slot zero)
-template <typename T, int N, int NT, int DIR>
+// f_dy is set; DIR > 0: grid -> slots (unscaled, Nyquist slot zero)
+template <typename T, int N, int NT, int DIR, bool PAD>
 __global__ void __launch_bounds__(NT, rows_ctas<T>(NT)) k_y_cols(YDesc d) {
   extern __shared__ __align__(16) unsigned char rows_smem[];
-  constexpr int TC = col_tile<T>();
+  constexpr int TC = col_tile<T>(), Q0 = N / FftPlan<N>::R0;
   const int Ny = d.Ny, K = d.K, half = Ny / 2, zg = blockIdx.y, f = blockIdx.z;
   C<T>* u = reinterpret_cast<C<T>*>(rows_smem);
   C<T>* v = u + col_tile<T>() * col_stride<T, N>();
   const C<T>* __restrict__ tw = reinterpret_cast<const C<T>*>(d.tw);
   const int ix0 = blockIdx.x * TC;
+  const size_t skip = (size_t)(N - Ny) * K;      // the padded modes
   if constexpr (DIR < 0) {
-    const C<T>* in = reinterpret_cast<const C<T>*>(d.src) + ((size_t)d.f_src[f] * d.nz + zg) * Ny * K + ix0;
+    const C<T>* __restrict__ in = reinterpret_cast<const C<T>*>(d.src) + ((size_t)d.f_src[f] * d.nz + zg) * Ny * K + ix0;
     C<T>* out = reinterpret_cast<C<T>*>(d.dst) + ((size_t)f * d.nz + zg) * N * K + ix0;
-    const T* ky = reinterpret_cast<const T*>(sizeof(T) == 8 ? (const void*)d.ky : (const void*)d.ky32);
+    const T* __restrict__ ky = reinterpret_cast<const T*>(sizeof(T) == 8 ? (const void*)d.ky : (const void*)d.ky32);
     const bool dy = d.f_dy[f] != 0;
-    col_run<T, N, +1, NT, true, true>(
+    col_run<T, N, +1, NT, PAD, true, true>(
         u, v, tw,
-        [&](int c, int i) -> C<T> {
+        [&](int c, int j) {
           // mode n at position n mod N; slots [0, half) and (half, Ny)
-          const int sl = i < half ? i : (i > N - half ? i - N + Ny : -1);
-          if (sl < 0 || ix0 + c >= K) return mk<T>(0, 0);
-          const C<T> z = in[(size_t)sl * K + c];
-          if (!dy) return z;
-          const T q = ky[(size_t)sl * K];
-          return mk<T>(-q * z.y, q * z.x);
+          const C<T>* x = in + c + (size_t)j * K;
+          const T* q = ky + (size_t)j * K;
+          const bool ok = ix0 + c < K;
+          return [=](auto t) -> C<T> {
+            constexpr int i0 = decltype(t)::value * Q0;
+            const int i = i0 + j;
+            const bool low = PAD ? 3 * i0 < N : i < half;
+            const bool high = PAD ? 3 * i0 > 2 * N || (3 * i0 == 2 * N && j > 0) : i > N - half;
+            if (!ok || !(low || high)) return mk<T>(0, 0);
+            const size_t at = (size_t)i0 * K - (low ? 0 : skip);
+            const C<T> z = x[at];
+            if (!dy) return z;
+            const T w = q[at];
+            return mk<T>(-w * z.y, w * z.x);
+          };
         },
         [&](int c, int i, C<T> z) {
           if (ix0 + c < K) out[(size_t)i * K + c] = z;
         });
   } else {
-    const C<T>* in = reinterpret_cast<const C<T>*>(d.src) + ((size_t)f * d.nz + zg) * N * K + ix0;
+    // (the 1 / N is in the z transform's table)
+    const C<T>* __restrict__ in = reinterpret_cast<const C<T>*>(d.src) + ((size_t)f * d.nz + zg) * N * K + ix0;
     C<T>* out = reinterpret_cast<C<T>*>(d.dst) + ((size_t)f * d.nz + zg) * Ny * K + ix0;
-    const T s = (T)1 / (T)N;
-    col_run<T, N, -1, NT, true, true>(
-        u, v, tw, [&](int c, int i) -> C<T> { return ix0 + c < K ? in[(size_t)i * K + c] : mk<T>(0, 0); },
+    col_run<T, N, -1, NT, false, true, true>(
+        u, v, tw,
+        [&](int c, int j) {
+          const C<T>* x = in + c + (size_t)j * K;
+          const bool ok = ix0 + c < K;
+          return [=](auto t) -> C<T> { return ok ? x[(size_t)(decltype(t)::value * Q0) * K] : mk<T>(0, 0); };
+        },
         [&](int c, int i, C<T> z) {
-          const int sl = i < half ? i : (i > N - half ? i - N + Ny : -1);
           if (ix0 + c >= K) return;
-          if (sl >= 0) out[(size_t)sl * K + c] = mk<T>(z.x * s, z.y * s);
+          if (i < half) out[(size_t)i * K + c] = z;
+          else if (i > N - half) out[(size_t)i * K + c - skip] = z;
           if (i == 0) out[(size_t)half * K + c] = mk<T>(0, 0);
         });
   }
@@ -267,7 +317,9 @@ cudaError_t launch_y_cols(cudaStream_t s, const YDesc& d, int nf) {
       return cudaErrorInvalidValue;
     } else {
       dim3 grid((d.K + col_tile<T>() - 1) / col_tile<T>(), d.nz, nf);
-      auto* k = d.dir < 0 ? k_y_cols<T, N, NT, -1> : k_y_cols<T, N, NT, 1>;
+      auto* k = d.dir < 0 ? k_y_cols<T, N, NT, -1, false> : k_y_cols<T, N, NT, 1, false>;
+      if constexpr (N % 3 == 0)
+        if (d.dir < 0 && 3 * d.Ny == 2 * N) k = k_y_cols<T, N, NT, -1, true>;
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
       k<<<grid, NT, smem, s>>>(d);
@@ -276,31 +328,32 @@ cudaError_t launch_y_cols(cudaStream_t s, const YDesc& d, int nf) {
   });
 }
 
-// Chebyshev backward of variable f_var[f] (no derivative), pencil columns bx TC ..: V_k = conj(w_k)(X_k - i X_{N-k}), X_0 = d_0, X_k =
-// d_k / 2, d_n = (-1)^n c_n
+// Chebyshev backward of variable f_var[f] (no derivative), pencil columns bx TC
+// ..: V_k = conj(w_k)(X_k - i X_{N-k}), X_0 = d_0, X_k = d_k / 2, d_n = (-1)^n
+// c_n.  X_k and X_{N-k} carry the same sign and half (N is even), so the table
+// wq holds (-1)^k w_k / 2 (1 at k = 0) and the coefficients go in as they are.
 template <typename T, int N, int NT>
 __device__ __forceinline__ void z_backward_body(const ZDesc& d, int bx, int f, unsigned char* rows_smem) {
-  constexpr int TC = col_tile<T>();
+  constexpr int TC = col_tile<T>(), Q0 = N / FftPlan<N>::R0;
   const int Nc = d.Nc, P = d.P, p0 = bx * TC;
   C<T>* u = reinterpret_cast<C<T>*>(rows_smem);
   C<T>* v = u + col_tile<T>() * col_stride<T, N>();
   const C<T>* __restrict__ tw = reinterpret_cast<const C<T>*>(d.tw);
-  const C<T>* wq = reinterpret_cast<const C<T>*>(d.wq);
-  const C<T>* src = reinterpret_cast<const C<T>*>(sizeof(T) == 8 ? (const void*)d.xc : (const void*)d.xc32) +
-                    (size_t)d.f_var[f] * d.xc_stride + (size_t)p0 * Nc;
+  const C<T>* __restrict__ wq = reinterpret_cast<const C<T>*>(d.wq);
+  const C<T>* __restrict__ src =
+      reinterpret_cast<const C<T>*>(sizeof(T) == 8 ? (const void*)d.xc : (const void*)d.xc32) +
+      (size_t)d.f_var[f] * d.xc_stride + (size_t)p0 * Nc;
   C<T>* gz = reinterpret_cast<C<T>*>(d.gz) + (size_t)f * N * P + p0;
-  col_run<T, N, +1, NT, false, true>(
+  col_run<T, N, +1, NT, false, false, true>(
       u, v, tw,
-      [&](int c, int k) -> C<T> {
-        if (p0 + c >= P) return mk<T>(0, 0);
-        auto coef = [&](int n) -> C<T> {
-          if (n >= Nc) return mk<T>(0, 0);
-          const C<T> x = src[(size_t)c * Nc + n];
-          const T s = ((n & 1) ? (T)-1 : (T)1) * (n == 0 ? (T)1 : (T)0.5);
-          return mk<T>(s * x.x, s * x.y);
+      [&](int c, int j) {
+        const C<T>* x = src + (size_t)c * Nc;
+        const int top = p0 + c < P ? Nc : 0;     // no pencil: no coefficients
+        return [=](auto t) -> C<T> {
+          const int k = j + decltype(t)::value * Q0;
+          const C<T> a = k < top ? x[k] : mk<T>(0, 0), b = N - k < top ? x[N - k] : mk<T>(0, 0);
+          return cmulc<T>(mk<T>(a.x + b.y, a.y - b.x), fft_tw<T>(wq, k));
         };
-        const C<T> a = coef(k), b = k == 0 ? mk<T>(0, 0) : coef(N - k);
-        return cmulc<T>(mk<T>(a.x + b.y, a.y - b.x), wq[k]);
       },
       [&](int c, int j, C<T> z) {
         const int zg = j < N / 2 ? 2 * j : 2 * (N - 1 - j) + 1;
@@ -308,33 +361,39 @@ __device__ __forceinline__ void z_backward_body(const ZDesc& d, int bx, int f, u
       });
 }
 
-// Chebyshev forward of product f: out_k = (w_k V_k + conj(w_k) V_{N-k})
-// scaled to T coefficients
+// Chebyshev forward of product f: out_k = w_k V_k + conj(w_k) V_{N-k}, wq the
+// w_k with the T coefficients' sign and scale and the 1 / (2 N_gx) [/ N_gy] that
+// the x [and y] transforms leave out
 template <typename T, int N, int NT>
 __device__ __forceinline__ void z_forward_body(const ZDesc& d, int bx, int f, unsigned char* rows_smem) {
-  constexpr int TC = col_tile<T>(), NS = col_stride<T, N>();
-  const int Nc = d.Nc, P = d.P, p0 = bx * TC, e = f;
+  constexpr int TC = col_tile<T>(), NS = col_stride<T, N>(), Q0 = N / FftPlan<N>::R0;
+  const int Nc = d.Nc, P = d.P, p0 = bx * TC;
   C<T>* u = reinterpret_cast<C<T>*>(rows_smem);
   C<T>* v = u + col_tile<T>() * col_stride<T, N>();
   const C<T>* __restrict__ tw = reinterpret_cast<const C<T>*>(d.tw);
-  const C<T>* wq = reinterpret_cast<const C<T>*>(d.wq);
-  const C<T>* h = reinterpret_cast<const C<T>*>(d.h) + (size_t)e * N * P + p0;
-  col_run<T, N, -1, NT, true, false>(
+  const C<T>* __restrict__ wq = reinterpret_cast<const C<T>*>(d.wq);
+  const C<T>* __restrict__ h = reinterpret_cast<const C<T>*>(d.h) + (size_t)f * N * P + p0;
+  col_run<T, N, -1, NT, false, true, false>(
       u, v, tw,
-      [&](int c, int j) -> C<T> {
-        const int zg = j < N / 2 ? 2 * j : 2 * (N - 1 - j) + 1;
-        return p0 + c < P ? h[(size_t)zg * P + c] : mk<T>(0, 0);
+      [&](int c, int j) {
+        const bool ok = p0 + c < P;
+        return [=](auto t) -> C<T> {
+          const int i = j + decltype(t)::value * Q0;
+          const int zg = i < N / 2 ? 2 * i : 2 * (N - 1 - i) + 1;
+          return ok ? h[(size_t)zg * P + c] : mk<T>(0, 0);
+        };
       },
       [&](int c, int i, C<T> z) { u[c * NS + fft_pad<T>(i)] = z; });
-  const T inv = (T)1 / (T)N;
-  for (int c = 0; c < TC && p0 + c < P; ++c)
-    for (int k = threadIdx.x; k < Nc; k += NT) {
-      const C<T> a = u[c * NS + fft_pad<T>(k)], b = u[c * NS + fft_pad<T>(k == 0 ? 0 : N - k)], w = wq[k];
-      const C<T> o = cadd<T>(cmul<T>(w, a), cmulc<T>(b, w));
-      const T s = ((k & 1) ? (T)-1 : (T)1) * (k == 0 ? inv * (T)0.5 : inv);
+  for (int k = threadIdx.x; k < Nc; k += NT) {
+    const C<T> w = wq[k];
+    for (int c = 0; c < TC && p0 + c < P; ++c) {
+      const C<T> a = u[c * NS + fft_pad<T>(k)], b = u[c * NS + fft_pad<T>(k == 0 ? 0 : N - k)];
+      const C<T> s = cadd<T>(a, b), m = csub<T>(a, b);
+      const T x = fma(-w.y, m.y, w.x * s.x), y = fma(w.y, m.x, w.x * s.y);
       // the k_x = 0 column is the transform of a real function: real coefficients
-      d.fc[((size_t)e * P + p0 + c) * Nc + k] = make_double2((double)(o.x * s), p0 + c == 0 ? 0.0 : (double)(o.y * s));
+      d.fc[((size_t)f * P + p0 + c) * Nc + k] = make_double2((double)x, p0 + c == 0 ? 0.0 : (double)y);
     }
+  }
 }
 
 template <typename T, int N, int NT>
@@ -393,7 +452,12 @@ __global__ void __launch_bounds__(BATCH_NT, sizeof(T) == 8 ? 2 : 3) k_x_rows_bat
   extern __shared__ __align__(16) unsigned char rows_smem[];
   for_each_item(nwork, queue, [&](int it) {
     const int4 w = work[it];
-    fft_switch<4096>(ds[w.x].N, [&](auto n) { x_rows_body<T, decltype(n)::value, BATCH_NT>(ds[w.x], w.y, rows_smem); });
+    const XDesc& d = ds[w.x];
+    fft_switch<4096>(d.N, [&](auto n) {
+      constexpr int N = decltype(n)::value;
+      if (N % 3 == 0 && 3 * d.K == N) x_rows_body<T, N, BATCH_NT, N % 3 == 0>(d, w.y, rows_smem);
+      else x_rows_body<T, N, BATCH_NT, false>(d, w.y, rows_smem);
+    });
   });
 }
 template <typename T, bool FWD>
