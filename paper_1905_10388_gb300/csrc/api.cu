@@ -138,8 +138,10 @@ struct Problem {
   // M~ on its own compact pattern (entries nonzero in at least one pencil)
   int64_t nnzM = 0;
   int32_t *d_indptrM = nullptr, *d_indicesM = nullptr;
-  int32_t* d_mrows = nullptr;   // rows of M~ with entries
-  int nmrows = 0;
+  // epilogue matvec rows (row, first entry, entries) of M~'s, L~'s and the transposed pattern
+  int4 *d_epM = nullptr, *d_epL = nullptr, *d_epT = nullptr;
+  int nmrows = 0;                                    // M~'s rows with entries
+  int32_t* d_row_item = nullptr;
   double* d_MvC = nullptr;
   int32_t *d_col_map = nullptr, *d_row_map = nullptr, *d_var_rec = nullptr, *d_var_ph = nullptr;
   int32_t *d_eq_diff = nullptr, *d_eq_ph = nullptr, *d_bc_rows = nullptr, *d_nl_eq = nullptr;
@@ -360,6 +362,17 @@ int default_forward_blocks(int npad) {
   return npad <= 1024 ? nch : near_divisor(nch, nch / 2);
 }
 
+// (row, first entry, entries) of a pattern's rows, those with entries first.
+std::vector<int4> row_list(const std::vector<int32_t>& indptr) {
+  std::vector<int4> v;
+  for (int with = 1; with >= 0; --with)
+    for (int r = 0; r + 1 < (int)indptr.size(); ++r) {
+      const int cnt = indptr[r + 1] - indptr[r];
+      if ((cnt > 0) == (with == 1)) v.push_back(make_int4(r, indptr[r], cnt, 0));
+    }
+  return v;
+}
+
 sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
   if (pr->uploaded) return SP_OK;
   if (!pr->has_layout) return fail(ctx, SP_ERR_STATE, "sp_set_layout has not been called");
@@ -389,16 +402,22 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
       for (int64_t k = 0; k < pr->nnzM; ++k) mv[(size_t)p * pr->nnzM + k] = pr->Mv[(size_t)p * pr->nnz + src[k]];
     CK(upload(&pr->d_indptrM, ip, s));
     CK(upload(&pr->d_indicesM, ix, s));
-    std::vector<int32_t> mrows;
-    for (int r = 0; r < pr->n; ++r)
-      if (ip[r + 1] > ip[r]) mrows.push_back(r);
-    pr->nmrows = (int)mrows.size();
-    if (mrows.empty()) mrows.push_back(0);
-    CK(upload(&pr->d_mrows, mrows, s));
+    CK(upload(&pr->d_epM, row_list(ip), s));
+    CK(upload(&pr->d_epL, row_list(pr->indptr), s));
+    pr->nmrows = 0;
+    for (int r = 0; r < pr->n; ++r) pr->nmrows += ip[r + 1] > ip[r];
     CK(upload(&pr->d_MvC, mv, s));
   }
   CK(upload(&pr->d_col_map, pr->col_map, s));
   CK(upload(&pr->d_row_map, pr->row_map, s));
+  std::vector<int32_t> item(pr->row_map.size());
+  for (size_t i = 0; i < item.size(); ++i) {
+    const int e = (int)(i / pr->Nz);
+    item[i] = pr->row_map[i] < 0 ? -1
+                                 : pr->row_map[i] << ROW_ITEM_BITS | (pr->eq_diff[e] ? ROW_ITEM_DIF : 0) |
+                                       (-pr->eq_ph[e] & 3);
+  }
+  CK(upload(&pr->d_row_item, item, s));
   CK(upload(&pr->d_var_rec, pr->var_rec, s));
   CK(upload(&pr->d_var_ph, pr->var_ph, s));
   CK(upload(&pr->d_eq_diff, pr->eq_diff, s));
@@ -585,7 +604,7 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
 
 void free_problem(Problem* pr) {
   auto F = [](void* p) { if (p) cudaFree(p); };
-  F(pr->d_indptr); F(pr->d_indices); F(pr->d_Mv); F(pr->d_Lv); F(pr->d_indptrM); F(pr->d_indicesM); F(pr->d_mrows); F(pr->d_MvC); F(pr->d_col_map); F(pr->d_row_map);
+  F(pr->d_indptr); F(pr->d_indices); F(pr->d_Mv); F(pr->d_Lv); F(pr->d_indptrM); F(pr->d_indicesM); F(pr->d_epM); F(pr->d_epL); F(pr->d_epT); F(pr->d_row_item); F(pr->d_MvC); F(pr->d_col_map); F(pr->d_row_map);
   F(pr->d_var_rec); F(pr->d_var_ph); F(pr->d_eq_diff); F(pr->d_eq_ph); F(pr->d_bc_rows); F(pr->d_nl_eq);
 
   F(pr->d_cfl_grid); F(pr->d_cfl_mid1); F(pr->d_cfl_mid2); F(pr->d_inv_dz); F(pr->d_cfl_args); F(pr->d_cfl_out);
@@ -747,13 +766,11 @@ sp_status eval_rhs(sp_ctx* ctx, Problem* pr, cudaStream_t s, double2* fc_out) {
 
 SolveArgs base_args(Problem* pr, sp_ctx* ctx, int fac) {
   SolveArgs a{};
-  a.P = pr->P; a.n = pr->n; a.Nz = pr->Nz; a.S = pr->S; a.nbc = pr->nbc; a.nnz = (int)pr->nnz;
+  a.P = pr->P; a.n = pr->n; a.Nz = pr->Nz; a.S = pr->S; a.nbc = pr->nbc;
   a.kl = pr->kl; a.kuu = pr->kl + pr->ku; a.npad = pr->npad; a.lpad = pr->lpad; a.upad = pr->upad;
   a.Lf = pr->fac[fac].L; a.piv = pr->fac[fac].piv; a.Uf = pr->fac[fac].U; a.rd = pr->fac[fac].rd;
-  a.indptr = pr->d_indptr; a.indices = pr->d_indices;
-  a.row_map = pr->d_row_map; a.col_map = pr->d_col_map;
+  a.row_item = pr->d_row_item; a.col_map = pr->d_col_map;
   a.var_recombine = pr->d_var_rec; a.var_phase = pr->d_var_ph;
-  a.eq_differential = pr->d_eq_diff; a.eq_phase = pr->d_eq_ph;
   a.nl_eq = pr->d_nl_eq; a.n_nl = (int)pr->nl_eqs.size();
   a.bc_rows = pr->d_bc_rows; a.bc_values = pr->d_bc_values;
   a.status = ctx->d_status;
@@ -771,12 +788,10 @@ void set_mv_M(Problem* pr, SolveArgs& a) {
   a.mv_vals = pr->d_MvC; a.mv_indptr = pr->d_indptrM; a.mv_indices = pr->d_indicesM; a.mv_nnz = (int)pr->nnzM;
 }
 void set_ep_M(Problem* pr, SolveArgs& a) {
-  a.ep_mv_vals = pr->d_MvC; a.ep_indptr = pr->d_indptrM; a.ep_indices = pr->d_indicesM; a.ep_nnz = (int)pr->nnzM;
-  a.ep_rows = pr->d_mrows; a.ep_nrows = pr->nmrows;
+  a.ep_mv_vals = pr->d_MvC; a.ep_list = pr->d_epM; a.ep_nl = pr->nmrows; a.ep_indices = pr->d_indicesM; a.ep_nnz = (int)pr->nnzM;
 }
 void set_ep_L(Problem* pr, SolveArgs& a) {
-  a.ep_mv_vals = pr->d_Lv; a.ep_indptr = pr->d_indptr; a.ep_indices = pr->d_indices; a.ep_nnz = (int)pr->nnz;
-  a.ep_rows = nullptr; a.ep_nrows = 0;
+  a.ep_mv_vals = pr->d_Lv; a.ep_list = pr->d_epL; a.ep_nl = pr->n; a.ep_indices = pr->d_indices; a.ep_nnz = (int)pr->nnz;
 }
 
 // Arguments of the lane substitution of `pr` with the listed factor `f`.
@@ -980,7 +995,6 @@ SolveArgs transposed_args(Problem* pr, sp_ctx* ctx) {
   a.ll = nullptr;
   a.spD = pr->facT.spD; a.spE = pr->facT.spE;    // null unless partitioned
   a.sp_nblk_f = pr->nblk; a.sp_u = pr->d_spT_u;
-  a.ep_rows = nullptr; a.ep_nrows = 0;   // the transposed patterns carry no row list
   return a;
 }
 
@@ -1962,6 +1976,7 @@ sp_status sp_adjoint_init(sp_ctx* ctx, int problem) {
         LT[(size_t)p * nnz + k] = pr->Lv[(size_t)p * nnz + where[k]];
       }
     CK(upload(&pr->d_indptrT, ipT, s));
+    CK(upload(&pr->d_epT, row_list(ipT), s));
     CK(upload(&pr->d_indicesT, ixT, s));
     CK(upload(&pr->d_MvT, MT, s));
     CK(upload(&pr->d_LvT, LT, s));
@@ -2071,7 +2086,7 @@ sp_status sp_step_adjoint(sp_ctx* ctx, int problem, double dt, const void* state
     t.vec[0] = pr->d_lamx; t.vec_coef[0] = 1.0; t.nvec = 1;
     t.xt_out = pr->d_mu[tb.s - 1];
     t.ep_mv_vals = tb.s == 2 ? pr->d_LvT : pr->d_MvT;
-    t.ep_indptr = pr->d_indptrT; t.ep_indices = pr->d_indicesT; t.ep_nnz = (int)pr->nnz;
+    t.ep_list = pr->d_epT; t.ep_nl = pr->n; t.ep_indices = pr->d_indicesT; t.ep_nnz = (int)pr->nnz;
     t.ep_mv_store = tb.s == 2 ? pr->d_LTmu : pr->d_MTmu;
     if ((st = solve(ctx, pr, s, t)) != SP_OK) return st;
   }
@@ -2086,7 +2101,7 @@ sp_status sp_step_adjoint(sp_ctx* ctx, int problem, double dt, const void* state
     SolveArgs t = transposed_args(pr, ctx);
     t.vec[0] = pr->d_JF; t.vec_coef[0] = 1.0; t.nvec = 1;
     t.xt_out = pr->d_mu[0];
-    t.ep_mv_vals = pr->d_MvT; t.ep_indptr = pr->d_indptrT; t.ep_indices = pr->d_indicesT;
+    t.ep_mv_vals = pr->d_MvT; t.ep_list = pr->d_epT; t.ep_nl = pr->n; t.ep_indices = pr->d_indicesT;
     t.ep_nnz = (int)pr->nnz; t.ep_mv_store = pr->d_MTmu; t.ep_mv_addvec = pr->d_mu[1];
     if ((st = solve(ctx, pr, s, t)) != SP_OK) return st;
   }

@@ -225,6 +225,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
   const int lp = mode == 0 ? a.lpad : 0, up = mode == 0 ? a.upad : 0;
   const int pp = block, tid = threadIdx.x;
   constexpr int nt = NT;
+  constexpr int PENCIL_U = MODE >= 0 ? 4 : 1;
   const int n = a.n;
   SolveSmem sm;
   {
@@ -294,7 +295,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
     __syncthreads();
   } else {
   // (mode 1, assembly only, then stores B~ for the substitution kernel)
-  pencil_assemble(a, pp, tid, nt, a.npad + 64, sm.B);
+  pencil_assemble<PENCIL_U>(a, pp, tid, nt, a.npad + 64, sm.B);
   if (mode == 1) {
     for (int r = tid; r < n; r += nt) a.bg[vec(r)] = sm.B[r];   // B~ for the substitution
     return;
@@ -480,7 +481,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
   }
   __syncthreads();
   const bool work = !*sm.abort_flag;
-  if (work) pencil_epilogue(a, pp, tid, nt, mode == 2, vec, sm.B);
+  if (work) pencil_epilogue<PENCIL_U>(a, pp, tid, nt, mode == 2, vec, sm.B);
 }
 
 // 256 threads: two pencils' CTAs fit on one SM (registers capped at 128 per

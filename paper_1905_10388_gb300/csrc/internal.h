@@ -155,9 +155,14 @@ cudaError_t launch_dz_adjoint(cudaStream_t s, int P, int Nz, double scale, const
 // stage takes M~X~^0 and three L~X~^j, and four F~^j.
 constexpr int SP_MAX_TERMS = 4;
 
+// Row items of the right-hand-side assembly: -1 where a mode has no row, else
+// row << 3 | differential << 2 | (-phase & 3).
+constexpr int ROW_ITEM_BITS = 3;
+constexpr int ROW_ITEM_DIF = 4;
+
 // Arguments of the pencil right-hand-side assembly + solve + epilogue kernel.
 struct SolveArgs {
-  int P, n, Nz, S, nbc, nnz;
+  int P, n, Nz, S, nbc;
   int kl, kuu, npad, lpad, upad;
   const double* Lf; const uint8_t* piv; const double* Uf; const double* rd;
   // prologue: B = sum_k vec_coef[k] vec[k] + mv_coef (Mat x) + sum_k fc_coef[k] P^L Fc_k + bc_coef g
@@ -179,13 +184,12 @@ struct SolveArgs {
   // stage's own right-hand side, when ep_from_b != 0 (mixed precision only)
   double ep_from_b, ep_alpha;
   const double2* ep_mv_addvec;                 // epilogue matvec acts on (X~ + addvec) if set
-  const int32_t* ep_indptr; const int32_t* ep_indices; int ep_nnz;    // pattern of ep_mv_vals
-  const int32_t* ep_rows; int ep_nrows;   // the pattern's non-empty rows (M~), or null: every row
+  const int4* ep_list; int ep_nl;              // (row, first entry, entries) of its ep_nl rows with entries
+  const int32_t* ep_indices; int ep_nnz;
   // tables (device)
-  const int32_t* indptr; const int32_t* indices;
-  const int32_t* row_map; const int32_t* col_map;
+  const int32_t* row_item;               // [equation][mode], see ROW_ITEM_BITS
+  const int32_t* col_map;
   const int32_t* var_recombine; const int32_t* var_phase;
-  const int32_t* eq_differential; const int32_t* eq_phase;
   const int32_t* nl_eq; int n_nl;        // equation index of each nonlinear slot
   const int32_t* bc_rows; const double2* bc_values;
   DevStatus* status;

@@ -12,63 +12,186 @@ constexpr int SPK_BW = 32;            // backward window rows (kl + ku <= 31)
 constexpr int SPK_CHUNK = 32;         // rows of a block: a multiple of this
 
 // ---------------------------------------------------------------------------
-// factorization time: the coupling matrices, one thread per (pencil, block,
-// unit inflow).  D_k[r][i]: forward window row r after block k for window
-// row i = 1 before it (no fresh right-hand side); E_k[r][t]: backward
-// outflow r (row j0 - kuu + r) for unit inflow t (row j1 - kuu + t), or, for
-// the lane substitution (by_row), b of row j0 + r for unit b of row j1 + t.
-// The arithmetic is the substitution's own, written per row.
+// factorization time: the coupling matrices, lane i carrying unit inflow i.
+// D_k[r][i]: forward window row r after block k for window row i = 1 before it
+// (no fresh right-hand side); E_k[r][t]: backward outflow r (row j0 - kuu + r)
+// for unit inflow t (row j1 - kuu + t), or, for the lane substitution (by_row),
+// b of row j0 + r for unit b of row j1 + t.  The arithmetic is the
+// substitution's own, written per row.  A warp takes a block's E, or its D with
+// a 32-row window, or four blocks' D with 8-row windows.
+//
+// Bound by the FP64 pipe (64 cycles per warp instruction) and, with few
+// pencils, by the row chain.  A 32-row window's row has 2 to 9 multipliers that
+// are not zero of up to 31: they are loaded one per lane, four rows ahead, and
+// a ballot picks the FMAs that are issued; the window stays in registers, the
+// shift by a row being the FMA's destination.  One thread per inflow with
+// indexed windows in local memory and every multiplier's FMA took 1625 us at
+// 512 x 256 (256 pencils, 28 forward and 4 back blocks), 241 us for the
+// 256 x 64 eigenvalue problem; this form 206 us and 87 us.
 // ---------------------------------------------------------------------------
-template <int FW>
-__global__ void k_spike_coupling(int P, int npad, int nblk_f, int nblk, int kl, int kuu, int lpad, int upad,
-                                 const double* __restrict__ L, const uint8_t* __restrict__ piv,
-                                 const double* __restrict__ U, double* __restrict__ D, double* __restrict__ E,
-                                 bool by_row) {
-  constexpr int FS = FW - 1;
-  const long long nf = (long long)P * nblk_f * FS;
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= nf + (long long)P * nblk * kuu) return;
-  if (idx < nf) {
-    const int i = (int)(idx % FS);
-    const int k = (int)((idx / FS) % nblk_f);
-    const int p = (int)(idx / ((long long)FS * nblk_f));
-    const int m = npad / nblk_f, j0 = k * m, j1 = j0 + m;
-    double win[FW];
-    for (int t = 0; t < FW; ++t) win[t] = (t == i) ? 1.0 : 0.0;
-    const double* Lp = L + (size_t)p * npad * lpad;
-    const uint8_t* pv = piv + (size_t)p * npad;
-    for (int j = j0; j < j1; ++j) {
-      const int off = pv[j];
-      const double y = win[off];        // the pivot row's value is y_j
-      win[off] = win[0];                // row j's value moves to the pivot row
-      for (int d = 1; d <= kl; ++d) win[d] = fma(-Lp[(size_t)j * lpad + d - 1], y, win[d]);
-      for (int t = 0; t < FW - 1; ++t) win[t] = win[t + 1];
-      win[FW - 1] = 0.0;
-    }
-    double* Dk = D + ((size_t)p * nblk_f + k) * FS * FW;
-    for (int r = 0; r < FS; ++r) Dk[r * FW + i] = win[r];
-  } else {
-    const long long jdx = idx - nf;
-    const int t0 = (int)(jdx % kuu);
-    const int k = (int)((jdx / kuu) % nblk);
-    const int p = (int)(jdx / ((long long)kuu * nblk));
-    const int m = npad / nblk, j0 = k * m, j1 = j0 + m;
-    double w[SPK_BW];                   // w[t]: pending row j - t
-    const double* Up = U + (size_t)p * npad * upad;
-    double* Ek = E + ((size_t)p * nblk + k) * kuu * SPK_BW;
-    // inflow t0: partial sum of row j1 - kuu + t0, or (by_row) b of row j1 + t0
-    for (int t = 0; t < SPK_BW; ++t)
-      w[t] = by_row ? ((t0 + 1 + t <= kuu && j1 + t0 < npad) ? -Up[(size_t)(j1 + t0) * upad + t0 + 1 + t] : 0.0)
-                    : (t == kuu - 1 - t0 ? 1.0 : 0.0);
-    for (int j = j1 - 1; j >= j0; --j) {
-      const double bj = w[0];
-      if (by_row && j - j0 < kuu) Ek[(j - j0) * SPK_BW + t0] = bj;
-      for (int t = 1; t <= kuu; ++t) w[t] = fma(-Up[(size_t)j * upad + t], bj, w[t]);
-      for (int t = 0; t < SPK_BW - 1; ++t) w[t] = w[t + 1];
-      w[SPK_BW - 1] = 0.0;
-    }
-    for (int r = 0; r < kuu && !by_row; ++r) Ek[r * SPK_BW + t0] = w[kuu - 1 - r];
+// window w of the row chain past one row with value y: w[t - 1] = w[t] - l_t y,
+// l_t held by lane t (zero where the row has no multiplier)
+__device__ __forceinline__ void window_step(double (&w)[SPK_BW], double l, double y) {
+  const unsigned on = __ballot_sync(0xffffffffu, (__double_as_longlong(l) << 1) != 0);
+#pragma unroll
+  for (int t = 1; t < SPK_BW; ++t) {
+    if ((on >> t) & 1u)
+      w[t - 1] = fma(-__shfl_sync(0xffffffffu, l, t), y, w[t]);
+    else
+      w[t - 1] = w[t];
   }
+  w[SPK_BW - 1] = 0.0;
+}
+
+constexpr int SPK_AHEAD = 4;          // rows loaded ahead (a divisor of SPK_CHUNK)
+
+// D of one block, 32-row window
+__device__ __forceinline__ void coupling_d32(int j0, int j1, int kl, int lpad, const double* __restrict__ Lp,
+                                             const uint8_t* __restrict__ pv, double* __restrict__ Dk) {
+  const int lane = threadIdx.x & 31;
+  double w[SPK_BW], l[SPK_AHEAD];
+#pragma unroll
+  for (int t = 0; t < SPK_BW; ++t) w[t] = (t == lane) ? 1.0 : 0.0;
+  uint32_t pw;
+  auto load = [&](int j, double (&l_)[SPK_AHEAD], uint32_t& pw_) {
+    const bool in = j < j1;
+    pw_ = in ? *reinterpret_cast<const uint32_t*>(pv + j) : 0u;
+#pragma unroll
+    for (int i = 0; i < SPK_AHEAD; ++i)
+      l_[i] = (in && lane >= 1 && lane <= kl) ? Lp[(size_t)(j + i) * lpad + lane - 1] : 0.0;
+  };
+  load(j0, l, pw);
+  for (int j = j0; j < j1; j += SPK_AHEAD) {
+    double ln[SPK_AHEAD];
+    uint32_t pn;
+    load(j + SPK_AHEAD, ln, pn);
+#pragma unroll
+    for (int i = 0; i < SPK_AHEAD; ++i) {
+      const int off = (pw >> (8 * i)) & 0xff;
+      double y = w[0];                  // the pivot row's value is y_j
+      if (off != 0) {
+#pragma unroll
+        for (int t = 1; t < SPK_BW; ++t)
+          if (t == off) { y = w[t]; w[t] = w[0]; }   // row j's value moves to the pivot row
+      }
+      window_step(w, l[i], y);
+    }
+    pw = pn;
+#pragma unroll
+    for (int i = 0; i < SPK_AHEAD; ++i) l[i] = ln[i];
+  }
+  if (lane < SPK_BW - 1) {
+#pragma unroll
+    for (int r = 0; r < SPK_BW - 1; ++r) Dk[r * SPK_BW + lane] = w[r];
+  }
+}
+
+// D of one block, 8-row window, by eight lanes
+__device__ __forceinline__ void coupling_d8(bool act, int j0, int m, int kl, int lpad, const double* __restrict__ Lp,
+                                            const uint8_t* __restrict__ pv, double* __restrict__ Dk) {
+  const int i = threadIdx.x & 7;
+  double w[SPK_FW], l[SPK_FS];
+#pragma unroll
+  for (int t = 0; t < SPK_FW; ++t) w[t] = (t == i) ? 1.0 : 0.0;
+  int off;
+  auto load = [&](int j, double (&l_)[SPK_FS], int& off_) {
+    const bool in = act && j < j0 + m;
+    off_ = in ? pv[j] : 0;
+#pragma unroll
+    for (int d = 0; d < SPK_FS; ++d) l_[d] = (in && d < kl) ? Lp[(size_t)j * lpad + d] : 0.0;
+  };
+  load(j0, l, off);
+  for (int j = j0; j < j0 + m; ++j) {
+    double ln[SPK_FS];
+    int on;
+    load(j + 1, ln, on);
+    double y = w[0];
+#pragma unroll
+    for (int t = 1; t < SPK_FW; ++t) {
+      const bool at = t == off;
+      y = at ? w[t] : y;
+      w[t] = at ? w[0] : w[t];
+    }
+#pragma unroll
+    for (int d = 0; d < SPK_FS; ++d) w[d] = fma(-l[d], y, w[d + 1]);
+    w[SPK_FW - 1] = 0.0;
+    off = on;
+#pragma unroll
+    for (int d = 0; d < SPK_FS; ++d) l[d] = ln[d];
+  }
+  if (act && i < SPK_FS) {
+#pragma unroll
+    for (int r = 0; r < SPK_FS; ++r) Dk[r * SPK_FW + i] = w[r];
+  }
+}
+
+// E of one block
+__device__ __forceinline__ void coupling_e(int j0, int j1, int kuu, int npad, int upad, bool by_row,
+                                           const double* __restrict__ Up, double* __restrict__ Ek) {
+  const int lane = threadIdx.x & 31;
+  double w[SPK_BW], l[SPK_AHEAD];     // w[t]: pending row j - t
+  // inflow `lane`: partial sum of row j1 - kuu + lane, or (by_row) b of row j1 + lane
+#pragma unroll
+  for (int t = 0; t < SPK_BW; ++t) {
+    if (by_row)
+      w[t] = (lane + 1 + t <= kuu && j1 + lane < npad) ? -Up[(size_t)(j1 + lane) * upad + lane + 1 + t] : 0.0;
+    else
+      w[t] = t == kuu - 1 - lane ? 1.0 : 0.0;
+  }
+  auto load = [&](int j, double (&l_)[SPK_AHEAD]) {     // rows j, j - 1, ..
+#pragma unroll
+    for (int i = 0; i < SPK_AHEAD; ++i)
+      l_[i] = (j >= j0 && lane >= 1 && lane <= kuu) ? Up[(size_t)(j - i) * upad + lane] : 0.0;
+  };
+  load(j1 - 1, l);
+  for (int j = j1 - 1; j >= j0; j -= SPK_AHEAD) {
+    double ln[SPK_AHEAD];
+    load(j - SPK_AHEAD, ln);
+#pragma unroll
+    for (int i = 0; i < SPK_AHEAD; ++i) {
+      const double bj = w[0];
+      if (by_row && j - i - j0 < kuu && lane < kuu) Ek[(j - i - j0) * SPK_BW + lane] = bj;
+      window_step(w, l[i], bj);
+    }
+#pragma unroll
+    for (int i = 0; i < SPK_AHEAD; ++i) l[i] = ln[i];
+  }
+  if (!by_row && lane < kuu) {
+#pragma unroll
+    for (int t = 0; t < SPK_BW; ++t)
+      if (t < kuu) Ek[(kuu - 1 - t) * SPK_BW + lane] = w[t];
+  }
+}
+
+constexpr int SPK_COUPLING_WARPS = 2;   // per CTA: few pencils spread over more SMs
+template <int FW>
+__global__ void __launch_bounds__(SPK_COUPLING_WARPS * 32)
+    k_spike_coupling(int P, int npad, int nblk_f, int nblk, int kl, int kuu, int lpad, int upad,
+                     const double* __restrict__ L, const uint8_t* __restrict__ piv, const double* __restrict__ U,
+                     double* __restrict__ D, double* __restrict__ E, bool by_row) {
+  constexpr int FS = FW - 1, PER = SPK_BW / FW;          // blocks of D per warp
+  const int nd = (P * nblk_f + PER - 1) / PER, ne = P * nblk;
+  int w = blockIdx.x * SPK_COUPLING_WARPS + (threadIdx.x >> 5);
+  // the back blocks, the longer chains, first
+  if (w < ne) {
+    const int p = w / nblk, k = w - p * nblk, m = npad / nblk;
+    coupling_e(k * m, (k + 1) * m, kuu, npad, upad, by_row, U + (size_t)p * npad * upad,
+               E + (size_t)w * kuu * SPK_BW);
+    return;
+  }
+  w -= ne;
+  if (w >= nd) return;
+  const int m = npad / nblk_f;
+  const int b = w * PER + (FW == 8 ? (threadIdx.x & 31) >> 3 : 0);
+  const bool act = b < P * nblk_f;
+  const int p = act ? b / nblk_f : 0, k = act ? b - p * nblk_f : 0;
+  const double* Lp = L + (size_t)p * npad * lpad;
+  const uint8_t* pv = piv + (size_t)p * npad;
+  double* Dk = D + ((size_t)p * nblk_f + k) * FS * FW;
+  if constexpr (FW == 8)
+    coupling_d8(act, k * m, m, kl, lpad, Lp, pv, Dk);
+  else
+    coupling_d32(k * m, (k + 1) * m, kl, lpad, Lp, pv, Dk);
 }
 
 cudaError_t launch_spike_coupling(cudaStream_t s, int P, int npad, int nblk_f, int nblk, int kl, int kuu, int lpad,
@@ -77,10 +200,10 @@ cudaError_t launch_spike_coupling(cudaStream_t s, int P, int npad, int nblk_f, i
       npad % (nblk_f * SPK_CHUNK))
     return cudaErrorInvalidValue;
   const bool wide = kl > SPK_FS;
-  const long long total = (long long)P * (nblk_f * (wide ? SPK_BW - 1 : SPK_FS) + nblk * kuu);
+  const long long warps = (long long)P * nblk + (wide ? (long long)P * nblk_f : ((long long)P * nblk_f + 3) / 4);
   auto* k = wide ? k_spike_coupling<SPK_BW> : k_spike_coupling<SPK_FW>;
-  k<<<(unsigned)((total + 127) / 128), 128, 0, s>>>(P, npad, nblk_f, nblk, kl, kuu, lpad, upad, f.L, f.piv, f.U,
-                                                   f.spD, f.spE, by_row);
+  k<<<(unsigned)((warps + SPK_COUPLING_WARPS - 1) / SPK_COUPLING_WARPS), SPK_COUPLING_WARPS * 32, 0, s>>>(
+      P, npad, nblk_f, nblk, kl, kuu, lpad, upad, f.L, f.piv, f.U, f.spD, f.spE, by_row);
   return cudaGetLastError();
 }
 

@@ -323,7 +323,7 @@ __device__ __forceinline__ void pencil_split_body(const SolveArgs& a, int p, dou
     const double g = uin[q];
     gs[q] = dfinite(g) ? g : 0.0;
   }
-  pencil_assemble(a, p, tid, NT, npad + 64, reinterpret_cast<double2*>(B));
+  pencil_assemble<1>(a, p, tid, NT, npad + 64, reinterpret_cast<double2*>(B));
   const size_t prow = (size_t)p * n;
   if (a.ep_from_b != 0.0)                        // the epilogue's L~X~ takes B~
     for (int r = tid; r < n; r += NT) a.bg[prow + r] = reinterpret_cast<double2*>(B)[r];
@@ -419,7 +419,7 @@ __device__ __forceinline__ void pencil_split_body(const SolveArgs& a, int p, dou
     for (int t = warp; t < (nblk - 1) * 2; t += NW) split_bwd<2>(a, p, t >> 1, t & 1, nblk, m, B, gs, us, o0);
     __syncthreads();
   }
-  pencil_epilogue(a, p, tid, NT, true, [&](int r) { return prow + r; }, reinterpret_cast<const double2*>(B));
+  pencil_epilogue<1>(a, p, tid, NT, true, [&](int r) { return prow + r; }, reinterpret_cast<const double2*>(B));
 }
 
 template <bool WIDE, int NT>
