@@ -13,7 +13,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libspectau.so")
 BUILD = os.path.join(HERE, "_build")
-SOURCES = ["api.cu", "band.cu", "lanes.cu", "split.cu", "spike.cu", "chebmma.cu", "transforms.cu", "rows_x32.cu", "rows_x64.cu", "rows_y32.cu", "rows_y64.cu",
+SOURCES = ["api.cu", "band.cu", "lanes.cu", "split.cu", "pair.cu", "spike.cu", "chebmma.cu", "transforms.cu", "rows_x32.cu", "rows_x64.cu", "rows_y32.cu", "rows_y64.cu",
            "rows_z32.cu", "rows_z64.cu", "rows_b32.cu", "rows_b64.cu", "static_transform.cu", "peak.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]

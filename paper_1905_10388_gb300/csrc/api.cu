@@ -1037,7 +1037,7 @@ struct Batch {
   std::vector<int> ids;
   int prec = 0, scheme = 0, nstage = 0, parity = 0;
   int tile = 8;
-  int max_ngz = 0, max_kuu = 0;
+  int max_ngz = 0, max_kl = 0, max_kuu = 0;
   size_t x_smem = 0, s_smem = 0;
   bool split = false;                        // every problem's solves in the partitioned kernel
   bool fast = false;                         // every problem's transforms on compile-time lengths
@@ -1097,15 +1097,20 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
     for (int e = 0; e < (int)pr->nl_eqs.size(); ++e)
       for (int t = 0; t < nt; ++t) zf.push_back({zc, make_int4((int)q, t, e, 0)});
     for (int r = 0; r < pr->Ngz; ++r) xr.push_back({(long long)pr->Ngx, make_int4((int)q, r, 0, 0)});
-    for (int p = 0; p < pr->P; ++p) sv.push_back({(long long)pr->n, make_int4((int)q, p, 0, 0)});
+    const int per = b->split ? 1 : pencil_pair_per(pr->npad, pencils);
+    for (int p = 0; p < pr->P; p += per)
+      sv.push_back({(long long)pr->n, make_int4((int)q, p, std::min(per, pr->P - p), 0)});
     b->max_ngz = std::max(b->max_ngz, pr->Ngz);
+    b->max_kl = std::max(b->max_kl, pr->kl);
     b->max_kuu = std::max(b->max_kuu, pr->kl + pr->ku);
     const int nf = (int)pr->gfields.size(), ne = (int)pr->nl_eqs.size();
     b->x_smem = std::max(b->x_smem, b->fast ? x_rows_bytes(pr->prec, pr->Ngx, nf, ne)
                                             : x_smem_bytes(pr->prec, pr->Ngx, 7, nf, ne));
     b->z_smem = std::max(b->z_smem, z_cols_bytes(pr->prec, pr->Ngz));
     b->s_smem = std::max(b->s_smem, b->split ? pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false)
-                                             : pencil_solve_smem(pr->npad, pr->lpad, pr->upad));
+                                             : pencil_pair_smem(pr->npad, per));
+    // (longer pencils than a lone problem's window kernel takes stay refused)
+    if (!b->split && pencil_solve_smem(pr->npad, pr->lpad, pr->upad) > 227 * 1024) CK(cudaErrorInvalidValue);
   }
   auto finish = [](std::vector<std::pair<long long, int4>>& v) {
     std::stable_sort(v.begin(), v.end(), [](const auto& a, const auto& c) { return a.first > c.first; });
@@ -1145,7 +1150,6 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
       zfv.push_back(zdesc_forward(ps[q], plans[q][i].fc_out));
       if (!b->fast) zfv.back().wq = zbv.back().wq;
       av.push_back(plans[q][i].args);
-      av.back().fwd16 = 1;            // throughput-bound: both parts' forward in one warp
       if (b->split) stage_lx(ps[q], av.back());
       fill_f_halves(av.back());
     }
@@ -1197,7 +1201,7 @@ sp_status batch_step(sp_ctx* ctx, Batch* b, cudaStream_t s) {
       CK(launch_cheb_forward_batched(s, b->prec, b->tile, st.d_zf, b->d_wzf, b->nzf, b->max_ngz, q2));
     }
     if (b->split) CK(launch_pencil_split_batched(s, st.d_args, b->d_ws, b->ns, b->s_smem));
-    else CK(launch_pencil_solve_batched(s, st.d_args, b->d_ws, b->ns, b->max_kuu, b->s_smem));
+    else CK(launch_pencil_pair_batched(s, st.d_args, b->d_ws, b->ns, b->max_kl, b->max_kuu, b->s_smem));
   }
   return SP_OK;
 }

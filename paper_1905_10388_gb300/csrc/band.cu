@@ -332,50 +332,8 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
       done = k + 1;
       return true;
     };
-    // forward: row interchanges and unit-lower multipliers.  With fwd16 and
-    // kl <= 15 warp 0 carries both parts in two 16-lane windows (lanes 0-15
-    // the real, 16-31 the imaginary part): one DFMA instruction per row for
-    // both, half the FP64 issue of a 32-lane window per part, the same
-    // arithmetic per element.  Warp 1 still joins every chunk's barrier
-    // (ring slots).  Batched: 6.36 -> 5.72 ms per 64-instance step; a lone
-    // 512 x 256 solve, bound by its chain latency, went 0.295 -> 0.309 ms.
-    if (a.fwd16 && a.kl <= 15) {
-      const int hl = lane & 15, hb = lane & 16;
-      double* Bh = reinterpret_cast<double*>(sm.B) + (lane >> 4);   // this half's part
-      double v = Bh[2 * hl];          // window element b[j + ((hl - j) & 15)]
-      double nv = Bh[2 * (hl + 16)];  // the element this lane takes next
-      double vs = v;
-      for (int c = 0; c < nchunks; ++c) {
-        const int s = c % SOLVE_RING;
-        if (!chunk_sync(&sm.barL[s], c, doneL)) { ok = false; break; }
-        if (tid == 0 && c >= 1 && c - 1 + SOLVE_RING < nchunks) {
-          fence_proxy_async();
-          issue_L(c - 1 + SOLVE_RING);   // both warps are past chunk c - 1
-        }
-        if (comp != 0) continue;
-        const double* Lc = sm.Lring + (size_t)s * SOLVE_CHUNK * a.lpad;
-        const uint32_t* Pw = reinterpret_cast<const uint32_t*>(sm.Pring + (size_t)s * SOLVE_CHUNK);
-        const int j0 = c * SOLVE_CHUNK;
-#pragma unroll
-        for (int jj = 0; jj < 32; ++jj) {
-          const int off = (Pw[jj >> 2] >> (8 * (jj & 3))) & 0xff;
-          const int q = jj & 15;
-          const int pl = ((q + off) & 15) | hb;
-          const int d = (hl - q) & 15;
-          const double l = (d >= 1 && d <= a.kl) ? Lc[jj * a.lpad + d - 1] : 0.0;
-          const double bj = __shfl_sync(0xffffffffu, vs, pl);        // pivot row value = y_j
-          const double vo = __shfl_sync(0xffffffffu, vs, q | hb);    // old b_j moves to the pivot row
-          const double nxt = Bh[2 * (j0 + jj + 32)];
-          v = (lane == pl) ? vo : v;
-          v = fma(-l, bj, v);
-          vs = v;
-          const bool own = (hl == q);
-          if (own) Bh[2 * (j0 + jj)] = bj;
-          v = own ? nv : v;
-          nv = own ? nxt : nv;
-        }
-      }
-    } else {
+    // forward: row interchanges and unit-lower multipliers
+    {
       double v = Bd[2 * lane];          // window element b[j + ((lane - j) & 31)]
       double nv = Bd[2 * (lane + 32)];  // the element this lane takes next
       // shuffle source: v before the owner lane swaps in its next element --
@@ -493,14 +451,6 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 2) k_pencil_solve(SolveArgs a) 
   extern __shared__ __align__(128) unsigned char smem_raw[];
   pencil_solve_body<RU, -1, SOLVE_THREADS>(a, blockIdx.x, smem_raw);
 }
-// 128 threads, three CTAs per SM: for more pencils than two CTAs per SM
-// hold, more concurrent chains outweigh the narrower assembly and epilogue
-template <int RU>
-__global__ void __launch_bounds__(128, 3) k_pencil_solve_narrow(SolveArgs a) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  pencil_solve_body<RU, -1, 128>(a, blockIdx.x, smem_raw);
-}
-
 // right-hand-side assembly only (MODE 1) or epilogue only (MODE 2), around
 // the lane substitution: shared memory for B~ alone, several CTAs per SM
 template <int MODE>
@@ -509,31 +459,7 @@ __global__ void __launch_bounds__(128, 6) k_pencil_stage(SolveArgs a) {
   pencil_solve_body<1, MODE>(a, blockIdx.x, smem_raw);
 }
 
-// a batch of problems: work item (problem, pencil) per CTA
-template <int RU>
-// (one CTA per pencil: its items are long dependent chains, so a
-// persistent grid buys nothing here; 128 registers keep three CTAs per SM)
-__global__ void __launch_bounds__(128, 4) k_pencil_solve_batched(const SolveArgs* __restrict__ args,
-                                                                 const int4* __restrict__ work) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  const int4 w = work[blockIdx.x];
-  pencil_solve_body<RU>(args[w.x], w.y, smem_raw);
-}
-
 size_t pencil_solve_smem(int npad, int lpad, int upad) { return solve_smem_bytes(npad, lpad, upad); }
-
-cudaError_t launch_pencil_solve_batched(cudaStream_t s, const SolveArgs* args, const int4* work, int nwork,
-                                        int max_kuu, size_t smem) {
-  if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  if (max_kuu <= 31) {
-    cudaFuncSetAttribute(k_pencil_solve_batched<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_pencil_solve_batched<1><<<nwork, 128, smem, s>>>(args, work);
-  } else {
-    cudaFuncSetAttribute(k_pencil_solve_batched<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_pencil_solve_batched<2><<<nwork, 128, smem, s>>>(args, work);
-  }
-  return cudaGetLastError();
-}
 
 cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
   SolveArgs a = args;
@@ -559,18 +485,10 @@ cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 1;
   }
-  // three CTAs of 128 threads per SM (228 KB of shared memory, 1 KB of it
-  // reserved per CTA) when the pencils fill more than one wave of two
-  if (a.P > 2 * sms && 3 * (smem + 1024) <= 228 * 1024) {
-    if (a.kuu <= 31) {
-      cudaFuncSetAttribute(k_pencil_solve_narrow<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_pencil_solve_narrow<1><<<grid, 128, smem, s>>>(a);
-    } else {
-      cudaFuncSetAttribute(k_pencil_solve_narrow<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_pencil_solve_narrow<2><<<grid, 128, smem, s>>>(a);
-    }
-    return cudaGetLastError();
-  }
+  // more pencils than one wave of two CTAs per SM: several pencils' chains per
+  // sub-partition instead of a CTA per pencil (where three of this kernel's CTAs
+  // would fit an SM, 228 KB of shared memory, 1 KB of it reserved per CTA)
+  if (a.P > 2 * sms && 3 * (smem + 1024) <= 228 * 1024) return launch_pencil_pair(s, a);
   if (a.kuu <= 31) {
     cudaFuncSetAttribute(k_pencil_solve<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_pencil_solve<1><<<grid, SOLVE_THREADS, smem, s>>>(a);

@@ -199,11 +199,6 @@ struct SolveArgs {
   // keeps B~ [p][n] in bg for the epilogue's L~X~
   int mode;
   double2* bg; const double2* xg;
-  // 1: with kl <= 15, one warp runs both parts' forward substitution in two
-  // 16-lane windows (half the FP64 issue; the batched solve, bound by the
-  // FP64 pipe, sets it; a lone problem's whole-row chains are bound by their
-  // latency and keep a 32-lane window per part)
-  int fwd16;
   // the factor's lists (host pointer; null: no lane substitution)
   const LaneList* ll;
   // coupling matrices of the partitioned substitution (null: not available)
@@ -286,9 +281,13 @@ cudaError_t launch_pencil_split(cudaStream_t s, const SolveArgs& a);
 cudaError_t launch_pencil_split_batched(cudaStream_t s, const SolveArgs* args, const int4* work, int nwork,
                                         size_t smem);
 size_t pencil_split_smem(int npad, int nblk, int nblk_f, int kuu, bool wide);
-// batched pencil solves: one CTA per (problem, pencil) work item
-cudaError_t launch_pencil_solve_batched(cudaStream_t s, const SolveArgs* args, const int4* work, int nwork,
-                                        int max_kuu, size_t smem);
+// whole-row-order solves of one or two pencils per CTA (pair.cu); batched: work
+// items (problem, first pencil, pencils)
+cudaError_t launch_pencil_pair(cudaStream_t s, const SolveArgs& a);
+cudaError_t launch_pencil_pair_batched(cudaStream_t s, const SolveArgs* args, const int4* work, int nwork, int max_kl,
+                                       int max_kuu, size_t smem);
+size_t pencil_pair_smem(int npad, int per);
+int pencil_pair_per(int npad, long long pencils);
 bool lanes_supported(int kl, int kuu);
 cudaError_t launch_coef_to_solve(cudaStream_t s, int P, int S, int Nz, const double2* xc,
                                  double2* xt, const int32_t* col_map, const int32_t* var_recombine,
