@@ -1,4 +1,5 @@
-"""Whole-row-order solves of one or two pencils per CTA (Sec. "Matrix solvers").
+"""Whole-row-order solves of one or two pencils per CTA and the register
+factorization (Sec. "Matrix solvers").
 
 * The pair kernel runs every FMA in the window kernel's order: a batch's
   states equal the problems stepped alone bit for bit, and a lone problem's
@@ -8,6 +9,8 @@
   factors) are reached only through their own solvers: a long channel's first
   pencils against the same pencils of a short one, and the adjoint step against
   its form in row blocks.
+* Factors of matrices as short as the 32-column window and longer, narrow and
+  wide bands, against the oracle after two steps.
 """
 import numpy as np
 import pytest
@@ -17,11 +20,13 @@ if not torch.cuda.is_available():
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
 import seeded_inputs as si
+from oracle import fisher as ofk
 from oracle import rb as orb
+from oracle import timesteppers as ots
 from paper_1905_10388_gb300 import _lib
 from paper_1905_10388_gb300.adjoint import RBAdjoint
-from paper_1905_10388_gb300.solver import Context, RB3DSolver, RBOnsetEVP, RBSolver, step_batched
-from gpu_util import rel_err
+from paper_1905_10388_gb300.solver import Context, FisherKPPSolver, RB3DSolver, RBOnsetEVP, RBSolver, step_batched
+from gpu_util import check_fields, oracle_floor, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -117,3 +122,44 @@ def test_adjoint_of_a_long_channel(ctx):
         out.append(Ld.cpu().numpy()[slot])
     for a, b in zip(*out):
         assert rel_err(b, a) < 1e-5
+
+
+@pytest.mark.parametrize("nz", [16, 32])
+def test_factor_of_small_matrices_rb(ctx, nz):
+    """n = 112, 224 with kl = 7.  Bar 1e-11: at these sizes w's error against the
+    oracle's other formulation is 1.1e-12 with either factorization."""
+    nx, ra, dt = 16, 1e5, 1e-3
+    xi = si.rb_noise(7, nz, nx)
+    s = RBSolver(ctx, nx, nz, ra, scheme="RK222")
+    s.factor(dt)
+    s.set_initial_state(xi)
+    s.step(2)
+    s.sync()
+
+    def stepper(sysr):
+        st = ots.RungeKuttaIMEX(sysr)
+        st.dt = dt
+        return st
+    ref, floor = oracle_floor(lambda m, lu: orb.RB2D(nx, nz, ra, cheb_method=m, lu_method=lu),
+                              lambda sysr: sysr.initial_state(xi), stepper, 2)
+    check_fields(s.get_state(), ref, floor, 1e-11, label=f"factor_{nx}x{nz}_rk222_fp64_2steps")
+
+
+@pytest.mark.parametrize("nz", [16, 32])
+def test_factor_of_small_matrices_fisher(ctx, nz):
+    """n = 32, 64 with kl = 2."""
+    nx, dt = 16, 1e-3
+    u0 = si.fisher_noise(5, nz, nx)
+    s = FisherKPPSolver(ctx, nx, nz, scheme="RK222")
+    s.factor(dt)
+    s.set_initial_state(u0)
+    s.step(2)
+    s.sync()
+    sysr = ofk.FisherKPP(nx, nz, s.D, s.R, s.Lx)
+    X = sysr.initial_state(u0)
+    st = ots.RungeKuttaIMEX(sysr, ots.RK222)
+    for _ in range(2):
+        X = st.step(X, dt)
+    got = s.get_state()
+    for i, v in enumerate(ofk.FISHER_VARIABLES):
+        assert rel_err(got[i], X[i]) < 1e-12, v
