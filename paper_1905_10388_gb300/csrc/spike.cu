@@ -208,21 +208,23 @@ cudaError_t launch_spike_coupling(cudaStream_t s, int P, int npad, int nblk_f, i
 }
 
 // forward inflows: s_0 = rows 0..6 of B~, s_1 from block 0 (exact), then
-// s_{k+1} = s0_{k+1} + D_k s_k; one warp per (pencil, part), lanes 0..6.
-// The next step's matrix row and outflow are loaded before this step's FMAs.
+// s_{k+1} = s0_{k+1} + D_k s_k; eight lanes per (pencil, part), four of them per
+// warp and FMA (a warp each, at seven FMAs a step, was bound by the FP64 pipe:
+// Fisher-KPP 2048 x 1024, 2048 chains, 18.8 us against 13.9 us).  The
+// next step's matrix row and outflow are loaded before this step's FMAs.
 __global__ void __launch_bounds__(128) k_spike_fwd_rec(LaneArgs s, const double* __restrict__ D) {
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= s.P * 2) return;
-  const int p = w >> 1, c = w & 1;
-  const int i = lane < SPK_FS ? lane : 0;
+  const int chain = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const bool act = chain < s.P * 2;
+  const int p = act ? chain >> 1 : 0, c = chain & 1;
+  const int q = threadIdx.x & 7, i = q < SPK_FS ? q : 0;
+  const bool own = act && q < SPK_FS;
   const double* Bp = reinterpret_cast<const double*>(s.bg + lane_index(p, i < s.n ? i : 0, s.npad)) + c;
   auto at = [&](int k) { return (((size_t)p * s.nblk_f + k) * 2 + c) * SPK_FW; };
   double st = i < s.n ? Bp[0] : 0.0;
-  if (lane < SPK_FS) s.sst[at(0) + i] = st;
+  if (own) s.sst[at(0) + i] = st;
   if (s.nblk_f < 2) return;
   st = s.s0[at(1) + i];
-  if (lane < SPK_FS) s.sst[at(1) + i] = st;
+  if (own) s.sst[at(1) + i] = st;
   double dn[SPK_FS], sn = 0.0;
   auto load = [&](int k) {
     const double* Dk = D + ((size_t)p * s.nblk_f + k) * SPK_FS * SPK_FW + i * SPK_FW;
@@ -238,11 +240,11 @@ __global__ void __launch_bounds__(128) k_spike_fwd_rec(LaneArgs s, const double*
     double acc = sn, acc2 = 0.0;      // two independent FMA chains per step
     if (k + 1 < s.nblk_f - 1) load(k + 1);
 #pragma unroll
-    for (int t = 0; t < SPK_FS; t += 2) acc = fma(dc[t], __shfl_sync(0xffffffffu, st, t), acc);
+    for (int t = 0; t < SPK_FS; t += 2) acc = fma(dc[t], __shfl_sync(0xffffffffu, st, t, 8), acc);
 #pragma unroll
-    for (int t = 1; t < SPK_FS; t += 2) acc2 = fma(dc[t], __shfl_sync(0xffffffffu, st, t), acc2);
+    for (int t = 1; t < SPK_FS; t += 2) acc2 = fma(dc[t], __shfl_sync(0xffffffffu, st, t, 8), acc2);
     st = acc + acc2;
-    if (lane < SPK_FS) s.sst[at(k + 1) + i] = st;
+    if (own) s.sst[at(k + 1) + i] = st;
   }
 }
 
@@ -304,6 +306,52 @@ __global__ void __launch_bounds__(SPK_REC_WARPS * 32) k_spike_bwd_rec(LaneArgs s
   }
 }
 
+// the same for kuu <= W (8 or 16), W lanes per (pencil, part): four or two
+// chains share each FMA and nothing waits at a barrier (the four-warp form
+// issues its 32 columns' FMAs whatever kuu: Fisher-KPP 2048 x 1024, kuu = 8,
+// 75 us against 21 us).
+template <int W>
+__global__ void __launch_bounds__(128) k_spike_bwd_rec_narrow(LaneArgs s, const double* __restrict__ E) {
+  const int chain = (blockIdx.x * blockDim.x + threadIdx.x) / W;
+  const bool act = chain < s.P * 2;
+  const int p = act ? chain >> 1 : 0, c = chain & 1;
+  const int r = threadIdx.x & (W - 1), kuu = s.kuu;
+  const bool in = act && r < kuu;
+  auto at = [&](int k) { return (((size_t)p * s.nblk + k) * 2 + c) * SPK_BW + r; };
+  if (s.nblk < 2) return;
+  double en[W], on = 0.0, gn = 0.0;
+  auto load = [&](int k) {
+    const double* Ek = E + (((size_t)p * s.nblk + k) * kuu + (in ? r : 0)) * SPK_BW;
+#pragma unroll
+    for (int t = 0; t < W; ++t) en[t] = (in && t < kuu) ? Ek[t] : 0.0;
+    on = in ? s.o0[at(k)] : 0.0;
+    gn = (in && k > 1) ? spike_guess(s.uin[at(k - 1)]) : 0.0;
+  };
+  double d;                           // u_k - g_k
+  {
+    const double u = in ? s.o0[at(s.nblk - 1)] : 0.0;
+    const double g = (in && s.nblk > 2) ? spike_guess(s.uin[at(s.nblk - 2)]) : 0.0;
+    d = u - g;
+    if (in) s.uin[at(s.nblk - 2)] = u;
+  }
+  if (s.nblk > 2) load(s.nblk - 2);
+  for (int k = s.nblk - 2; k >= 1; --k) {
+    double ec[W];
+#pragma unroll
+    for (int t = 0; t < W; ++t) ec[t] = en[t];
+    const double o = on, g = gn;
+    if (k > 1) load(k - 1);
+    double acc = 0.0, acc2 = 0.0;     // two independent FMA chains per step
+#pragma unroll
+    for (int t = 0; t < W; t += 2) acc = fma(ec[t], __shfl_sync(0xffffffffu, d, t, W), acc);
+#pragma unroll
+    for (int t = 1; t < W; t += 2) acc2 = fma(ec[t], __shfl_sync(0xffffffffu, d, t, W), acc2);
+    const double u = o + (acc + acc2);
+    if (in) s.uin[at(k - 1)] = u;
+    d = u - g;
+  }
+}
+
 bool spike_supported(int kl, int kuu, int npad, int nblk) {
   return kl <= SPK_FS && spike_bwd_supported(kuu, npad, nblk);
 }
@@ -316,13 +364,19 @@ bool spike_bwd_supported(int kuu, int npad, int nblk) {
 // the recurrences alone, between the passes of the lane substitution
 cudaError_t launch_spike_forward_rec(cudaStream_t st, const LaneArgs& s, const double* D) {
   const int T = 128;
-  k_spike_fwd_rec<<<(unsigned)((s.P * 2 * 32 + T - 1) / T), T, 0, st>>>(s, D);
+  k_spike_fwd_rec<<<(unsigned)(((size_t)s.P * 2 * 8 + T - 1) / T), T, 0, st>>>(s, D);
   return cudaGetLastError();
 }
 
 cudaError_t launch_spike_backward_rec(cudaStream_t st, const LaneArgs& s, const double* E) {
   if (s.nblk < 2) return cudaSuccess;
-  k_spike_bwd_rec<<<s.P * 2, SPK_REC_WARPS * 32, 0, st>>>(s, E);
+  const int T = 128;
+  if (s.kuu <= 8)
+    k_spike_bwd_rec_narrow<8><<<(unsigned)(((size_t)s.P * 2 * 8 + T - 1) / T), T, 0, st>>>(s, E);
+  else if (s.kuu <= 16)
+    k_spike_bwd_rec_narrow<16><<<(unsigned)(((size_t)s.P * 2 * 16 + T - 1) / T), T, 0, st>>>(s, E);
+  else
+    k_spike_bwd_rec<<<s.P * 2, SPK_REC_WARPS * 32, 0, st>>>(s, E);
   return cudaGetLastError();
 }
 
