@@ -58,15 +58,14 @@ STAGES = {"RK222": 2, "RK443": 4, "RK111": 1, "SBDF1": 1, "SBDF2": 1, "SBDF3": 1
 
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one pencil
-# solve of the 512x256 SBDF2 FP64 step, summed over its eight launches
-# (assembly, partitioned substitution, epilogue), from one ncu capture of
-# `bench.py --precision fp64 --no-cpu-baseline --no-error --steps 3 --warmup 3`
-# (metrics gpu__time_duration.sum, dram__bytes_read.sum, dram__bytes_write.sum;
-# -k regex:"k_spike|k_pencil_stage_wide" -s 16 -c 8).  It is reported only
-# while the kernels' sources hash to the captured ones.
+# solve of the 512x256 SBDF2 FP64 step (one launch of k_pencil_split), from one
+# ncu capture of `bench.py --precision fp64 --no-cpu-baseline --no-error --steps 3
+# --warmup 3` (metrics gpu__time_duration.sum, dram__bytes_read.sum,
+# dram__bytes_write.sum; -k regex:k_pencil_split -s 4 -c 2).  It is reported only
+# while the kernel's sources hash to the captured ones.
 SOLVE_TRAFFIC = {"workload": "rb2d_512x256_sbdf2", "precision": "fp64", "bytes": 306.3032e6,
                  "sources_sha256": "272a9c00e27801bc99b3c01e82e5e5fe76e6aac3c3de33546d1b504c131c687a"}
-SOLVE_SOURCES = ("paper_1905_10388_gb300/csrc/band.cu", "paper_1905_10388_gb300/csrc/spike.cu",
+SOLVE_SOURCES = ("paper_1905_10388_gb300/csrc/split.cu", "paper_1905_10388_gb300/csrc/pencil.cuh",
                  "paper_1905_10388_gb300/csrc/internal.h", "paper_1905_10388_gb300/csrc/common.cuh",
                  "paper_1905_10388_gb300/csrc/tma.cuh")
 
@@ -394,24 +393,25 @@ def run_ours(args):
     flops, nbytes = solve_flops_bytes(s)
     n_, kl_, ku_ = s.band()
     # the library's automatic choice of substitution kernel (sp_set_solve_kernel):
-    # lane substitution (assembly, lanes, epilogue: three launches), the
-    # partitioned substitution (assembly, two forward passes and their
-    # recurrence, two backward passes and theirs, epilogue: eight launches),
-    # or the single window kernel
-    lanes = s.P >= 4096 and (kl_, kl_ + ku_) in ((9, 38), (7, 29))
+    # lane substitution of whole pencils (assembly, forward, back, epilogue:
+    # four launches) or of row blocks (two passes each way and the recurrences
+    # over blocks between them: eight), the partitioned solve of a pencil per
+    # CTA, two pencils per CTA, or the window kernel (one launch each)
     nblk = s.spike_blocks()
     factor_mb = s.P * s.solve_work()[1] / 1e6
     achieved = flops / (solve_ms * 1e-3) / 1e12
     peaks = measured_peaks()
-    if lanes:
-        kernel, solve_launches_per = "k_pencil_stage<1> + k_pencil_lanes + k_pencil_stage<2>", 3
-    elif nblk > 0:
-        kernel = (f"partitioned substitution, {nblk} row blocks per pencil: k_pencil_stage_wide<1> + "
-                  "k_spike_fwd<1> + k_spike_fwd_rec + k_spike_fwd<2> + k_spike_bwd<1> + k_spike_bwd_rec + "
-                  "k_spike_bwd<2> + k_pencil_stage_wide<2>")
+    if nblk > 0 and s.P >= 608:
+        kernel = (f"lane substitution, {nblk} row blocks per pencil: k_pencil_stage<1> + k_lane_fwd<1> + "
+                  "k_spike_fwd_rec + k_lane_fwd<2> + k_lane_bwd<1> + k_spike_bwd_rec + k_lane_bwd<2> + "
+                  "k_pencil_stage<2>")
         solve_launches_per = 8
+    elif nblk > 0:
+        kernel, solve_launches_per = f"k_pencil_split, {nblk} row blocks per pencil", 1
+    elif s.P >= 2048:
+        kernel, solve_launches_per = "k_pencil_stage<1> + k_lane_fwd<0> + k_lane_bwd<0> + k_pencil_stage<2>", 4
     else:
-        kernel, solve_launches_per = "k_pencil_solve", 1
+        kernel, solve_launches_per = "k_pencil_pair" if s.P > 304 else "k_pencil_solve", 1
     roof = {"kernel": kernel, "bound": "alu", "achieved": achieved, "peak": fp64_peak,
             "unit": "TFLOP/s", "frac": achieved / fp64_peak,
             "traffic": solve_traffic(args.workload, head), "algorithmic_bytes": nbytes,

@@ -245,10 +245,9 @@ sp_status sp_set_batch_persistent(sp_ctx* ctx, int nproblems, const int* problem
  * sp_adjoint_init: after sp_factor, factors the transposed pencils
  *   A~^T = M~^T + dt H_ii L~^T (banded LU with partial pivoting, FP64) and
  *   allocates the adjoint work buffers; for problems on the partitioned
- *   substitution it also computes the transposed factor's back-substitution
- *   coupling matrices (the transposed solves substitute forward whole-row,
- *   since kl' = ku is wider than the partitioned forward windows, and back
- *   in blocks) and zeroes their inflow guesses.
+ *   substitution it also computes the transposed factor's coupling matrices
+ *   (kl' = ku is wider than the 8-lane forward windows: the transposed
+ *   solves use 32-lane windows both ways) and zeroes their inflow guesses.
  * sp_step_adjoint: given the states of one forward step (states_dev,
  *   device, nstates consecutive arrays of S*P*N_z complex: X^n alone
  *   (nstates = 1; the first stage is then recomputed from X^n) or X^n
@@ -352,11 +351,11 @@ sp_status sp_cfl_dt(double freq, double dt_prev, double safety, double min_dt, d
  * with U), for the factor that the steady steps use (the last one of
  * sp_factor: SBDF2's, not its SBDF1 start):
  *   fma_per_row   multiply-adds per row and real right-hand side, forward
- *                 plus back.  Window kernel: kl + (kl + ku), every band
- *                 entry.  Lane kernel: kl + the mean number of listed
- *                 superdiagonal entries of U per column (the union of the
- *                 pencils' nonzero patterns); one multiply by 1/U_jj per row
- *                 comes on top in both.
+ *                 plus back.  Window and partitioned kernels: kl + (kl +
+ *                 ku), every band entry.  Lane kernel: the mean number of
+ *                 listed multipliers and superdiagonal entries of U per row
+ *                 (the union of 16 pencils' nonzero patterns); one multiply
+ *                 by 1/U_jj per row comes on top in all.
  *   factor_bytes  bytes of stored factor one pencil's substitution reads
  *                 (multipliers, U entries including 1/U_jj, pivot bytes).
  * Either pointer may be NULL.  SP_ERR_NOT_FACTORED before sp_factor. */
@@ -372,39 +371,39 @@ sp_status sp_get_solve_work(sp_ctx* ctx, int problem, double* fma_per_row, doubl
 sp_status sp_set_timing(sp_ctx* ctx, int problem, int max_launches);
 
 /* Choice of the substitution kernel of the pencil solves (Sec. "Matrix
- * solvers"; the arithmetic is the same, the order of every FMA too, so both
- * give identical results): SP_SOLVE_AUTO picks SP_SOLVE_LANES for problems
- * with at least 4096 pencils when (kl, kl + ku) is (9, 38) or (7, 29), else
- * SP_SOLVE_WINDOW.  WINDOW: one warp per pencil and real/imaginary part,
- * the band across the lanes (latency-bound few-pencil problems).  LANES:
- * one lane per pencil and real/imaginary part (throughput-bound
- * many-pencil problems; SP_ERR_ARG for other band widths).  SPIKE: the
- * partitioned substitution below (few long pencils; SP_ERR_ARG unless
- * kl <= 7 and kl + ku <= 31).  Must precede
- * the first call that moves the problem to the device (sp_factor,
- * sp_set_field, sp_transform): SP_ERR_STATE afterwards. */
+ * solvers").  WINDOW: whole pencils, the band across the lanes of a warp.
+ * LANES: whole pencils, one lane per pencil and real/imaginary part on the
+ * factor's listed entries (throughput-bound many-pencil problems; SP_ERR_ARG
+ * unless (kl, kl + ku) is (9, 38) or (7, 29)).  Both run every FMA in the same
+ * order and give identical results.  SPIKE: the partitioned substitution below
+ * (few pencils; SP_ERR_ARG unless kl <= 7 and kl + ku <= 31).  SP_SOLVE_AUTO
+ * picks LANES from 2048 pencils on where SPIKE does not apply, SPIKE as stated
+ * below, else WINDOW.  Must precede the first call that moves the problem to
+ * the device (sp_factor, sp_set_field, sp_transform): SP_ERR_STATE
+ * afterwards. */
 typedef enum { SP_SOLVE_AUTO = 0, SP_SOLVE_WINDOW = 1, SP_SOLVE_LANES = 2, SP_SOLVE_SPIKE = 3 } sp_solve_kernel;
 sp_status sp_set_solve_kernel(sp_ctx* ctx, int problem, int kind);
 
 /* Partitioned substitution (SP_SOLVE_SPIKE; Sec. "Matrix solvers": the
  * pencil solves are O(n) with the stored factor).  With fewer pencils than
  * the GPU has dependent-chain slots, each pencil's back substitution is cut
- * into nblk blocks of whole 32-row chunks (the forward one into blocks of
- * about 128 rows), substituted in parallel: a pass per block from guessed
+ * into nblk blocks of whole 32-row chunks (the forward one into blocks of 32
+ * to 64 rows), substituted in parallel: a pass per block from guessed
  * inflows, a recurrence over blocks with coupling matrices computed at
- * sp_factor (kl x kl forward, (kl+ku) x (kl+ku) backward per block), then a
- * pass with the true inflows.  The back substitution's guesses are the true
- * inflows of the problem's previous solve (zero after sp_factor or
- * sp_set_field, and for a guess that is not finite): exact for any guess,
- * and consecutive time-step solves then correct by small differences, so no
- * rounding is amplified by cancellation.  Results equal the whole-row-order
- * substitution to rounding.  SP_SOLVE_AUTO picks it for 2D problems with
- * fewer than 608 pencils of at least 512 rows when kl <= 7 and kl + ku <= 31.
- * sp_set_spike_blocks sets nblk (0: automatic, about 1024 / P blocks);
- * SP_ERR_ARG if the padded rows do not split into nblk whole 32-row chunks,
- * SP_ERR_STATE once the problem is on the device (like sp_set_solve_kernel).
- * sp_get_spike_blocks returns the block count in use (0: not partitioned,
- * or the problem not yet on the device). */
+ * sp_factor, then a pass with the true inflows.  The back substitution's
+ * guesses are the true inflows of the problem's previous solve (zero after
+ * sp_factor or sp_set_field, and for a guess that is not finite): exact for
+ * any guess, and consecutive time-step solves then correct by small
+ * differences, so no rounding is amplified by cancellation.  Results equal
+ * the whole-row-order substitution to rounding.  SP_SOLVE_AUTO picks it for
+ * problems with fewer than 4096 pencils of at least 512 padded rows, and with
+ * at most 304 pencils of at least 96, when kl + ku <= 31 and kl <= 7 (fewer than
+ * 608 pencils: kl <= 30) and the block counts fit shared memory.
+ * sp_set_spike_blocks sets nblk (0: automatic); SP_ERR_ARG if the padded rows
+ * do not split into nblk whole 32-row chunks, SP_ERR_STATE once the problem is
+ * on the device (like sp_set_solve_kernel).  sp_get_spike_blocks returns the
+ * block count in use (0: not partitioned, or the problem not yet on the
+ * device). */
 sp_status sp_set_spike_blocks(sp_ctx* ctx, int problem, int nblk);
 
 /* Chebyshev backward transform of the mixed form (Sec. "Chebyshev basis":

@@ -102,9 +102,8 @@ cudaError_t launch_spike_backward_rec(cudaStream_t s, const LaneArgs& a, const d
 
 // Problems with at least this many pencils use the lane substitution on whole
 // pencils.  Its time is the chain's (about 0.93 us per row and solve) up to
-// 608 groups, the window kernel's grows with the pencils: 288 rows of 3D
-// Rayleigh-Benard take 0.27 ms against 0.17 ms for 1024 pencils and 0.34 ms
-// for 2048.
+// 608 groups, the whole-row-order kernel's (pair.cu) grows with the pencils:
+// 288 rows of 3D Rayleigh-Benard take 0.27 ms against 0.14 ms for 1024 pencils.
 constexpr int LANE_MIN_PENCILS = 2048;
 
 // Chebyshev backward transform on the tensor cores (chebmma.cu): the split
