@@ -64,7 +64,7 @@ STAGES = {"RK222": 2, "RK443": 4, "RK111": 1, "SBDF1": 1, "SBDF2": 1, "SBDF3": 1
 # dram__bytes_write.sum; -k regex:k_pencil_split -s 4 -c 2).  It is reported only
 # while the kernel's sources hash to the captured ones.
 SOLVE_TRAFFIC = {"workload": "rb2d_512x256_sbdf2", "precision": "fp64", "bytes": 203.8e6,
-                 "sources_sha256": "7d83527d4c29b09065443b4a6ebeedfa2e060531cf4e92f5bb0b9dbc9735f21b"}
+                 "sources_sha256": "8189e88e12277a8a9be603e2271ccc22ed4f801dc07efa1b3ba7d6d40ee45eed"}
 SOLVE_SOURCES = ("paper_1905_10388_gb300/csrc/split.cu", "paper_1905_10388_gb300/csrc/pencil.cuh",
                  "paper_1905_10388_gb300/csrc/internal.h", "paper_1905_10388_gb300/csrc/common.cuh",
                  "paper_1905_10388_gb300/csrc/tma.cuh")

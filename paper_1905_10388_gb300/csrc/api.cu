@@ -564,7 +564,7 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
   pr->spike = !pr->lanes && split_fits && bands &&
               (pr->solve_kind == SP_SOLVE_SPIKE ||
                (pr->solve_kind == SP_SOLVE_AUTO && pr->P < SPIKE_MAX_PENCILS &&
-                (pr->npad >= SPIKE_MIN_ROWS || (pr->P <= SPLIT_MAX_PENCILS && pr->n >= SPLIT_MIN_ROWS))));
+                (pr->npad >= SPIKE_MIN_ROWS || (pr->P <= SPLIT_MAX_PENCILS && pr->npad >= SPLIT_MIN_ROWS))));
   if (pr->spike) {
     pr->by_group = pr->P >= LANE_SPLIT_PENCILS;
     const size_t nv = (size_t)pr->P * pr->nblk * 2, nvf = (size_t)pr->P * pr->nblk_f * 2;

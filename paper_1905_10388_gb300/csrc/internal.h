@@ -90,10 +90,9 @@ constexpr int SPIKE_MAX_PENCILS = 4096;
 constexpr int LANE_SPLIT_PENCILS = 608;
 constexpr int SPIKE_MIN_ROWS = 512;
 // Problems that have at most two CTAs per SM take it from fewer rows on (64 x
-// 32, 224 rows: 16 RK222 steps 2.27 ms with the window kernel, 2.10 ms; Fisher-
-// KPP 128 x 64, 128 rows, the shortest measured: 43 us a solve, 33 us).
+// 32, 224 rows: 16 RK222 steps 2.27 ms with the window kernel, 2.10 ms).
 constexpr int SPLIT_MAX_PENCILS = 304;
-constexpr int SPLIT_MIN_ROWS = 128;
+constexpr int SPLIT_MIN_ROWS = 96;
 bool spike_supported(int kl, int kuu, int npad, int nblk);
 bool spike_bwd_supported(int kuu, int npad, int nblk);
 cudaError_t launch_spike_coupling(cudaStream_t s, int P, int npad, int nblk_f, int nblk, int kl, int kuu, int lpad,
