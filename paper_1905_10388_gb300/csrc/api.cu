@@ -795,7 +795,7 @@ void set_ep_L(Problem* pr, SolveArgs& a) {
 }
 
 // Arguments of the lane substitution of `pr` with the listed factor `f`.
-LaneArgs lane_args(sp_ctx* ctx, Problem* pr, const LaneList& f, int kl, int kuu) {
+LaneArgs lane_args(sp_ctx* ctx, Problem* pr, const LaneList& f, int kl, int kuu, int cold) {
   LaneArgs la{};
   la.P = pr->P; la.n = pr->n; la.npad = pr->npad; la.kl = kl; la.kuu = kuu;
   la.nblk = pr->spike ? pr->nblk : 1; la.m = pr->npad / la.nblk;
@@ -804,6 +804,7 @@ LaneArgs lane_args(sp_ctx* ctx, Problem* pr, const LaneList& f, int kl, int kuu)
   la.Lv = f.Lv; la.Uv = f.Uv; la.lco = f.lco; la.uco = f.uco; la.pg = f.pg;
   la.bg = pr->d_bg; la.yg = reinterpret_cast<double*>(pr->d_yg); la.xg = pr->d_xg;
   la.status = ctx->d_status;
+  la.cold = cold;
   la.s0 = pr->d_sp_s0; la.sst = pr->d_sp_s; la.o0 = pr->d_sp_o0; la.uin = pr->d_sp_u;
   return la;
 }
@@ -836,7 +837,7 @@ sp_status solve(sp_ctx* ctx, Problem* pr, cudaStream_t s, const SolveArgs& args)
     // assembly -> lane substitution, whole or partitioned -> epilogue
     a.mode = 1;
     CK(launch_pencil_solve(s, a));
-    const LaneArgs la = lane_args(ctx, pr, *a.ll, a.kl, a.kuu);
+    const LaneArgs la = lane_args(ctx, pr, *a.ll, a.kl, a.kuu, a.sp_cold);
     if (pr->lanes) {
       CK(launch_lane_forward(s, la, 0));
       CK(launch_lane_backward(s, la, 0));
@@ -1559,6 +1560,7 @@ sp_status sp_solve_lbvp(sp_ctx* ctx, int problem, int nslots, const int32_t* eqs
   a.xc_out = pr->d_Xc;
   a.xt_out = pr->d_Xt;
   a.ep_mv_vals = nullptr;
+  a.sp_cold = 1;                      // one inversion's solution says nothing about the next one's
   if ((st = solve(ctx, pr, s, a)) != SP_OK) return st;
   CK(cudaStreamSynchronize(s));
   pr->xt_valid = true;

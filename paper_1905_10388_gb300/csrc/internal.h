@@ -70,6 +70,7 @@ struct LaneArgs {
   double2* xg;                  // b = U_jj x~
   double* s0; double* sst;      // forward outflows / inflows [p][nblk_f][2][8]
   double* o0; double* uin;      // backward outflows / inflows [p][nblk][2][32]
+  int cold;                     // 1: pass 1 starts from zero inflows instead of uin
   DevStatus* status;
 };
 // pass 0: whole pencils; 1: blocks from zero / guessed inflows; 2: from the true ones
@@ -204,6 +205,9 @@ struct SolveArgs {
   const double* spD; const double* spE;
   int sp_nblk, sp_nblk_f;       // back- and forward-substitution blocks per pencil
   double* sp_u;                 // back-substitution inflows, the next solve's guesses [p][nblk][2][32]
+  // 1: start from zero inflows; 0: from the previous solve's, for right-hand
+  // sides that change little from solve to solve (rounding errors scale with the guess)
+  int sp_cold;
 };
 
 // fc_half / fc_mhalf from fc_coef (exact scalings), before a launch

@@ -246,7 +246,7 @@ __device__ __forceinline__ void lane_bwd_body(const LaneArgs& a, int g, int blk,
   const size_t bidx = (((size_t)(p0 + (act ? i : 0)) * a.nblk + blk) * 2 + comp) * 32;
   X[XR * 32 + lane] = 0.0;
   if (PASS != 0) {
-    const bool in = act && (PASS == 2 || blk < a.nblk - 1);
+    const bool in = act && (PASS == 2 || (blk < a.nblk - 1 && !a.cold));
 #pragma unroll 8
     for (int r = 0; r < XR; ++r) {
       const double v = (in && r < kuu) ? a.uin[bidx + r] : 0.0;

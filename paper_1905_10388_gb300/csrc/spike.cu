@@ -248,7 +248,11 @@ __global__ void __launch_bounds__(128) k_spike_fwd_rec(LaneArgs s, const double*
   }
 }
 
-__device__ __forceinline__ double spike_guess(double g) { return dfinite(g) ? g : 0.0; }
+// the inflow that pass 1 started a block from
+__device__ __forceinline__ double spike_guess(const LaneArgs& s, size_t i) {
+  const double g = s.uin[i];
+  return (!s.cold && dfinite(g)) ? g : 0.0;
+}
 
 // backward inflows: u_{nblk-2} = o_{nblk-1} (exact), then
 // u_{k-1} = o_k + E_k (u_k - g_k), g_k the guess PASS 1 started block k
@@ -268,7 +272,7 @@ __global__ void __launch_bounds__(SPK_REC_WARPS * 32) k_spike_bwd_rec(LaneArgs s
   if (s.nblk < 2) return;
   if (wq == 0) {
     const double u = r < kuu ? s.o0[at(s.nblk - 1) + r] : 0.0;
-    const double g = (r < kuu && s.nblk > 2) ? spike_guess(s.uin[at(s.nblk - 2) + r]) : 0.0;
+    const double g = (r < kuu && s.nblk > 2) ? spike_guess(s, at(s.nblk - 2) + r) : 0.0;
     ucur[r] = u - g;                                 // u_k - g_k for the next step
     if (r < kuu) s.uin[at(s.nblk - 2) + r] = u;
   }
@@ -298,7 +302,7 @@ __global__ void __launch_bounds__(SPK_REC_WARPS * 32) k_spike_bwd_rec(LaneArgs s
       double u = o;
 #pragma unroll
       for (int q = 0; q < SPK_REC_WARPS; ++q) u += part[q][r];
-      const double g = (r < kuu && k > 1) ? spike_guess(s.uin[at(k - 1) + r]) : 0.0;
+      const double g = (r < kuu && k > 1) ? spike_guess(s, at(k - 1) + r) : 0.0;
       ucur[r] = r < kuu ? u - g : 0.0;
       if (r < kuu) s.uin[at(k - 1) + r] = u;
     }
@@ -325,12 +329,12 @@ __global__ void __launch_bounds__(128) k_spike_bwd_rec_narrow(LaneArgs s, const 
 #pragma unroll
     for (int t = 0; t < W; ++t) en[t] = (in && t < kuu) ? Ek[t] : 0.0;
     on = in ? s.o0[at(k)] : 0.0;
-    gn = (in && k > 1) ? spike_guess(s.uin[at(k - 1)]) : 0.0;
+    gn = (in && k > 1) ? spike_guess(s, at(k - 1)) : 0.0;
   };
   double d;                           // u_k - g_k
   {
     const double u = in ? s.o0[at(s.nblk - 1)] : 0.0;
-    const double g = (in && s.nblk > 2) ? spike_guess(s.uin[at(s.nblk - 2)]) : 0.0;
+    const double g = (in && s.nblk > 2) ? spike_guess(s, at(s.nblk - 2)) : 0.0;
     d = u - g;
     if (in) s.uin[at(s.nblk - 2)] = u;
   }

@@ -321,7 +321,7 @@ __device__ __forceinline__ void pencil_split_body(const SolveArgs& a, int p, dou
   double* uin = a.sp_u + (size_t)p * nblk * 2 * SPL_W;
   for (int q = tid; q < nblk * 2 * SPL_W; q += NT) {
     const double g = uin[q];
-    gs[q] = dfinite(g) ? g : 0.0;
+    gs[q] = (!a.sp_cold && dfinite(g)) ? g : 0.0;
   }
   pencil_assemble<1>(a, p, tid, NT, npad + 64, reinterpret_cast<double2*>(B));
   const size_t prow = (size_t)p * n;
