@@ -247,7 +247,8 @@ sp_status sp_set_batch_persistent(sp_ctx* ctx, int nproblems, const int* problem
  *   allocates the adjoint work buffers; for problems on the partitioned
  *   substitution it also computes the transposed factor's coupling matrices
  *   (kl' = ku is wider than the 8-lane forward windows: the transposed
- *   solves use 32-lane windows both ways) and zeroes their inflow guesses.
+ *   solves use 32-lane windows both ways, and always start from zero
+ *   inflows).
  * sp_step_adjoint: given the states of one forward step (states_dev,
  *   device, nstates consecutive arrays of S*P*N_z complex: X^n alone
  *   (nstates = 1; the first stage is then recomputed from X^n) or X^n

@@ -205,7 +205,7 @@ struct Problem {
   int spike_blocks = 0;                      // requested (0: automatic)
   int nblk = 0, nblk_f = 0;
   double *d_sp_s0 = nullptr, *d_sp_s = nullptr, *d_sp_o0 = nullptr, *d_sp_u = nullptr;
-  double* d_spT_u = nullptr;                 // inflow guesses of the transposed solves
+  double* d_spT_u = nullptr;                 // inflows of the transposed solves
   std::map<std::pair<int, int>, TransformPlan> plans;
   // stepping state
   int iteration = 0;
@@ -321,15 +321,11 @@ sp_status make_plan(sp_ctx* ctx, Problem* pr, int Nc, int Ng, TransformPlan** ou
 }
 
 // the partitioned back substitution starts its blocks from the previous
-// solve's inflows (spike.cu); zero them, the transposed solves' too, so that
-// a run (or a gradient) from a set state repeats bit for bit
+// solve's inflows (split.cu, spike.cu); zero them, so that a run from a set
+// state repeats bit for bit
 cudaError_t reset_spike_guess(Problem* pr, cudaStream_t s) {
   if (!pr->spike) return cudaSuccess;
-  const size_t bytes = (size_t)pr->P * pr->nblk * 2 * 32 * sizeof(double);
-  cudaError_t e = cudaSuccess;
-  if (pr->d_sp_u) e = cudaMemsetAsync(pr->d_sp_u, 0, bytes, s);
-  if (e == cudaSuccess && pr->d_spT_u) e = cudaMemsetAsync(pr->d_spT_u, 0, bytes, s);
-  return e;
+  return cudaMemsetAsync(pr->d_sp_u, 0, (size_t)pr->P * pr->nblk * 2 * 32 * sizeof(double), s);
 }
 
 // the divisor of `whole` nearest to `target`
@@ -996,6 +992,7 @@ SolveArgs transposed_args(Problem* pr, sp_ctx* ctx) {
   a.ll = nullptr;
   a.spD = pr->facT.spD; a.spE = pr->facT.spE;    // null unless partitioned
   a.sp_nblk_f = pr->nblk; a.sp_u = pr->d_spT_u;
+  a.sp_cold = 1;                        // lambda need not come from the last call
   return a;
 }
 
@@ -2028,7 +2025,6 @@ sp_status sp_adjoint_init(sp_ctx* ctx, int problem) {
     if (!pr->facT.spD) CK(dalloc(&pr->facT.spD, (size_t)pr->P * pr->nblk * (pr->klT > 7 ? 31 * 32 : 7 * 8)));
     if (!pr->facT.spE) CK(dalloc(&pr->facT.spE, (size_t)pr->P * pr->nblk * kuuT * 32));
     if (!pr->d_spT_u) CK(dalloc(&pr->d_spT_u, (size_t)pr->P * pr->nblk * 2 * 32));
-    CK(cudaMemsetAsync(pr->d_spT_u, 0, (size_t)pr->P * pr->nblk * 2 * 32 * sizeof(double), s));
     CK(launch_spike_coupling(s, pr->P, pr->npad, pr->nblk, pr->nblk, pr->klT, kuuT, pr->lpadT, pr->upad, pr->facT,
                              false));
     CK(cudaStreamSynchronize(s));
@@ -2075,6 +2071,7 @@ sp_status sp_step_adjoint(sp_ctx* ctx, int problem, double dt, const void* state
     a.bc_coef = dt * tb.A[1][0];
     a.xc_out = pr->d_Xc;
     a.xc32_out = nullptr;
+    a.sp_cold = 1;                      // nor X^n from the last one's
     if ((st = solve(ctx, pr, s, a)) != SP_OK) return st;
     X1 = pr->d_Xc;
   }

@@ -10,7 +10,8 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
-from paper_1905_10388_gb300.solver import Context, QGInversion
+from paper_1905_10388_gb300 import _lib
+from paper_1905_10388_gb300.solver import Context, QGInversion, RBSolver
 
 pytestmark = pytest.mark.gpu
 
@@ -37,3 +38,30 @@ def test_inversion_does_not_depend_on_the_one_before(ctx, nx, nz):
     later.invert(q1 * 1e12)
     assert later.spike_blocks() > 1
     assert np.array_equal(later.invert(q2), want)
+
+
+@pytest.mark.parametrize("nx,nz,scheme", [(64, 32, "RK222"), (64, 64, "RK111"), (256, 128, "RK222")])
+def test_adjoint_step_does_not_depend_on_the_one_before(ctx, nx, nz, scheme):
+    h, dt = ctx.handle, 1e-3
+    rng = np.random.default_rng(6)
+
+    def solver():
+        s = RBSolver(ctx, nx, nz, 1e6, scheme=scheme)
+        s.factor(dt)
+        _lib.check(h, _lib.lib().sp_adjoint_init(h, s.pid))
+        return s
+
+    def adjoint(s, X, lam):
+        X, lam = (torch.as_tensor(a, device="cuda") for a in (X, lam))
+        _lib.check(h, _lib.lib().sp_step_adjoint(h, s.pid, dt, X.data_ptr(), 1, lam.data_ptr()))
+        ctx.sync_status()
+        return lam.cpu().numpy()
+    first, later = solver(), solver()
+    shape = (first.S, first.P, nz)
+    (x1, l1), (x2, l2) = [[(rng.standard_normal(shape) + 1j * rng.standard_normal(shape)) / (1 + np.arange(nz)) ** 2
+                           for _ in range(2)] for _ in range(2)]
+    want = adjoint(first, x2, l2)
+    adjoint(later, x1 * 1e3, l1 * 1e10)
+    assert later.spike_blocks() > 1
+    assert np.isfinite(want).all()
+    assert np.array_equal(adjoint(later, x2, l2), want)
