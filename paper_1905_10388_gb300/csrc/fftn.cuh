@@ -9,15 +9,16 @@
 // immediate: at run-time lengths the index arithmetic alone was most of the
 // FP32 kernels' instructions.
 //
-// Twiddled butterflies split even and odd inputs with one common factor:
-// E_q = sum_s a_{2s} w^{2s} r^{2qs}, O_q the same sum of a_{2s+1}, X_{q, q+R/2} =
-// E_q +- w r^q O_q (r = exp(sign 2 pi i / R)), down to single elements.  Each
-// two-point step is four FMAs for E + w O and, in FP64, whose pipe is the
-// bound, two for E - w O = 2 E - (E + w O): 72 FP64 instructions and 4 twiddle
-// loads for radix 8, against 84 and 7 with the inputs multiplied first (errors
-// of the right-hand side against a dense evaluation 5.6e-14 against 5.8e-14 at
-// 256 x 256).  FP32, bound by other instructions, takes four for it, as exact
-// as a product and a difference.
+// A twiddled butterfly multiplies its inputs once and then runs the plain DFT,
+// whose two-point steps with a constant root are four FMAs for E + w O and, in
+// FP64, whose pipe is the bound, two for E - w O = 2 E - (E + w O); FP32, bound by
+// other instructions, takes four for it, as exact as a product and a difference.
+// A twiddle at every level (two-point steps with the common factors w, w^2, w^4:
+// 72 FP64 instructions and 4 twiddle loads for radix 8 against 80 and 7) rounds
+// each element three times more: errors of the right-hand side against extended
+// precision 1.51e-15 (FP64) and 4.52e-7 (mixed) against 1.33e-15 and 4.29e-7 here,
+// geometric means over lengths of 48 to 768.  It was 5 % faster in FP64 (512 x
+// 256 RK222 step 754 against 795 us, mixed 415 against 417).
 //
 // Buffers are padded by one element every 128 bytes, so the first pass's
 // stride-R writes spread over the banks.
@@ -80,34 +81,8 @@ __device__ __forceinline__ void bfly(C<T> e, C<T> o, C<T> w, C<T>& p, C<T>& m) {
   }
 }
 
-// DFT of length R (a power of two) of a[0], a[S], a[2S], ... with the common
-// twiddle w: out[q] = sum_t a[t S] w^t r^{qt}; tw[base] = conj-adjusted powers.
-// `at(m, q, R)` returns w^m exp(SIGN 2 pi i q / R) for q < R / 4.
-template <typename T, int SIGN, int R, int S, int M, typename W>
-struct DitTw {
-  static __device__ __forceinline__ void run(const C<T>* a, C<T>* out, const W& at) {
-    C<T> e[R / 2], o[R / 2];
-    DitTw<T, SIGN, R / 2, 2 * S, 2 * M, W>::run(a, e, at);
-    DitTw<T, SIGN, R / 2, 2 * S, 2 * M, W>::run(a + S, o, at);
-    if (R == 2) {
-      bfly<T>(e[0], o[0], at(M, 0, 2), out[0], out[1]);
-    } else {
-#pragma unroll
-      for (int q = 0; q < R / 4; ++q) {
-        const C<T> w = at(M, q, R);
-        bfly<T>(e[q], o[q], w, out[q], out[q + R / 2]);
-        bfly<T>(e[q + R / 4], o[q + R / 4], rot90<T, SIGN>(w), out[q + R / 4], out[q + 3 * R / 4]);
-      }
-    }
-  }
-};
-template <typename T, int SIGN, int S, int M, typename W>
-struct DitTw<T, SIGN, 1, S, M, W> {
-  static __device__ __forceinline__ void run(const C<T>* a, C<T>* out, const W&) { out[0] = a[0]; }
-};
-
-// The same without twiddles (first pass): constant roots, the trivial ones as
-// sums and differences.
+// DFT of length R (a power of two) of a[0], a[S], a[2S], ...: constant roots, the
+// trivial ones as sums and differences.
 template <typename T, int SIGN, int R, int S>
 struct Dit {
   static __device__ __forceinline__ void run(const C<T>* a, C<T>* out) {
@@ -137,6 +112,16 @@ template <typename T, int SIGN, int S>
 struct Dit<T, SIGN, 1, S> {
   static __device__ __forceinline__ void run(const C<T>* a, C<T>* out) { out[0] = a[0]; }
 };
+
+// The same of a[t] w^t; `at(t)` returns w^t.
+template <typename T, int SIGN, int R, typename W>
+__device__ __forceinline__ void dft_twiddled(const C<T>* a, C<T>* out, const W& at) {
+  C<T> b[R];
+  b[0] = a[0];
+#pragma unroll
+  for (int t = 1; t < R; ++t) b[t] = cmul<T>(at(t), a[t]);
+  Dit<T, SIGN, R, 1>::run(b, out);
+}
 
 // 3-point DFT: sums, differences and FMAs with -1/2 and sqrt(3)/2.  Z: an input
 // known to be zero (-1: none).
@@ -239,11 +224,10 @@ __device__ __forceinline__ void fft_pass_tw(const C<T>* __restrict__ x, const C<
 #pragma unroll
     for (int t = 0; t < R; ++t) a[t] = xb[fft_pad<T>(j + t * Q)];
     const unsigned w0 = k * STEP;
-    auto at = [&](int m, int q, int r) {
-      const C<T> w = fft_tw<T>(tw, m * w0 + q * (N / r));
+    dft_twiddled<T, SIGN, R>(a, y, [&](int t) {
+      const C<T> w = fft_tw<T>(tw, t * w0);
       return SIGN > 0 ? mk<T>(w.x, -w.y) : w;
-    };
-    DitTw<T, SIGN, R, 1, 1, decltype(at)>::run(a, y, at);
+    });
     const int o = g * R * Ns + k;
 #pragma unroll
     for (int q = 0; q < R; ++q) out(b, o + q * Ns, y[q]);

@@ -225,11 +225,10 @@ __device__ __forceinline__ void col_run(C<T>* u, C<T>* v, const C<T>* tw, OPEN&&
 #pragma unroll
       for (int t = 0; t < R; ++t) a[t] = xc[fft_pad<T>(j + t * Q)];
       const unsigned w0 = k * STEP;
-      auto at = [&](int m, int q, int rr) {
-        const C<T> w = fft_tw<T>(tw, m * w0 + q * (N / rr));
+      dft_twiddled<T, SIGN, R>(a, y, [&](int t) {
+        const C<T> w = fft_tw<T>(tw, t * w0);
         return SIGN > 0 ? mk<T>(w.x, -w.y) : w;
-      };
-      DitTw<T, SIGN, R, 1, 1, decltype(at)>::run(a, y, at);
+      });
       const int o = j / Ns * (R * Ns) + k;
 #pragma unroll
       for (int q = 0; q < R; ++q) out(c, o + q * Ns, y[q]);
