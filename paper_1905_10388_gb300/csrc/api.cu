@@ -461,7 +461,9 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
     // w_k = exp(-i pi k / (2 N)) with what the transforms fold into it (rows.cuh)
     std::vector<double2> zb(pr->Ngz), zf(pr->Ngz);
     const double pi = 3.14159265358979323846;
-    const double hs = 1.0 / (2.0 * pr->Ngx) / (pr->ndim == 3 ? pr->Ngy : 1);
+    double hs = 1.0 / (2.0 * pr->Ngx) / (pr->ndim == 3 ? pr->Ngy : 1);
+    if (pr->prec)                                // what the x and y transforms leave of it
+      hs = std::ldexp(hs, rows_shift(2 * pr->Ngx) + (pr->ndim == 3 ? rows_shift(pr->Ngy) : 0));
     for (int k = 0; k < pr->Ngz; ++k) {
       const double c = std::cos(pi * k / (2.0 * pr->Ngz)), n = -std::sin(pi * k / (2.0 * pr->Ngz));
       const double b = k == 0 ? 1.0 : (k % 2 ? -0.5 : 0.5), f = (k % 2 ? -1.0 : 1.0) * (k == 0 ? 0.5 : 1.0) * hs / pr->Ngz;

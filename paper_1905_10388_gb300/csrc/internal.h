@@ -334,6 +334,14 @@ inline size_t x_rows_bytes(int prec, int N, int nf, int ne) {
   const int nbi = (nf + 1) / 2, nbo = (ne + 1) / 2;
   return (nbi + (nbi > 2 * nbo ? nbi : 2 * nbo)) * rows_padded(prec, N);
 }
+// Forward sums leave the FP32 x transform times 2^-rows_shift(2 N), the y
+// transform times 2^-rows_shift(N): exact, and no sum grows past its own
+// transform's length.  The z transform's table takes the rest of 1 / (2 N_gx N_gy).
+__host__ __device__ constexpr int rows_shift(int n) {
+  int e = 0;
+  while ((1 << e) < n) ++e;
+  return e;
+}
 inline int z_cols_tile(int prec) { return prec ? 8 : 4; }
 inline size_t z_cols_bytes(int prec, int N) {   // two buffers of tile columns, each one element over a multiple of 16
   const size_t el = N + (prec ? N / 16 : N / 8);

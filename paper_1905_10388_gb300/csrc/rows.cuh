@@ -35,6 +35,14 @@ constexpr size_t ROWS_SMEM = ROWS_SMEM_MAX;
 __device__ __forceinline__ double neg_bits(double x) { return dneg(x); }
 __device__ __forceinline__ float neg_bits(float x) { return -x; }
 
+// Factor that a forward transform's results leave with: 1 in FP64; in FP32 an
+// exact 2^-rows_shift(N), else the sums over all axes would overflow where each
+// product and each axis' sum still fits
+template <typename T, int N>
+__host__ __device__ constexpr T rows_scale() {
+  return sizeof(T) == 4 ? (T)1 / (T)(1 << rows_shift(N)) : (T)1;
+}
+
 // threads of a CTA: about the butterflies of four sequences, in whole warps
 template <typename T, int N>
 constexpr int rows_threads() {
@@ -147,12 +155,13 @@ __device__ __forceinline__ void x_rows_body(const XDesc& d, int row, unsigned ch
       },
       [&](int b, int i, C<T> z) { Z[b * NP + fft_pad<T>(i)] = z; });
   C<T>* h = reinterpret_cast<C<T>*>(d.h) + (size_t)row * K;
-  // (the 1 / (2 N) of the forward transform is in the z transform's table)
+  // (1 / (2 N), in FP32 what rows_scale leaves of it, is in the z transform's table)
+  constexpr T sc = rows_scale<T, 2 * N>();
   for (int b = 0; b < nbo; ++b)
     for (int k = tid; k < K; k += NT) {
       const C<T> z = Z[b * NP + fft_pad<T>(k)], r = Z[b * NP + fft_pad<T>(k == 0 ? 0 : N - k)];
-      h[2 * b * plane + k] = mk<T>(z.x + r.x, z.y - r.y);
-      if (2 * b + 1 < ne) h[(2 * b + 1) * plane + k] = mk<T>(z.y + r.y, r.x - z.x);
+      h[2 * b * plane + k] = mk<T>(sc * (z.x + r.x), sc * (z.y - r.y));
+      if (2 * b + 1 < ne) h[(2 * b + 1) * plane + k] = mk<T>(sc * (z.y + r.y), sc * (r.x - z.x));
     }
 }
 
@@ -287,7 +296,8 @@ __global__ void __launch_bounds__(NT, rows_ctas<T>(NT)) k_y_cols(YDesc d) {
           if (ix0 + c < K) out[(size_t)i * K + c] = z;
         });
   } else {
-    // (the 1 / N is in the z transform's table)
+    // (1 / N, in FP32 what rows_scale leaves of it, is in the z transform's table)
+    constexpr T sc = rows_scale<T, N>();
     const C<T>* __restrict__ in = reinterpret_cast<const C<T>*>(d.src) + ((size_t)f * d.nz + zg) * N * K + ix0;
     C<T>* out = reinterpret_cast<C<T>*>(d.dst) + ((size_t)f * d.nz + zg) * Ny * K + ix0;
     col_run<T, N, -1, NT, false, true, true>(
@@ -299,8 +309,8 @@ __global__ void __launch_bounds__(NT, rows_ctas<T>(NT)) k_y_cols(YDesc d) {
         },
         [&](int c, int i, C<T> z) {
           if (ix0 + c >= K) return;
-          if (i < half) out[(size_t)i * K + c] = z;
-          else if (i > N - half) out[(size_t)i * K + c - skip] = z;
+          if (i < half) out[(size_t)i * K + c] = cscale<T>(z, sc);
+          else if (i > N - half) out[(size_t)i * K + c - skip] = cscale<T>(z, sc);
           if (i == 0) out[(size_t)half * K + c] = mk<T>(0, 0);
         });
   }
@@ -361,8 +371,8 @@ __device__ __forceinline__ void z_backward_body(const ZDesc& d, int bx, int f, u
 }
 
 // Chebyshev forward of product f: out_k = w_k V_k + conj(w_k) V_{N-k}, wq the
-// w_k with the T coefficients' sign and scale and the 1 / (2 N_gx) [/ N_gy] that
-// the x [and y] transforms leave out
+// w_k with the T coefficients' sign and scale and the part of 1 / (2 N_gx)
+// [/ N_gy] that the x [and y] transforms leave out
 template <typename T, int N, int NT>
 __device__ __forceinline__ void z_forward_body(const ZDesc& d, int bx, int f, unsigned char* rows_smem) {
   constexpr int TC = col_tile<T>(), NS = col_stride<T, N>(), Q0 = N / FftPlan<N>::R0;

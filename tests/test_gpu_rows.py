@@ -143,3 +143,27 @@ def test_rhs_one_field(ctx, nx, nz, prec):
 def test_rhs_3d(ctx, nx, ny, nz, scale, prec):
     s = RB3DSolver(ctx, nx, ny, nz, 1e5, precision=prec, dealias=scale)
     _check(s, rbmod.BILINEAR_TERMS_3D, scale, prec)
+
+
+@pytest.mark.parametrize("shape", [(64, 32), (256, 64), (64, 32, 32)])
+def test_products_near_the_top_of_single_precision(ctx, shape):
+    """Products of 4e35 and sums of them over one axis fit FP32 (3.4e38); no
+    transform may carry the sum over two.  Single modes: errors of a few FP32
+    units, 3e-7 measured, bar 1e-6."""
+    out = []
+    for prec in ("fp64", "mixed"):
+        if len(shape) == 3:
+            s = RB3DSolver(ctx, *shape, 1e5, precision=prec)
+            nh = (shape[1], shape[0])
+        else:
+            s = RBSolver(ctx, *shape, 1e5, precision=prec)
+            nh = (shape[0],)
+        z = np.pi * rbmod.chebyshev_nodes(s.Nz).reshape((-1,) + (1,) * len(nh))
+        x = 2 * np.pi * np.arange(nh[-1]) / nh[-1]
+        for i, v in enumerate(("b", "u", "w")):
+            s.set_field(v, 3e17 * np.sin((i + 1) * z) * np.cos((i + 1) * x + i) * np.ones((s.Nz,) + nh), layout="g")
+        out.append(s.eval_rhs())
+    size = max(np.linalg.norm(f) for f in out[0].values())     # (3D: v's products are zero but for rounding)
+    for e in out[0]:
+        assert np.isfinite(out[1][e]).all(), e
+        assert np.linalg.norm(out[1][e] - out[0][e]) < 1e-6 * size, e
