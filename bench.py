@@ -392,26 +392,13 @@ def run_ours(args):
 
     flops, nbytes = solve_flops_bytes(s)
     n_, kl_, ku_ = s.band()
-    # the library's automatic choice of substitution kernel (sp_set_solve_kernel):
-    # lane substitution of whole pencils (assembly, forward, back, epilogue:
-    # four launches) or of row blocks (two passes each way and the recurrences
-    # over blocks between them: eight), the partitioned solve of a pencil per
-    # CTA, two pencils per CTA, or the window kernel (one launch each)
     nblk = s.spike_blocks()
     factor_mb = s.P * s.solve_work()[1] / 1e6
     achieved = flops / (solve_ms * 1e-3) / 1e12
     peaks = measured_peaks()
-    if nblk > 0 and s.P >= 608:
-        kernel = (f"lane substitution, {nblk} row blocks per pencil: k_pencil_stage<1> + k_lane_fwd<1> + "
-                  "k_spike_fwd_rec + k_lane_fwd<2> + k_lane_bwd<1> + k_spike_bwd_rec + k_lane_bwd<2> + "
-                  "k_pencil_stage<2>")
-        solve_launches_per = 8
-    elif nblk > 0:
-        kernel, solve_launches_per = f"k_pencil_split, {nblk} row blocks per pencil", 1
-    elif s.P >= 2048:
-        kernel, solve_launches_per = "k_pencil_stage<1> + k_lane_fwd<0> + k_lane_bwd<0> + k_pencil_stage<2>", 4
-    else:
-        kernel, solve_launches_per = "k_pencil_pair" if s.P > 304 else "k_pencil_solve", 1
+    names = s.solve_kernels()
+    solve_launches_per = len(names)
+    kernel = " + ".join(names) + (f", {nblk} row blocks per pencil" if nblk > 0 else "")
     roof = {"kernel": kernel, "bound": "alu", "achieved": achieved, "peak": fp64_peak,
             "unit": "TFLOP/s", "frac": achieved / fp64_peak,
             "traffic": solve_traffic(args.workload, head), "algorithmic_bytes": nbytes,

@@ -37,7 +37,7 @@ EXPORTS = (
     "sp_cfl_frequency", "sp_cfl_dt", "sp_eig_target", "sp_measure_fma_peak",
     "sp_set_spike_blocks", "sp_get_spike_blocks", "sp_set_z_transform", "sp_get_z_transform",
     "sp_solve_lbvp", "sp_eig_residual", "sp_batch_persistent",
-    "sp_set_batch_persistent",
+    "sp_set_batch_persistent", "sp_get_solve_kernels",
 )
 
 
@@ -97,6 +97,7 @@ _SIGS = {
     "sp_measure_fma_peak": [I, I, ctypes.POINTER(D)],
     "sp_set_spike_blocks": [P, I, I],
     "sp_get_spike_blocks": [P, I, ctypes.POINTER(I)],
+    "sp_get_solve_kernels": [P, I, ctypes.POINTER(ctypes.c_char_p), ctypes.POINTER(I)],
     "sp_set_z_transform": [P, I, I],
     "sp_get_z_transform": [P, I, ctypes.POINTER(I)],
     "sp_solve_lbvp": [P, I, I, I32P, P],

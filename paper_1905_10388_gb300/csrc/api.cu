@@ -349,7 +349,7 @@ int default_spike_blocks(int npad, int P) {
   const int nch = npad / SOLVE_CHUNK;
   const int groups = (P + LANE_GROUP - 1) / LANE_GROUP;
   if (P >= LANE_SPLIT_PENCILS) return near_divisor(nch, std::max(2, 1024 / groups));
-  return near_divisor(nch, P <= 152 ? 8 : 4);
+  return near_divisor(nch, P <= GPU_SMS ? 8 : 4);
 }
 // Forward blocks: of about 32 rows, 64 for long pencils (a block costs a step
 // of the recurrence over blocks, about as long as three rows of its two passes).
@@ -2591,6 +2591,30 @@ sp_status sp_get_spike_blocks(sp_ctx* ctx, int problem, int* nblk) {
   if (!pr || !nblk) return fail(ctx, SP_ERR_ARG, "bad context, problem id or output");
   ctx->err.clear();
   *nblk = (pr->uploaded && pr->spike) ? pr->nblk : 0;
+  return SP_OK;
+}
+
+sp_status sp_get_solve_kernels(sp_ctx* ctx, int problem, const char** names, int* launches) {
+  Problem* pr = get(ctx, problem);
+  if (!pr) return fail(ctx, SP_ERR_ARG, "bad context or problem id");
+  ctx->err.clear();
+  if (!pr->uploaded) return fail(ctx, SP_ERR_STATE, "the problem is not on the device yet");
+  const char* s;
+  int n = 1;
+  if (pr->lanes) {
+    s = "k_pencil_stage<1> + k_lane_fwd<0> + k_lane_bwd<0> + k_pencil_stage<2>";
+    n = 4;
+  } else if (pr->by_group) {
+    s = "k_pencil_stage<1> + k_lane_fwd<1> + k_spike_fwd_rec + k_lane_fwd<2> + k_lane_bwd<1> + k_spike_bwd_rec + "
+        "k_lane_bwd<2> + k_pencil_stage<2>";
+    n = 8;
+  } else if (pr->spike) {
+    s = "k_pencil_split";
+  } else {
+    s = whole_row_kernel(pr->P, pr->npad, pr->lpad, pr->upad) == WHOLE_PAIR ? "k_pencil_pair" : "k_pencil_solve";
+  }
+  if (names) *names = s;
+  if (launches) *launches = n;
   return SP_OK;
 }
 

@@ -628,6 +628,13 @@ __global__ void __launch_bounds__(128, 6) k_pencil_stage(SolveArgs a) {
 
 size_t pencil_solve_smem(int npad, int lpad, int upad) { return solve_smem_bytes(npad, lpad, upad); }
 
+// More pencils than one wave of two CTAs per SM: several pencils' chains per
+// sub-partition instead of a CTA per pencil (where three of this kernel's CTAs
+// would fit an SM, 228 KB of shared memory, 1 KB of it reserved per CTA).
+WholeRowKernel whole_row_kernel(int P, int npad, int lpad, int upad) {
+  return P > 2 * GPU_SMS && 3 * (solve_smem_bytes(npad, lpad, upad) + 1024) <= 228 * 1024 ? WHOLE_PAIR : WHOLE_WINDOW;
+}
+
 cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
   SolveArgs a = args;
   fill_f_halves(a);
@@ -646,16 +653,7 @@ cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
   const size_t smem = solve_smem_bytes(a.npad, a.lpad, a.upad);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   const int grid = a.P;
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 1;
-  }
-  // more pencils than one wave of two CTAs per SM: several pencils' chains per
-  // sub-partition instead of a CTA per pencil (where three of this kernel's CTAs
-  // would fit an SM, 228 KB of shared memory, 1 KB of it reserved per CTA)
-  if (a.P > 2 * sms && 3 * (smem + 1024) <= 228 * 1024) return launch_pencil_pair(s, a);
+  if (whole_row_kernel(a.P, a.npad, a.lpad, a.upad) == WHOLE_PAIR) return launch_pencil_pair(s, a);
   if (a.kuu <= 31) {
     cudaFuncSetAttribute(k_pencil_solve<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     k_pencil_solve<1><<<grid, SOLVE_THREADS, smem, s>>>(a);

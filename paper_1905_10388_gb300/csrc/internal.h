@@ -11,6 +11,8 @@
 
 namespace spectau {
 
+constexpr int GPU_SMS = 152;           // GB300
+
 // Column chunk streamed per bulk copy by the pencil-solve kernel, and the
 // ring depth.  Factor arrays are padded to a multiple of SOLVE_CHUNK columns.
 constexpr int SOLVE_CHUNK = 32;
@@ -92,7 +94,7 @@ constexpr int LANE_SPLIT_PENCILS = 608;
 constexpr int SPIKE_MIN_ROWS = 512;
 // Problems that have at most two CTAs per SM take it from fewer rows on (64 x
 // 32, 224 rows: 16 RK222 steps 2.27 ms with the window kernel, 2.10 ms).
-constexpr int SPLIT_MAX_PENCILS = 304;
+constexpr int SPLIT_MAX_PENCILS = 2 * GPU_SMS;
 constexpr int SPLIT_MIN_ROWS = 96;
 bool spike_supported(int kl, int kuu, int npad, int nblk);
 bool spike_bwd_supported(int kuu, int npad, int nblk);
@@ -279,6 +281,9 @@ cudaError_t launch_eig_residual(cudaStream_t s, int P, int n, int nnz, const int
                                 const double* Mv, const double* Lv, const double2* x, const double2* sig,
                                 double* res);
 size_t pencil_solve_smem(int npad, int lpad, int upad);
+// the kernel that solves P pencils in whole-row order, one launch
+enum WholeRowKernel { WHOLE_WINDOW, WHOLE_PAIR };
+WholeRowKernel whole_row_kernel(int P, int npad, int lpad, int upad);
 // partitioned pencil solve, one CTA per pencil (split.cu)
 cudaError_t launch_pencil_split(cudaStream_t s, const SolveArgs& a);
 cudaError_t launch_pencil_split_batched(cudaStream_t s, const SolveArgs* args, const int4* work, int nwork,

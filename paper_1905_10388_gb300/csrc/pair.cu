@@ -202,11 +202,11 @@ __global__ void __launch_bounds__(PAIR_THREADS, 5) k_pencil_pair_batched(const S
 
 size_t pencil_pair_smem(int npad, int per) { return (size_t)per * (npad + 64) * sizeof(double2); }
 
-// Two pencils per CTA once single-pencil CTAs would not all be resident (152
-// SMs, four each), as long as five such CTAs fit an SM's shared memory: longer
+// Two pencils per CTA once single-pencil CTAs would not all be resident (four
+// per SM), as long as five such CTAs fit an SM's shared memory: longer
 // pencils (more than 1344 rows) go one per CTA.
 int pencil_pair_per(int npad, long long pencils) {
-  return pencils > 4 * 152 && pencil_pair_smem(npad, 2) <= 44 * 1024 ? 2 : 1;
+  return pencils > 4 * GPU_SMS && pencil_pair_smem(npad, 2) <= 44 * 1024 ? 2 : 1;
 }
 
 // f(kernel) for the instance that serves bands up to kl, kuu

@@ -442,8 +442,6 @@ size_t pencil_split_smem(int npad, int nblk, int nblk_f, int kuu, bool wide) {
 
 // One CTA of 512 threads per SM while every pencil has an SM of its own, two
 // of 256 beyond that.
-constexpr int SPL_SMS = 152;
-
 cudaError_t launch_pencil_split(cudaStream_t s, const SolveArgs& args) {
   SolveArgs a = args;
   fill_f_halves(a);
@@ -460,7 +458,7 @@ cudaError_t launch_pencil_split(cudaStream_t s, const SolveArgs& args) {
       e = cudaGetLastError();
     }
   };
-  if (a.P <= SPL_SMS) {
+  if (a.P <= GPU_SMS) {
     if (wide) go(k_pencil_split<true, 512>, 512);
     else go(k_pencil_split<false, 512>, 512);
   } else {
@@ -480,7 +478,7 @@ cudaError_t launch_pencil_split_batched(cudaStream_t s, const SolveArgs* args, c
       e = cudaGetLastError();
     }
   };
-  if (nwork <= SPL_SMS) go(k_pencil_split_batched<512>, 512);
+  if (nwork <= GPU_SMS) go(k_pencil_split_batched<512>, 512);
   else go(k_pencil_split_batched<256>, 256);
   return e;
 }

@@ -147,6 +147,15 @@ class TauSolver:
         L.check(h, L.lib().sp_get_spike_blocks(h, self.pid, ctypes.byref(out)))
         return out.value
 
+    def solve_kernels(self):
+        """Names of the kernels of one pencil solve, in order (a list)."""
+        names, n = ctypes.c_char_p(), ctypes.c_int()
+        h = self.ctx.handle
+        L.check(h, L.lib().sp_get_solve_kernels(h, self.pid, ctypes.byref(names), ctypes.byref(n)))
+        names = names.value.decode().split(" + ")
+        assert len(names) == n.value
+        return names
+
     def set_bilinear(self, terms):
         ops = {"ID": L.SP_OP_ID, "DX": L.SP_OP_DX, "DY": L.SP_OP_DY}
         eq = np.array([self.eq[t[0]] for t in terms], np.int32)
