@@ -378,10 +378,10 @@ sp_status sp_set_timing(sp_ctx* ctx, int problem, int max_launches);
  * unless (kl, kl + ku) is (9, 38) or (7, 29)).  Both run every FMA in the same
  * order and give identical results.  SPIKE: the partitioned substitution below
  * (few pencils; SP_ERR_ARG unless kl <= 7 and kl + ku <= 31).  SP_SOLVE_AUTO
- * picks LANES from 2048 pencils on where SPIKE does not apply, SPIKE as stated
- * below, else WINDOW.  Must precede the first call that moves the problem to
- * the device (sp_factor, sp_set_field, sp_transform): SP_ERR_STATE
- * afterwards. */
+ * picks SPIKE as stated below, else LANES from 2048 pencils on (any band the
+ * factorization takes), else WINDOW.  Must precede the first call that moves
+ * the problem to the device (sp_factor, sp_set_field, sp_transform):
+ * SP_ERR_STATE afterwards. */
 typedef enum { SP_SOLVE_AUTO = 0, SP_SOLVE_WINDOW = 1, SP_SOLVE_LANES = 2, SP_SOLVE_SPIKE = 3 } sp_solve_kernel;
 sp_status sp_set_solve_kernel(sp_ctx* ctx, int problem, int kind);
 

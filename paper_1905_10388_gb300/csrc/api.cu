@@ -532,9 +532,6 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
   pr->upad = kuu <= 31 ? 32 : 64;
   // SBDFq keeps q factors (its start-up orders); the Runge-Kutta schemes one
   const int nfactors = is_cnab(pr->scheme) ? 1 : std::max(1, sbdf_order(pr->scheme));
-  // thousands of pencils: one lane per right-hand side, whole pencils
-  pr->lanes = pr->solve_kind == SP_SOLVE_LANES ||
-              (pr->solve_kind == SP_SOLVE_AUTO && pr->P >= LANE_MIN_PENCILS);
   // mixed precision: the Chebyshev backward transform on the tensor cores
   // (SP_ZT_MMA, or SP_ZT_AUTO on three-dimensional problems), when its sizes fit
   pr->zmma = pr->prec == SP_PREC_MIXED && cheb_mma_supported(pr->Nz, pr->Ngz) &&
@@ -547,9 +544,8 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
       if (pr->zkind == SP_ZT_MMA) CK(e);
     }
   }
-  // a few hundred pencils are too few chains for the GPU: cut each pencil's
-  // rows into blocks substituted in parallel (spike.cu)
-  pr->by_group = pr->lanes;
+  // up to a few thousand pencils are too few chains for the GPU: cut each
+  // pencil's rows into blocks substituted in parallel (split.cu, lanes.cu)
   pr->nblk = pr->spike_blocks > 0 ? pr->spike_blocks : default_spike_blocks(pr->npad, pr->P);
   // (a lower band wider than the 8-lane forward windows: forward blocks as
   // long as the back ones, in the one-CTA form only)
@@ -559,12 +555,15 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
                           pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, kuu, wide) <= 227 * 1024;
   const bool bands = wide ? pr->kl <= 30 && pr->P < LANE_SPLIT_PENCILS && spike_bwd_supported(kuu, pr->npad, pr->nblk)
                           : spike_supported(pr->kl, kuu, pr->npad, pr->nblk);
-  pr->spike = !pr->lanes && split_fits && bands &&
+  pr->spike = split_fits && bands &&
               (pr->solve_kind == SP_SOLVE_SPIKE ||
                (pr->solve_kind == SP_SOLVE_AUTO && pr->P < SPIKE_MAX_PENCILS &&
                 (pr->npad >= SPIKE_MIN_ROWS || (pr->P <= SPLIT_MAX_PENCILS && pr->npad >= SPLIT_MIN_ROWS))));
+  // thousands of pencils else: one lane per right-hand side, whole pencils
+  pr->lanes = pr->solve_kind == SP_SOLVE_LANES ||
+              (pr->solve_kind == SP_SOLVE_AUTO && !pr->spike && pr->P >= LANE_MIN_PENCILS);
+  pr->by_group = pr->lanes || (pr->spike && pr->P >= LANE_SPLIT_PENCILS);
   if (pr->spike) {
-    pr->by_group = pr->P >= LANE_SPLIT_PENCILS;
     const size_t nv = (size_t)pr->P * pr->nblk * 2, nvf = (size_t)pr->P * pr->nblk_f * 2;
     CK(dalloc(&pr->d_sp_u, nv * 32));
     CK(reset_spike_guess(pr, ctx->stream));

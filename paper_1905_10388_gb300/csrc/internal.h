@@ -107,6 +107,8 @@ cudaError_t launch_spike_backward_rec(cudaStream_t s, const LaneArgs& a, const d
 // pencils.  Its time is the chain's (about 0.93 us per row and solve) up to
 // 608 groups, the whole-row-order kernel's (pair.cu) grows with the pencils:
 // 288 rows of 3D Rayleigh-Benard take 0.27 ms against 0.14 ms for 1024 pencils.
+// Pencils that row blocks serve take those first (2048 pencils of Fisher-KPP, per
+// solve: 512 rows 0.28 ms whole, 0.17 ms in blocks; 2048 rows 1.13 and 0.55).
 constexpr int LANE_MIN_PENCILS = 2048;
 
 // Chebyshev backward transform on the tensor cores (chebmma.cu): the split

@@ -9,6 +9,7 @@ if not torch.cuda.is_available():
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
 from paper_1905_10388_gb300.solver import Context, FisherKPPSolver, QGInversion, RB3DSolver, RBSolver
+from gpu_util import rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -32,3 +33,27 @@ def test_kernels_asked_for_by_name(ctx, kind, kernels):
     s = RBSolver(ctx, 64, 64, 1e6)
     s.set_solve_kernel(kind)
     assert _upload(s) == kernels
+
+
+# 2048 pencils: 512 rows in row blocks, 128 rows whole (the same bits as the
+# window order, for a band that cannot be asked for by name)
+@pytest.mark.parametrize("nz,blocks", [(256, True), (64, False)])
+def test_row_blocks_come_before_whole_pencils(ctx, nz, blocks):
+    out = []
+    for kind in ("window", "auto"):
+        s = FisherKPPSolver(ctx, 4096, nz, scheme="SBDF2", precision="mixed", dealias=(1, 1))
+        s.set_solve_kernel(kind)
+        s.factor(1e-3)
+        if kind == "auto":
+            assert ("k_lane_fwd<1>" in s.solve_kernels()) == blocks
+            assert ("k_lane_fwd<0>" in s.solve_kernels()) != blocks
+        s.set_initial_state(np.random.default_rng(1).random((nz, 4096)))
+        s.step(3)
+        s.sync()
+        out.append(s.get_state())
+    assert np.isfinite(out[0]).all()
+    if blocks:
+        for a, b in zip(*out):
+            assert rel_err(b, a) < 1e-9
+    else:
+        assert np.array_equal(*out)
