@@ -2610,7 +2610,8 @@ sp_status sp_get_solve_kernels(sp_ctx* ctx, int problem, const char** names, int
   } else if (pr->spike) {
     s = "k_pencil_split";
   } else {
-    s = whole_row_kernel(pr->P, pr->npad, pr->lpad, pr->upad) == WHOLE_PAIR ? "k_pencil_pair" : "k_pencil_solve";
+    const WholeRowKernel k = whole_row_kernel(pr->P, pr->npad, pr->lpad, pr->upad);
+    s = k == WHOLE_PAIR ? "k_pencil_pair" : k == WHOLE_NARROW ? "k_pencil_solve_narrow" : "k_pencil_solve";
   }
   if (names) *names = s;
   if (launches) *launches = n;

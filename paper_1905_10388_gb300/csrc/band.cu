@@ -618,6 +618,13 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 2) k_pencil_solve(SolveArgs a) 
   extern __shared__ __align__(128) unsigned char smem_raw[];
   pencil_solve_body<RU, -1, SOLVE_THREADS>(a, blockIdx.x, smem_raw);
 }
+// 128 threads, up to four CTAs per SM: for more pencils than two CTAs per SM hold,
+// more concurrent chains outweigh the narrower assembly and epilogue
+template <int RU>
+__global__ void __launch_bounds__(128, 4) k_pencil_solve_narrow(SolveArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  pencil_solve_body<RU, -1, 128>(a, blockIdx.x, smem_raw);
+}
 // right-hand-side assembly only (MODE 1) or epilogue only (MODE 2), around
 // the lane substitution: shared memory for B~ alone, several CTAs per SM
 template <int MODE>
@@ -628,11 +635,15 @@ __global__ void __launch_bounds__(128, 6) k_pencil_stage(SolveArgs a) {
 
 size_t pencil_solve_smem(int npad, int lpad, int upad) { return solve_smem_bytes(npad, lpad, upad); }
 
-// More pencils than one wave of two CTAs per SM: several pencils' chains per
-// sub-partition instead of a CTA per pencil (where three of this kernel's CTAs
-// would fit an SM, 228 KB of shared memory, 1 KB of it reserved per CTA).
+// One wave of two wide CTAs per SM; beyond that narrow ones, where three fit an
+// SM (228 KB of shared memory, 1 KB of it reserved per CTA); from more than four
+// pencils per SM on two pencils per CTA without factor rings.  Its chains, with
+// the factor from global memory, are longer, so up to there it loses (per
+// solve: 448 rows of 384 pencils 86 us narrow, 101 us in pairs, 512 pencils 97
+// and 111; 3D 32 x 32 x 32, 512 pencils, 89 and 112; beyond, pair.cu).
 WholeRowKernel whole_row_kernel(int P, int npad, int lpad, int upad) {
-  return P > 2 * GPU_SMS && 3 * (solve_smem_bytes(npad, lpad, upad) + 1024) <= 228 * 1024 ? WHOLE_PAIR : WHOLE_WINDOW;
+  if (P <= 2 * GPU_SMS || 3 * (solve_smem_bytes(npad, lpad, upad) + 1024) > 228 * 1024) return WHOLE_WINDOW;
+  return P <= PAIR_MIN_PENCILS ? WHOLE_NARROW : WHOLE_PAIR;
 }
 
 cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
@@ -652,16 +663,17 @@ cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
   }
   const size_t smem = solve_smem_bytes(a.npad, a.lpad, a.upad);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  const int grid = a.P;
-  if (whole_row_kernel(a.P, a.npad, a.lpad, a.upad) == WHOLE_PAIR) return launch_pencil_pair(s, a);
-  if (a.kuu <= 31) {
-    cudaFuncSetAttribute(k_pencil_solve<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_pencil_solve<1><<<grid, SOLVE_THREADS, smem, s>>>(a);
-  } else {
-    cudaFuncSetAttribute(k_pencil_solve<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_pencil_solve<2><<<grid, SOLVE_THREADS, smem, s>>>(a);
+  auto go = [&](auto kernel, int threads) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<a.P, threads, smem, s>>>(a);
+    return cudaGetLastError();
+  };
+  switch (whole_row_kernel(a.P, a.npad, a.lpad, a.upad)) {
+    case WHOLE_PAIR: return launch_pencil_pair(s, a);
+    case WHOLE_NARROW: return a.kuu <= 31 ? go(k_pencil_solve_narrow<1>, 128) : go(k_pencil_solve_narrow<2>, 128);
+    default: return a.kuu <= 31 ? go(k_pencil_solve<1>, SOLVE_THREADS) : go(k_pencil_solve<2>, SOLVE_THREADS);
   }
-  return cudaGetLastError();
 }
 
 // bands for which the lane substitution can be asked for by name

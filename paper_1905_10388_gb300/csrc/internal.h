@@ -284,7 +284,7 @@ cudaError_t launch_eig_residual(cudaStream_t s, int P, int n, int nnz, const int
                                 double* res);
 size_t pencil_solve_smem(int npad, int lpad, int upad);
 // the kernel that solves P pencils in whole-row order, one launch
-enum WholeRowKernel { WHOLE_WINDOW, WHOLE_PAIR };
+enum WholeRowKernel { WHOLE_WINDOW, WHOLE_NARROW, WHOLE_PAIR };
 WholeRowKernel whole_row_kernel(int P, int npad, int lpad, int upad);
 // partitioned pencil solve, one CTA per pencil (split.cu)
 cudaError_t launch_pencil_split(cudaStream_t s, const SolveArgs& a);
@@ -298,6 +298,7 @@ cudaError_t launch_pencil_pair_batched(cudaStream_t s, const SolveArgs* args, co
                                        int max_kuu, size_t smem);
 size_t pencil_pair_smem(int npad, int per);
 int pencil_pair_per(int npad, long long pencils);
+constexpr int PAIR_MIN_PENCILS = 4 * GPU_SMS;
 bool lanes_supported(int kl, int kuu);
 cudaError_t launch_coef_to_solve(cudaStream_t s, int P, int S, int Nz, const double2* xc,
                                  double2* xt, const int32_t* col_map, const int32_t* var_recombine,

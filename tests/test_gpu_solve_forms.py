@@ -57,3 +57,10 @@ def test_row_blocks_come_before_whole_pencils(ctx, nz, blocks):
             assert rel_err(b, a) < 1e-9
     else:
         assert np.array_equal(*out)
+
+
+@pytest.mark.parametrize("nx,nz,kernel", [(768, 64, "k_pencil_solve_narrow"), (1024, 64, "k_pencil_solve_narrow"),
+                                          (1536, 12, "k_pencil_pair")])
+def test_whole_row_kernel_by_pencils(ctx, nx, nz, kernel):
+    d = (3, 2) if nx == 1024 else (4, 3) if nz % 3 == 0 else (2, 1)
+    assert _upload(RBSolver(ctx, nx, nz, 1e6, precision="mixed", dealias=d)) == [kernel]
