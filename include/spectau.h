@@ -423,8 +423,8 @@ sp_status sp_set_z_transform(sp_ctx* ctx, int problem, int kind);
 sp_status sp_get_z_transform(sp_ctx* ctx, int problem, int* kind);
 sp_status sp_get_spike_blocks(sp_ctx* ctx, int problem, int* nblk);
 
-/* The kernels of one pencil solve of this problem, in order ("a + b + ..."; a
- * static string), and how many launches they are.  Either pointer may be
+/* The kernels of one pencil solve of this problem, in order ("a + b + ...", held
+ * by the problem), and how many launches they are.  Either pointer may be
  * NULL.  SP_ERR_STATE while the problem is not on the device. */
 sp_status sp_get_solve_kernels(sp_ctx* ctx, int problem, const char** names, int* launches);
 sp_status sp_last_solve_time(sp_ctx* ctx, int problem, double* ms_per_launch, int* launches);

@@ -202,9 +202,13 @@ struct Problem {
   // inflow/outflow vectors of the blocks
   bool spike = false;
   bool by_group = false;                     // the lane substitution serves the problem (whole or partitioned)
+  std::string solve_names;                   // sp_get_solve_kernels
+  bool passes = false;                       // row blocks in launches of their own (spike.cu)
   int spike_blocks = 0;                      // requested (0: automatic)
   int nblk = 0, nblk_f = 0;
   double *d_sp_s0 = nullptr, *d_sp_s = nullptr, *d_sp_o0 = nullptr, *d_sp_u = nullptr;
+  int nblkT = 0;                             // row blocks of the transposed solves
+  bool passesT = false;
   double* d_spT_u = nullptr;                 // inflows of the transposed solves
   std::map<std::pair<int, int>, TransformPlan> plans;
   // stepping state
@@ -336,26 +340,40 @@ int near_divisor(int whole, int target) {
   return best;
 }
 
-// Blocks per pencil of the partitioned back substitution, each a whole number
-// of 32-row chunks.  In the one-CTA-per-pencil form (split.cu) a block and
-// part is a warp's: eight blocks for a CTA of 16 warps, four for one of 8
-// (512 x 256 SBDF2 mixed, 16 steps: 2 blocks 4.79 ms, 4 blocks 3.76, 8 blocks
-// 4.15; 500-step adjoint sizes, 20 steps: 4 blocks 17.8 ms, 7 16.6, 14 18.7).
-// From LANE_SPLIT_PENCILS pencils on the lane substitution takes them: about
-// 1024 groups of 16 pencils x blocks, a warp or two for each of the GPU's 608
-// sub-partitions (Fisher-KPP 2048 x 1024, four steps: 512 warps 5.20 ms, 1024
-// 4.91 ms, 2048 5.77 ms).
-int default_spike_blocks(int npad, int P) {
-  const int nch = npad / SOLVE_CHUNK;
-  const int groups = (P + LANE_GROUP - 1) / LANE_GROUP;
-  if (P >= LANE_SPLIT_PENCILS) return near_divisor(nch, std::max(2, 1024 / groups));
-  return near_divisor(nch, P <= GPU_SMS ? 8 : 4);
+// Row blocks of a problem's partitioned substitution; their rows are whole
+// 32-row chunks.
+struct RowBlocks {
+  int nblk, nblk_f;             // back and forward
+};
+// One CTA per pencil (split.cu): a back block and part is a warp's, eight blocks
+// for a CTA of 16 warps, four for one of 8 (512 x 256 SBDF2 mixed, 16 steps: 2
+// blocks 4.79 ms, 4 blocks 3.76, 8 blocks 4.15; 500-step adjoint sizes, 20 steps:
+// 4 blocks 17.8 ms, 7 16.6, 14 18.7).  Forward blocks of about 32 rows, 64 for
+// long pencils (a block costs a step of the recurrence over blocks, about as
+// long as three rows of its two passes); with a lower band wider than the
+// 8-lane forward windows as long as the back ones.
+RowBlocks split_blocks(int npad, int P, bool wide) {
+  const int nch = npad / SOLVE_CHUNK, nblk = near_divisor(nch, P <= GPU_SMS ? 8 : 4);
+  return {nblk, wide ? nblk : npad <= 1024 ? nch : near_divisor(nch, nch / 2)};
 }
-// Forward blocks: of about 32 rows, 64 for long pencils (a block costs a step
-// of the recurrence over blocks, about as long as three rows of its two passes).
-int default_forward_blocks(int npad) {
-  const int nch = npad / SOLVE_CHUNK;
-  return npad <= 1024 ? nch : near_divisor(nch, nch / 2);
+// Lane substitution in row blocks: about 1024 groups of 16 pencils x blocks, a
+// warp or two for each of the GPU's 608 sub-partitions (Fisher-KPP 2048 x 1024,
+// four steps: 512 warps 5.20 ms, 1024 4.91 ms, 2048 5.77 ms).
+RowBlocks lane_blocks(int npad, int P) {
+  const int groups = (P + LANE_GROUP - 1) / LANE_GROUP, nblk = near_divisor(npad / SOLVE_CHUNK, std::max(2, 1024 / groups));
+  return {nblk, nblk};
+}
+// Passes in launches of their own (spike.cu): about 1024 / P back blocks, two to
+// four chains per sub-partition with their two parts, of at least 64 rows (256
+// pencils of 1792 rows: 4 blocks 0.224 ms per solve, 7 blocks 0.254, 14 blocks
+// 0.253, whole pencils 0.289); forward blocks of 128 rows, or 64 or 32 where
+// those divide the rows.
+RowBlocks pass_blocks(int npad, int P) {
+  const int nch = npad / SOLVE_CHUNK, target = std::max(2, (1024 + P - 1) / P);
+  int nblk = 1;
+  for (int d = 2; d <= nch / 2; ++d)
+    if (nch % d == 0 && std::abs(d - target) < std::abs(nblk - target)) nblk = d;
+  return {nblk, nch % 4 == 0 ? nch / 4 : nch % 2 == 0 ? nch / 2 : nch};
 }
 
 // (row, first entry, entries) of a pattern's rows, those with entries first.
@@ -546,19 +564,24 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
   }
   // up to a few thousand pencils are too few chains for the GPU: cut each
   // pencil's rows into blocks substituted in parallel (split.cu, lanes.cu)
-  pr->nblk = pr->spike_blocks > 0 ? pr->spike_blocks : default_spike_blocks(pr->npad, pr->P);
-  // (a lower band wider than the 8-lane forward windows: forward blocks as
-  // long as the back ones, in the one-CTA form only)
-  const bool wide = pr->kl > 7;
-  pr->nblk_f = pr->P >= LANE_SPLIT_PENCILS || wide ? pr->nblk : default_forward_blocks(pr->npad);
-  const bool split_fits = pr->P >= LANE_SPLIT_PENCILS ||
-                          pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, kuu, wide) <= 227 * 1024;
-  const bool bands = wide ? pr->kl <= 30 && pr->P < LANE_SPLIT_PENCILS && spike_bwd_supported(kuu, pr->npad, pr->nblk)
-                          : spike_supported(pr->kl, kuu, pr->npad, pr->nblk);
-  pr->spike = split_fits && bands &&
-              (pr->solve_kind == SP_SOLVE_SPIKE ||
-               (pr->solve_kind == SP_SOLVE_AUTO && pr->P < SPIKE_MAX_PENCILS &&
-                (pr->npad >= SPIKE_MIN_ROWS || (pr->P <= SPLIT_MAX_PENCILS && pr->npad >= SPLIT_MIN_ROWS))));
+  const bool by_name = pr->solve_kind == SP_SOLVE_SPIKE, wide = pr->kl > 7;
+  const bool automatic = pr->solve_kind == SP_SOLVE_AUTO && pr->P < SPIKE_MAX_PENCILS;
+  auto use = [&](RowBlocks rb) {
+    pr->nblk = pr->spike_blocks > 0 ? pr->spike_blocks : rb.nblk;
+    pr->nblk_f = (wide || pr->P >= LANE_SPLIT_PENCILS) ? pr->nblk : rb.nblk_f;
+    return wide ? pr->kl <= 30 && spike_bwd_supported(kuu, pr->npad, pr->nblk)
+                : spike_supported(pr->kl, kuu, pr->npad, pr->nblk);
+  };
+  if (pr->P >= LANE_SPLIT_PENCILS) {
+    pr->spike = (by_name || (automatic && pr->npad >= SPIKE_MIN_ROWS)) && !wide && use(lane_blocks(pr->npad, pr->P));
+  } else {
+    pr->spike = (by_name || (automatic && (pr->npad >= SPIKE_MIN_ROWS ||
+                                           (pr->P <= SPLIT_MAX_PENCILS && pr->npad >= SPLIT_MIN_ROWS)))) &&
+                use(split_blocks(pr->npad, pr->P, wide)) &&
+                split_serves(pr->P, pr->npad, wide, pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, kuu, wide));
+    if (!pr->spike && !wide && (by_name || (automatic && pr->npad >= SPIKE_MIN_ROWS)))
+      pr->spike = pr->passes = use(pass_blocks(pr->npad, pr->P));
+  }
   // thousands of pencils else: one lane per right-hand side, whole pencils
   pr->lanes = pr->solve_kind == SP_SOLVE_LANES ||
               (pr->solve_kind == SP_SOLVE_AUTO && !pr->spike && pr->P >= LANE_MIN_PENCILS);
@@ -567,12 +590,15 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
     const size_t nv = (size_t)pr->P * pr->nblk * 2, nvf = (size_t)pr->P * pr->nblk_f * 2;
     CK(dalloc(&pr->d_sp_u, nv * 32));
     CK(reset_spike_guess(pr, ctx->stream));
-    if (pr->by_group) {
+    if (pr->by_group || pr->passes) {
       CK(dalloc(&pr->d_sp_s0, nvf * 8));
       CK(dalloc(&pr->d_sp_s, nvf * 8));
       CK(dalloc(&pr->d_sp_o0, nv * 32));
-    } else {
-      CK(dalloc(&pr->d_bg, (size_t)pr->P * pr->n));
+    }
+    if (!pr->by_group) CK(dalloc(&pr->d_bg, (size_t)pr->P * pr->n));
+    if (pr->passes) {
+      CK(dalloc(&pr->d_xg, (size_t)pr->P * pr->n));
+      CK(dalloc(&pr->d_yg, (size_t)pr->P * pr->n));
     }
   }
   if (pr->by_group) {
@@ -777,7 +803,8 @@ SolveArgs base_args(Problem* pr, sp_ctx* ctx, int fac) {
   a.spD = pr->spike ? pr->fac[fac].spD : nullptr;   // null unless partitioned substitution
   a.spE = pr->spike ? pr->fac[fac].spE : nullptr;
   a.sp_nblk = pr->nblk; a.sp_nblk_f = pr->nblk_f; a.sp_u = pr->d_sp_u;
-  a.bg = pr->d_bg; a.xg = pr->d_xg;
+  a.sp_passes = pr->passes;
+  a.bg = pr->d_bg; a.xg = pr->d_xg; a.yg = pr->d_yg; a.by_pencil = !pr->by_group;
   return a;
 }
 
@@ -791,18 +818,24 @@ void set_ep_L(Problem* pr, SolveArgs& a) {
   a.ep_mv_vals = pr->d_Lv; a.ep_list = pr->d_epL; a.ep_nl = pr->n; a.ep_indices = pr->d_indices; a.ep_nnz = (int)pr->nnz;
 }
 
-// Arguments of the lane substitution of `pr` with the listed factor `f`.
-LaneArgs lane_args(sp_ctx* ctx, Problem* pr, const LaneList& f, int kl, int kuu, int cold) {
+// Arguments of the substitution launches of `pr` with the solve's factor, its
+// lists for the lane substitution.
+LaneArgs lane_args(sp_ctx* ctx, Problem* pr, const SolveArgs& a) {
   LaneArgs la{};
-  la.P = pr->P; la.n = pr->n; la.npad = pr->npad; la.kl = kl; la.kuu = kuu;
-  la.nblk = pr->spike ? pr->nblk : 1; la.m = pr->npad / la.nblk;
-  la.nblk_f = pr->spike ? pr->nblk_f : 1; la.m_f = pr->npad / la.nblk_f;
-  la.lcap = f.lcap; la.ucap = f.ucap; la.lrecs = f.lrecs; la.urecs = f.urecs;
-  la.Lv = f.Lv; la.Uv = f.Uv; la.lco = f.lco; la.uco = f.uco; la.pg = f.pg;
+  la.P = pr->P; la.n = pr->n; la.npad = pr->npad; la.kl = a.kl; la.kuu = a.kuu;
+  la.nblk = pr->spike ? a.sp_nblk : 1; la.m = pr->npad / la.nblk;
+  la.nblk_f = pr->spike && a.sp_nblk_f > 0 ? a.sp_nblk_f : 1; la.m_f = pr->npad / la.nblk_f;
+  if (a.ll) {
+    const LaneList& f = *a.ll;
+    la.lcap = f.lcap; la.ucap = f.ucap; la.lrecs = f.lrecs; la.urecs = f.urecs;
+    la.Lv = f.Lv; la.Uv = f.Uv; la.lco = f.lco; la.uco = f.uco; la.pg = f.pg;
+  }
+  la.L = a.Lf; la.piv = a.piv; la.U = a.Uf; la.lpad = a.lpad; la.upad = a.upad;
+  la.by_pencil = a.by_pencil;
   la.bg = pr->d_bg; la.yg = reinterpret_cast<double*>(pr->d_yg); la.xg = pr->d_xg;
   la.status = ctx->d_status;
-  la.cold = cold;
-  la.s0 = pr->d_sp_s0; la.sst = pr->d_sp_s; la.o0 = pr->d_sp_o0; la.uin = pr->d_sp_u;
+  la.cold = a.sp_cold;
+  la.s0 = pr->d_sp_s0; la.sst = pr->d_sp_s; la.o0 = pr->d_sp_o0; la.uin = a.sp_u;
   return la;
 }
 
@@ -831,10 +864,10 @@ sp_status solve(sp_ctx* ctx, Problem* pr, cudaStream_t s, const SolveArgs& args)
   if (t) CK(cudaEventRecord(pr->ev[pr->ev_used], s));
   SolveArgs a = args;
   if (a.ll) {
-    // assembly -> lane substitution, whole or partitioned -> epilogue
+    // assembly -> lane substitution, whole or in row blocks -> epilogue
     a.mode = 1;
     CK(launch_pencil_solve(s, a));
-    const LaneArgs la = lane_args(ctx, pr, *a.ll, a.kl, a.kuu, a.sp_cold);
+    const LaneArgs la = lane_args(ctx, pr, a);
     if (pr->lanes) {
       CK(launch_lane_forward(s, la, 0));
       CK(launch_lane_backward(s, la, 0));
@@ -846,6 +879,23 @@ sp_status solve(sp_ctx* ctx, Problem* pr, cudaStream_t s, const SolveArgs& args)
       CK(launch_spike_backward_rec(s, la, a.spE));
       CK(launch_lane_backward(s, la, 2));
     }
+    a.mode = 2;
+    stage_lx(pr, a);
+    CK(launch_pencil_solve(s, a));
+  } else if (a.spE && a.sp_passes) {
+    // assembly -> passes over the row blocks -> epilogue (a wide lower band:
+    // the forward substitution whole, with the assembly)
+    const LaneArgs la = lane_args(ctx, pr, a);
+    a.mode = a.sp_nblk_f > 0 ? 1 : 3;
+    CK(launch_pencil_solve(s, a));
+    if (a.sp_nblk_f > 0) {
+      CK(launch_spike_forward(s, la, 1));
+      CK(launch_spike_forward_rec(s, la, a.spD));
+      CK(launch_spike_forward(s, la, 2));
+    }
+    CK(launch_spike_backward(s, la, 1));
+    CK(launch_spike_backward_rec(s, la, a.spE));
+    CK(launch_spike_backward(s, la, 2));
     a.mode = 2;
     stage_lx(pr, a);
     CK(launch_pencil_solve(s, a));
@@ -992,7 +1042,8 @@ SolveArgs transposed_args(Problem* pr, sp_ctx* ctx) {
   a.xs32_out = nullptr;
   a.ll = nullptr;
   a.spD = pr->facT.spD; a.spE = pr->facT.spE;    // null unless partitioned
-  a.sp_nblk_f = pr->nblk; a.sp_u = pr->d_spT_u;
+  a.sp_nblk = pr->nblkT; a.sp_nblk_f = pr->passesT ? 0 : pr->nblkT; a.sp_u = pr->d_spT_u;
+  a.sp_passes = pr->passesT; a.by_pencil = 1;
   a.sp_cold = 1;                        // lambda need not come from the last call
   return a;
 }
@@ -1083,7 +1134,8 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
   for (Problem* pr : ps) {
     pencils += pr->P;
     b->fast = b->fast && pr->rows_fast;
-    b->split = b->split && pr->spike && !pr->by_group && pr->kl <= 7;
+    b->split = b->split && pr->spike && !pr->by_group && pr->kl <= 7 &&
+               pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false) <= 227 * 1024;
   }
   b->split = b->split && pencils <= SPLIT_MAX_PENCILS;
   for (size_t q = 0; q < ps.size(); ++q) {
@@ -2017,17 +2069,25 @@ sp_status sp_adjoint_init(sp_ctx* ctx, int problem) {
   CK(e);
   pr->facT.alpha = pr->fac[0].alpha;
   pr->facT.beta = pr->fac[0].beta;
-  // the transposed solves are partitioned like the forward ones, their wider
-  // lower band (kl' = ku) in forward blocks as long as the back ones
+  // the transposed solves, with their wider lower band (kl' = ku): one CTA per
+  // pencil, its forward blocks as long as the back ones, or passes over the back
+  // blocks after a whole-row forward substitution
   const int kuuT = pr->klT + pr->kuT;
-  if (pr->spike && !pr->by_group && pr->upad == 32 && pr->klT <= 30 &&
-      spike_bwd_supported(kuuT, pr->npad, pr->nblk) &&
-      pencil_split_smem(pr->npad, pr->nblk, pr->nblk, kuuT, pr->klT > 7) <= 227 * 1024) {
-    if (!pr->facT.spD) CK(dalloc(&pr->facT.spD, (size_t)pr->P * pr->nblk * (pr->klT > 7 ? 31 * 32 : 7 * 8)));
-    if (!pr->facT.spE) CK(dalloc(&pr->facT.spE, (size_t)pr->P * pr->nblk * kuuT * 32));
-    if (!pr->d_spT_u) CK(dalloc(&pr->d_spT_u, (size_t)pr->P * pr->nblk * 2 * 32));
-    CK(launch_spike_coupling(s, pr->P, pr->npad, pr->nblk, pr->nblk, pr->klT, kuuT, pr->lpadT, pr->upad, pr->facT,
-                             false));
+  const bool wideT = pr->klT > 7;
+  pr->nblkT = pr->passes ? split_blocks(pr->npad, pr->P, wideT).nblk : pr->nblk;
+  bool partT = pr->spike && !pr->by_group && pr->upad == 32 && pr->klT <= 30 &&
+               spike_bwd_supported(kuuT, pr->npad, pr->nblkT) &&
+               split_serves(pr->P, pr->npad, wideT, pencil_split_smem(pr->npad, pr->nblkT, pr->nblkT, kuuT, wideT));
+  if (!partT && pr->passes && pr->upad == 32 && spike_bwd_supported(kuuT, pr->npad, pr->nblk)) {
+    partT = pr->passesT = true;
+    pr->nblkT = pr->nblk;
+  }
+  if (partT) {
+    if (!pr->facT.spD && !pr->passesT) CK(dalloc(&pr->facT.spD, (size_t)pr->P * pr->nblkT * (wideT ? 31 * 32 : 7 * 8)));
+    if (!pr->facT.spE) CK(dalloc(&pr->facT.spE, (size_t)pr->P * pr->nblkT * kuuT * 32));
+    if (!pr->d_spT_u) CK(dalloc(&pr->d_spT_u, (size_t)pr->P * pr->nblkT * 2 * 32));
+    CK(launch_spike_coupling(s, pr->P, pr->npad, pr->passesT ? 0 : pr->nblkT, pr->nblkT, pr->klT, kuuT, pr->lpadT,
+                             pr->upad, pr->facT, false));
     CK(cudaStreamSynchronize(s));
   }
   return SP_OK;
@@ -2343,7 +2403,7 @@ sp_status sp_eig_target(sp_ctx* ctx, int problem, double sigma_t, int iters, con
   cudaError_t e = launch_band_factor(s, pr->P, pr->n, (int)pr->nnz, pr->kl, pr->ku, pr->d_indptr, pr->d_indices,
                                      pr->d_Mv, pr->d_Lv, sigma_t, 1.0, work, pr->fac[0], pr->npad, pr->lpad,
                                      pr->upad, ctx->d_status);
-  const bool split = pr->spike && !pr->by_group;
+  const bool split = pr->spike && !pr->by_group && !pr->passes;
   if (e == cudaSuccess && split) {
     e = reset_spike_guess(pr, s);
     if (e == cudaSuccess)
@@ -2535,7 +2595,7 @@ sp_status sp_set_solve_kernel(sp_ctx* ctx, int problem, int kind) {
                 pr->kl, pr->kl + pr->ku);
   if (kind == SP_SOLVE_SPIKE) {
     const int npad = (pr->n + SOLVE_CHUNK - 1) / SOLVE_CHUNK * SOLVE_CHUNK;
-    const int nblk = pr->spike_blocks > 0 ? pr->spike_blocks : default_spike_blocks(npad, pr->P);
+    const int nblk = pr->spike_blocks > 0 ? pr->spike_blocks : 1;
     if (pr->nnz < 0 || !spike_supported(pr->kl, pr->kl + pr->ku, npad, nblk))
       return fail(ctx, SP_ERR_ARG, "no partitioned substitution for kl = %d, kl + ku = %d, %d rows in %d blocks "
                   "(needs kl <= 7, kl + ku <= 31, whole 32-row chunks per block; set the pencils first)",
@@ -2598,23 +2658,32 @@ sp_status sp_get_solve_kernels(sp_ctx* ctx, int problem, const char** names, int
   if (!pr) return fail(ctx, SP_ERR_ARG, "bad context or problem id");
   ctx->err.clear();
   if (!pr->uploaded) return fail(ctx, SP_ERR_STATE, "the problem is not on the device yet");
-  const char* s;
-  int n = 1;
-  if (pr->lanes) {
-    s = "k_pencil_stage<1> + k_lane_fwd<0> + k_lane_bwd<0> + k_pencil_stage<2>";
-    n = 4;
-  } else if (pr->by_group) {
-    s = "k_pencil_stage<1> + k_lane_fwd<1> + k_spike_fwd_rec + k_lane_fwd<2> + k_lane_bwd<1> + k_spike_bwd_rec + "
-        "k_lane_bwd<2> + k_pencil_stage<2>";
-    n = 8;
+  std::vector<const char*> k;
+  if (pr->by_group || pr->passes) {
+    const bool wide = pr->P < STAGE_WIDE_PENCILS;
+    k.push_back(wide ? "k_pencil_stage_wide<1>" : "k_pencil_stage<1>");
+    if (pr->lanes) {
+      k.insert(k.end(), {"k_lane_fwd<0>", "k_lane_bwd<0>"});
+    } else {
+      if (pr->nblk_f > 1) k.push_back(pr->passes ? "k_spike_fwd<1>" : "k_lane_fwd<1>");
+      k.insert(k.end(), {"k_spike_fwd_rec", pr->passes ? "k_spike_fwd<2>" : "k_lane_fwd<2>",
+                         pr->passes ? "k_spike_bwd<1>" : "k_lane_bwd<1>"});
+      if (pr->nblk > 1) {
+        k.push_back(pr->kl + pr->ku <= 16 ? "k_spike_bwd_rec_narrow" : "k_spike_bwd_rec");
+        k.push_back(pr->passes ? "k_spike_bwd<2>" : "k_lane_bwd<2>");
+      }
+    }
+    k.push_back(wide ? "k_pencil_stage_wide<2>" : "k_pencil_stage<2>");
   } else if (pr->spike) {
-    s = "k_pencil_split";
+    k.push_back("k_pencil_split");
   } else {
-    const WholeRowKernel k = whole_row_kernel(pr->P, pr->npad, pr->lpad, pr->upad);
-    s = k == WHOLE_PAIR ? "k_pencil_pair" : k == WHOLE_NARROW ? "k_pencil_solve_narrow" : "k_pencil_solve";
+    const WholeRowKernel w = whole_row_kernel(pr->P, pr->npad, pr->lpad, pr->upad);
+    k.push_back(w == WHOLE_PAIR ? "k_pencil_pair" : w == WHOLE_NARROW ? "k_pencil_solve_narrow" : "k_pencil_solve");
   }
-  if (names) *names = s;
-  if (launches) *launches = n;
+  pr->solve_names.clear();
+  for (const char* name : k) pr->solve_names += (pr->solve_names.empty() ? "" : " + ") + std::string(name);
+  if (names) *names = pr->solve_names.c_str();
+  if (launches) *launches = (int)k.size();
   return SP_OK;
 }
 

@@ -389,7 +389,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
   // MODE >= 0 fixes the stage at compile time (assembly-only and
   // epilogue-only kernels carry neither the factor ring nor the substitution)
   const int mode = MODE >= 0 ? MODE : a.mode;
-  const int lp = mode == 0 ? a.lpad : 0, up = mode == 0 ? a.upad : 0;
+  const int lp = (mode == 0 || mode == 3) ? a.lpad : 0, up = mode == 0 ? a.upad : 0;
   const int pp = block, tid = threadIdx.x;
   constexpr int nt = NT;
   constexpr int PENCIL_U = MODE >= 0 ? 4 : 1;
@@ -433,26 +433,29 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
 
   if (tid == 0) {
     *sm.abort_flag = 0;
-    if (mode == 0) {
+    if (mode == 0 || mode == 3) {
       for (int s = 0; s < SOLVE_RING; ++s) {
         mbar_init(&sm.barL[s], 1);
         mbar_init(&sm.barU[s], 1);
       }
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       // the factor does not depend on the prologue: start streaming now
+      // (mode 3, forward substitution only: L alone)
       for (int c = 0; c < min(SOLVE_RING, nchunks); ++c) issue_L(c);
-      for (int k = 0; k < min(SOLVE_RING, nchunks); ++k) issue_U(k);
+      if (mode == 0)
+        for (int k = 0; k < min(SOLVE_RING, nchunks); ++k) issue_U(k);
     }
   }
 
   // ---- prologue: B~ = linear combination of stored vectors, one matvec,
   //      left-preconditioned F~ (T-to-U conversion, tau rows dropped) and
   //      boundary values
-  // element r of this pencil in the lane substitution's vectors
-  const size_t v0 = lane_index(pp, 0, a.npad);
-  auto vec = [&](int r) { return v0 + (size_t)r * LANE_GROUP; };
+  // element r of this pencil in the substitution kernels' vectors
+  const size_t v0 = a.by_pencil ? (size_t)pp * n : lane_index(pp, 0, a.npad);
+  const int vstep = a.by_pencil ? 1 : LANE_GROUP;
+  auto vec = [&](int r) { return v0 + (size_t)r * vstep; };
   if (mode == 2) {
-    // epilogue only: X~ = b / U_jj, b from the lane substitution
+    // epilogue only: X~ = b / U_jj, b from the substitution
     const double* rdp = a.rd + (size_t)pp * a.npad;
     for (int r = tid; r < n; r += nt) {
       const double2 b = a.xg[vec(r)];
@@ -485,7 +488,7 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
   //      Both warps read each ring slot; named barrier 1 (64 threads) at the
   //      top of every chunk both agrees on a timed-out wait and frees the
   //      previous slot for refilling.
-  if (mode == 0 && tid < 64) {
+  if ((mode == 0 || mode == 3) && tid < 64) {
     const int lane = tid & 31;
     const int comp = tid >> 5;                 // 0: real part, 1: imaginary part
     double* Bd = reinterpret_cast<double*>(sm.B) + comp;   // element j at Bd[2 j]
@@ -540,6 +543,8 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
     asm volatile("bar.sync 1, 64;" ::: "memory");
     // backward: scaled U columns (U_{j-t,j}/U_jj), window of 32*RU entries;
     // x_j = b_j / U_jj is applied once per chunk, lane l to row j0 + l
+    // (mode 3 stops after the forward pass: y is in B)
+    if (mode == 0) {
     constexpr int W = 32 * RU;
     const double* rdp = a.rd + (size_t)pp * a.npad;
     const int npad = a.npad;
@@ -594,18 +599,24 @@ __device__ __forceinline__ void pencil_solve_body(const SolveArgs& a, int block,
       }
       Bd[2 * (j0 + lane)] = xo * rdl;
     }
+    }
     if (!ok && tid == 0) {
       // report, then let every copy in flight land before the CTA exits
       raise_status(a.status, SP_ERR_TIMEOUT, pp);
       // chunks issued: RING up front, then chunk q - 1 + RING at the top of chunk q
       const int issL = min(nchunks, doneL == 0 ? SOLVE_RING : doneL - 1 + SOLVE_RING);
-      const int issU = min(nchunks, doneU == 0 ? SOLVE_RING : doneU - 1 + SOLVE_RING);
+      const int issU = mode == 0 ? min(nchunks, doneU == 0 ? SOLVE_RING : doneU - 1 + SOLVE_RING) : 0;
       for (int q = doneL; q < issL; ++q) bounded_wait(&sm.barL[q % SOLVE_RING], (q / SOLVE_RING) & 1);
       for (int q = doneU; q < issU; ++q) bounded_wait(&sm.barU[q % SOLVE_RING], (q / SOLVE_RING) & 1);
     }
   }
   __syncthreads();
   const bool work = !*sm.abort_flag;
+  if (mode == 3) {
+    // y = L^-1 P B~ for the partitioned back substitution
+    for (int r = tid; work && r < n; r += nt) a.yg[(size_t)pp * n + r] = sm.B[r];
+    return;
+  }
   if (work) pencil_epilogue<PENCIL_U>(a, pp, tid, nt, mode == 2, vec, sm.B);
 }
 
@@ -633,6 +644,14 @@ __global__ void __launch_bounds__(128, 6) k_pencil_stage(SolveArgs a) {
   pencil_solve_body<1, MODE>(a, blockIdx.x, smem_raw);
 }
 
+// the same with 512-thread CTAs, for problems with few pencils (one CTA per
+// pencil would leave most of the GPU idle at 128 threads)
+template <int MODE>
+__global__ void __launch_bounds__(512, 2) k_pencil_stage_wide(SolveArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  pencil_solve_body<1, MODE, 512>(a, blockIdx.x, smem_raw);
+}
+
 size_t pencil_solve_smem(int npad, int lpad, int upad) { return solve_smem_bytes(npad, lpad, upad); }
 
 // One wave of two wide CTAs per SM; beyond that narrow ones, where three fit an
@@ -649,19 +668,8 @@ WholeRowKernel whole_row_kernel(int P, int npad, int lpad, int upad) {
 cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
   SolveArgs a = args;
   fill_f_halves(a);
-  if (a.mode == 1 || a.mode == 2) {
-    const size_t smem = solve_smem_bytes(a.npad, 0, 0);
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
-    if (a.mode == 1) {
-      cudaFuncSetAttribute(k_pencil_stage<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_pencil_stage<1><<<a.P, 128, smem, s>>>(a);
-    } else {
-      cudaFuncSetAttribute(k_pencil_stage<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_pencil_stage<2><<<a.P, 128, smem, s>>>(a);
-    }
-    return cudaGetLastError();
-  }
-  const size_t smem = solve_smem_bytes(a.npad, a.lpad, a.upad);
+  const bool stage = a.mode == 1 || a.mode == 2;
+  const size_t smem = stage ? solve_smem_bytes(a.npad, 0, 0) : solve_smem_bytes(a.npad, a.lpad, a.upad);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   auto go = [&](auto kernel, int threads) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -669,6 +677,9 @@ cudaError_t launch_pencil_solve(cudaStream_t s, const SolveArgs& args) {
     kernel<<<a.P, threads, smem, s>>>(a);
     return cudaGetLastError();
   };
+  if (stage && a.P < STAGE_WIDE_PENCILS)
+    return a.mode == 1 ? go(k_pencil_stage_wide<1>, 512) : go(k_pencil_stage_wide<2>, 512);
+  if (stage) return a.mode == 1 ? go(k_pencil_stage<1>, 128) : go(k_pencil_stage<2>, 128);
   switch (whole_row_kernel(a.P, a.npad, a.lpad, a.upad)) {
     case WHOLE_PAIR: return launch_pencil_pair(s, a);
     case WHOLE_NARROW: return a.kuu <= 31 ? go(k_pencil_solve_narrow<1>, 128) : go(k_pencil_solve_narrow<2>, 128);

@@ -57,8 +57,9 @@ struct BandFactor {
   LaneList ll;                  // lists of the lane substitution (whole or partitioned)
 };
 
-// Lane substitution of one problem's pencils, whole (nblk = nblk_f = 1) or in
-// row blocks.
+// Substitution of one problem's pencils in launches of their own: by lanes,
+// whole (nblk = nblk_f = 1) or in row blocks (lanes.cu), or row blocks of a warp's
+// window (spike.cu).
 struct LaneArgs {
   int P, n, npad, kl, kuu;
   int nblk, m, nblk_f, m_f;     // blocks per pencil and their rows, back and forward
@@ -66,7 +67,10 @@ struct LaneArgs {
   const double* Lv; const double* Uv;
   const int32_t* lco; const int32_t* uco;
   const uint16_t* pg;
+  const double* L; const uint8_t* piv; const double* U; int lpad, upad;   // spike.cu: the factor itself
   // right-hand sides by group, [G][npad][16 pencils] complex, zero beyond n
+  // (spike.cu: by pencil, [p][n])
+  int by_pencil;
   const double2* bg;            // B~
   double* yg;                   // y = L^-1 P B~
   double2* xg;                  // b = U_jj x~
@@ -82,24 +86,41 @@ cudaError_t lane_list_build(cudaStream_t s, int P, int n, int npad, int kl, int 
                             const double* L, const uint8_t* piv, const double* U, LaneList& f);
 void lane_list_free(LaneList& f);
 
-// Problems with fewer pencils than this (and kl <= 7, kl + ku <= 31, at
-// least SPIKE_MIN_ROWS rows) use the partitioned substitution by default,
-// from LANE_SPLIT_PENCILS pencils on in its lane form (Fisher-KPP 2048 x 1024,
-// 1024 pencils: 0.41 ms per solve against 0.78 ms with the window kernel),
-// below that one CTA per pencil (2D Rayleigh-Benard 256 x 128, 128 pencils: 65
-// us per solve; eight launches of separate pass kernels took 110 us; 512 x 256,
-// 256 pencils: 188 us, the lane form 207 us).
+// Problems with fewer pencils than this, of at least SPIKE_MIN_ROWS rows with kl
+// <= 7 and kl + ku <= 31, use a partitioned substitution by default: from
+// LANE_SPLIT_PENCILS pencils on in its lane form (Fisher-KPP 2048 x 1024, 1024
+// pencils: 0.41 ms per solve against 0.78 ms with the window kernel), below
+// that one CTA per pencil where split_serves says so, else passes over the
+// blocks in launches of their own.
 constexpr int SPIKE_MAX_PENCILS = 4096;
-constexpr int LANE_SPLIT_PENCILS = 608;
+constexpr int LANE_SPLIT_PENCILS = 4 * GPU_SMS;
 constexpr int SPIKE_MIN_ROWS = 512;
-// Problems that have at most two CTAs per SM take it from fewer rows on (64 x
-// 32, 224 rows: 16 RK222 steps 2.27 ms with the window kernel, 2.10 ms).
+// Problems that have at most two CTAs per SM take one CTA per pencil from fewer
+// rows on (64 x 32, 224 rows: 16 RK222 steps 2.27 ms with the window kernel, 2.10 ms).
 constexpr int SPLIT_MAX_PENCILS = 2 * GPU_SMS;
 constexpr int SPLIT_MIN_ROWS = 96;
+// Whether one CTA of `smem` bytes per pencil beats passes in separate launches
+// (us per solve, one CTA against passes).  All pencils have to be on the GPU at
+// once (512 x 512: 592 against 373 with one CTA on each SM at a time).  Its time
+// is that of the fullest SM, the passes' goes with the pencils, so it wins with
+// most SMs' places taken (256 x 128, 128 pencils: 65 against 110; 512 x 256, 256
+// pencils: 186 against 209; 256 x 512: 217 against 223), and with fewer pencils
+// as long as their chains are short (64 x 256, 1792 rows: faster; 64 x 384, 2688
+// rows: 166 against 136; 192 pencils of 1344 rows 167 against 159).  A wide lower
+// band has no such passes forward: there one CTA wins wherever all fit (adjoint
+// step at 128 x 512: 1.83 ms against 2.12).
+inline bool split_serves(int P, int npad, bool wide, size_t smem) {
+  const int per_sm = (P + GPU_SMS - 1) / GPU_SMS;
+  if (P > SPLIT_MAX_PENCILS || smem > 227 * 1024 || per_sm * (smem + 1024) > 228 * 1024) return false;
+  return wide || 4 * P >= 3 * per_sm * GPU_SMS || npad * per_sm <= 2048;
+}
 bool spike_supported(int kl, int kuu, int npad, int nblk);
 bool spike_bwd_supported(int kuu, int npad, int nblk);
 cudaError_t launch_spike_coupling(cudaStream_t s, int P, int npad, int nblk_f, int nblk, int kl, int kuu, int lpad,
                                   int upad, const BandFactor& f, bool by_row);
+// the passes over row blocks of a warp's window: 1 from zero / guessed inflows, 2 from the true ones
+cudaError_t launch_spike_forward(cudaStream_t s, const LaneArgs& a, int pass);
+cudaError_t launch_spike_backward(cudaStream_t s, const LaneArgs& a, int pass);
 cudaError_t launch_spike_forward_rec(cudaStream_t s, const LaneArgs& a, const double* D);
 cudaError_t launch_spike_backward_rec(cudaStream_t s, const LaneArgs& a, const double* E);
 
@@ -198,16 +219,18 @@ struct SolveArgs {
   const int32_t* bc_rows; const double2* bc_values;
   DevStatus* status;
   // mode 0: assembly, substitution and epilogue in one kernel; 1: assembly
-  // only, B~ to bg; 2: epilogue only, from xg (the lane substitution runs in
-  // between: bg, xg by group, xg holds b = U_jj x~).  The partitioned kernel
-  // keeps B~ [p][n] in bg for the epilogue's L~X~
-  int mode;
-  double2* bg; const double2* xg;
+  // only, B~ to bg; 2: epilogue only, from xg (the substitution runs in between:
+  // bg, xg by group or by pencil, xg holds b = U_jj x~); 3: assembly and
+  // whole-row forward substitution, y to yg (by pencil).  The one-CTA partitioned
+  // kernel keeps B~ [p][n] in bg for the epilogue's L~X~
+  int mode, by_pencil;
+  double2* bg; const double2* xg; double2* yg;
   // the factor's lists (host pointer; null: no lane substitution)
   const LaneList* ll;
   // coupling matrices of the partitioned substitution (null: not available)
   const double* spD; const double* spE;
-  int sp_nblk, sp_nblk_f;       // back- and forward-substitution blocks per pencil
+  int sp_passes;                // 1: row blocks in launches of their own (spike.cu), 0: in one (split.cu)
+  int sp_nblk, sp_nblk_f;       // back- and forward-substitution blocks per pencil (nblk_f 0: forward whole)
   double* sp_u;                 // back-substitution inflows, the next solve's guesses [p][nblk][2][32]
   // 1: start from zero inflows; 0: from the previous solve's, for right-hand
   // sides that change little from solve to solve (rounding errors scale with the guess)
@@ -299,6 +322,8 @@ cudaError_t launch_pencil_pair_batched(cudaStream_t s, const SolveArgs* args, co
 size_t pencil_pair_smem(int npad, int per);
 int pencil_pair_per(int npad, long long pencils);
 constexpr int PAIR_MIN_PENCILS = 4 * GPU_SMS;
+// assembly and epilogue launches with fewer pencils use 512 threads per pencil
+constexpr int STAGE_WIDE_PENCILS = 2 * GPU_SMS;
 bool lanes_supported(int kl, int kuu);
 cudaError_t launch_coef_to_solve(cudaStream_t s, int P, int S, int Nz, const double2* xc,
                                  double2* xt, const int32_t* col_map, const int32_t* var_recombine,

@@ -1,8 +1,11 @@
-// Coupling matrices of the partitioned substitutions (split.cu, lanes.cu) and
-// the lane form's recurrences over row blocks (sm_103a).
+// Partitioned substitution in launches of their own (sm_103a): the coupling
+// matrices of every partitioned form (split.cu has the method), the recurrences
+// over row blocks, and, for pencils that one CTA each does not suit (too many for
+// one wave of them, or long and few), passes over the blocks of all pencils.
 #include <algorithm>
 
 #include "internal.h"
+#include "tma.cuh"
 
 namespace spectau {
 
@@ -196,8 +199,9 @@ __global__ void __launch_bounds__(SPK_COUPLING_WARPS * 32)
 
 cudaError_t launch_spike_coupling(cudaStream_t s, int P, int npad, int nblk_f, int nblk, int kl, int kuu, int lpad,
                                   int upad, const BandFactor& f, bool by_row) {
-  if (kl > SPK_BW - 2 || kuu >= SPK_BW || nblk < 1 || nblk_f < 1 || npad % (nblk * SPK_CHUNK) ||
-      npad % (nblk_f * SPK_CHUNK))
+  // (nblk_f 0: E alone)
+  if (kl > SPK_BW - 2 || kuu >= SPK_BW || nblk < 1 || nblk_f < 0 || npad % (nblk * SPK_CHUNK) ||
+      (nblk_f > 0 && npad % (nblk_f * SPK_CHUNK)))
     return cudaErrorInvalidValue;
   const bool wide = kl > SPK_FS;
   const long long warps = (long long)P * nblk + (wide ? (long long)P * nblk_f : ((long long)P * nblk_f + 3) / 4);
@@ -218,7 +222,9 @@ __global__ void __launch_bounds__(128) k_spike_fwd_rec(LaneArgs s, const double*
   const int p = act ? chain >> 1 : 0, c = chain & 1;
   const int q = threadIdx.x & 7, i = q < SPK_FS ? q : 0;
   const bool own = act && q < SPK_FS;
-  const double* Bp = reinterpret_cast<const double*>(s.bg + lane_index(p, i < s.n ? i : 0, s.npad)) + c;
+  const int r0 = i < s.n ? i : 0;
+  const double* Bp =
+      reinterpret_cast<const double*>(s.bg + (s.by_pencil ? (size_t)p * s.n + r0 : lane_index(p, r0, s.npad))) + c;
   auto at = [&](int k) { return (((size_t)p * s.nblk_f + k) * 2 + c) * SPK_FW; };
   double st = i < s.n ? Bp[0] : 0.0;
   if (own) s.sst[at(0) + i] = st;
@@ -354,6 +360,192 @@ __global__ void __launch_bounds__(128) k_spike_bwd_rec_narrow(LaneArgs s, const 
     if (in) s.uin[at(k - 1)] = u;
     d = u - g;
   }
+}
+
+// ---------------------------------------------------------------------------
+// forward substitution of one block per 8-lane segment, four segments
+// (chains: pencil, block, real or imaginary part) per warp.  Lane q of a
+// segment holds row j + ((q - j) & 7) at step j.  PASS 1: zero inflow
+// (the first block: its true rows 0..7), writes the outflow; PASS 2: the
+// true inflow, writes y.
+// ---------------------------------------------------------------------------
+template <int PASS>
+__global__ void __launch_bounds__(128) k_spike_fwd(LaneArgs s) {
+  const int gl = blockIdx.x * blockDim.x + threadIdx.x;
+  const int q = threadIdx.x & 7;
+  const int nk = PASS == 1 ? s.nblk_f - 1 : s.nblk_f;   // PASS 1 skips the last block (no next block)
+  const int ch = gl >> 3;
+  const bool act = ch < s.P * nk * 2;
+  const int chv = act ? ch : 0;
+  const int c = chv & 1, k = (chv >> 1) % nk, p = (chv >> 1) / nk;
+  const int j0 = k * s.m_f, j1 = j0 + s.m_f, n = s.n;
+  const double* Bp = reinterpret_cast<const double*>(s.bg + (size_t)p * n) + c;   // row r at Bp[2 r]
+  auto fresh = [&](int r) -> double { return (act && r < n) ? Bp[2 * r] : 0.0; };
+  const size_t sidx = (((size_t)p * s.nblk_f + k) * 2 + c) * SPK_FW;
+  double v;
+  if (PASS == 1)
+    v = (k == 0 || q == SPK_FS) ? fresh(j0 + q) : 0.0;
+  else
+    v = (q < SPK_FS) ? (act ? s.sst[sidx + q] : 0.0) : fresh(j0 + q);
+  const double* Lp = s.L + (size_t)p * s.npad * s.lpad;
+  const uint8_t* pv = s.piv + (size_t)p * s.npad;
+  double* Yp = s.yg + (size_t)p * n * 2 + c;
+  const int kl = s.kl, lpad = s.lpad;
+  // each 8-row chunk's pivots, multipliers and fresh right-hand side are
+  // loaded one chunk ahead (warps issue in order: a load consumed in the
+  // same chunk would stall the chain)
+  unsigned long long pw;
+  double lv[SPK_FW], nv;
+  auto load = [&](int j8, unsigned long long& pw_, double* lv_, double& nv_) {
+    const bool in = act && j8 < j1;
+    pw_ = in ? *reinterpret_cast<const unsigned long long*>(pv + j8) : 0ull;
+#pragma unroll
+    for (int i = 0; i < SPK_FW; ++i) {
+      const int d = (q - i) & 7;
+      lv_[i] = (in && d >= 1 && d <= kl) ? Lp[(size_t)(j8 + i) * lpad + d - 1] : 0.0;
+    }
+    nv_ = in ? fresh(j8 + SPK_FW + q) : 0.0;
+  };
+  load(j0, pw, lv, nv);
+  for (int j8 = j0; j8 < j1; j8 += SPK_FW) {
+    unsigned long long pw2;
+    double lv2[SPK_FW], nv2;
+    load(j8 + SPK_FW, pw2, lv2, nv2);
+#pragma unroll
+    for (int i = 0; i < SPK_FW; ++i) {
+      const int off = (int)((pw >> (8 * i)) & 0xff);
+      const int pl = (i + off) & 7;
+      const double bj = __shfl_sync(0xffffffffu, v, pl, 8);   // pivot row value = y_j
+      const double vo = __shfl_sync(0xffffffffu, v, i, 8);    // old row j value moves to the pivot row
+      v = (q == pl) ? vo : v;
+      v = fma(-lv[i], bj, v);
+      if (PASS == 2 && act && q == i && j8 + i < n) Yp[2 * (j8 + i)] = bj;
+      v = (q == i) ? nv : v;                                   // row j + 8 enters in row j's slot
+    }
+    pw = pw2;
+    nv = nv2;
+#pragma unroll
+    for (int i = 0; i < SPK_FW; ++i) lv[i] = lv2[i];
+  }
+  // lane q now holds row j1 + q: the outflow is rows j1 .. j1 + 6
+  if (PASS == 1 && act && q < SPK_FS) s.s0[(((size_t)p * s.nblk_f + k + 1) * 2 + c) * SPK_FW + q] = v;
+}
+
+// ---------------------------------------------------------------------------
+// back substitution of one block, one CTA of two warps (real and imaginary
+// part) per block, with the scaled U columns (U_{j-t,j} / U_jj) streamed chunk by
+// chunk into a shared-memory ring.  Lane l holds the row congruent to l mod 32
+// of rows j - 31 .. j.  PASS 1 (blocks 1 .. nblk - 1, or the one block): the
+// guessed inflow, zero for the last block, writes the outflow (and b for the
+// last block, which has no inflow); PASS 2 (blocks 0 .. nblk - 2): the true
+// inflow, writes b = U_jj x for the block's rows.
+// ---------------------------------------------------------------------------
+constexpr int SPK_RING = 2;           // U chunks in flight per block (16 KB: about 11 blocks per SM)
+template <int PASS>
+__global__ void __launch_bounds__(64, 10) k_spike_bwd(LaneArgs s) {
+  __shared__ __align__(128) double Uring[SPK_RING * SPK_CHUNK * SPK_BW];
+  __shared__ __align__(8) uint64_t bar[SPK_RING];
+  __shared__ int abort_flag;
+  // PASS 1 skips block 0 (its outflow has no use); PASS 2 the last block,
+  // final after PASS 1
+  const int k0 = (PASS == 1 && s.nblk > 1) ? 1 : 0;
+  const int nk = s.nblk > 1 ? s.nblk - 1 : 1;
+  const int p = blockIdx.x / nk, k = k0 + (blockIdx.x - p * nk);
+  const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;
+  const int m = s.m, j0 = k * m, j1 = j0 + m, n = s.n, kuu = s.kuu;
+  const int nch = m / SPK_CHUNK, chi = j1 / SPK_CHUNK - 1;     // chunks chi, chi - 1, ..., chi - nch + 1
+  const double* Usrc = s.U + (size_t)p * s.npad * s.upad;
+  const uint32_t ubytes = SPK_CHUNK * SPK_BW * 8;
+  auto issue = [&](int q) {                       // q-th chunk of the block in backward order
+    const int sl = q % SPK_RING;
+    mbar_expect_tx(&bar[sl], ubytes);
+    bulk_g2s(Uring + (size_t)sl * SPK_CHUNK * SPK_BW, Usrc + (size_t)(chi - q) * SPK_CHUNK * s.upad, ubytes,
+             &bar[sl]);
+  };
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int sl = 0; sl < SPK_RING; ++sl) mbar_init(&bar[sl], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int q = 0; q < min(nch, SPK_RING); ++q) issue(q);
+  }
+  __syncthreads();
+  const double* Yp = s.yg + (size_t)p * n * 2 + c;
+  auto yv = [&](int r) -> double { return (r >= j0 && r < n) ? Yp[2 * r] : 0.0; };
+  double w = yv(j1 - SPK_BW + lane);
+  const int first_in = SPK_BW - kuu;              // lanes first_in .. 31 hold the inflow rows
+  const size_t bidx = (((size_t)p * s.nblk + k) * 2 + c) * SPK_BW;
+  if (lane >= first_in) {
+    if (PASS == 2) w += s.uin[bidx + lane - first_in];
+    else if (k < s.nblk - 1) w += spike_guess(s, bidx + lane - first_in);
+  }
+  // lane l takes row jc - 32 + l when it owns column jc + l of the chunk
+  // at jc: nw holds that row, loaded one chunk ahead
+  double nw = yv(j1 - 2 * SPK_BW + lane);
+  double ws = w;   // shuffle source: w before the owner swaps in its next row (the
+                   // next column's owner is another lane, so the swap stays off the chain)
+  const bool store = PASS == 2 || k == s.nblk - 1;
+  double* Xp = reinterpret_cast<double*>(s.xg + (size_t)p * n) + c;
+  int done = 0;
+  bool ok = true;
+  for (int q = 0; q < nch; ++q) {
+    const int sl = q % SPK_RING;
+    const bool got = bounded_wait(&bar[sl], (q / SPK_RING) & 1);
+    if (!got) atomicOr(&abort_flag, 1);
+    __syncthreads();
+    if (abort_flag) { ok = false; break; }
+    done = q + 1;
+    if (threadIdx.x == 0 && q >= 1 && q - 1 + SPK_RING < nch) {
+      fence_proxy_async();
+      issue(q - 1 + SPK_RING);                    // both warps are past chunk q - 1
+    }
+    const double* Uc = Uring + (size_t)sl * SPK_CHUNK * SPK_BW;
+    const int jc = (chi - q) * SPK_CHUNK;
+    const double nxt = yv(jc - 2 * SPK_BW + lane);   // this lane's row of the next chunk
+    double xo = 0.0;
+#pragma unroll
+    for (int jj = SPK_CHUNK - 1; jj >= 0; --jj) {
+      const double bj = __shfl_sync(0xffffffffu, ws, jj);
+      const int t = (jj - lane) & 31;
+      const double u = (t >= 1) ? Uc[jj * SPK_BW + t] : 0.0;
+      w = fma(-u, bj, w);
+      ws = w;
+      const bool own = lane == jj;
+      xo = own ? bj : xo;
+      w = own ? nw : w;
+    }
+    nw = nxt;
+    if (store && jc + lane < n) Xp[2 * (jc + lane)] = xo;
+  }
+  if (!ok) {
+    if (threadIdx.x == 0) {
+      raise_status(s.status, SP_ERR_TIMEOUT, p);
+      const int issued = min(nch, done == 0 ? SPK_RING : done - 1 + SPK_RING);
+      for (int q = done; q < issued; ++q) bounded_wait(&bar[q % SPK_RING], (q / SPK_RING) & 1);
+    }
+    return;
+  }
+  // lane l holds row j0 - 32 + l: the outflow is rows j0 - kuu .. j0 - 1
+  if (PASS == 1 && k > 0 && lane >= first_in) s.o0[bidx + lane - first_in] = w;
+}
+
+cudaError_t launch_spike_forward(cudaStream_t st, const LaneArgs& s, int pass) {
+  if (!spike_supported(s.kl, s.kuu, s.npad, s.nblk) || s.nblk_f < 1 || s.m_f * s.nblk_f != s.npad || s.m_f % SPK_FW)
+    return cudaErrorInvalidValue;
+  const int T = 128;
+  const long long lanes = (long long)s.P * (pass == 1 ? s.nblk_f - 1 : s.nblk_f) * 2 * SPK_FW;
+  if (lanes == 0) return cudaSuccess;
+  if (pass == 1) k_spike_fwd<1><<<(unsigned)((lanes + T - 1) / T), T, 0, st>>>(s);
+  else k_spike_fwd<2><<<(unsigned)((lanes + T - 1) / T), T, 0, st>>>(s);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_spike_backward(cudaStream_t st, const LaneArgs& s, int pass) {
+  if (!spike_bwd_supported(s.kuu, s.npad, s.nblk) || s.m * s.nblk != s.npad || s.upad != SPK_BW)
+    return cudaErrorInvalidValue;
+  const unsigned grid = s.P * (s.nblk > 1 ? s.nblk - 1 : 1);
+  if (pass == 1) k_spike_bwd<1><<<grid, 64, 0, st>>>(s);
+  else if (s.nblk > 1) k_spike_bwd<2><<<grid, 64, 0, st>>>(s);
+  return cudaGetLastError();
 }
 
 bool spike_supported(int kl, int kuu, int npad, int nblk) {

@@ -8,7 +8,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
-from paper_1905_10388_gb300.solver import Context, FisherKPPSolver, QGInversion, RB3DSolver, RBSolver
+from paper_1905_10388_gb300.solver import Context, FisherKPPSolver, RBSolver, step_batched
 from gpu_util import rel_err
 
 pytestmark = pytest.mark.gpu
@@ -27,8 +27,8 @@ def _upload(s):
 
 
 @pytest.mark.parametrize("kind,kernels", [("window", ["k_pencil_solve"]), ("spike", ["k_pencil_split"]),
-                                          ("lanes", ["k_pencil_stage<1>", "k_lane_fwd<0>", "k_lane_bwd<0>",
-                                                     "k_pencil_stage<2>"])])
+                                          ("lanes", ["k_pencil_stage_wide<1>", "k_lane_fwd<0>", "k_lane_bwd<0>",
+                                                     "k_pencil_stage_wide<2>"])])
 def test_kernels_asked_for_by_name(ctx, kind, kernels):
     s = RBSolver(ctx, 64, 64, 1e6)
     s.set_solve_kernel(kind)
@@ -64,3 +64,67 @@ def test_row_blocks_come_before_whole_pencils(ctx, nz, blocks):
 def test_whole_row_kernel_by_pencils(ctx, nx, nz, kernel):
     d = (3, 2) if nx == 1024 else (4, 3) if nz % 3 == 0 else (2, 1)
     assert _upload(RBSolver(ctx, nx, nz, 1e6, precision="mixed", dealias=d)) == [kernel]
+
+
+PASSES = ["k_spike_fwd<1>", "k_spike_fwd_rec", "k_spike_fwd<2>", "k_spike_bwd<1>", "k_spike_bwd_rec", "k_spike_bwd<2>"]
+
+
+# one CTA per pencil where all are on the GPU at once and most of it is taken, or
+# the chains are short; else passes in launches of their own
+@pytest.mark.parametrize("nx,nz,d,passes", [
+    (64, 256, (3, 2), False), (64, 384, (2, 1), True), (64, 1024, (3, 2), True), (256, 512, (3, 2), False),
+    (256, 1024, (3, 2), True), (384, 96, (4, 3), False), (384, 192, (4, 3), True), (512, 256, (3, 2), False),
+    (512, 512, (3, 2), True), (768, 96, (4, 3), True), (1024, 256, (3, 2), True)])
+def test_partitioned_form_by_size(ctx, nx, nz, d, passes):
+    k = _upload(RBSolver(ctx, nx, nz, 1e6, precision="mixed", dealias=d))
+    assert k[1:-1] == PASSES if passes else k == ["k_pencil_split"]
+
+
+# (nx, nz, dealias, precision, blocks asked for): few long pencils, more than one
+# wave of CTAs, N_z = 1024 at two pencil counts, and block counts that one CTA's
+# shared memory does not hold
+@pytest.mark.parametrize("nx,nz,d,prec,blocks", [
+    (64, 384, (2, 1), "fp64", 0), (768, 48, (4, 3), "mixed", 11), (768, 96, (4, 3), "mixed", 0), (1024, 128, (3, 2), "mixed", 0),
+    (32, 1024, (3, 2), "fp64", 0), (32, 1024, (3, 2), "fp64", 112), (256, 1024, (3, 2), "mixed", 0)])
+def test_passes_equal_window_to_rounding(ctx, nx, nz, d, prec, blocks):
+    xi = np.random.default_rng(4).standard_normal((nz, nx))
+    out = []
+    for kind in ("window", "spike" if blocks else "auto"):
+        s = RBSolver(ctx, nx, nz, 1e6, scheme="SBDF2", precision=prec, dealias=d)
+        s.set_solve_kernel(kind)
+        if blocks and kind != "window":
+            s.set_spike_blocks(blocks)
+        s.factor(1e-4)
+        if kind != "window":
+            assert s.solve_kernels()[1:-1] == PASSES
+            assert s.spike_blocks() == blocks if blocks else s.spike_blocks() > 1
+        s.set_initial_state(xi, amplitude=1e-2)
+        s.step(4, graph=True)
+        s.sync()
+        out.append(s.get_state())
+    assert np.isfinite(out[0]).all()
+    for a, b in zip(*out):                         # the bars of the partitioned substitution elsewhere
+        assert rel_err(b, a) < (1e-11 if prec == "fp64" else 1e-5)
+
+
+def test_batch_of_long_problems_equals_them_alone_to_rounding(ctx):
+    """Two problems that run in passes alone, in one CTA per pencil together."""
+    def make():
+        out = []
+        for i, (nx, nz, d) in enumerate(((64, 384, (2, 1)), (32, 512, (3, 2)))):
+            s = RBSolver(ctx, nx, nz, 1e6, scheme="SBDF2", dealias=d)
+            s.factor(1e-4)
+            assert s.solve_kernels()[1:-1] == PASSES
+            s.set_initial_state(np.random.default_rng(i).standard_normal((nz, nx)), amplitude=1e-2)
+            out.append(s)
+        return out
+    alone, batch = make(), make()
+    for s in alone:
+        s.step(4)
+    step_batched(batch, 4)
+    ctx.sync_status()
+    for a, b in zip(alone, batch):
+        X, Y = a.get_state(), b.get_state()
+        assert np.isfinite(X).all()
+        for x, y in zip(X, Y):
+            assert rel_err(y, x) < 1e-11
