@@ -108,11 +108,15 @@ constexpr int SPLIT_MIN_ROWS = 96;
 // as long as their chains are short (64 x 256, 1792 rows: faster; 64 x 384, 2688
 // rows: 166 against 136; 192 pencils of 1344 rows 167 against 159).  A wide lower
 // band has no such passes forward: there one CTA wins wherever all fit (adjoint
-// step at 128 x 512: 1.83 ms against 2.12).
+// step at 128 x 512: 1.83 ms against 2.12) from the rows on at which its 32-lane
+// windows repay the second pass (us per eigenvalue iteration, one CTA against the
+// window kernel: 128 pencils of 224 rows 50 against 44, 448 rows 69 against 79; 256
+// pencils of 448 rows 100 against 86, 896 rows 154 against 155).
 inline bool split_serves(int P, int npad, bool wide, size_t smem) {
   const int per_sm = (P + GPU_SMS - 1) / GPU_SMS;
   if (P > SPLIT_MAX_PENCILS || smem > 227 * 1024 || per_sm * (smem + 1024) > 228 * 1024) return false;
-  return wide || 4 * P >= 3 * per_sm * GPU_SMS || npad * per_sm <= 2048;
+  if (wide) return npad >= (per_sm == 1 ? 384 : 512);
+  return 4 * P >= 3 * per_sm * GPU_SMS || npad * per_sm <= 2048;
 }
 bool spike_supported(int kl, int kuu, int npad, int nblk);
 bool spike_bwd_supported(int kuu, int npad, int nblk);

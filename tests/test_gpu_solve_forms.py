@@ -8,7 +8,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
-from paper_1905_10388_gb300.solver import Context, FisherKPPSolver, RBSolver, step_batched
+from paper_1905_10388_gb300.solver import Context, FisherKPPSolver, RBOnsetEVP, RBSolver, step_batched
 from gpu_util import rel_err
 
 pytestmark = pytest.mark.gpu
@@ -128,3 +128,11 @@ def test_batch_of_long_problems_equals_them_alone_to_rounding(ctx):
         assert np.isfinite(X).all()
         for x, y in zip(X, Y):
             assert rel_err(y, x) < 1e-11
+
+
+# kl = 8: 32-lane windows both ways
+@pytest.mark.parametrize("nx,nz,kernel", [(256, 32, "k_pencil_solve"), (256, 64, "k_pencil_split"),
+                                          (512, 64, "k_pencil_solve"), (512, 128, "k_pencil_split"),
+                                          (1024, 128, "k_pencil_solve_narrow")])
+def test_wide_lower_band_by_rows(ctx, nx, nz, kernel):
+    assert _upload(RBOnsetEVP(ctx, nx, nz, 2000.0)) == [kernel]
