@@ -10,6 +10,7 @@
 #include <cstring>
 #include <map>
 #include <memory>
+#include <queue>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -1090,6 +1091,7 @@ struct Batch {
   int max_ngz = 0, max_kl = 0, max_kuu = 0;
   size_t x_smem = 0, s_smem = 0;
   bool split = false;                        // every problem's solves in the partitioned kernel
+  bool pairs = false;                        // else: in the kernel of two pencils per CTA, or the window kernel
   bool fast = false;                         // every problem's transforms on compile-time lengths
   size_t z_smem = 0;
   int4 *d_wzb = nullptr, *d_wx = nullptr, *d_wzf = nullptr, *d_ws = nullptr;
@@ -1118,6 +1120,45 @@ cudaError_t upload_vec(T** d, const std::vector<T>& v) {
 }
 
 // Work lists in descending cost order (largest items first).
+// Time at which the last of `items`, longest first, ends on `slots` places.
+double last_end(const std::vector<double>& items, int slots) {
+  std::priority_queue<double, std::vector<double>, std::greater<double>> free;
+  double last = 0;
+  for (double d : items) {
+    double t = 0;
+    if ((int)free.size() >= slots) { t = free.top(); free.pop(); }
+    free.push(t + d);
+    last = std::max(last, t + d);
+  }
+  return last;
+}
+// Whole-row solves of a batch: pairs (pair.cu) or the window kernel.  A pencil's
+// time goes with its rows; against the window kernel, up to four CTAs per SM, its
+// chains are 1.18 times as long in the pair kernel alone in its CTA and 1.4
+// times with another, of which five fit (us per RK222 step, window and pairs:
+// 512 pencils of 896 rows 459 and 531, 1024 854 and 709; 1792 rows, 640 pencils
+// 1508 and 1097, 1024 1641 and 1920, 2048 3185 and 3045; 704 of 448 to 1792 rows
+// 799 and 931).
+bool batch_in_pairs(const std::vector<Problem*>& ps, int pencils) {
+  std::vector<std::pair<int, int>> rows;          // (rows, pencils)
+  size_t window = 0, pair = 0;
+  for (Problem* pr : ps) {
+    rows.push_back({pr->npad, pr->P});
+    window = std::max(window, pencil_solve_smem(pr->npad, pr->lpad, pr->upad));
+    pair = std::max(pair, pencil_pair_smem(pr->npad, pencil_pair_per(pr->npad, pencils)));
+  }
+  std::sort(rows.rbegin(), rows.rend());
+  std::vector<double> w, p;
+  for (auto [n, count] : rows) {
+    const int per = pencil_pair_per(n, pencils);
+    w.insert(w.end(), count, n);
+    p.insert(p.end(), (count + per - 1) / per, per == 2 ? 1.4 * n : 1.18 * n);
+  }
+  std::sort(p.rbegin(), p.rend());
+  auto slots = [](size_t smem, int most) { return GPU_SMS * std::max(1, std::min(most, (int)(228 * 1024 / (smem + 1024)))); };
+  return last_end(p, slots(pair, 5)) < last_end(w, slots(window, 4));
+}
+
 sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::vector<int>& ids, int tile,
                       int parity, bool persist, Batch* b) {
   b->ids = ids;
@@ -1138,6 +1179,7 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
                pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false) <= 227 * 1024;
   }
   b->split = b->split && pencils <= SPLIT_MAX_PENCILS;
+  b->pairs = !b->split && batch_in_pairs(ps, pencils);
   for (size_t q = 0; q < ps.size(); ++q) {
     Problem* pr = ps[q];
     const int tl = b->fast ? z_cols_tile(pr->prec) : tile;
@@ -1148,7 +1190,7 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
     for (int e = 0; e < (int)pr->nl_eqs.size(); ++e)
       for (int t = 0; t < nt; ++t) zf.push_back({zc, make_int4((int)q, t, e, 0)});
     for (int r = 0; r < pr->Ngz; ++r) xr.push_back({(long long)pr->Ngx, make_int4((int)q, r, 0, 0)});
-    const int per = b->split ? 1 : pencil_pair_per(pr->npad, pencils);
+    const int per = b->pairs ? pencil_pair_per(pr->npad, pencils) : 1;
     for (int p = 0; p < pr->P; p += per)
       sv.push_back({(long long)pr->n, make_int4((int)q, p, std::min(per, pr->P - p), 0)});
     b->max_ngz = std::max(b->max_ngz, pr->Ngz);
@@ -1158,10 +1200,11 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
     b->x_smem = std::max(b->x_smem, b->fast ? x_rows_bytes(pr->prec, pr->Ngx, nf, ne)
                                             : x_smem_bytes(pr->prec, pr->Ngx, 7, nf, ne));
     b->z_smem = std::max(b->z_smem, z_cols_bytes(pr->prec, pr->Ngz));
+    const size_t window = pencil_solve_smem(pr->npad, pr->lpad, pr->upad);
     b->s_smem = std::max(b->s_smem, b->split ? pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false)
-                                             : pencil_pair_smem(pr->npad, per));
+                                    : b->pairs ? pencil_pair_smem(pr->npad, per) : window);
     // (longer pencils than a lone problem's window kernel takes stay refused)
-    if (!b->split && pencil_solve_smem(pr->npad, pr->lpad, pr->upad) > 227 * 1024) CK(cudaErrorInvalidValue);
+    if (!b->split && window > 227 * 1024) CK(cudaErrorInvalidValue);
   }
   auto finish = [](std::vector<std::pair<long long, int4>>& v) {
     std::stable_sort(v.begin(), v.end(), [](const auto& a, const auto& c) { return a.first > c.first; });
@@ -1252,7 +1295,8 @@ sp_status batch_step(sp_ctx* ctx, Batch* b, cudaStream_t s) {
       CK(launch_cheb_forward_batched(s, b->prec, b->tile, st.d_zf, b->d_wzf, b->nzf, b->max_ngz, q2));
     }
     if (b->split) CK(launch_pencil_split_batched(s, st.d_args, b->d_ws, b->ns, b->s_smem));
-    else CK(launch_pencil_pair_batched(s, st.d_args, b->d_ws, b->ns, b->max_kl, b->max_kuu, b->s_smem));
+    else if (b->pairs) CK(launch_pencil_pair_batched(s, st.d_args, b->d_ws, b->ns, b->max_kl, b->max_kuu, b->s_smem));
+    else CK(launch_pencil_solve_batched(s, st.d_args, b->d_ws, b->ns, b->max_kuu, b->s_smem));
   }
   return SP_OK;
 }

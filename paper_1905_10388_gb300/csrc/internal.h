@@ -313,6 +313,8 @@ size_t pencil_solve_smem(int npad, int lpad, int upad);
 // the kernel that solves P pencils in whole-row order, one launch
 enum WholeRowKernel { WHOLE_WINDOW, WHOLE_NARROW, WHOLE_PAIR };
 WholeRowKernel whole_row_kernel(int P, int npad, int lpad, int upad);
+cudaError_t launch_pencil_solve_batched(cudaStream_t s, const SolveArgs* args, const int4* work, int nwork, int max_kuu,
+                                        size_t smem);
 // partitioned pencil solve, one CTA per pencil (split.cu)
 cudaError_t launch_pencil_split(cudaStream_t s, const SolveArgs& a);
 cudaError_t launch_pencil_split_batched(cudaStream_t s, const SolveArgs* args, const int4* work, int nwork,

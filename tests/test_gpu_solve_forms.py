@@ -136,3 +136,26 @@ def test_batch_of_long_problems_equals_them_alone_to_rounding(ctx):
                                           (1024, 128, "k_pencil_solve_narrow")])
 def test_wide_lower_band_by_rows(ctx, nx, nz, kernel):
     assert _upload(RBOnsetEVP(ctx, nx, nz, 2000.0)) == [kernel]
+
+
+# whole-row batches: the window kernel (332 pencils), pencils alone in the pair
+# kernel (640 of 1792 rows), two to a CTA (1280 of 224 rows)
+@pytest.mark.parametrize("shapes", [[(512, 16), (128, 32), (24, 12)], [(256, 256)] * 5, [(64, 32)] * 40])
+def test_whole_row_batches_equal_window_bit_for_bit(ctx, shapes):
+    def make():
+        out = []
+        for i, (nx, nz) in enumerate(shapes):
+            s = RBSolver(ctx, nx, nz, 1e6, scheme="SBDF2", precision="mixed", dealias=(4, 3) if nx % 3 == 0 else (3, 2))
+            s.set_solve_kernel("window")
+            s.factor(1e-4)
+            s.set_initial_state(np.random.default_rng(i).standard_normal((nz, nx)), amplitude=1e-2)
+            out.append(s)
+        return out
+    alone, batch = make(), make()
+    for s in alone:
+        s.step(3)
+    step_batched(batch, 3)
+    ctx.sync_status()
+    for a, b in zip(alone, batch):
+        assert np.isfinite(a.get_state()).all()
+        assert np.array_equal(a.get_state(), b.get_state())
