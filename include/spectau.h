@@ -398,7 +398,7 @@ sp_status sp_set_solve_kernel(sp_ctx* ctx, int problem, int kind);
  * differences, so no rounding is amplified by cancellation.  Results equal
  * the whole-row-order substitution to rounding.  SP_SOLVE_AUTO picks it for
  * problems with fewer than 4096 pencils of at least 512 padded rows, and with
- * at most 304 pencils of at least 96, when kl + ku <= 31 and kl <= 7 (fewer than
+ * at most 304 pencils of at least 192, when kl + ku <= 31 and kl <= 7 (fewer than
  * 608 pencils: kl <= 30) and the block counts fit shared memory.
  * sp_set_spike_blocks sets nblk (0: automatic); SP_ERR_ARG if the padded rows
  * do not split into nblk whole 32-row chunks, SP_ERR_STATE once the problem is

@@ -1084,21 +1084,22 @@ sp_status adjoint_rhs(sp_ctx* ctx, Problem* pr, cudaStream_t s, const double2* x
 struct BatchStage {
   ZDesc* d_zb = nullptr; ZDesc* d_zf = nullptr; XDesc* d_x = nullptr; SolveArgs* d_args = nullptr;
 };
+constexpr int BATCH_COUNTERS = 6;
 struct Batch {
   std::vector<int> ids;
   int prec = 0, scheme = 0, nstage = 0, parity = 0;
   int tile = 8;
   int max_ngz = 0, max_kl = 0, max_kuu = 0;
-  size_t x_smem = 0, s_smem = 0;
-  bool split = false;                        // every problem's solves in the partitioned kernel
-  bool pairs = false;                        // else: in the kernel of two pencils per CTA, or the window kernel
-  bool fast = false;                         // every problem's transforms on compile-time lengths
-  size_t z_smem = 0;
-  int4 *d_wzb = nullptr, *d_wx = nullptr, *d_wzf = nullptr, *d_ws = nullptr;
-  int nzb = 0, nx = 0, nzf = 0, ns = 0;
+  // work lists, each problem's items in the one of the kernels it uses alone:
+  // transforms [1] on compile-time lengths or [0] not, solves [1] in the
+  // partitioned kernel or [0] in whole-row order (pairs: pair.cu, else band.cu)
+  size_t z_smem = 0, x_smem[2] = {0, 0}, s_smem[2] = {0, 0};
+  bool pairs = false;
+  int4 *d_wzb[2] = {}, *d_wx[2] = {}, *d_wzf[2] = {}, *d_ws[2] = {};
+  int nzb[2] = {}, nx[2] = {}, nzf[2] = {}, ns[2] = {};
   std::vector<BatchStage> stages;
   std::map<int, cudaGraphExec_t> graphs;     // by block length
-  // persistent launches: four work counters per stage, zeroed once per step
+  // persistent launches: BATCH_COUNTERS work counters per stage, zeroed once per step
   bool persist = false;
   int* d_queue = nullptr;
 };
@@ -1107,7 +1108,8 @@ namespace {
 
 void free_batch(Batch* b) {
   auto F = [](void* p) { if (p) cudaFree(p); };
-  F(b->d_wzb); F(b->d_wx); F(b->d_wzf); F(b->d_ws); F(b->d_queue);
+  for (int k = 0; k < 2; ++k) { F(b->d_wzb[k]); F(b->d_wx[k]); F(b->d_wzf[k]); F(b->d_ws[k]); }
+  F(b->d_queue);
   for (auto& st : b->stages) { F(st.d_zb); F(st.d_zf); F(st.d_x); F(st.d_args); }
   for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
 }
@@ -1167,57 +1169,63 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
   b->scheme = ps[0]->scheme;
   b->tile = tile;
   b->parity = parity;
-  std::vector<std::pair<long long, int4>> zb, xr, zf, sv;
-  // few pencils in all: the solves' latency counts, so each problem's
-  // partitioned form; more: the FP64 pipe does, so whole pencils
+  std::vector<std::pair<long long, int4>> zb[2], xr[2], zf[2], sv[2];
+  // few pencils in all: the solves' latency counts, so the partitioned form where
+  // a problem has one; more: the FP64 pipe does, so whole pencils
   int pencils = 0;
-  b->split = b->fast = true;
+  for (Problem* pr : ps) pencils += pr->P;
+  std::vector<bool> split;
+  std::vector<Problem*> whole;
   for (Problem* pr : ps) {
-    pencils += pr->P;
-    b->fast = b->fast && pr->rows_fast;
-    b->split = b->split && pr->spike && !pr->by_group && pr->kl <= 7 &&
-               pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false) <= 227 * 1024;
+    split.push_back(pencils <= SPLIT_MAX_PENCILS && pr->spike && !pr->by_group && pr->kl <= 7 &&
+                    pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false) <= 227 * 1024);
+    if (!split.back()) whole.push_back(pr);
   }
-  b->split = b->split && pencils <= SPLIT_MAX_PENCILS;
-  b->pairs = !b->split && batch_in_pairs(ps, pencils);
+  int whole_pencils = 0;
+  for (Problem* pr : whole) whole_pencils += pr->P;
+  b->pairs = batch_in_pairs(whole, whole_pencils);
   for (size_t q = 0; q < ps.size(); ++q) {
     Problem* pr = ps[q];
-    const int tl = b->fast ? z_cols_tile(pr->prec) : tile;
+    const int fast = pr->rows_fast;
+    const int tl = fast ? z_cols_tile(pr->prec) : tile;
     const int nt = (pr->P + tl - 1) / tl;
     const long long zc = (long long)pr->Ngz * 100 + pr->Nz;
-    for (int f = 0; f < (int)(b->fast ? pr->zvars.size() : pr->gfields.size()); ++f)
-      for (int t = 0; t < nt; ++t) zb.push_back({zc, make_int4((int)q, t, f, 0)});
+    for (int f = 0; f < (int)(fast ? pr->zvars.size() : pr->gfields.size()); ++f)
+      for (int t = 0; t < nt; ++t) zb[fast].push_back({zc, make_int4((int)q, t, f, 0)});
     for (int e = 0; e < (int)pr->nl_eqs.size(); ++e)
-      for (int t = 0; t < nt; ++t) zf.push_back({zc, make_int4((int)q, t, e, 0)});
-    for (int r = 0; r < pr->Ngz; ++r) xr.push_back({(long long)pr->Ngx, make_int4((int)q, r, 0, 0)});
-    const int per = b->pairs ? pencil_pair_per(pr->npad, pencils) : 1;
+      for (int t = 0; t < nt; ++t) zf[fast].push_back({zc, make_int4((int)q, t, e, 0)});
+    for (int r = 0; r < pr->Ngz; ++r) xr[fast].push_back({(long long)pr->Ngx, make_int4((int)q, r, 0, 0)});
+    const int nf = (int)pr->gfields.size(), ne = (int)pr->nl_eqs.size();
+    b->x_smem[fast] = std::max(b->x_smem[fast], fast ? x_rows_bytes(pr->prec, pr->Ngx, nf, ne)
+                                                     : x_smem_bytes(pr->prec, pr->Ngx, 7, nf, ne));
+    if (fast) b->z_smem = std::max(b->z_smem, z_cols_bytes(pr->prec, pr->Ngz));
+    else b->max_ngz = std::max(b->max_ngz, pr->Ngz);
+    const int per = !split[q] && b->pairs ? pencil_pair_per(pr->npad, whole_pencils) : 1;
     for (int p = 0; p < pr->P; p += per)
-      sv.push_back({(long long)pr->n, make_int4((int)q, p, std::min(per, pr->P - p), 0)});
-    b->max_ngz = std::max(b->max_ngz, pr->Ngz);
+      sv[split[q]].push_back({(long long)pr->n, make_int4((int)q, p, std::min(per, pr->P - p), 0)});
+    const size_t window = pencil_solve_smem(pr->npad, pr->lpad, pr->upad);
+    b->s_smem[split[q]] = std::max(
+        b->s_smem[split[q]], split[q] ? pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false)
+                             : b->pairs ? pencil_pair_smem(pr->npad, per) : window);
+    if (split[q]) continue;
     b->max_kl = std::max(b->max_kl, pr->kl);
     b->max_kuu = std::max(b->max_kuu, pr->kl + pr->ku);
-    const int nf = (int)pr->gfields.size(), ne = (int)pr->nl_eqs.size();
-    b->x_smem = std::max(b->x_smem, b->fast ? x_rows_bytes(pr->prec, pr->Ngx, nf, ne)
-                                            : x_smem_bytes(pr->prec, pr->Ngx, 7, nf, ne));
-    b->z_smem = std::max(b->z_smem, z_cols_bytes(pr->prec, pr->Ngz));
-    const size_t window = pencil_solve_smem(pr->npad, pr->lpad, pr->upad);
-    b->s_smem = std::max(b->s_smem, b->split ? pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, pr->kl + pr->ku, false)
-                                    : b->pairs ? pencil_pair_smem(pr->npad, per) : window);
     // (longer pencils than a lone problem's window kernel takes stay refused)
-    if (!b->split && window > 227 * 1024) CK(cudaErrorInvalidValue);
+    if (window > 227 * 1024) CK(cudaErrorInvalidValue);
   }
-  auto finish = [](std::vector<std::pair<long long, int4>>& v) {
-    std::stable_sort(v.begin(), v.end(), [](const auto& a, const auto& c) { return a.first > c.first; });
-    std::vector<int4> out;
-    for (auto& x : v) out.push_back(x.second);
-    return out;
-  };
-  auto wzb = finish(zb), wx = finish(xr), wzf = finish(zf), ws = finish(sv);
-  b->nzb = (int)wzb.size(); b->nx = (int)wx.size(); b->nzf = (int)wzf.size(); b->ns = (int)ws.size();
-  CK(upload_vec(&b->d_wzb, wzb));
-  CK(upload_vec(&b->d_wx, wx));
-  CK(upload_vec(&b->d_wzf, wzf));
-  CK(upload_vec(&b->d_ws, ws));
+  for (int k = 0; k < 2; ++k) {
+    auto put = [&](std::vector<std::pair<long long, int4>>& v, int4** d, int* n) {
+      std::stable_sort(v.begin(), v.end(), [](const auto& a, const auto& c) { return a.first > c.first; });
+      std::vector<int4> out;
+      for (auto& x : v) out.push_back(x.second);
+      *n = (int)out.size();
+      return upload_vec(d, out);
+    };
+    CK(put(zb[k], &b->d_wzb[k], &b->nzb[k]));
+    CK(put(xr[k], &b->d_wx[k], &b->nx[k]));
+    CK(put(zf[k], &b->d_wzf[k], &b->nzf[k]));
+    CK(put(sv[k], &b->d_ws[k], &b->ns[k]));
+  }
   // per-stage descriptor tables from the single-problem plans, planned at
   // the requested schedule phase (multistep schemes rotate their buffers)
   std::vector<std::vector<StagePlan>> plans;
@@ -1235,16 +1243,10 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
     std::vector<SolveArgs> av;
     for (size_t q = 0; q < ps.size(); ++q) {
       zbv.push_back(zdesc_backward(ps[q]));
-      if (!b->fast && ps[q]->rows_fast) {    // the run-time-length kernels' tables and fields
-        const TransformPlan& pz = ps[q]->plans.at({ps[q]->Nz, ps[q]->Ngz});
-        zbv.back().wq = ps[q]->prec ? pz.dct32 : pz.dct64;
-        zbv.back().f_var = ps[q]->d_gvar;
-      }
       xv.push_back(xdesc_rows(ps[q]));
       zfv.push_back(zdesc_forward(ps[q], plans[q][i].fc_out));
-      if (!b->fast) zfv.back().wq = zbv.back().wq;
       av.push_back(plans[q][i].args);
-      if (b->split) stage_lx(ps[q], av.back());
+      if (split[q]) stage_lx(ps[q], av.back());
       fill_f_halves(av.back());
     }
     BatchStage st;
@@ -1254,7 +1256,7 @@ sp_status build_batch(sp_ctx* ctx, const std::vector<Problem*>& ps, const std::v
     CK(upload_vec(&st.d_args, av));
     b->stages.push_back(st);
   }
-  CK(dalloc(&b->d_queue, (size_t)4 * std::max(1, b->nstage)));
+  CK(dalloc(&b->d_queue, (size_t)BATCH_COUNTERS * std::max(1, b->nstage)));
   return SP_OK;
 }
 
@@ -1276,27 +1278,30 @@ void drop_batches(sp_ctx* ctx, int problem) {
 }
 
 sp_status batch_step(sp_ctx* ctx, Batch* b, cudaStream_t s) {
-  if (b->persist) CK(cudaMemsetAsync(b->d_queue, 0, (size_t)4 * b->nstage * sizeof(int), s));
+  if (b->persist) CK(cudaMemsetAsync(b->d_queue, 0, (size_t)BATCH_COUNTERS * b->nstage * sizeof(int), s));
   for (int i = 0; i < b->nstage; ++i) {
     const BatchStage& st = b->stages[i];
-    int* q = b->persist ? b->d_queue + 4 * i : nullptr;
-    int *q1 = q ? q + 1 : nullptr, *q2 = q ? q + 2 : nullptr;
-    if (b->fast && b->prec) {
-      CK(launch_z_cols_batched<float>(s, false, st.d_zb, b->d_wzb, b->nzb, b->z_smem, q));
-      CK(launch_x_rows_batched<float>(s, st.d_x, b->d_wx, b->nx, b->x_smem, q1));
-      CK(launch_z_cols_batched<float>(s, true, st.d_zf, b->d_wzf, b->nzf, b->z_smem, q2));
-    } else if (b->fast) {
-      CK(launch_z_cols_batched<double>(s, false, st.d_zb, b->d_wzb, b->nzb, b->z_smem, q));
-      CK(launch_x_rows_batched<double>(s, st.d_x, b->d_wx, b->nx, b->x_smem, q1));
-      CK(launch_z_cols_batched<double>(s, true, st.d_zf, b->d_wzf, b->nzf, b->z_smem, q2));
-    } else {
-      CK(launch_cheb_backward_batched(s, b->prec, b->tile, st.d_zb, b->d_wzb, b->nzb, b->max_ngz, q));
-      CK(launch_fourier_rows_batched(s, b->prec, st.d_x, b->d_wx, b->nx, b->x_smem, q1));
-      CK(launch_cheb_forward_batched(s, b->prec, b->tile, st.d_zf, b->d_wzf, b->nzf, b->max_ngz, q2));
-    }
-    if (b->split) CK(launch_pencil_split_batched(s, st.d_args, b->d_ws, b->ns, b->s_smem));
-    else if (b->pairs) CK(launch_pencil_pair_batched(s, st.d_args, b->d_ws, b->ns, b->max_kl, b->max_kuu, b->s_smem));
-    else CK(launch_pencil_solve_batched(s, st.d_args, b->d_ws, b->ns, b->max_kuu, b->s_smem));
+    auto counter = [&](int k) { return b->persist ? b->d_queue + BATCH_COUNTERS * i + k : nullptr; };
+    auto z = [&](bool forward, const ZDesc* d, int4* const* w, const int* n, int k) -> cudaError_t {
+      cudaError_t e = cudaSuccess;
+      if (n[1])
+        e = b->prec ? launch_z_cols_batched<float>(s, forward, d, w[1], n[1], b->z_smem, counter(k))
+                    : launch_z_cols_batched<double>(s, forward, d, w[1], n[1], b->z_smem, counter(k));
+      if (e == cudaSuccess && n[0])
+        e = forward ? launch_cheb_forward_batched(s, b->prec, b->tile, d, w[0], n[0], b->max_ngz, counter(k + 1))
+                    : launch_cheb_backward_batched(s, b->prec, b->tile, d, w[0], n[0], b->max_ngz, counter(k + 1));
+      return e;
+    };
+    CK(z(false, st.d_zb, b->d_wzb, b->nzb, 0));
+    if (b->nx[1])
+      CK(b->prec ? launch_x_rows_batched<float>(s, st.d_x, b->d_wx[1], b->nx[1], b->x_smem[1], counter(2))
+                 : launch_x_rows_batched<double>(s, st.d_x, b->d_wx[1], b->nx[1], b->x_smem[1], counter(2)));
+    if (b->nx[0]) CK(launch_fourier_rows_batched(s, b->prec, st.d_x, b->d_wx[0], b->nx[0], b->x_smem[0], counter(3)));
+    CK(z(true, st.d_zf, b->d_wzf, b->nzf, 4));
+    if (b->ns[1]) CK(launch_pencil_split_batched(s, st.d_args, b->d_ws[1], b->ns[1], b->s_smem[1]));
+    if (b->ns[0])
+      CK(b->pairs ? launch_pencil_pair_batched(s, st.d_args, b->d_ws[0], b->ns[0], b->max_kl, b->max_kuu, b->s_smem[0])
+                  : launch_pencil_solve_batched(s, st.d_args, b->d_ws[0], b->ns[0], b->max_kuu, b->s_smem[0]));
   }
   return SP_OK;
 }
@@ -1901,8 +1906,8 @@ sp_status sp_step_batched(sp_ctx* ctx, int nproblems, const int* problem_ids, co
       float tot = 0;
       for (int rep = 0; rep < 4; ++rep) {
         CK(cudaEventRecord(e0, ctx->stream));
-        CK(launch_cheb_backward_batched(ctx->stream, b->prec, tile, sg.d_zb, b->d_wzb, b->nzb, b->max_ngz));
-        CK(launch_cheb_forward_batched(ctx->stream, b->prec, tile, sg.d_zf, b->d_wzf, b->nzf, b->max_ngz));
+        CK(launch_cheb_backward_batched(ctx->stream, b->prec, tile, sg.d_zb, b->d_wzb[0], b->nzb[0], b->max_ngz));
+        CK(launch_cheb_forward_batched(ctx->stream, b->prec, tile, sg.d_zf, b->d_wzf[0], b->nzf[0], b->max_ngz));
         CK(cudaEventRecord(e1, ctx->stream));
         CK(cudaEventSynchronize(e1));
         float ms;

@@ -96,9 +96,12 @@ constexpr int SPIKE_MAX_PENCILS = 4096;
 constexpr int LANE_SPLIT_PENCILS = 4 * GPU_SMS;
 constexpr int SPIKE_MIN_ROWS = 512;
 // Problems that have at most two CTAs per SM take one CTA per pencil from fewer
-// rows on (64 x 32, 224 rows: 16 RK222 steps 2.27 ms with the window kernel, 2.10 ms).
+// rows on (64 x 32, 224 rows: 16 RK222 steps 2.27 ms with the window kernel, 2.10
+// ms).  Below it gains nothing and the coupling matrices cost (us, window against
+// one CTA: 32 x 16, 128 rows, a solve 28 and 28, a factorization 265 and 291; 512
+// x 16 a solve 29 and 33).
 constexpr int SPLIT_MAX_PENCILS = 2 * GPU_SMS;
-constexpr int SPLIT_MIN_ROWS = 96;
+constexpr int SPLIT_MIN_ROWS = 192;
 // Whether one CTA of `smem` bytes per pencil beats passes in separate launches
 // (us per solve, one CTA against passes).  All pencils have to be on the GPU at
 // once (512 x 512: 592 against 373 with one CTA on each SM at a time).  Its time

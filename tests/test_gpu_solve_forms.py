@@ -159,3 +159,34 @@ def test_whole_row_batches_equal_window_bit_for_bit(ctx, shapes):
     for a, b in zip(alone, batch):
         assert np.isfinite(a.get_state()).all()
         assert np.array_equal(a.get_state(), b.get_state())
+
+
+@pytest.mark.parametrize("nx,nz,kernel", [(32, 16, "k_pencil_solve"), (512, 16, "k_pencil_solve"), (48, 24, "k_pencil_split"),
+                                          (512, 32, "k_pencil_split")])
+def test_short_pencils_keep_the_window_kernel(ctx, nx, nz, kernel):
+    assert _upload(RBSolver(ctx, nx, nz, 1e6, dealias=(4, 3) if nx % 3 == 0 else (3, 2))) == [kernel]
+
+
+def test_batch_of_unlike_kernels_equals_problems_alone_bit_for_bit(ctx):
+    """Partitioned (64 x 32) and whole-row solves (32 x 16), transforms on
+    compile-time lengths and, on 12 points in z, on run-time ones."""
+    def make():
+        out = [RBSolver(ctx, nx, nz, 1e5, scheme="RK222", precision="mixed") for nx, nz in ((64, 32), (32, 16))]
+        out.append(FisherKPPSolver(ctx, 64, 8, scheme="RK222", precision="mixed"))
+        for i, s in enumerate(out):
+            s.factor(1e-4)
+            rng = np.random.default_rng(i)
+            if i < 2:
+                s.set_initial_state(rng.standard_normal((s.Nz, s.Nx)), amplitude=1e-2)
+            else:
+                s.set_initial_state(rng.random((s.Nz, s.Nx)))
+        return out
+    alone, batch = make(), make()
+    assert [s.solve_kernels() for s in batch] == [["k_pencil_split"], ["k_pencil_solve"], ["k_pencil_solve"]]
+    for s in alone:
+        s.step(5)
+    step_batched(batch, 5)
+    ctx.sync_status()
+    for a, b in zip(alone, batch):
+        assert np.isfinite(a.get_state()).all()
+        assert np.array_equal(a.get_state(), b.get_state())
