@@ -197,6 +197,7 @@ __device__ __forceinline__ void lane_fwd_body(const LaneArgs& a, int g, int blk,
   }
   if (!ok) {
     ln_lost(bar, done, min(nch, done + LN_BUFS), p0, a.status, lane);
+    if (lane == 0) bounded_wait(bar + LN_BUFS, 0);   // the first rows' copy
     return;
   }
   if (PASS == 1 && act) {

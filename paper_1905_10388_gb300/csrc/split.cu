@@ -331,7 +331,10 @@ __device__ __forceinline__ void pencil_split_body(const SolveArgs& a, int p, dou
     const int k = q / FW;
     reinterpret_cast<double2*>(raw)[q] = reinterpret_cast<double2*>(B)[k * mf + q - k * FW];
   }
-  if (!bounded_wait(bar, 0)) raise_status(a.status, SP_ERR_TIMEOUT, p);   // (latched; the CTA ends as usual)
+  if (!bounded_wait(bar, 0)) {                   // (latched; the CTA ends as usual, its copies given time to land)
+    raise_status(a.status, SP_ERR_TIMEOUT, p);
+    bounded_wait(bar, 0);
+  }
   __syncthreads();
 
   // ---- forward
