@@ -354,15 +354,17 @@ static cudaError_t launch_fwd(cudaStream_t s, const LaneArgs& a) {
   const int G = (a.P + LANE_GROUP - 1) / LANE_GROUP;
   const int warps = G * (PASS == 0 ? 1 : (PASS == 1 ? a.nblk_f - 1 : a.nblk_f));
   const int wr = lane_window(a.kl), d = lane_fwd_doubles(wr, a.lrecs);
-  if (wr == 32) return lane_launch(k_lane_fwd<32, PASS>, s, a, warps, d);
-  return lane_launch(k_lane_fwd<64, PASS>, s, a, warps, d);
+  if constexpr (PASS == 0)                        // (row blocks: kl <= 7, 32 rows)
+    if (wr == 64) return lane_launch(k_lane_fwd<64, PASS>, s, a, warps, d);
+  return lane_launch(k_lane_fwd<32, PASS>, s, a, warps, d);
 }
 template <int PASS>
 static cudaError_t launch_bwd(cudaStream_t s, const LaneArgs& a) {
   const int G = (a.P + LANE_GROUP - 1) / LANE_GROUP;
   const int warps = G * ((PASS == 0 || a.nblk < 2) ? 1 : a.nblk - 1);
-  if (lane_ring(a.kuu) == 32) return lane_launch(k_lane_bwd<32, PASS>, s, a, warps, lane_bwd_doubles(32, a.urecs));
-  return lane_launch(k_lane_bwd<64, PASS>, s, a, warps, lane_bwd_doubles(64, a.urecs));
+  if constexpr (PASS == 0)                        // (row blocks: kuu <= 31, 32 rows)
+    if (lane_ring(a.kuu) == 64) return lane_launch(k_lane_bwd<64, PASS>, s, a, warps, lane_bwd_doubles(64, a.urecs));
+  return lane_launch(k_lane_bwd<32, PASS>, s, a, warps, lane_bwd_doubles(32, a.urecs));
 }
 
 cudaError_t launch_lane_forward(cudaStream_t s, const LaneArgs& a, int pass) {
@@ -395,12 +397,12 @@ __global__ void __launch_bounds__(256) k_lane_mask(int P, int n, int npad, int k
   bool l = false, u0 = false, u1 = false;
   for (int p = g * LANE_GROUP; p < p1; ++p) {
     const size_t col = (size_t)p * npad + j;
-    if (L && lane >= 1 && lane <= kl) l |= L[col * lpad + lane - 1] != 0.0;
+    if (lane >= 1 && lane <= kl) l |= L[col * lpad + lane - 1] != 0.0;
     if (lane <= kuu) u0 |= U[col * upad + lane] != 0.0;
     if (lane + 32 <= kuu) u1 |= U[col * upad + lane + 32] != 0.0;
   }
   const uint32_t lb = __ballot_sync(0xffffffffu, l);
-  if (L && lane == 0) lmask[(size_t)g * npad + j] = lb;
+  if (lane == 0) lmask[(size_t)g * npad + j] = lb;
   unsigned long long* um = umask + (size_t)g * npad;
   if (lane >= 1 && u0 && j - lane >= 0) atomicOr(um + j - lane, 1ull << lane);
   if (u1 && j - lane - 32 >= 0) atomicOr(um + j - lane - 32, 1ull << (lane + 32));
@@ -458,7 +460,6 @@ __global__ void __launch_bounds__(256) k_lane_pack(int P, int n, int npad, int l
   const int total = npad / LN_ROWS, c = j / LN_ROWS;
   const size_t row = (size_t)g * npad + j;
   const bool fwd = lane < 16;
-  if (fwd && !L) return;
   if (fwd) f.pg[row * LANE_GROUP + i] = (uint16_t)(((j + ((act && j < n) ? piv[(size_t)p * npad + j] : 0)) & (wr - 1)) * 256);
   const unsigned long long* um = f.umask + (size_t)g * npad;
   const uint32_t* lm = f.lmask + (size_t)g * npad;
@@ -497,8 +498,8 @@ void lane_list_free(LaneList& f) {
   f = LaneList{};
 }
 
-// Lists of the factor (L, piv, U) of P pencils; L null: the back
-// substitution's only.  Reads the entry counts back (synchronous).
+// Lists of the factor (L, piv, U) of P pencils.  Reads the entry counts back
+// (synchronous).
 cudaError_t lane_list_build(cudaStream_t s, int P, int n, int npad, int kl, int kuu, int lpad, int upad,
                             const double* L, const uint8_t* piv, const double* U, LaneList& f) {
   const int G = (P + LANE_GROUP - 1) / LANE_GROUP, total = npad / LN_ROWS;

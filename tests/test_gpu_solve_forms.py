@@ -8,7 +8,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
-from paper_1905_10388_gb300.solver import Context, FisherKPPSolver, RBOnsetEVP, RBSolver, step_batched
+from paper_1905_10388_gb300.solver import Context, FisherKPPSolver, QGInversion, RBOnsetEVP, RBSolver, step_batched
 from gpu_util import rel_err
 
 pytestmark = pytest.mark.gpu
@@ -190,3 +190,47 @@ def test_batch_of_unlike_kernels_equals_problems_alone_bit_for_bit(ctx):
     for a, b in zip(alone, batch):
         assert np.isfinite(a.get_state()).all()
         assert np.array_equal(a.get_state(), b.get_state())
+
+
+# the lane form's row blocks with bands wider than the reaction-diffusion one:
+# kl + ku = 29 (recurrence of four warps per chain), several block counts
+@pytest.mark.parametrize("nx,nz,d,blocks", [(1536, 96, (4, 3), 0), (1536, 96, (4, 3), 3), (1536, 96, (4, 3), 7),
+                                            (2048, 128, (1, 1), 0)])
+def test_lane_row_blocks_of_a_wide_band_equal_window_to_rounding(ctx, nx, nz, d, blocks):
+    xi = np.random.default_rng(4).standard_normal((nz, nx))
+    out = []
+    for kind in ("window", "auto"):
+        s = RBSolver(ctx, nx, nz, 1e6, scheme="SBDF2", precision="mixed", dealias=d)
+        s.set_solve_kernel(kind)
+        if blocks and kind == "auto":
+            s.set_spike_blocks(blocks)
+        s.factor(1e-4)
+        if kind == "auto":
+            assert {"k_lane_fwd<1>", "k_spike_bwd_rec"} <= set(s.solve_kernels())
+            assert s.spike_blocks() == blocks if blocks else s.spike_blocks() > 1
+        s.set_initial_state(xi, amplitude=1e-2)
+        s.step(4)
+        s.sync()
+        out.append(s.get_state())
+    assert np.isfinite(out[0]).all()
+    for a, b in zip(*out):
+        assert rel_err(b, a) < 1e-5
+
+
+# kl + ku = 9 (recurrence in 16 lanes per chain), FP64: the partitioned bar
+@pytest.mark.parametrize("nx,nz,blocks", [(2048, 256, 0), (2048, 512, 4)])
+def test_lane_row_blocks_of_an_inversion_equal_window_to_rounding(ctx, nx, nz, blocks):
+    rng = np.random.default_rng(8)
+    q = (rng.standard_normal((nx // 2, nz)) + 1j * rng.standard_normal((nx // 2, nz))) / (1 + np.arange(nz))
+    q[0] = q[0].real
+    out = []
+    for kind in ("window", "auto"):
+        s = QGInversion(ctx, nx, nz, [1.688, 0.75, 0.063])
+        s.set_solve_kernel(kind)
+        if blocks and kind == "auto":
+            s.set_spike_blocks(blocks)
+        out.append(s.invert(q))
+        if kind == "auto":
+            assert {"k_lane_fwd<1>", "k_spike_bwd_rec_narrow"} <= set(s.solve_kernels())
+    for a, b in zip(*out):
+        assert rel_err(b, a) < 1e-11
