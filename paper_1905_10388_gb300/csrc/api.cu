@@ -1550,6 +1550,8 @@ sp_status sp_set_bilinear_rhs(sp_ctx* ctx, int problem, int nterms, const int32_
 // pencil (and, per solve kernel, the lane layout or the partitioned
 // substitution's coupling matrices); synchronous.
 static sp_status factor_matrices(sp_ctx* ctx, Problem* pr, int nf, const double (*ab)[2]) {
+  // (no step on what a failure here leaves: freed lists, half a factor)
+  pr->factored = pr->lbvp_factored = false;
   CK(reset_spike_guess(pr, ctx->stream));
   const int ldab = 2 * pr->kl + pr->ku + 1;
   double* work = nullptr;

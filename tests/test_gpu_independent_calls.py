@@ -23,8 +23,8 @@ def ctx():
     c.close()
 
 
-# one CTA per pencil (128 and 512 rows) and row blocks of the lane form (512 rows)
-@pytest.mark.parametrize("nx,nz", [(64, 64), (512, 256), (2048, 256)])
+# one CTA per pencil (256 and 512 rows) and row blocks of the lane form (512 rows)
+@pytest.mark.parametrize("nx,nz", [(64, 128), (512, 256), (2048, 256)])
 def test_inversion_does_not_depend_on_the_one_before(ctx, nx, nz):
     rng = np.random.default_rng(5)
 

@@ -234,3 +234,28 @@ def test_lane_row_blocks_of_an_inversion_equal_window_to_rounding(ctx, nx, nz, b
             assert {"k_lane_fwd<1>", "k_spike_bwd_rec_narrow"} <= set(s.solve_kernels())
     for a, b in zip(*out):
         assert rel_err(b, a) < 1e-11
+
+
+@pytest.mark.parametrize("scheme,prec", [("RK222", "fp64"), ("SBDF2", "mixed")])
+def test_batch_beyond_304_pencils_equals_problems_alone_to_rounding(ctx, scheme, prec):
+    """On the automatic kernels: whole-row order together (320 pencils), one CTA
+    per pencil alone."""
+    def make():
+        out = []
+        for i, (nx, nz) in enumerate(((512, 32), (64, 64), (64, 32))):
+            s = RBSolver(ctx, nx, nz, 1e6, scheme=scheme, precision=prec)
+            s.factor(1e-4)
+            assert s.solve_kernels() == ["k_pencil_split"]
+            s.set_initial_state(np.random.default_rng(i).standard_normal((nz, nx)), amplitude=1e-2)
+            out.append(s)
+        return out
+    alone, batch = make(), make()
+    for s in alone:
+        s.step(5)
+    step_batched(batch, 5)
+    ctx.sync_status()
+    for a, b in zip(alone, batch):
+        X, Y = a.get_state(), b.get_state()
+        assert np.isfinite(X).all()
+        for x, y in zip(X, Y):                     # the bars of partitioned against whole-row solves
+            assert rel_err(y, x) < (1e-11 if prec == "fp64" else 1e-5)
