@@ -214,10 +214,16 @@ sp_status sp_step_graph(sp_ctx* ctx, int problem, double dt, int nsteps);
  * problem is listed (largest items first) in one grid, so small problems
  * fill the SMs left idle by large ones.  dts[q] must equal problem q's
  * factored dt.  Problems not yet in their steady schedule (fresh state,
- * SBDF2 first step) are first stepped one by one.  On the first call for a
- * set of ids the pencil tile of the z-transform kernels is autotuned (4, 8
- * or 16 columns per CTA, fastest kept; sp_batch_tile reports it).
- * use_graph = 1 records blocks of up to 16 batch steps in CUDA graphs and
+ * SBDF2 first step) are first stepped one by one.  Up to 304 pencils in all,
+ * each problem's transforms and solves run the arithmetic they run alone
+ * (unless it takes the partitioned solve's passes or its lane form alone), so
+ * its states equal its own steps bit for bit; with more, solves are in
+ * whole-row order, and states equal those of partitioned problems alone to
+ * rounding, bit for bit those of problems on SP_SOLVE_WINDOW.  The pencil tile of the
+ * z transforms is fixed by the precision (8 columns, FP64 4); for problems
+ * whose grid has no compile-time transform (fewer than 16 points) it is
+ * autotuned on the first call for a set of ids (4, 8 or 16, fastest kept).
+ * sp_batch_tile reports it.  use_graph = 1 records blocks of up to 16 batch steps in CUDA graphs and
  * replays them.  Asynchronous. */
 sp_status sp_step_batched(sp_ctx* ctx, int nproblems, const int* problem_ids, const double* dts,
                           int nsteps, int use_graph);
@@ -227,8 +233,8 @@ sp_status sp_batch_tile(sp_ctx* ctx, int nproblems, const int* problem_ids, int*
  * batched step: *persistent = 1 when the batched transform kernels run as
  * persistent grids (as many CTAs as the GPU holds at once) pulling (problem,
  * tile) work items from a device counter, largest items first; 0 when each
- * work item has a CTA of its own.  The batched pencil solves always take one
- * CTA per pencil.  The autotuner times one batch step of
+ * work item has a CTA of its own.  The batched pencil solves always take a
+ * CTA per item, of one pencil or two.  The autotuner times one batch step of
  * each shape (with the z tile it picked) on a saved copy of every buffer a
  * step writes, then restores them.  SP_ERR_STATE before that step. */
 sp_status sp_batch_persistent(sp_ctx* ctx, int nproblems, const int* problem_ids, int* persistent);
@@ -389,22 +395,26 @@ sp_status sp_set_solve_kernel(sp_ctx* ctx, int problem, int kind);
  * pencil solves are O(n) with the stored factor).  With fewer pencils than
  * the GPU has dependent-chain slots, each pencil's back substitution is cut
  * into nblk blocks of whole 32-row chunks (the forward one into blocks of 32
- * to 64 rows), substituted in parallel: a pass per block from guessed
+ * to 128 rows), substituted in parallel: a pass per block from guessed
  * inflows, a recurrence over blocks with coupling matrices computed at
- * sp_factor, then a pass with the true inflows.  The back substitution's
- * guesses are the true inflows of the problem's previous solve (zero after
- * sp_factor or sp_set_field, and for a guess that is not finite): exact for
- * any guess, and consecutive time-step solves then correct by small
- * differences, so no rounding is amplified by cancellation.  Results equal
- * the whole-row-order substitution to rounding.  SP_SOLVE_AUTO picks it for
- * problems with fewer than 4096 pencils of at least 512 padded rows, and with
- * at most 304 pencils of at least 192, when kl + ku <= 31 and kl <= 7 (fewer than
- * 608 pencils: kl <= 30) and the block counts fit shared memory.
- * sp_set_spike_blocks sets nblk (0: automatic); SP_ERR_ARG if the padded rows
- * do not split into nblk whole 32-row chunks, SP_ERR_STATE once the problem is
- * on the device (like sp_set_solve_kernel).  sp_get_spike_blocks returns the
- * block count in use (0: not partitioned, or the problem not yet on the
- * device). */
+ * sp_factor, then a pass with the true inflows.  In a run the back
+ * substitution's guesses are the true inflows of the problem's previous
+ * solve (zero after sp_factor or sp_set_field, and for a guess that is not
+ * finite): exact for any guess, and consecutive time-step solves then correct
+ * by small differences, so no rounding is amplified by cancellation.
+ * sp_solve_lbvp and sp_step_adjoint always start from zero: their results do
+ * not depend on the calls before.  Results equal the whole-row-order
+ * substitution to rounding.  SP_SOLVE_AUTO picks it for problems with fewer
+ * than 4096 pencils of at least 512 padded rows, and with at most 304 pencils
+ * of at least 192, when kl <= 7 and kl + ku <= 31; for kl of 8 to 30 with at
+ * most 304 pencils of at least 384 rows (512 beyond 152 pencils).  It runs as
+ * one kernel with a CTA per pencil where that serves (sp_get_solve_kernels
+ * says what runs), from 608 pencils on by lanes, else in launches of its own
+ * per pass.  sp_set_spike_blocks sets nblk (0: automatic); SP_ERR_ARG if the
+ * padded rows do not split into nblk whole 32-row chunks, SP_ERR_STATE once
+ * the problem is on the device (like sp_set_solve_kernel).
+ * sp_get_spike_blocks returns the block count in use (0: not partitioned, or
+ * the problem not yet on the device). */
 sp_status sp_set_spike_blocks(sp_ctx* ctx, int problem, int nblk);
 
 /* Chebyshev backward transform of the mixed form (Sec. "Chebyshev basis":

@@ -1,7 +1,7 @@
 // Host runtime behind the C ABI (include/spectau.h): problem objects,
 // validation, device tables, transform plans, factor/step orchestration,
 // CUDA-graph replay and launch timing.  No computation of the step happens
-// on the host; every stage is one of the kernels in band.cu / transforms.cu.
+// on the host; every stage is one of the kernels of this directory.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>

@@ -688,7 +688,8 @@ __global__ void __launch_bounds__(128, 4) k_pencil_solve_batched(const SolveArgs
   pencil_solve_body<RU, 0, 128, true>(args[w.x], w.y, smem_raw);
 }
 // right-hand-side assembly only (MODE 1) or epilogue only (MODE 2), around
-// the lane substitution: shared memory for B~ alone, several CTAs per SM
+// substitution in launches of its own: shared memory for B~ alone, several CTAs
+// per SM
 template <int MODE>
 __global__ void __launch_bounds__(128, 6) k_pencil_stage(SolveArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];

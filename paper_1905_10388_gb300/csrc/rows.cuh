@@ -2,7 +2,7 @@
 // side's x rows with the dealiased products, the y transforms and the
 // Chebyshev (z) transforms.  Conventions and data layouts as in
 // transforms.cu, whose run-time-length kernels serve the other transforms
-// (set-up, batches of uneven problems, adjoint) and lengths.
+// (set-up, CFL, adjoint) and lengths.
 //
 // Derivatives i k_x and i k_y commute with the transforms of the other axes:
 // z transforms run once per variable, y transforms once per variable and once
