@@ -9,16 +9,16 @@
 // immediate: at run-time lengths the index arithmetic alone was most of the
 // FP32 kernels' instructions.
 //
-// A twiddled butterfly multiplies its inputs once and then runs the plain DFT,
-// whose two-point steps with a constant root are four FMAs for E + w O and, in
-// FP64, whose pipe is the bound, two for E - w O = 2 E - (E + w O); FP32, bound by
-// other instructions, takes four for it, as exact as a product and a difference.
-// A twiddle at every level (two-point steps with the common factors w, w^2, w^4:
-// 72 FP64 instructions and 4 twiddle loads for radix 8 against 80 and 7) rounds
-// each element three times more: errors of the right-hand side against extended
-// precision 1.51e-15 (FP64) and 4.52e-7 (mixed) against 1.33e-15 and 4.29e-7 here,
-// geometric means over lengths of 48 to 768.  It was 5 % faster in FP64 (512 x
-// 256 RK222 step 754 against 795 us, mixed 415 against 417).
+// A twiddled butterfly multiplies each input once, half of them within the first
+// two-point steps: E + w O in four FMAs and, in FP64, whose pipe is the bound, E -
+// w O = 2 E - (E + w O) in two (FP32, bound by other instructions, takes four for
+// it, as exact as a product and a difference): 72 FP64 instructions for radix 8,
+// 80 with the products first.  Error of the right-hand side against extended
+// precision, FP64 and mixed, geometric means over lengths of 48 to 768, and an
+// FP64 512 x 256 RK222 step: here 1.37e-15, 4.30e-7, 770 us; products first
+// 1.33e-15, 4.29e-7, 796 us; a twiddle at each of the three levels (72
+// instructions, 4 twiddle loads for 7) 1.51e-15, 4.52e-7, 754 us; the run-time
+// kernels of transforms.cu 1.33e-15, 4.31e-7.
 //
 // Buffers are padded by one element every 128 bytes, so the first pass's
 // stride-R writes spread over the banks.
@@ -81,14 +81,16 @@ __device__ __forceinline__ void bfly(C<T> e, C<T> o, C<T> w, C<T>& p, C<T>& m) {
   }
 }
 
-// DFT of length R (a power of two) of a[0], a[S], a[2S], ...: constant roots, the
+// DFT of length R (a power of two) of elements I, I + S, I + 2 S, ...: the two-point
+// steps on the elements themselves by `leaf(i, j, p, m)`, which sets p, m to the
+// sum and difference of elements i and j, the others with constant roots, the
 // trivial ones as sums and differences.
-template <typename T, int SIGN, int R, int S>
+template <typename T, int SIGN, int R, int S, int I, typename LEAF>
 struct Dit {
-  static __device__ __forceinline__ void run(const C<T>* a, C<T>* out) {
+  static __device__ __forceinline__ void run(C<T>* out, const LEAF& leaf) {
     C<T> e[R / 2], o[R / 2];
-    Dit<T, SIGN, R / 2, 2 * S>::run(a, e);
-    Dit<T, SIGN, R / 2, 2 * S>::run(a + S, o);
+    Dit<T, SIGN, R / 2, 2 * S, I, LEAF>::run(e, leaf);
+    Dit<T, SIGN, R / 2, 2 * S, I + S, LEAF>::run(o, leaf);
 #pragma unroll
     for (int q = 0; q < R / 2; ++q) {
       if (q == 0) {
@@ -108,19 +110,29 @@ struct Dit {
     }
   }
 };
-template <typename T, int SIGN, int S>
-struct Dit<T, SIGN, 1, S> {
-  static __device__ __forceinline__ void run(const C<T>* a, C<T>* out) { out[0] = a[0]; }
+template <typename T, int SIGN, int S, int I, typename LEAF>
+struct Dit<T, SIGN, 2, S, I, LEAF> {
+  static __device__ __forceinline__ void run(C<T>* out, const LEAF& leaf) { leaf(I, I + S, out[0], out[1]); }
 };
-
-// The same of a[t] w^t; `at(t)` returns w^t.
+template <typename T, int SIGN, int R>
+__device__ __forceinline__ void dft_plain(const C<T>* a, C<T>* out) {
+  if constexpr (R == 1) {
+    out[0] = a[0];
+  } else {
+    auto leaf = [&](int i, int j, C<T>& p, C<T>& m) {
+      p = cadd<T>(a[i], a[j]);
+      m = csub<T>(a[i], a[j]);
+    };
+    Dit<T, SIGN, R, 1, 0, decltype(leaf)>::run(out, leaf);
+  }
+}
+// The DFT of a[t] w^t; `at(t)` returns w^t.
 template <typename T, int SIGN, int R, typename W>
 __device__ __forceinline__ void dft_twiddled(const C<T>* a, C<T>* out, const W& at) {
-  C<T> b[R];
-  b[0] = a[0];
-#pragma unroll
-  for (int t = 1; t < R; ++t) b[t] = cmul<T>(at(t), a[t]);
-  Dit<T, SIGN, R, 1>::run(b, out);
+  auto leaf = [&](int i, int j, C<T>& p, C<T>& m) {
+    bfly<T>(i == 0 ? a[0] : cmul<T>(at(i), a[i]), a[j], at(j), p, m);
+  };
+  Dit<T, SIGN, R, 1, 0, decltype(leaf)>::run(out, leaf);
 }
 
 // 3-point DFT: sums, differences and FMAs with -1/2 and sqrt(3)/2.  Z: an input
@@ -164,7 +176,7 @@ __device__ __forceinline__ void dft_first(const C<T>* a, C<T>* out) {
 #pragma unroll
     for (int k1 = 0; k1 < 3; ++k1) {
       C<T> o[H];
-      Dit<T, SIGN, H, 1>::run(b[k1], o);
+      dft_plain<T, SIGN, H>(b[k1], o);
 #pragma unroll
       for (int k2 = 0; k2 < H; ++k2) {
         // the k in [0, R) with H k = k1 H (mod 3 H) after the maps: k = k1 (H
@@ -175,7 +187,7 @@ __device__ __forceinline__ void dft_first(const C<T>* a, C<T>* out) {
       }
     }
   } else {
-    Dit<T, SIGN, R, 1>::run(a, out);
+    dft_plain<T, SIGN, R>(a, out);
   }
 }
 

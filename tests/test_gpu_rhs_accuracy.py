@@ -3,7 +3,7 @@ dealiasing") against an evaluation in extended precision, for FFT lengths of
 two and three passes with and without the factor three.
 
 A butterfly that multiplies an element by a twiddle at every level rounds it
-more often than one multiplication before plain butterflies does.  The plain
+more often than one that multiplies each input once.  The plain
 Stockham kernels (transforms.cu) have a mean error (geometric, over the sizes
 here) of 1.328e-15 in FP64 and 4.311e-7 in the mixed form; the right-hand side
 may be 4 % above that.  Level-by-level twiddles are 14 % and 5 % above it.
