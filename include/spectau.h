@@ -406,7 +406,8 @@ sp_status sp_set_solve_kernel(sp_ctx* ctx, int problem, int kind);
  * not depend on the calls before.  Results equal the whole-row-order
  * substitution to rounding.  SP_SOLVE_AUTO picks it for problems with fewer
  * than 4096 pencils of at least 512 padded rows, and with at most 304 pencils
- * of at least 192, when kl <= 7 and kl + ku <= 31; for kl of 8 to 30 with at
+ * of at least 192 (128 where kl + ku <= 16 and there are at most 152
+ * pencils), when kl <= 7 and kl + ku <= 31; for kl of 8 to 30 with at
  * most 304 pencils of at least 384 rows (512 beyond 152 pencils).  It runs as
  * one kernel with a CTA per pencil where that serves (sp_get_solve_kernels
  * says what runs), from 608 pencils on by lanes, else in launches of its own

@@ -577,7 +577,7 @@ sp_status upload_problem(sp_ctx* ctx, Problem* pr) {
     pr->spike = (by_name || (automatic && pr->npad >= SPIKE_MIN_ROWS)) && !wide && use(lane_blocks(pr->npad, pr->P));
   } else {
     pr->spike = (by_name || (automatic && (pr->npad >= SPIKE_MIN_ROWS ||
-                                           (pr->P <= SPLIT_MAX_PENCILS && pr->npad >= SPLIT_MIN_ROWS)))) &&
+                                           (pr->P <= SPLIT_MAX_PENCILS && pr->npad >= split_min_rows(pr->P, kuu))))) &&
                 use(split_blocks(pr->npad, pr->P, wide)) &&
                 split_serves(pr->P, pr->npad, wide, pencil_split_smem(pr->npad, pr->nblk, pr->nblk_f, kuu, wide));
     if (!pr->spike && !wide && (by_name || (automatic && pr->npad >= SPIKE_MIN_ROWS)))

@@ -9,16 +9,15 @@
 // immediate: at run-time lengths the index arithmetic alone was most of the
 // FP32 kernels' instructions.
 //
-// A twiddled butterfly multiplies each input once, half of them within the first
-// two-point steps: E + w O in four FMAs and, in FP64, whose pipe is the bound, E -
-// w O = 2 E - (E + w O) in two (FP32, bound by other instructions, takes four for
-// it, as exact as a product and a difference): 72 FP64 instructions for radix 8,
-// 80 with the products first.  Error of the right-hand side against extended
-// precision, FP64 and mixed, geometric means over lengths of 48 to 768, and an
-// FP64 512 x 256 RK222 step: here 1.37e-15, 4.30e-7, 770 us; products first
-// 1.33e-15, 4.29e-7, 796 us; a twiddle at each of the three levels (72
-// instructions, 4 twiddle loads for 7) 1.51e-15, 4.52e-7, 754 us; the run-time
-// kernels of transforms.cu 1.33e-15, 4.31e-7.
+// A twiddled butterfly multiplies each input once.  In FP64, whose pipe is the
+// bound, half of the products sit in the first two-point steps, E + w O in four
+// FMAs and E - w O = 2 E - (E + w O) in two: 72 instructions for radix 8 instead of
+// 80.  FP32 has no fewer instructions that way.  Error of the right-hand side
+// against extended precision, geometric means over lengths of 48 to 768, and an
+// FP64 512 x 256 RK222 step: FP64 here 1.37e-15 (770 us), products first 1.33e-15
+// (796 us), a twiddle at each of the three levels (72 instructions, 4 twiddle
+// loads for 7) 1.51e-15 (754 us), the run-time kernels of transforms.cu 1.33e-15;
+// FP32 here 4.29e-7, a twiddle at each level 4.52e-7, the run-time kernels 4.31e-7.
 //
 // Buffers are padded by one element every 128 bytes, so the first pass's
 // stride-R writes spread over the banks.
@@ -130,7 +129,14 @@ __device__ __forceinline__ void dft_plain(const C<T>* a, C<T>* out) {
 template <typename T, int SIGN, int R, typename W>
 __device__ __forceinline__ void dft_twiddled(const C<T>* a, C<T>* out, const W& at) {
   auto leaf = [&](int i, int j, C<T>& p, C<T>& m) {
-    bfly<T>(i == 0 ? a[0] : cmul<T>(at(i), a[i]), a[j], at(j), p, m);
+    const C<T> e = i == 0 ? a[0] : cmul<T>(at(i), a[i]);
+    if constexpr (sizeof(T) == 8) {
+      bfly<T>(e, a[j], at(j), p, m);
+    } else {
+      const C<T> o = cmul<T>(at(j), a[j]);
+      p = cadd<T>(e, o);
+      m = csub<T>(e, o);
+    }
   };
   Dit<T, SIGN, R, 1, 0, decltype(leaf)>::run(out, leaf);
 }

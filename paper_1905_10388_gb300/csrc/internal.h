@@ -96,12 +96,14 @@ constexpr int SPIKE_MAX_PENCILS = 4096;
 constexpr int LANE_SPLIT_PENCILS = 4 * GPU_SMS;
 constexpr int SPIKE_MIN_ROWS = 512;
 // Problems that have at most two CTAs per SM take one CTA per pencil from fewer
-// rows on (64 x 32, 224 rows: 16 RK222 steps 2.27 ms with the window kernel, 2.10
-// ms).  Below it gains nothing and the coupling matrices cost (us, window against
-// one CTA: 32 x 16, 128 rows, a solve 28 and 28, a factorization 265 and 291; 512
-// x 16 a solve 29 and 33).
+// rows on (us per RK222 step, window kernel and one CTA: 48 x 24, 192 rows, 108 and
+// 102; 384 x 24 155 and 147; 64 x 32, 224 rows, 16 steps 2.27 and 2.10 ms).  Below
+// it gains nothing and the coupling matrices cost (32 x 16, 128 rows: a step 84 and
+// 85, a factorization 163 and 188), but for narrow bands, whose back recurrence
+// is short, while every pencil has an SM of its own (Fisher-KPP, 128 rows: 32
+// pencils 65 and 63, 128 pencils 68 and 66, 256 pencils 72 and 74; 96 rows 82 and 86).
 constexpr int SPLIT_MAX_PENCILS = 2 * GPU_SMS;
-constexpr int SPLIT_MIN_ROWS = 192;
+inline int split_min_rows(int P, int kuu) { return kuu <= 16 && P <= GPU_SMS ? 128 : 192; }
 // Whether one CTA of `smem` bytes per pencil beats passes in separate launches
 // (us per solve, one CTA against passes).  All pencils have to be on the GPU at
 // once (512 x 512: 592 against 373 with one CTA on each SM at a time).  Its time

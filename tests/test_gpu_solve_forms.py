@@ -167,6 +167,12 @@ def test_short_pencils_keep_the_window_kernel(ctx, nx, nz, kernel):
     assert _upload(RBSolver(ctx, nx, nz, 1e6, dealias=(4, 3) if nx % 3 == 0 else (3, 2))) == [kernel]
 
 
+@pytest.mark.parametrize("nx,nz,kernel", [(96, 48, "k_pencil_solve"), (128, 64, "k_pencil_split"), (256, 64, "k_pencil_split"),
+                                          (512, 64, "k_pencil_solve"), (512, 128, "k_pencil_split")])
+def test_short_pencils_of_a_narrow_band(ctx, nx, nz, kernel):
+    assert _upload(FisherKPPSolver(ctx, nx, nz, dealias=(4, 3) if nx % 3 == 0 else (3, 2))) == [kernel]
+
+
 def test_batch_of_unlike_kernels_equals_problems_alone_bit_for_bit(ctx):
     """Partitioned (64 x 32) and whole-row solves (32 x 16), transforms on
     compile-time lengths and, on 12 points in z, on run-time ones."""
