@@ -16,10 +16,10 @@
 // instruction issue (57 % active, FMA pipe 20 %): a run-time length, a branch or
 // an address per element costs more than the arithmetic.  Per launch, the
 // run-time-length kernels before and these now: x rows 512 x 256 FP64 171 ->
-// 119 us (pipe 69 % busy, 82 % on the SMs with three of the 384 rows), FP32 28
-// -> 16; 3D 128 x 128 x 64 FP32 390 -> 160; Fisher-KPP 2048 x 1024 FP32 137 ->
-// 60; y of the 3D case 139 and 40 -> 64 and 20; z 512 x 256 FP64 76 and 40 -> 41
-// and 29.
+// 125 us (three of the 384 rows on some SMs, two on most), FP32 28 -> 17; 3D 128 x
+// 128 x 64 FP32 390 -> 163; Fisher-KPP 2048 x 1024 FP32 137 -> 72 (its radix-16
+// passes load 15 twiddles each); y of the 3D case 139 and 40 -> 66 and 21; z 512 x
+// 256 FP64 76 and 40 -> 43 and 30.
 #pragma once
 #include <algorithm>
 #include <type_traits>
